@@ -94,7 +94,7 @@ NLINV_API int nlinv_supported_size(int n);
 NLINV_API nlinv_status nlinv_default_params(nlinv_params* p, int n, int ncoils);
 
 /* Creates a context on the current CUDA device: validates *params, allocates the device workspace (about
- * 9 (1+J) n^2 complex values) and builds the transform tables.  stream is a cudaStream_t on which the context
+ * 8 (1+J) n^2 complex values) and builds the transform tables.  stream is a cudaStream_t on which the context
  * queues its work; NULL makes the context create (and later destroy) a non-blocking stream of its own, since the
  * legacy default stream cannot be captured into a graph.  On success *out owns the context.  Blocks until set-up
  * is done.  Errors: EINVAL (bad params, NULL out), ENOMEM (the workspace allocation failed; the environment
@@ -240,7 +240,7 @@ NLINV_API nlinv_status nlinv_reconstruct_batch(nlinv_batch* batch, int nframes, 
  * batch's stream, on the workspaces left by the last nlinv_reconstruct_batch (whose CG state it advances; every
  * frame's solve is first marked running, so that each kernel does its full work): each kernel is launched for all
  * grid sides, one side after another, reps times back to back between two events.  ms_out (HOST, 6 doubles) gets
- * the mean duration of one launch set, in the order of nlinv_profile_cg.  Waits for the stream.  Errors: EINVAL
+ * the mean duration of one launch set, in the order of nlinv_profile_cg (a batch runs six kernels an iteration).  Waits for the stream.  Errors: EINVAL
  * (reps < 1, NULL pointers, no reconstruction yet, fewer than two CG iterations), ECUDA. */
 NLINV_API nlinv_status nlinv_batch_profile_cg(nlinv_batch* batch, int reps, double* ms_out);
 
@@ -252,20 +252,22 @@ NLINV_API nlinv_status nlinv_batch_destroy(nlinv_batch* batch);
 
 /* Waits up to timeout_s seconds (< 0: no limit) for the context's queued work.  ETIMEOUT if it is still running,
  * EBREAKDOWN if a CG breakdown was flagged since the last check (the flag is then cleared), ECUDA on a CUDA
- * error or when a kernel's wait for its own asynchronous copies or tensor-core stage ran past its time limit (about
- * a second; the kernel then stopped waiting and its results are not valid). */
+ * error or when a kernel's wait for its own tensor-core stage ran past its time limit (about a second; the kernel then
+ * stopped waiting and its results are not valid). */
 NLINV_API nlinv_status nlinv_wait(nlinv_ctx* ctx, double timeout_s);
 
 /* Times the kernels of one CG iteration of Eq. 3 with CUDA events on the context's stream, on the workspace left
- * by the last nlinv_reconstruct (whose CG state it advances -- a solve that had stopped at its rounding floor is
- * marked running again, so that every kernel does its full work; x is not changed): each kernel is launched reps times
- * back to back between two events, so ms_out gets its steady-state launch duration (consecutive launches overlap
- * their ramp and drain, as the passes of a graph replay do; the first one and the CG step issue their loads of p, r and
- * dx after their wait here, since back to back each launch would read what the one before writes, while in a
- * reconstruction they issue them before).  With reps = 1 the six kernels run once each, in order.  ms_out (HOST, 6 doubles) receives the mean duration in milliseconds of, in order:
+ * by the last nlinv_reconstruct (whose CG state it advances -- the solve is marked as running with no rounding floor, so
+ * that every kernel does its full work; x is not changed): each kernel is launched reps times back to back between two
+ * events, so ms_out gets its steady-state launch duration (consecutive launches overlap their ramp and drain, as the
+ * passes of a graph replay do; the row update pass issues its loads of p and r after its wait here, since back to back
+ * each launch would read what the one before writes, while in a reconstruction it issues them before).  An iteration is
+ * four passes: a column pass [1], a row pass [2], a column pass [3] and a row update pass that does the work of [0], [4]
+ * and [5]; its duration is divided among those three in proportion to the vector planes each part moves (2 : 1 : 2), so
+ * the six entries add up to the iteration.  ms_out (HOST, 6 doubles) receives the mean duration in milliseconds of:
  *   [0] row pass  p = r + beta p, W^-1 (first axis)   [1] column pass  W^-1, C (products), FFT
  *   [2] row pass  PSF                                  [3] column pass  FFT^-1, C^H (channel products), FFT
- *   [4] row pass  W^-H + alpha p, Re<p, q>             [5] CG step  dx += alpha p, r -= alpha q, |r|^2
+ *   [4] row pass  W^-H + alpha p                       [5] CG step  dx += alpha p, r -= alpha q, |r|^2
  * Waits for the stream.  Errors: EINVAL (reps < 1, NULL pointers, no reconstruction yet), ECUDA. */
 NLINV_API nlinv_status nlinv_profile_cg(nlinv_ctx* ctx, int reps, double* ms_out);
 

@@ -18,6 +18,14 @@ template <int N1, int N2> void side_smem(MultiKernels& m) {
         std::max(m.col_smem[mode], col_smem(mode, S::N, NLV_COL_C, S::SM_LANE_COL, S::N / 2).total);
 }
 
+// the batches' CG passes (frames of a batch have the standard field of view)
+void add_batch_cg(MultiKernels& k) {
+  k.row[ROW_BCG_RHS] = (const void*)row_pass_multi<ROW_BCG_RHS, false>;
+  k.row_std[ROW_BCG_DIR] = (const void*)row_pass_multi<ROW_BCG_DIR, true>;
+  k.row_std[ROW_BCG_NORMAL] = (const void*)row_pass_multi<ROW_BCG_NORMAL, true>;
+  k.col_std[COL_BCG_DIR] = (const void*)col_pass_multi<COL_BCG_DIR, true>;
+}
+
 MultiKernels make_multi() {
   MultiKernels m{};
   m.row[ROW_W_IFFT] = (const void*)row_pass_multi<ROW_W_IFFT, false>;
@@ -27,7 +35,6 @@ MultiKernels make_multi() {
   m.row[ROW_P_IFFT] = (const void*)row_pass_multi<ROW_P_IFFT, false>;
   m.row[ROW_FFT_W_ADJ] = (const void*)row_pass_multi<ROW_FFT_W_ADJ, false>;
   m.row[ROW_FFT_W_NORMAL] = (const void*)row_pass_multi<ROW_FFT_W_NORMAL, false>;
-  m.row[ROW_FFT_W_RHS] = (const void*)row_pass_multi<ROW_FFT_W_RHS, false>;
   m.col[COL_IFFT_C] = (const void*)col_pass_multi<COL_IFFT_C, false>;
   m.col[COL_PROD_FFT] = (const void*)col_pass_multi<COL_PROD_FFT, false>;
   m.col[COL_SIM_FFT] = (const void*)col_pass_multi<COL_SIM_FFT, false>;
@@ -37,6 +44,7 @@ MultiKernels make_multi() {
   m.row_std[ROW_PSF] = (const void*)row_pass_multi<ROW_PSF, true>;
   m.row_std[ROW_FFT_W_NORMAL] = (const void*)row_pass_multi<ROW_FFT_W_NORMAL, true>;
   m.col_std[COL_IFFT_PROD_FFT] = (const void*)col_pass_multi<COL_IFFT_PROD_FFT, true>;
+  add_batch_cg(m);
   side_smem<8, 16>(m);
   side_smem<12, 16>(m);
   side_smem<16, 16>(m);

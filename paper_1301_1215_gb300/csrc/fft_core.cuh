@@ -243,9 +243,13 @@ struct NoTc {
 // as one block-wide tensor-core contraction instead (every thread takes part; threads without data pass zeros).
 // TRAIL = false drops the closing barrier (CUDA-core stages only): for the last exchange of a pass, when every
 // later write to the exchange area comes after another block-wide barrier (the next round's or work item's).
-template <int P1, int P2, int D, int E, class TC = NoTc, bool TRAIL = true>
+// mid() runs between the shared-memory writes and the barrier of the exchange (loads to overlap with it).
+struct NoMid {
+  __device__ __forceinline__ void operator()() const {}
+};
+template <int P1, int P2, int D, int E, class TC = NoTc, bool TRAIL = true, class Mid = NoMid>
 __device__ __forceinline__ void fft_AtoB2(float2 (&v)[E], float2* sm_in, int in_idx, bool in_ok, float2* sm_out,
-                                          int out_idx, bool out_ok, const float2* tw, TC* tc = nullptr) {
+                                          int out_idx, bool out_ok, const float2* tw, TC* tc = nullptr, Mid mid = Mid()) {
   constexpr int S = P1 + 1;
   constexpr bool tc1 = TC::enabled && P2 == 16;
   constexpr bool tc3 = TC::enabled && P1 == 16;
@@ -259,6 +263,7 @@ __device__ __forceinline__ void fft_AtoB2(float2 (&v)[E], float2* sm_in, int in_
       sm_in[k2 * S + in_idx] = (k2 == 0) ? v[k2] : cmul(v[k2], w);
     });
   }
+  mid();
   __syncthreads();
   if (out_ok) {
     static_for<P1>([&](auto nc) { constexpr int n1 = decltype(nc)::value; v[n1] = sm_out[out_idx * S + n1]; });

@@ -9,6 +9,7 @@
 //
 // Vectors of the unknown x = (rho, chat_1 .. chat_J) hold 1 + J planes: plane 0 is rho, planes 1..J chat_j.
 #pragma once
+#include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
 #include "fft_core.cuh"
@@ -26,27 +27,35 @@ enum Reduce : int {
 constexpr int kMaxNewton = 64;
 
 // Scalars of the CG and Newton iterations, kept in device memory (FP64).
+// The values that one launch writes while its other blocks still read the value of the iteration before have two
+// slots, indexed by the parity of the CG iteration.
 struct Scalars {
-  double rr;                     // |r|^2 of the current CG residual (numerator of alpha)
+  double rr[2];                  // |r_i|^2 of iteration i in slot i & 1 (batches: slot 0)
   double rr0;                    // |b|^2 of the current CG solve (the reference of the rounding floor)
-  double rr_prev;                // |r|^2 of the previous CG residual (denominator of the next beta)
-  double alpha;                  // CG step length
+  double rr_prev;                // batches: |r|^2 of the previous CG residual (denominator of the next beta)
+  double alpha;                  // batches: CG step length
   double beta;                   // CG direction update
   double pq;                     // last Re<p, A p>
+  float step[2];                 // CG step length a_i of iteration i in slot i & 1, as the FP32 updates use it
+  float beta_f;                  // beta likewise
   double last;                   // result of a RED_NONE reduction
   double resid[kMaxNewton + 1];  // |y - F x_n| per Newton step
-  int cg_stop[kMaxNewton];       // per Newton step: the CG iteration that reached the rounding floor, -1 if none
-  int flags;                     // bit 0: CG breakdown (a non-finite |r|^2 or Re<p, A p>);
-                                 // bit 1: the current CG solve has reached the rounding floor (latched)
+  int cg_stop[kMaxNewton + 1];   // per Newton step: the CG iteration that reached the rounding floor, -1 if none
+                                 // (the last entry: the solve of the timing calls)
+  int flags;                     // bit 0: CG breakdown (a non-finite |r|^2 or Re<p, A p>)
   unsigned ticket;               // completion counter of the last-block reduction
 };
 
 constexpr int kFlagBreakdown = 1;
-constexpr int kFlagCgStopped = 2;
 // Rounding floor of CG: the solve stops once |r|^2 <= kCgFloor2 |b|^2, i.e. |r| at the FP32 unit roundoff 2^-24
 // relative to |b| (further iterations cannot improve a single-precision solution; left to run, the recursive
 // residual decays into the FP32 denormal range, where the step lengths lose their precision).
 constexpr double kCgFloor2 = 0x1p-48;
+
+// An unevaluated sum of two floats (see pair_add).
+struct Pair {
+  float h, l;
+};
 
 struct KArgs {
   int N, J, f, Wc;          // grid side, coils, half-width of Omega, compact width 2f
@@ -55,7 +64,6 @@ struct KArgs {
   int rho_per_cta;          // row passes with a rho part: consecutive rho-plane pixels handled by one block
   const float* wtab;        // Sobolev weight w(k) = (1 + a |k|^2)^(-l/2), N x N natural order
   float alpha;              // alpha_n of Eq. 3 for the normal operator and the right-hand side
-  int pupd;                 // CG passes: first form p = r + beta p (beta from Scalars) and write it back
   const float2* src;        // main input planes
   float2* dst;              // main output planes
   const float2* rho;        // rho of the linearisation point (natural N x N)
@@ -69,31 +77,38 @@ struct KArgs {
   const float2* x;          // Newton iterate, (1+J) planes
   const float2* xref;       // regularisation centre, (1+J) planes
   float2* r;                // CG residual, (1+J) planes
-  float2* pout;             // CG direction written by the right-hand side pass
   float2* dx;               // CG solution, (1+J) planes
+  float2* U;                // CG direction pass: W^-1 p on Omega, compact J x Wc x Wc, carried from iteration to iteration
   const float2* twA;        // twiddles of the split (N1, N2)
   const float2* twB;        // twiddles of the split (N2, N1)
   double* partials;         // one double per block
   Scalars* sc;
   int reduce;               // Reduce
-  int slot;                 // RED_RESID index; RED_RR_INIT and the CG step: the Newton step
-  int iter;                 // CG step: index of the CG iteration
-  const float2* q;          // CG step: A p
-  long n2;                  // vector passes: number of float4 (two complex values each)
-  // Re<p, A p> without a last-block tail: the normal-operator pass of the CG iteration only writes one FP64
-  // partial per block into pq_part; the CG step, its one consumer, adds the n_pq partials itself to form alpha.
+  int slot;                 // RED_RESID index; RED_RR_INIT and the CG passes: the Newton step
+  int iter;                 // CG passes: index of the CG iteration; cg_finish: number of scheduled iterations
+  int last;                 // CG update pass: the last scheduled iteration (its row transform would not be read)
+  int scalars;              // DF^H column pass of a CG iteration: one more block forms the step length (cg_decide)
+  const float2* q;          // vector passes: second operand; batch CG step: A p
+  float2* pout;             // batches: CG direction written by the right-hand side pass
+  // Batches: the normal-operator pass writes one FP64 partial of Re<p, A p> per block into pq_part (the CG step adds
+  // the n_pq partials to form alpha), the CG step one of |r|^2 into brr_part (the first pass of the next iteration adds
+  // the n_rr partials to form beta; NULL: beta from Scalars).
   double* pq_part;
   int n_pq;
-  // |r|^2 likewise: the CG step writes one partial per block into rr_part, and the first pass of the next CG
-  // iteration (its one consumer) adds the n_rr partials to form beta.  rr_part = NULL: beta from Scalars.
-  double* rr_part;
+  double* brr_part;
+  long n2;                  // vector passes: number of float4 (two complex values each)
+  // Sums without a last-block tail: a pass writes one partial per block and a later launch adds them.
+  Pair* dd_part;            // PSF pass: partials of |P FFT(...)|^2 = |DF p|^2 (n_dd of them)
+  int n_dd;
+  Pair* rr_part;            // CG update pass: partials of |r|^2, then of Re<r, p>, then of |p|^2 (n_rr of each)
   int n_rr;
   float coef;               // vector passes: second coefficient of out = alpha X + coef Y
   const void* tcB;          // tensor-core passes: the B tiles of the radix-16 DFT stage (tc_dft.cuh)
-  int cgskip;               // a launch of the CG iteration: it returns at once when the solve has stopped
-                            // (kCgSkipAfterWait, kCgSkipEarly: see cg_flags_early)
-  int src_early;            // inputs written two or more launches back, read before the dependent-launch wait:
-                            // the first CG pass's p (its first round's main loads), the CG step's r, dx and p
+  int skip;                 // a launch of the CG iteration: it returns at once when the solve stopped before CG
+                            // iteration `skip` (0: never; see cg_stop_early)
+  int skip_after;           // the stop is read after the dependent-launch wait (the CG update pass)
+  int src_early;            // CG update pass: its rows of p, written two or more launches back, are staged before the
+                            // dependent-launch wait
 };
 
 // ------------------------------------------------------------------------------- dependent launches ----
@@ -106,38 +121,34 @@ __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// True for a pass of the CG iteration whose solve has stopped at its rounding floor (Scalars::flags, latched by the
-// CG step): the pass then skips its work -- the stopped solve's remaining iterations are empty steps (the dx they
-// would leave is the one already there).  Only the CG step writes the flag, and every pass starts after the CG step
-// before it has completed (dependent-launch wait), so all threads of a pass read the same value: each reads it
-// itself, with no barrier.  (The CG step takes its own decision block-wide, inside cg_step_body.)
+// A pass of CG iteration i whose solve has stopped (Scalars::cg_stop) skips its work: the remaining iterations of a
+// stopped solve are empty steps (the dx they would leave is the one already there).  Two passes of iteration i may
+// record the stop, the direction pass and the DF^H column pass, while other blocks of theirs, or early blocks of the
+// pass after, read it; what they record is i.  So the first three passes of an iteration skip for a stop before i
+// (KArgs::skip = i) and take no notice of a stop at i -- what they then compute is not read --, and the update pass,
+// after its wait, skips for a stop at i as well (skip = i + 1): all threads of a launch always decide alike.
+//
+// What a kernel may read before its wait: a kernel is scheduled only once every block of the kernel before it has
+// passed its own wait (pdl_enter: wait, then launch_dependents), i.e. once the kernel two launches back has completed,
+// so anything written two or more launches back (or before the stream reached the library's first kernel) is in
+// place.  A stop before iteration i was recorded at least two launches before each pass of iteration i, so the first
+// three passes read it before their wait, overlapping the kernel before.
+constexpr int kNoStop = -1;      // as unsigned: after every iteration
+__device__ __forceinline__ int cg_stop_early(const KArgs& A) {
+  return A.skip > 0 && !A.skip_after ? *(volatile const int*)&A.sc->cg_stop[A.slot] : kNoStop;
+}
 __device__ __forceinline__ bool cg_stopped(const KArgs& A) {
-  return A.cgskip && (*(volatile const int*)&A.sc->flags & kFlagCgStopped) != 0;
+  return A.skip > 0 && (unsigned)*(volatile const int*)&A.sc->cg_stop[A.slot] < (unsigned)A.skip;
 }
-
-// cgskip values.  kCgSkipEarly marks a pass whose flag may be read before its dependent-launch wait, so that the
-// read overlaps the kernel before it instead of delaying this pass's first loads.  What a kernel may read before
-// its wait: a kernel is scheduled only once every block of the kernel before it has passed its own wait (pdl_enter:
-// wait, then launch_dependents), i.e. once the kernel two launches back has completed, so anything written two or
-// more launches back (or before the stream reached the library's first kernel) is in place.  For the second to
-// fifth passes of the CG iteration the flag's writer (the previous CG step) is two or more launches back; for the
-// first pass it is the kernel just before.
-constexpr int kCgSkipAfterWait = 1, kCgSkipEarly = 2;
-__device__ __forceinline__ int cg_flags_early(const KArgs& A) {
-  return A.cgskip == kCgSkipEarly ? *(volatile const int*)&A.sc->flags : 0;
-}
-// The stop test of a single-frame pass, given what cg_flags_early read before the wait.
-__device__ __forceinline__ bool cg_stopped_after(const KArgs& A, int early_flags) {
-  return A.cgskip == kCgSkipEarly ? (early_flags & kFlagCgStopped) != 0 : cg_stopped(A);
+// The stop test of a single-frame pass, given what cg_stop_early read before the wait.
+__device__ __forceinline__ bool cg_stopped_after(const KArgs& A, int early_stop) {
+  return A.skip_after ? cg_stopped(A) : (unsigned)early_stop < (unsigned)A.skip;
 }
 
 // ------------------------------------------------------------------------------------------- geometry ----
 __device__ __forceinline__ bool in_omega(int e, int N, int f) { return e < f || e >= N - f; }
 __device__ __forceinline__ int to_compact(int e, int N, int f) { return e < f ? e : e - (N - 2 * f); }
 __device__ __forceinline__ int to_natural(int cc, int N, int f) { return cc < f ? cc : cc + (N - 2 * f); }
-
-// beta of the pending direction update p = r + beta p (CG, Table 1)
-__device__ __forceinline__ float cg_beta(const KArgs& A) { return (float)A.sc->beta; }
 
 // ----------------------------------------------------------------------------------------- reductions ----
 // Butterfly sum over the lanes of this warp that exist: lanes 0..cnt-1 (a block's last warp may be partial, and a
@@ -180,14 +191,73 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   return s;
 }
 
+// Sums over the threads and blocks of a CG iteration are kept as an unevaluated pair of floats h + l: Knuth's two-sum
+// gives the exact rounding error of every addition to h, which collects in l, so a sum of n terms is good to about
+// n 2^-48.  The terms themselves are FP32 sums of at most 16 products, good to 2^-22 or so, and the scalars formed
+// from the sums (|r|^2, beta, the step length) are FP64.  FP64 additions run at 1/64 of the FP32 rate on sm_103a: a
+// tree sum in FP64 cost the PSF pass 1.2 us of 7.4 at 384 x 384 with 10 coils, and the update pass, with three, 3 us.
+__device__ __forceinline__ void pair_add(Pair& s, float x, float lo) {
+  const float t = __fadd_rn(s.h, x);
+  const float z = __fsub_rn(t, s.h);
+  const float e = __fadd_rn(__fsub_rn(s.h, __fsub_rn(t, z)), __fsub_rn(x, z));
+  s.h = t;
+  s.l = __fadd_rn(s.l, __fadd_rn(e, lo));
+}
+// The sums over a block carry a factor kBlockScale and those over the blocks of a launch kGridScale more, so that no
+// FP32 sum overflows where its terms do not (at most 2^13 terms of a block's threads, 2^12 blocks); powers of two, so
+// nothing is rounded short of the denormal range.
+constexpr float kBlockScale = 0x1p-13f, kGridScale = 0x1p-12f;
+// The value of a sum over the blocks of a launch.
+__device__ __forceinline__ double grid_value(const Pair& s) { return ((double)s.h + (double)s.l) * 0x1p25; }
+// Butterfly sum over the existing lanes of the calling warp (all of them call it), valid in lane 0.
+__device__ __forceinline__ Pair warp_sum(Pair s, int cnt) {
+  const unsigned mask = cnt >= 32 ? 0xffffffffu : (1u << cnt) - 1u;
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h = __shfl_xor_sync(mask, s.h, o), l = __shfl_xor_sync(mask, s.l, o);
+    if ((lane ^ o) < cnt) pair_add(s, h, l);
+  }
+  return s;
+}
+// scale times the sum of the n pairs at src (global or shared memory) by the calling warp, in a fixed order, valid in
+// lane 0.
+__device__ __forceinline__ Pair warp_sum_of(const Pair* src, int n, float scale) {
+  constexpr int D = 12;            // loads in flight
+  const int lane = threadIdx.x & 31, nl = warp_lanes();
+  Pair s = {0.f, 0.f};
+  for (int k0 = lane; k0 < n; k0 += D * nl) {
+    Pair t[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const bool ok = k0 + d * nl < n;
+      t[d].h = ok ? src[k0 + d * nl].h : 0.f;
+      t[d].l = ok ? src[k0 + d * nl].l : 0.f;
+    }
+#pragma unroll
+    for (int d = 0; d < D; ++d) pair_add(s, t[d].h * scale, t[d].l * scale);
+  }
+  return warp_sum(s, nl);
+}
+// Block sums of K pairs per thread that every thread has stored at sums[k * blockDim.x + threadIdx.x], a barrier ago:
+// the block's last warps (in most splits they have no part in the layout-A steps) add one each and write out[k].
+template <int K> __device__ __forceinline__ void block_pairs(const Pair* sums, Pair* const (&out)[K]) {
+  const int nw = ((int)blockDim.x + 31) >> 5, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    if (warp == nw - 1 - k % nw) {
+      const Pair s = warp_sum_of(sums + k * blockDim.x, blockDim.x, 1.f);
+      if ((threadIdx.x & 31) == 0) *out[k] = s;
+    }
+}
+
 __device__ __forceinline__ void finalize_scalar(Scalars* sc, int reduce, int slot, double total) {
   switch (reduce) {
     case RED_RESID: sc->resid[slot] = sqrt(total); break;
     case RED_RR_INIT:           // a new CG solve starts: nothing has stopped yet
-      sc->rr = total;
+      sc->rr[0] = total;
       sc->rr0 = total;
       sc->beta = 0.0;
-      sc->flags &= ~kFlagCgStopped;
       sc->cg_stop[slot] = -1;
       break;
     default: sc->last = total; break;
@@ -267,46 +337,63 @@ enum RowMode : int {
   ROW_FFT_RESID = 3,     // dst <- y - P * FFT_row(T) / sqrt N, |dst|^2                  (Newton residual)
   ROW_P_IFFT = 4,        // T <- compact cols of FFT^-1_row(P * src / sqrt N)            (DF^H input)
   ROW_FFT_W_ADJ = 5,     // dst coil planes <- w FFT_row(T)/sqrt N; rho plane <- sum_j zsum_j (DF^H output)
-  ROW_FFT_W_NORMAL = 6,  // as ADJ, plus alpha p; Re<p, q>                               (normal operator)
-  ROW_FFT_W_RHS = 7,     // as ADJ, minus alpha (x - xref); r = p = b, dx = 0, |b|^2     (right-hand side)
-  NUM_ROW_MODES = 8
+  ROW_FFT_W_NORMAL = 6,  // as ADJ, plus alpha p                                          (normal operator)
+  // single frames
+  ROW_CG_RHS = 7,        // as ADJ, minus alpha (x - xref); r = b, |b|^2; T <- FFT^-1_row(w r)  (right-hand side)
+  ROW_CG_UPDATE = 8,     // q = w FFT_row(T)/sqrt N + alpha p; the CG updates; T <- FFT^-1_row(w r)
+  ROW_CG_PSF = 9,        // as PSF; |P FFT_row(T)|^2
+  // batches
+  ROW_BCG_RHS = 10,      // as ADJ, minus alpha (x - xref); r = p = b, dx = 0, |b|^2     (right-hand side)
+  ROW_BCG_DIR = 11,      // p = r + beta p; T <- compact cols of FFT^-1_row(w p / sqrt N)
+  ROW_BCG_NORMAL = 12,   // as NORMAL with the rho part of p = r + beta p; Re<p, q>
+  NUM_ROW_MODES = 13
 };
-
-template <int MODE> struct RowTraits {
-  static constexpr bool load_compact = !(MODE == ROW_W_IFFT || MODE == ROW_P_IFFT);
-  static constexpr bool inverse_first = (MODE == ROW_W_IFFT || MODE == ROW_P_IFFT);
-  static constexpr bool has_rho = (MODE == ROW_FFT_W_ADJ || MODE == ROW_FFT_W_NORMAL || MODE == ROW_FFT_W_RHS);
-  static constexpr bool reduces = (MODE == ROW_FFT_RESID || MODE == ROW_FFT_W_NORMAL || MODE == ROW_FFT_W_RHS);
-  // side inputs staged per row: sampling-pattern row (bytes), weight row (floats), complex rows
-  static constexpr bool s_mask = (MODE == ROW_PSF || MODE == ROW_FFT_P_OUT || MODE == ROW_FFT_RESID);
-  static constexpr bool s_w = has_rho || MODE == ROW_W_IFFT;
-};
-
-// Shared-memory layout of a row pass (byte offsets), identical on host and device.
-struct RowSmem {
-  size_t xch, tw, mask, w, cplx, total;
-};
-__host__ __device__ inline RowSmem row_smem(int mode, int N, int lanes, int sm_lane) {
-  RowSmem L{};
-  const bool m = (mode == ROW_PSF || mode == ROW_FFT_P_OUT || mode == ROW_FFT_RESID);
-  const bool w = (mode == ROW_FFT_W_ADJ || mode == ROW_FFT_W_NORMAL || mode == ROW_FFT_W_RHS || mode == ROW_W_IFFT);
-  L.xch = 0;
-  L.tw = align16((size_t)lanes * sm_lane * 8);
-  L.mask = L.tw + align16((size_t)2 * N * 8);
-  L.w = L.mask + (m ? align16((size_t)lanes * N) : 0);
-  L.cplx = L.w + (w ? align16((size_t)lanes * N * 4) : 0);
-  L.total = L.cplx + ((mode == ROW_FFT_RESID) ? (size_t)lanes * N * 8 : 0);
-  return L;
-}
-
-#ifndef NLV_COL_C
-#define NLV_COL_C 8
-#endif
 
 // Row passes run kRowCtasPerSM blocks per SM; a block holds up to kRowMaxThreads threads (whole lanes of TL
 // threads) and loops over its share of rows when they do not fit at once.
 constexpr int kRowMaxThreads = 320;
 constexpr int kRowCtasPerSM = 2;
+
+template <int MODE> struct RowTraits {
+  static constexpr bool inverse_first = (MODE == ROW_W_IFFT || MODE == ROW_P_IFFT || MODE == ROW_BCG_DIR);
+  static constexpr bool load_compact = !inverse_first;
+  static constexpr bool psf = (MODE == ROW_PSF || MODE == ROW_CG_PSF);
+  static constexpr bool normal = (MODE == ROW_FFT_W_NORMAL || MODE == ROW_BCG_NORMAL);
+  static constexpr bool rhs = (MODE == ROW_CG_RHS || MODE == ROW_BCG_RHS);
+  static constexpr bool has_rho = (MODE == ROW_FFT_W_ADJ || normal || rhs);
+  static constexpr bool reduces = (MODE == ROW_FFT_RESID || MODE == ROW_BCG_NORMAL || rhs);
+  // a second transform follows the first one in the same pass
+  static constexpr bool two = (psf || MODE == ROW_CG_RHS || MODE == ROW_CG_UPDATE);
+  // side inputs staged per row: sampling-pattern row (bytes), weight row (floats), complex rows
+  static constexpr bool s_mask = (psf || MODE == ROW_FFT_P_OUT || MODE == ROW_FFT_RESID);
+  static constexpr bool s_w = has_rho || MODE == ROW_W_IFFT || MODE == ROW_BCG_DIR || MODE == ROW_CG_UPDATE;
+};
+
+// Shared-memory layout of a row pass (byte offsets), identical on host and device.
+struct RowSmem {
+  size_t xch, tw, mask, w, cplx, sums, total;
+};
+// Floats per staged weight row: w(g) = w(-g), so the CG update pass, short of shared memory, keeps g = 0 .. N/2.
+__host__ __device__ constexpr int w_pitch(int mode, int N);
+__host__ __device__ inline RowSmem row_smem(int mode, int N, int lanes, int sm_lane) {
+  RowSmem L{};
+  const bool m = (mode == ROW_PSF || mode == ROW_CG_PSF || mode == ROW_FFT_P_OUT || mode == ROW_FFT_RESID);
+  const bool w = !m && mode != ROW_P_IFFT;
+  L.xch = 0;
+  L.tw = align16((size_t)lanes * sm_lane * 8);
+  L.mask = L.tw + align16((size_t)2 * N * 8);
+  L.w = L.mask + (m ? align16((size_t)lanes * N) : 0);
+  L.cplx = L.w + (w ? align16((size_t)lanes * w_pitch(mode, N) * 4) : 0);
+  L.sums = L.cplx + ((mode == ROW_FFT_RESID || mode == ROW_CG_UPDATE) ? (size_t)lanes * N * 8 : 0);
+  L.total = L.sums + (mode == ROW_CG_UPDATE ? (size_t)3 * kRowMaxThreads * sizeof(Pair) : 0);
+  return L;
+}
+__host__ __device__ constexpr int w_pitch(int mode, int N) { return mode == ROW_CG_UPDATE ? N / 2 + 4 : N; }
+
+#ifndef NLV_COL_C
+#define NLV_COL_C 8
+#endif
+
 
 // rho plane of the adjoint / normal / right-hand-side outputs: the sum of the channel products over the coils on
 // Omega (the channel summation of Table 1) plus the mode's alpha term.  Every block takes an equal slice of the
@@ -314,76 +401,127 @@ constexpr int kRowCtasPerSM = 2;
 // o + blockDim.x) and issues every load of both before the first use; the coil sum of a pixel runs over even and
 // odd coils in two partial sums added at the end.
 // Dot-product partials: a thread sums at most 32 products in FP32 (one row round, or two pixels of the rho slice)
-// before adding them to its FP64 partial, so the FP32 summation length is bounded whatever the problem size.
+// before adding them to its FP64 partial, so the FP32 summation length is bounded whatever the problem size.  In the
+// single-frame CG passes the real and imaginary products of a thread go to two FP32 sums of at most 16 products each
+// (one row round of at most 16 complex values, or one step of the rho slice) before they are added to its pair.
+__device__ __forceinline__ void dot_acc(float2& acc, float2 a, float2 b) {     // acc += (Re a Re b, Im a Im b)
+  acc.x = fmaf(a.x, b.x, acc.x);
+  acc.y = fmaf(a.y, b.y, acc.y);
+}
+
+__device__ __forceinline__ void dot_flush(float2& acc, Pair& sum) {
+  pair_add(sum, acc.x * kBlockScale, 0.f);
+  pair_add(sum, acc.y * kBlockScale, 0.f);
+  acc = make_float2(0.f, 0.f);
+}
+
+// The two pixels o0 and o0 + blockDim.x of a rho-plane step: which exist (ok), which lie on Omega (om, with their
+// compact offset zo).  Pixel and channel-product offsets fit 32 bits: a plane has at most 1024^2 pixels, the J
+// channel-product planes at most 64 x 512^2 entries.
+template <int N>
+__device__ __forceinline__ void rho_pixels(int o0, int e_end, int f, int Wc, bool (&ok)[2], bool (&om)[2], int (&zo)[2]) {
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int o = o0 + k * (int)blockDim.x;
+    const int e1 = o / N, e2 = o - e1 * N;
+    ok[k] = o < e_end;
+    om[k] = ok[k] && in_omega(e1, N, f) && in_omega(e2, N, f);
+    zo[k] = om[k] ? to_compact(e1, N, f) * Wc + to_compact(e2, N, f) : 0;
+  }
+}
+// Channel sums of those two pixels, over even and odd coils in two partial sums added at the end.  Eight coils' loads of
+// both pixels are in flight at once: with two, a frame of 10 coils paid the L2 latency five times.
+__device__ __forceinline__ void rho_channel_sum(const KArgs& A, const bool (&om)[2], const int (&zo)[2], int stride,
+                                                float2 (&z)[2]) {
+  constexpr int D = 8;
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 s[2][2] = {{zero, zero}, {zero, zero}};
+  const float2* z0 = A.zsum + zo[0];
+  const float2* z1 = A.zsum + zo[1];
+  int j = 0;
+  for (; j + D <= A.J; j += D) {
+    float2 a[D], b[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      a[d] = om[0] ? z0[d * stride] : zero;
+      b[d] = om[1] ? z1[d * stride] : zero;
+    }
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      s[0][d & 1] = cadd(s[0][d & 1], a[d]);
+      s[1][d & 1] = cadd(s[1][d & 1], b[d]);
+    }
+    z0 += D * stride;
+    z1 += D * stride;
+  }
+  if (j < A.J) {
+    float2 a[D], b[D];
+#pragma unroll
+    for (int d = 0; d < D - 1; ++d) {
+      a[d] = om[0] && j + d < A.J ? z0[d * stride] : zero;
+      b[d] = om[1] && j + d < A.J ? z1[d * stride] : zero;
+    }
+#pragma unroll
+    for (int d = 0; d < D - 1; ++d) {
+      s[0][d & 1] = cadd(s[0][d & 1], a[d]);
+      s[1][d & 1] = cadd(s[1][d & 1], b[d]);
+    }
+  }
+  z[0] = cadd(s[0][0], s[0][1]);
+  z[1] = cadd(s[1][0], s[1][1]);
+}
+
 template <int N, int MODE, bool STDF>
 __device__ __forceinline__ double rho_slice(const KArgs& A, int bid) {
-  // pixel and channel-product offsets in 32 bits: a plane has at most 1024^2 pixels, the J channel-product planes
-  // at most 64 x 512^2 entries
-  const int f = STDF ? N / 4 : A.f, Wc = STDF ? N / 2 : A.Wc, J = A.J;
+  const int f = STDF ? N / 4 : A.f, Wc = STDF ? N / 2 : A.Wc;
   constexpr int plane = N * N;
   const int e_begin = bid * A.rho_per_cta;
   const int e_end = min(e_begin + A.rho_per_cta, plane);
-  const float beta = (MODE == ROW_FFT_W_NORMAL && A.pupd) ? cg_beta(A) : 0.f;
-  const int stride = Wc * Wc;
+  const float beta = MODE == ROW_BCG_NORMAL ? (float)A.sc->beta : 0.f;
   const int bd = blockDim.x;
   double accd = 0.0;
   for (int o0 = e_begin + threadIdx.x; o0 < e_end; o0 += 2 * bd) {
     float acc = 0.f;
-    float2 a[2], b[2];
+    float2 a[2], b[2], z[2];
     int zo[2];
     bool ok[2], om[2];
+    rho_pixels<N>(o0, e_end, f, Wc, ok, om, zo);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int o = o0 + k * bd;
-      const int e1 = o / N, e2 = o - e1 * N;
-      ok[k] = o < e_end;
-      om[k] = ok[k] && in_omega(e1, N, f) && in_omega(e2, N, f);
-      zo[k] = om[k] ? to_compact(e1, N, f) * Wc + to_compact(e2, N, f) : 0;
       a[k] = b[k] = make_float2(0.f, 0.f);
       if (ok[k]) {
-        if constexpr (MODE == ROW_FFT_W_NORMAL) {
-          a[k] = A.p[o];
-          if (A.pupd) b[k] = A.r[o];
-        } else if constexpr (MODE == ROW_FFT_W_RHS) {
+        if constexpr (RowTraits<MODE>::normal) a[k] = A.p[o];
+        if constexpr (MODE == ROW_BCG_NORMAL) b[k] = A.r[o];
+        if constexpr (RowTraits<MODE>::rhs) {
           a[k] = A.x[o];
           b[k] = A.xref[o];
         }
       }
     }
-    const float2 zero = make_float2(0.f, 0.f);
-    float2 z00 = zero, z01 = zero, z10 = zero, z11 = zero;
-    int j = 0;
-    for (; j + 2 <= J; j += 2) {
-      if (om[0]) { z00 = cadd(z00, A.zsum[zo[0]]); z01 = cadd(z01, A.zsum[zo[0] + stride]); }
-      if (om[1]) { z10 = cadd(z10, A.zsum[zo[1]]); z11 = cadd(z11, A.zsum[zo[1] + stride]); }
-      zo[0] += 2 * stride;
-      zo[1] += 2 * stride;
-    }
-    if (j < J) {
-      if (om[0]) z00 = cadd(z00, A.zsum[zo[0]]);
-      if (om[1]) z10 = cadd(z10, A.zsum[zo[1]]);
-    }
-    const float2 z[2] = {cadd(z00, z01), cadd(z10, z11)};
+    rho_channel_sum(A, om, zo, Wc * Wc, z);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       if (!ok[k]) continue;
       const int o = o0 + k * bd;
       if constexpr (MODE == ROW_FFT_W_ADJ) {
         A.dst[o] = z[k];
-      } else if constexpr (MODE == ROW_FFT_W_NORMAL) {
+      } else if constexpr (RowTraits<MODE>::normal) {
         float2 pv = a[k];
-        if (A.pupd) {
+        if constexpr (MODE == ROW_BCG_NORMAL) {
           pv = make_float2(fmaf(beta, pv.x, b[k].x), fmaf(beta, pv.y, b[k].y));
           const_cast<float2*>(A.p)[o] = pv;
         }
         const float2 q = make_float2(fmaf(A.alpha, pv.x, z[k].x), fmaf(A.alpha, pv.y, z[k].y));
         A.dst[o] = q;
-        acc += pv.x * q.x + pv.y * q.y;
+        if constexpr (MODE == ROW_BCG_NORMAL) acc += pv.x * q.x + pv.y * q.y;
       } else {
         const float2 bb = make_float2(z[k].x - A.alpha * (a[k].x - b[k].x), z[k].y - A.alpha * (a[k].y - b[k].y));
         A.r[o] = bb;
-        A.pout[o] = bb;
-        A.dx[o] = make_float2(0.f, 0.f);
+        if constexpr (MODE == ROW_BCG_RHS) {
+          A.pout[o] = bb;
+          A.dx[o] = make_float2(0.f, 0.f);
+        }
         acc += bb.x * bb.x + bb.y * bb.y;
       }
     }
@@ -392,18 +530,116 @@ __device__ __forceinline__ double rho_slice(const KArgs& A, int bid) {
   return accd;
 }
 
+// The scalars of one CG update (see cg_point).
+struct CgStep {
+  float a, a_prev, beta, alpha;
+  bool first, odd;              // iteration 0 (p = r); an odd iteration (the one that updates dx)
+};
+struct CgDots {                 // sums of |r|^2, Re<r, p> and |p|^2 of the new r and p
+  float2 rr, rp, pp;
+};
+// One element of the CG update:  p = r + beta p_old;  q = z + alpha p (z: the element of DF^H DF p);  r -= a q.
+// Returns the new r; p: in the old, out the new direction; g: what the pair of iterations adds to dx (odd
+// iterations: a_prev p_old + a p).
+__device__ __forceinline__ float2 cg_point(const CgStep& c, float2 z, float2 r, float2& p, float2& g, CgDots& acc) {
+  const float2 po = p;
+  p = c.first ? r : make_float2(fmaf(c.beta, po.x, r.x), fmaf(c.beta, po.y, r.y));
+  const float2 q = make_float2(fmaf(c.alpha, p.x, z.x), fmaf(c.alpha, p.y, z.y));
+  r = make_float2(fmaf(-c.a, q.x, r.x), fmaf(-c.a, q.y, r.y));
+  g = make_float2(fmaf(c.a_prev, po.x, c.a * p.x), fmaf(c.a_prev, po.y, c.a * p.y));
+  dot_acc(acc.rr, r, r);
+  dot_acc(acc.rp, r, p);
+  dot_acc(acc.pp, p, p);
+  return r;
+}
+
+// dx += g (odd iterations; the first one, iteration 1, writes it).  The addition happens in L2, so no thread waits for
+// dx or holds it: read and written by the pass it cost 6 of 55 us at 512 x 512 with 16 coils and, held in registers
+// across the second transform, spilled 300 bytes a thread.
+__device__ __forceinline__ void cg_add_dx(const KArgs& A, int o, float2 g) {
+  if (A.iter > 1)
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(A.dx + o), "f"(g.x), "f"(g.y) : "memory");
+  else
+    A.dx[o] = g;
+}
+
+// Adds a thread's products to its three sums at sums[k * blockDim.x]; first: they hold nothing yet.
+__device__ __forceinline__ void cg_flush(CgDots& d, Pair* sums, bool first) {
+  float2* v[3] = {&d.rr, &d.rp, &d.pp};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    Pair s = {0.f, 0.f};
+    if (!first) s = sums[k * blockDim.x];
+    dot_flush(*v[k], s);
+    sums[k * blockDim.x] = s;
+  }
+}
+
+// The rho plane's slice of the CG update pass.
+template <int N, bool STDF>
+__device__ __forceinline__ void rho_cg_slice(const KArgs& A, int bid, const CgStep c, Pair* sums) {
+  const int f = STDF ? N / 4 : A.f, Wc = STDF ? N / 2 : A.Wc;
+  constexpr int plane = N * N;
+  const int e_begin = bid * A.rho_per_cta;
+  const int e_end = min(e_begin + A.rho_per_cta, plane);
+  const int bd = blockDim.x;
+  for (int o0 = e_begin + threadIdx.x; o0 < e_end; o0 += 2 * bd) {
+    CgDots acc;
+    acc.rr = acc.rp = acc.pp = make_float2(0.f, 0.f);
+    float2 p[2], r[2], z[2];
+    int zo[2];
+    bool ok[2], om[2];
+    rho_pixels<N>(o0, e_end, f, Wc, ok, om, zo);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int o = o0 + k * bd;
+      p[k] = r[k] = make_float2(0.f, 0.f);
+      if (ok[k]) {
+        r[k] = A.r[o];
+        if (!c.first) p[k] = A.p[o];
+      }
+    }
+    rho_channel_sum(A, om, zo, Wc * Wc, z);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      if (!ok[k]) continue;
+      const int o = o0 + k * bd;
+      float2 g;
+      A.r[o] = cg_point(c, z[k], r[k], p[k], g, acc);
+      const_cast<float2*>(A.p)[o] = p[k];
+      if (c.odd) cg_add_dx(A, o, g);
+    }
+    cg_flush(acc, sums, false);
+  }
+}
+
 // Side rows of the round starting at row R0 (sampling pattern, weights, data).  Every launch sequence writes these,
 // if at all, two or more launches before the pass that stages them (the data rows of the gradient's second
 // residual are the first residual, three launches back), never in the launch just before, so that a single-frame
-// pass may stage them before its dependent-launch wait (see cg_flags_early for why that suffices).
+// pass may stage them before its dependent-launch wait (see cg_stop_early for why that suffices).
 template <int N, int MODE>
 __device__ __forceinline__ void row_stage_side(const KArgs& A, const RowSmem& L, int R0, int r_end, int LANES,
                                                unsigned char* smem_raw) {
   using T = RowTraits<MODE>;
   const int nr = min(LANES, r_end - R0);
   if constexpr (T::s_mask) stage_rows(smem_raw + L.mask, A.mask, R0, nr, N, N, true);
-  if constexpr (T::s_w) stage_rows(smem_raw + L.w, A.wtab, R0, nr, N * 4, N, true);
+  if constexpr (MODE == ROW_CG_UPDATE) {
+    constexpr int W = w_pitch(MODE, N), Q = W / 4;               // 16-byte chunks
+    for (int i = threadIdx.x; i < nr * Q; i += blockDim.x) {
+      const int l = i / Q, c = i - l * Q;
+      cp_async16(smem_raw + L.w + (size_t)i * 16, A.wtab + (size_t)((R0 + l) % N) * N + 4 * c);
+    }
+  } else if constexpr (T::s_w) {
+    stage_rows(smem_raw + L.w, A.wtab, R0, nr, N * 4, N, true);
+  }
   if constexpr (MODE == ROW_FFT_RESID) stage_rows(smem_raw + L.cplx, A.y, R0, nr, N * 8, N, false);
+}
+
+// Rows of the CG direction p (coil planes) of the round starting at row R0; in iteration 0 p = r and none is read.
+template <int N>
+__device__ __forceinline__ void cg_stage_p(const KArgs& A, const RowSmem& L, int R0, int r_end, int LANES,
+                                           unsigned char* smem_raw) {
+  if (A.iter > 0) stage_rows(smem_raw + L.cplx, A.p + (size_t)N * N, R0, min(LANES, r_end - R0), N * 8, N, false);
 }
 
 // The twiddles and the first round's side rows of a single-frame row pass, issued before its dependent-launch
@@ -418,21 +654,25 @@ __device__ __forceinline__ void row_pass_prestage(const KArgs& A, int bid, unsig
   const int r_end = min(r_begin + A.rows_per_cta, A.nrows);
   stage_bytes(smem_raw + L.tw, A.twA, N * 8);
   stage_bytes(smem_raw + L.tw + N * 8, A.twB, N * 8);
-  if (r_begin < r_end) row_stage_side<N, MODE>(A, L, r_begin, r_end, LANES, smem_raw);
+  if (r_begin < r_end) {
+    row_stage_side<N, MODE>(A, L, r_begin, r_end, LANES, smem_raw);
+    if constexpr (MODE == ROW_CG_UPDATE)
+      if (A.src_early) cg_stage_p<N>(A, L, r_begin, r_end, LANES, smem_raw);
+  }
 }
 
 // Row pass: block b takes the coil rows [b*rows_per_cta, (b+1)*rows_per_cta) of the stacked J*N rows, one lane
 // (TL threads) per row, in as many rounds as its lanes need; passes with a rho part then take a slice of the rho
 // plane.  All threads of the block run every round (inactive lanes carry zeros) because of the barriers.
 // PRE: the twiddles and the first round's side rows were staged by row_pass_prestage, and the body itself waits for
-// the kernel before (pdl_enter) and applies the stop test: before its first loads, or, for the first CG pass with
-// src_early, right after the first round's main loads are issued.
+// the kernel before (pdl_enter) and applies the stop test before its first loads.
 template <int N1, int N2, int MODE, bool STDF = false, class TC = NoTc, bool PRE = false>
 __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk, unsigned char* smem_raw,
-                                              TC* tc = nullptr, int early_flags = 0) {
+                                              TC* tc = nullptr, int early_stop = kNoStop) {
   using S = Split<N1, N2>;
   using T = RowTraits<MODE>;
   constexpr int N = S::N, TL = S::TL, E = S::E;
+  constexpr bool CG = MODE == ROW_CG_UPDATE;
   static_assert(N2 == TL, "row passes assume N1 <= N2");
   const int LANES = blockDim.x / TL;
   // Two thread maps onto the rows of a round: layout A (N1 threads per row) packs the rows densely so that the
@@ -456,32 +696,35 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
     stage_bytes(smem_raw + L.tw, A.twA, N * 8);
     stage_bytes(smem_raw + L.tw + N * 8, A.twB, N * 8);
   }
-  __shared__ float s_beta;       // beta of the direction update p = r + beta p (ROW_W_IFFT with pupd)
   bool waited = !PRE;
   // the dependent-launch wait and the stop test (the same for every thread of the block); true: leave the pass
   auto enter = [&]() -> bool {
     pdl_enter();
     waited = true;
-    if (cg_stopped_after(A, early_flags)) {
+    if (cg_stopped_after(A, early_stop)) {
       cp_async_wait_all();
       return true;
     }
     return false;
   };
-  // with src_early the first CG pass issues its main loads (p) before the wait; every other pass waits first
-  const bool early_main = PRE && MODE == ROW_W_IFFT && A.src_early;
-  if (PRE && !early_main && enter()) return;
+  if (!waited) {
+    if (enter()) return;
+  }
+  __shared__ CgStep s_cg;          // CG update: its scalars, and the threads' sums (live registers across the transforms
+  [[maybe_unused]] Pair* sums = (Pair*)(smem_raw + L.sums) + threadIdx.x;      // would spill)
+  __shared__ Pair s_pairs[MODE == ROW_CG_PSF ? kRowMaxThreads : 1];
+  [[maybe_unused]] float2 dd = make_float2(0.f, 0.f);      // PSF pass: this round's |DF p|^2
+  __shared__ float s_beta;       // beta of the batches' direction update p = r + beta p
 
   for (int R0 = r_begin; R0 < r_end; R0 += LANES) {
   const int RA = R0 + laneA, RB = R0 + laneB;               // rows of the stacked coil planes in the two maps
   const bool activeA = mapA && RA < r_end, activeB = mapB && RB < r_end;
   const int e1A = RA % N;
+  const int rowB = (N + RB) * N + idxB;        // coil planes follow the rho plane (at most 65 x 512^2 elements)
   float2 v[E];
 
-  // ---- direction update: the rows of r go to the exchange buffer (natural order, pitch N) while p is loaded
-  if constexpr (MODE == ROW_W_IFFT) {
-    if (A.pupd && waited) stage_rows(smem_raw + L.xch, A.r, R0, min(LANES, r_end - R0), N * 8, N, false);
-  }
+  // ---- batches' direction update: the rows of r go to the exchange buffer (natural order, pitch N) while p is loaded
+  if constexpr (MODE == ROW_BCG_DIR) stage_rows(smem_raw + L.xch, A.r, R0, min(LANES, r_end - R0), N * 8, N, false);
 
   // ---- main loads, layout A: thread a < N1 holds row elements a + N1*m (no stores until all are issued)
   if (mapA) {
@@ -492,9 +735,9 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
       if (activeA) {
         if constexpr (T::load_compact) {
           if (in_omega(e2, N, f)) val = A.src[(size_t)RA * Wc + to_compact(e2, N, f)];
-        } else if constexpr (MODE == ROW_W_IFFT) {
-          val = __ldcg(A.src + (size_t)RA * N + e2);     // from L2 (issued before the wait with src_early)
-        } else {  // ROW_P_IFFT
+        } else if constexpr (MODE != ROW_P_IFFT) {
+          val = A.src[(size_t)RA * N + e2];
+        } else {
           const float2 sv = A.src[(size_t)RA * N + e2];
           val = A.mask[(size_t)e1A * N + e2] ? sv : make_float2(0.f, 0.f);
         }
@@ -502,54 +745,65 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
       v[m] = val;
     }
   }
-  if (!waited) {                 // src_early: the main loads are in flight; now the inputs of the kernel before
-    if (enter()) return;
-    if constexpr (MODE == ROW_W_IFFT) {
-      if (A.pupd) stage_rows(smem_raw + L.xch, A.r, R0, min(LANES, r_end - R0), N * 8, N, false);
-    }
-  }
 
   // ---- staged side inputs (the twiddles were issued before the first round)
   if (!PRE || R0 != r_begin) row_stage_side<N, MODE>(A, L, R0, r_end, LANES, smem_raw);
-  // beta from the |r|^2 partials of the CG step before, while the loads above are in flight (same order in every
-  // block; block 0 publishes |r|^2 and beta for the CG step and the later passes of this iteration)
-  if constexpr (MODE == ROW_W_IFFT) {
-    if (A.pupd && R0 == r_begin) {
-      if (A.rr_part) {
+  if constexpr (CG) {
+    if (!PRE || !A.src_early || R0 != r_begin) cg_stage_p<N>(A, L, R0, r_end, LANES, smem_raw);
+    if (R0 == r_begin && threadIdx.x == 0) {
+      CgStep cg;
+      cg.first = A.iter == 0;
+      cg.odd = (A.iter & 1) != 0;
+      cg.alpha = A.alpha;
+      cg.a = A.sc->step[A.iter & 1];
+      cg.a_prev = cg.first ? 0.f : A.sc->step[(A.iter & 1) ^ 1];
+      cg.beta = cg.first ? 0.f : A.sc->beta_f;
+      s_cg = cg;
+    }
+  }
+  // batches: beta from the |r|^2 partials of the CG step before, while the loads above are in flight (same order in
+  // every block; block 0 publishes |r|^2 and beta for the CG step and the later passes of this iteration)
+  if constexpr (MODE == ROW_BCG_DIR) {
+    if (R0 == r_begin) {
+      if (A.brr_part) {
         __shared__ double red[32];
         double t = 0.0;
-        for (int k = threadIdx.x; k < A.n_rr; k += blockDim.x) t += A.rr_part[k];
+        for (int k = threadIdx.x; k < A.n_rr; k += blockDim.x) t += A.brr_part[k];
         t = block_sum(t, red);
         if (threadIdx.x == 0) {
           const double rp = A.sc->rr_prev;
           const double b = (rp != 0.0) ? t / rp : 0.0;
           s_beta = (float)b;
-          if (bid == 0) { A.sc->rr = t; A.sc->beta = b; }
+          if (bid == 0) { A.sc->rr[0] = t; A.sc->beta = b; }
         }
       } else if (threadIdx.x == 0) {
-        s_beta = cg_beta(A);
+        s_beta = (float)A.sc->beta;
       }
     }
   }
   cp_async_wait_all();
   __syncthreads();
 
-  if constexpr (MODE == ROW_W_IFFT) {
+  if constexpr (MODE == ROW_BCG_DIR) {
     // p = r + beta p (r from the exchange buffer) written back, then weight
     const float* sw = (const float*)(smem_raw + L.w) + (size_t)laneA * N;
     const float2* sr = (const float2*)(smem_raw + L.xch) + (size_t)laneA * N;
     if (activeA) {
 #pragma unroll
       for (int m = 0; m < N2; ++m) {
-        if (A.pupd) {
-          const float2 rv = sr[idxA + N1 * m];
-          v[m] = make_float2(fmaf(s_beta, v[m].x, rv.x), fmaf(s_beta, v[m].y, rv.y));
-          const_cast<float2*>(A.src)[(size_t)RA * N + idxA + N1 * m] = v[m];
-        }
+        const float2 rv = sr[idxA + N1 * m];
+        v[m] = make_float2(fmaf(s_beta, v[m].x, rv.x), fmaf(s_beta, v[m].y, rv.y));
+        const_cast<float2*>(A.src)[(size_t)RA * N + idxA + N1 * m] = v[m];
         v[m] = cscale(v[m], sw[idxA + N1 * m] * rs);
       }
     }
-    if (A.pupd) __syncthreads();   // the exchange below overwrites the staged rows of r
+    __syncthreads();   // the exchange below overwrites the staged rows of r
+  } else if constexpr (MODE == ROW_W_IFFT) {
+    const float* sw = (const float*)(smem_raw + L.w) + (size_t)laneA * N;
+    if (activeA) {
+#pragma unroll
+      for (int m = 0; m < N2; ++m) v[m] = cscale(v[m], sw[idxA + N1 * m] * rs);
+    }
   } else if constexpr (MODE == ROW_P_IFFT) {
     if (mapA) {
 #pragma unroll
@@ -571,50 +825,93 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
     // single-frame normal-operator pass: its rows of p (layout B) are loaded before the transform, so that their
     // latency overlaps it (the batched pass, HBM-bound, loads them after it: the early loads cost it 2.5 %)
     constexpr bool kEarlyP = MODE == ROW_FFT_W_NORMAL && PRE;
-    float2 pB[kEarlyP ? N1 : 1];
+    float2 a0[T::normal ? N1 : 1];
     if constexpr (kEarlyP) {
       if (activeB) {
 #pragma unroll
-        for (int m = 0; m < N1; ++m) pB[m] = A.p[(size_t)N * N + (size_t)RB * N + idxB + N2 * m];
+        for (int m = 0; m < N1; ++m) a0[m] = A.p[rowB + N2 * m];
       }
     }
-    // the PSF pass exchanges again right after: keep the closing barrier there
-    fft_AtoB2<N1, N2, -1, E, TC, MODE == ROW_PSF>(v, smA, idxA, mapA, smB, idxB, mapB, twA, tc);
-    const unsigned char* smask = smem_raw + L.mask + (size_t)laneB * N;
-    if constexpr (MODE == ROW_PSF) {
-      {
+    // passes with a second transform exchange again right after: keep the closing barrier there
+    // the CG update issues its loads of r while the first transform is on its way (the registers of its layout-A
+    // elements are free by then: loaded before it, they spilled 400 bytes a thread)
+    float2 rB[CG ? N1 : 1];
+    fft_AtoB2<N1, N2, -1, E, TC, T::two>(v, smA, idxA, mapA, smB, idxB, mapB, twA, tc, [&] {
+      if constexpr (CG) {
+        if (activeB) {
 #pragma unroll
-        for (int m = 0; m < N1; ++m) {
-          const float sc = (activeB && smask[idxB + N2 * m]) ? rs * rs : 0.f;
-          v[m] = cscale(v[m], sc);
+          for (int m = 0; m < N1; ++m) rB[m] = A.r[rowB + N2 * m];
         }
       }
-      fft_AtoB2<N2, N1, +1, E, TC, false>(v, smB, idxB, mapB, smA, idxA, mapA, twB, tc);
-      if (activeA) {
+    });
+    const unsigned char* smask = smem_raw + L.mask + (size_t)laneB * N;
+    const float* sw = (const float*)(smem_raw + L.w) + (size_t)laneB * N;
+    // staged rows of y (residual) or of p (CG update)
+    float2* scp = (float2*)(smem_raw + L.cplx) + (size_t)laneB * N;
+    if constexpr (T::psf) {
 #pragma unroll
-        for (int m = 0; m < N2; ++m) {
-          const int e2 = idxA + N1 * m;
-          if (in_omega(e2, N, f)) A.dst[(size_t)RA * Wc + to_compact(e2, N, f)] = v[m];
+      for (int m = 0; m < N1; ++m) {
+        v[m] = (activeB && smask[idxB + N2 * m]) ? cscale(v[m], rs * rs) : make_float2(0.f, 0.f);
+        if constexpr (MODE == ROW_CG_PSF) dot_acc(dd, v[m], v[m]);
+      }
+      if constexpr (MODE == ROW_CG_PSF) {           // |DF p|^2 of these rows (the values carry one more factor 1/sqrt(N))
+        Pair t = {0.f, 0.f};
+        if (R0 != r_begin) t = s_pairs[threadIdx.x];
+        dot_flush(dd, t);
+        s_pairs[threadIdx.x] = t;
+      }
+    } else if constexpr (CG) {
+      const CgStep cg = s_cg;
+      const float* swh = (const float*)(smem_raw + L.w) + (size_t)laneB * w_pitch(MODE, N);
+      CgDots dots;
+      dots.rr = dots.rp = dots.pp = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int m = 0; m < N1; ++m) {
+        const int e2 = idxB + N2 * m;
+        float2 out = make_float2(0.f, 0.f);
+        if (activeB) {
+          const float w = swh[N2 * m < N / 2 ? e2 : N - e2] * rs;
+          float2 p = cg.first ? make_float2(0.f, 0.f) : scp[e2], g;
+          const float2 rn = cg_point(cg, cscale(v[m], w), rB[m], p, g, dots);
+          A.r[rowB + N2 * m] = rn;
+          const_cast<float2*>(A.p)[rowB + N2 * m] = p;
+          if (cg.odd) cg_add_dx(A, rowB + N2 * m, g);
+          out = cscale(rn, w);
         }
+        v[m] = out;
+      }
+      cg_flush(dots, sums, R0 == r_begin);
+    } else if constexpr (T::rhs) {
+      float2 x0[N1], x1[N1];          // x and x_ref, loaded before any store
+      if (activeB) {
+#pragma unroll
+        for (int m = 0; m < N1; ++m) {
+          x0[m] = A.x[rowB + N2 * m];
+          x1[m] = A.xref[rowB + N2 * m];
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < N1; ++m) {
+        float2 out = make_float2(0.f, 0.f);
+        if (activeB) {
+          const float w = sw[idxB + N2 * m] * rs;
+          const float2 val = cscale(v[m], w), xv = x0[m], xr = x1[m];
+          const float2 b = make_float2(val.x - A.alpha * (xv.x - xr.x), val.y - A.alpha * (xv.y - xr.y));
+          A.r[rowB + N2 * m] = b;
+          if constexpr (MODE == ROW_BCG_RHS) {
+            A.pout[rowB + N2 * m] = b;
+            A.dx[rowB + N2 * m] = make_float2(0.f, 0.f);
+          }
+          acc += b.x * b.x + b.y * b.y;
+          out = cscale(b, w);
+        }
+        v[m] = out;
       }
     } else {
-      const float* sw = (const float*)(smem_raw + L.w) + (size_t)laneB * N;
-      // staged rows of y; p, or x and x_ref, loaded into registers before any store
-      const float2* scp = (const float2*)(smem_raw + L.cplx) + (size_t)laneB * N;
-      constexpr int NV = (MODE == ROW_FFT_W_RHS) ? 2 : (MODE == ROW_FFT_W_NORMAL) ? 1 : 0;
-      float2 a0[NV ? N1 : 1], a1[NV == 2 ? N1 : 1];
-      if (NV && activeB) {
+      if constexpr (T::normal && !kEarlyP) {      // loaded before any store
+        if (activeB) {
 #pragma unroll
-        for (int m = 0; m < N1; ++m) {
-          const size_t oc = (size_t)N * N + (size_t)RB * N + idxB + N2 * m;
-          if constexpr (MODE == ROW_FFT_W_NORMAL) {
-            if constexpr (kEarlyP) a0[m] = pB[m];
-            else a0[m] = A.p[oc];
-          }
-          if constexpr (MODE == ROW_FFT_W_RHS) {
-            a0[m] = A.x[oc];
-            a1[m] = A.xref[oc];
-          }
+          for (int m = 0; m < N1; ++m) a0[m] = A.p[rowB + N2 * m];
         }
       }
       if (activeB) {
@@ -631,22 +928,27 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
             acc += rv.x * rv.x + rv.y * rv.y;
           } else {
             const float2 val = cscale(v[m], sw[e2] * rs);
-            const size_t oc = (size_t)N * N + o;      // coil planes follow the rho plane
             if constexpr (MODE == ROW_FFT_W_ADJ) {
-              A.dst[oc] = val;
-            } else if constexpr (MODE == ROW_FFT_W_NORMAL) {
+              A.dst[rowB + N2 * m] = val;
+            } else {
               const float2 pv = a0[m];
               const float2 q = make_float2(fmaf(A.alpha, pv.x, val.x), fmaf(A.alpha, pv.y, val.y));
-              A.dst[oc] = q;
-              acc += pv.x * q.x + pv.y * q.y;
-            } else {  // ROW_FFT_W_RHS
-              const float2 xv = a0[m], xr = a1[m];
-              const float2 b = make_float2(val.x - A.alpha * (xv.x - xr.x), val.y - A.alpha * (xv.y - xr.y));
-              A.r[oc] = b;
-              A.pout[oc] = b;
-              A.dx[oc] = make_float2(0.f, 0.f);
-              acc += b.x * b.x + b.y * b.y;
+              A.dst[rowB + N2 * m] = q;
+              if constexpr (MODE == ROW_BCG_NORMAL) acc += pv.x * q.x + pv.y * q.y;
             }
+          }
+        }
+      }
+    }
+    if constexpr (T::two) {
+      if (!CG || !A.last) {
+        fft_AtoB2<N2, N1, +1, E, TC, false>(v, smB, idxB, mapB, smA, idxA, mapA, twB, tc);
+        float2* dst = A.dst;
+        if (activeA) {
+#pragma unroll
+          for (int m = 0; m < N2; ++m) {
+            const int e2 = idxA + N1 * m;
+            if (in_omega(e2, N, f)) dst[(size_t)RA * Wc + to_compact(e2, N, f)] = v[m];
           }
         }
       }
@@ -660,21 +962,26 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
   }  // rounds
 
   if constexpr (T::has_rho) accd += rho_slice<N, MODE, STDF>(A, bid);
-  if constexpr (T::reduces) {
-    if (MODE == ROW_FFT_W_NORMAL && A.pq_part) {
-      __shared__ double red[32];
-      const double sblk = block_sum(accd, red);
-      if (threadIdx.x == 0) A.pq_part[bid] = sblk;
-    } else {
-      grid_reduce(accd, A, bid, nblk);
-    }
+  if constexpr (CG) {
+    rho_cg_slice<N, STDF>(A, bid, s_cg, sums);
+    __syncthreads();
+    block_pairs<3>(sums - threadIdx.x, {A.rr_part + bid, A.rr_part + A.n_rr + bid, A.rr_part + 2 * A.n_rr + bid});
+  }
+  // the pairs were stored before the second transform's barrier
+  if constexpr (MODE == ROW_CG_PSF) block_pairs<1>(s_pairs, {A.dd_part + bid});
+  if constexpr (MODE == ROW_BCG_NORMAL) {
+    __shared__ double red[32];
+    const double sblk = block_sum(accd, red);
+    if (threadIdx.x == 0) A.pq_part[bid] = sblk;
+  } else if constexpr (T::reduces) {
+    grid_reduce(accd, A, bid, nblk);
   }
 }
 
 template <int N1, int N2, int MODE, bool STDF = false>
 __global__ void __launch_bounds__(kRowMaxThreads, kRowCtasPerSM) row_pass(const KArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int early = cg_flags_early(A);
+  const int early = cg_stop_early(A);
   row_pass_prestage<N1, N2, MODE>(A, blockIdx.x, smem_raw);
   row_pass_body<N1, N2, MODE, STDF, NoTc, true>(A, blockIdx.x, gridDim.x, smem_raw, nullptr, early);
 }
@@ -686,7 +993,9 @@ enum ColMode : int {
   COL_SIM_FFT = 2,        // T <- FFT_col(M rho cimg_j) / sqrt N                          (data simulation)
   COL_IFFT_PROD_FFT = 3,  // u = FFT^-1_col(T); T <- FFT_col(M (drho c_j + rho u))        (DF)
   COL_IFFT_ADJ_FFT = 4,   // z = M FFT^-1_col(T); zsum_j = conj(c_j) z; T <- FFT_col(conj(rho) z)   (DF^H)
-  NUM_COL_MODES = 5
+  COL_CG_DIR = 5,         // single frames: U <- FFT^-1_col(T) + beta U;  T <- FFT_col(M ((r + beta p)_rho c_j + rho U))
+  COL_BCG_DIR = 6,        // batches: COL_IFFT_PROD_FFT for the rho part of p = r + beta p
+  NUM_COL_MODES = 7
 };
 
 // Shared-memory layout of a column pass (byte offsets): exchange, twiddles, then `nside` side arrays of
@@ -697,7 +1006,7 @@ struct ColSmem {
 };
 __host__ __device__ inline ColSmem col_smem(int mode, int N, int C, int sm_lane, int Wc) {
   ColSmem L{};
-  L.nside = (mode == COL_IFFT_PROD_FFT) ? 4 : (mode == COL_IFFT_ADJ_FFT) ? 2 : 0;
+  L.nside = (mode == COL_CG_DIR || mode == COL_BCG_DIR) ? 4 : (mode == COL_IFFT_PROD_FFT) ? 3 : (mode == COL_IFFT_ADJ_FFT) ? 2 : 0;
   L.xch = 0;
   L.tw = align16((size_t)C * sm_lane * 8);
   L.side = L.tw + align16((size_t)2 * N * 8);
@@ -740,8 +1049,11 @@ __device__ __forceinline__ void stage_natural_cols(float2* sdst, const float2* p
   }
 }
 
+// Side inputs of a column pass.  `before`: those that no launch just before writes (the twiddles, the coil map and
+// rho), which a single-frame pass stages before its dependent-launch wait; else the rest: drho, for the CG direction
+// pass the rho planes of p and r that the CG update pass just before has written.
 template <int N1, int N2, int MODE, bool STDF, int CC>
-__device__ __forceinline__ void col_stage_side(const KArgs& A, int bid, unsigned char* smem_raw) {
+__device__ __forceinline__ void col_stage_side(const KArgs& A, int bid, unsigned char* smem_raw, bool before) {
   using S = Split<N1, N2>;
   constexpr int N = S::N, C = ColCfg<N1, N2, CC>::C;
   const int f = STDF ? N / 4 : A.f, Wc = STDF ? N / 2 : A.Wc;
@@ -749,28 +1061,103 @@ __device__ __forceinline__ void col_stage_side(const KArgs& A, int bid, unsigned
   const int j = bid / strips;
   const int cc0 = (bid % strips) * C;
   const ColSmem L = col_smem(MODE, N, C, S::SM_LANE_COL, Wc);
-  stage_bytes(smem_raw + L.tw, A.twA, N * 8);
-  stage_bytes(smem_raw + L.tw + N * 8, A.twB, N * 8);
-  if (j < A.nrows) {
-    float2* sd = (float2*)(smem_raw + L.side);
-    const size_t sstride = (size_t)Wc * C;
-    if constexpr (MODE == COL_IFFT_PROD_FFT || MODE == COL_IFFT_ADJ_FFT) {
-      stage_compact_cols(sd, A.coil + (size_t)j * Wc * Wc, cc0, C, Wc);
-      stage_natural_cols(sd + sstride, A.rho, cc0, C, Wc, N, f);
+  float2* sd = (float2*)(smem_raw + L.side);
+  const size_t sstride = (size_t)Wc * C;
+  if (before) {
+    stage_bytes(smem_raw + L.tw, A.twA, N * 8);
+    stage_bytes(smem_raw + L.tw + N * 8, A.twB, N * 8);
+    if constexpr (MODE == COL_IFFT_PROD_FFT || MODE == COL_IFFT_ADJ_FFT || MODE == COL_CG_DIR || MODE == COL_BCG_DIR) {
+      if (j < A.nrows) {
+        stage_compact_cols(sd, A.coil + (size_t)j * Wc * Wc, cc0, C, Wc);
+        stage_natural_cols(sd + sstride, A.rho, cc0, C, Wc, N, f);
+      }
     }
-    if constexpr (MODE == COL_IFFT_PROD_FFT) {
-      stage_natural_cols(sd + 2 * sstride, A.drho, cc0, C, Wc, N, f);
-      if (A.pupd) stage_natural_cols(sd + 3 * sstride, A.r, cc0, C, Wc, N, f);
+  } else if constexpr (MODE == COL_IFFT_PROD_FFT) {
+    if (j < A.nrows) stage_natural_cols(sd + 2 * sstride, A.drho, cc0, C, Wc, N, f);
+  } else if constexpr (MODE == COL_CG_DIR || MODE == COL_BCG_DIR) {
+    if (j < A.nrows) {
+      if (MODE == COL_BCG_DIR || A.iter > 0) stage_natural_cols(sd + 2 * sstride, A.drho, cc0, C, Wc, N, f);
+      stage_natural_cols(sd + 3 * sstride, A.r, cc0, C, Wc, N, f);
     }
   }
 }
 
-// prestaged: the twiddles and side inputs were staged by col_stage_side before the dependent-launch wait.
+// beta_i = |r_i|^2 / |r_{i-1}|^2 of the CG direction pass from the partials that the CG update pass before wrote, by
+// the block's last warp (in most splits it has no part in the first register DFT), in the same order in every block.
+// Block 0 publishes |r_i|^2 and beta and records the stop when |r_i| has reached the rounding floor (or is not finite);
+// s_stop: the same for every block.
+__device__ __forceinline__ void cg_direction_scalars(const KArgs& A, int bid, float& s_beta, int& s_stop) {
+  if (threadIdx.x < ((blockDim.x - 1) & ~31u)) return;
+  const double rp = A.sc->rr[(A.iter & 1) ^ 1], rr0 = A.sc->rr0;
+  const Pair s = warp_sum_of(A.rr_part, A.n_rr, kGridScale);
+  if ((threadIdx.x & 31) == 0) {
+    const double t = grid_value(s);
+    const double b = (rp != 0.0) ? t / rp : 0.0;
+    const bool stop = !(t > kCgFloor2 * rr0) || !isfinite(t);
+    s_beta = (float)b;
+    s_stop = stop ? 1 : 0;
+    if (bid == 0) {
+      A.sc->rr[A.iter & 1] = t;
+      A.sc->beta = b;
+      A.sc->beta_f = (float)b;
+      if (stop) {
+        A.sc->cg_stop[A.slot] = A.iter;
+        if (!isfinite(t)) atomicOr(&A.sc->flags, kFlagBreakdown);
+      }
+    }
+  }
+}
+
+// Step length of a CG iteration, by one block of the DF^H column pass that has no columns: Re<p, A p> =
+// |DF p|^2 + alpha |p|^2 with |DF p|^2 from the PSF pass's partials and, for p = r + beta p_old,
+// |p|^2 = |r|^2 + 2 beta Re<r, p_old> + beta^2 |p_old|^2 from those of the CG update pass before.  The solve stops at the
+// rounding floor: |r|^2 <= kCgFloor2 |b|^2 (|r| at the FP32 unit roundoff relative to |b|, including b = 0),
+// Re<p, A p> <= 0 (impossible in exact arithmetic for the positive definite system of Eq. 3) or a non-finite value.
+// This iteration and every later one of the same solve are then empty (cg_stopped).  Non-finite values also set the
+// breakdown flag.
+template <int N>
+__device__ __forceinline__ void cg_decide(const KArgs& A) {
+  __shared__ Pair tot[3];
+  const int nw = ((int)blockDim.x + 31) >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    if (warp == k % nw) {
+      const Pair s = k == 0 ? warp_sum_of(A.dd_part, A.n_dd, kGridScale)
+                            : warp_sum_of(A.rr_part + k * A.n_rr, A.iter > 0 ? A.n_rr : 0, kGridScale);
+      if (lane == 0) tot[k] = s;
+    }
+  __syncthreads();
+  if (threadIdx.x != 0 || A.sc->cg_stop[A.slot] == A.iter) return;    // stopped by the direction pass already
+  const double rr = A.sc->rr[A.iter & 1], beta = A.iter > 0 ? A.sc->beta : 0.0;
+  const double pp = rr + beta * (2.0 * grid_value(tot[1]) + beta * grid_value(tot[2]));
+  // the PSF pass's values carry one more transform factor rs ~ 1/sqrt(N) than DF p; it is divided out as the passes
+  // round it (N in its place is off by up to 5e-7, and CG loses its orthogonality that much sooner)
+  const double rs = (double)rsqrtf((float)N);
+  const double t = grid_value(tot[0]) / (rs * rs) + (double)A.alpha * pp;
+  const bool finite = isfinite(t) && isfinite(rr);
+  A.sc->pq = t;
+  if (finite && rr > kCgFloor2 * A.sc->rr0 && t > 0.0) {
+    A.sc->step[A.iter & 1] = (float)(rr / t);
+  } else {
+    A.sc->cg_stop[A.slot] = A.iter;
+    if (!finite) atomicOr(&A.sc->flags, kFlagBreakdown);
+  }
+}
+
+// prestaged: the twiddles and the side inputs that no launch just before writes were staged by col_stage_side before
+// the dependent-launch wait.
 template <int N1, int N2, int MODE, bool STDF = false, class TC = NoTc, int CC = NLV_COL_C>
-__device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, unsigned char* smem_raw, TC* tc = nullptr,
-                                              bool prestaged = false) {
+__device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, int nblk, unsigned char* smem_raw,
+                                              TC* tc = nullptr, bool prestaged = false) {
   using S = Split<N1, N2>;
   constexpr int N = S::N, E = S::E, C = ColCfg<N1, N2, CC>::C;
+  if constexpr (MODE == COL_IFFT_ADJ_FFT) {
+    if (A.scalars && bid == nblk - 1) {
+      cp_async_wait_all();
+      cg_decide<N>(A);
+      return;
+    }
+  }
   const int lane = threadIdx.x % C, idx = threadIdx.x / C;
   const int f = STDF ? N / 4 : A.f, Wc = STDF ? N / 2 : A.Wc;
   const int strips = (Wc + C - 1) / C;
@@ -807,8 +1194,27 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, unsigned 
       v[m] = val;
     }
   }
+  // ---- CG direction: the W^-1 p of the iteration before on this thread's Omega elements (layout B)
+  [[maybe_unused]] float2 uo[MODE == COL_CG_DIR ? N1 : 1];
+  [[maybe_unused]] float beta = 0.f;
+  __shared__ float s_beta;
+  __shared__ int s_stop;
+  if constexpr (MODE == COL_CG_DIR) {
+    if (idx < N2) {
+#pragma unroll
+      for (int m = 0; m < N1; ++m) {
+        const int e1 = idx + N2 * m;
+        uo[m] = make_float2(0.f, 0.f);
+        if (A.iter > 0 && active && in_omega(e1, N, f)) uo[m] = A.U[cbase + (size_t)to_compact(e1, N, f) * Wc];
+      }
+    }
+  }
   // ---- staged side inputs (Omega rows of this block's columns) and twiddles
-  if (!prestaged) col_stage_side<N1, N2, MODE, STDF, CC>(A, bid, smem_raw);
+  if (!prestaged) col_stage_side<N1, N2, MODE, STDF, CC>(A, bid, smem_raw, true);
+  col_stage_side<N1, N2, MODE, STDF, CC>(A, bid, smem_raw, false);
+  if constexpr (MODE == COL_CG_DIR) {      // while the loads above are in flight; read after the first transform
+    if (A.iter > 0) cg_direction_scalars(A, bid, s_beta, s_stop);
+  }
   cp_async_wait_all();
   __syncthreads();
 
@@ -834,8 +1240,14 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, unsigned 
       }
       return;
     } else {
+      if constexpr (MODE == COL_CG_DIR) {
+        if (A.iter > 0) {
+          if (s_stop) return;          // the same in every block and thread: |r| has reached the rounding floor
+          beta = s_beta;
+        }
+      }
+      if constexpr (MODE == COL_BCG_DIR) beta = (float)A.sc->beta;
       const size_t sstride = (size_t)Wc * C;
-      const float beta = (MODE == COL_IFFT_PROD_FFT && A.pupd) ? cg_beta(A) : 0.f;
       if (idx < N2) {
 #pragma unroll
         for (int m = 0; m < N1; ++m) {
@@ -843,19 +1255,30 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, unsigned 
           float2 out = make_float2(0.f, 0.f);
           if (active && in_omega(e1, N, f)) {
             const int cr = to_compact(e1, N, f);
-            const float2 u = cscale(v[m], rs);
+            float2 u = cscale(v[m], rs);
             const float2 c = side[(size_t)cr * C + lane];
             const float2 rh = side[sstride + (size_t)cr * C + lane];
-            if constexpr (MODE == COL_IFFT_PROD_FFT) {
-              float2 dr = side[2 * sstride + (size_t)cr * C + lane];
-              if (A.pupd) {          // rho part of p = r + beta p (written later by the last row pass)
-                const float2 rv = side[3 * sstride + (size_t)cr * C + lane];
-                dr = make_float2(fmaf(beta, dr.x, rv.x), fmaf(beta, dr.y, rv.y));
-              }
-              out = cadd(cmul(dr, c), cmul(rh, u));
-            } else {  // COL_IFFT_ADJ_FFT
+            if constexpr (MODE == COL_IFFT_ADJ_FFT) {
               A.zsum[cbase + (size_t)cr * Wc] = cmulc(c, u);
               out = cmulc(rh, u);
+            } else {
+              float2 dr;
+              if constexpr (MODE == COL_CG_DIR) {      // W^-1 p and the rho part of p = r + beta p
+                dr = side[3 * sstride + (size_t)cr * C + lane];
+                if (A.iter > 0) {
+                  const float2 po = side[2 * sstride + (size_t)cr * C + lane];
+                  dr = make_float2(fmaf(beta, po.x, dr.x), fmaf(beta, po.y, dr.y));
+                  u = make_float2(fmaf(beta, uo[m].x, u.x), fmaf(beta, uo[m].y, u.y));
+                }
+                A.U[cbase + (size_t)cr * Wc] = u;
+              } else {
+                dr = side[2 * sstride + (size_t)cr * C + lane];
+                if constexpr (MODE == COL_BCG_DIR) {   // the rho part of p = r + beta p (written by the last row pass)
+                  const float2 rv = side[3 * sstride + (size_t)cr * C + lane];
+                  dr = make_float2(fmaf(beta, dr.x, rv.x), fmaf(beta, dr.y, rv.y));
+                }
+              }
+              out = cadd(cmul(dr, c), cmul(rh, u));
             }
           }
           v[m] = out;
@@ -877,17 +1300,17 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, unsigned 
 template <int N1, int N2, int MODE, bool STDF = false, int CC = NLV_COL_C>
 __global__ void __launch_bounds__(ColCfg<N1, N2, CC>::THREADS) col_pass(const KArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int early = cg_flags_early(A);
+  const int early = cg_stop_early(A);
   // before the wait only through L2 (16-byte copies): an odd f stages the natural planes with 8-byte copies,
   // which go through L1, after the wait
   const bool pre = STDF || (A.f & 1) == 0;
-  if (pre) col_stage_side<N1, N2, MODE, STDF, CC>(A, blockIdx.x, smem_raw);
+  if (pre) col_stage_side<N1, N2, MODE, STDF, CC>(A, blockIdx.x, smem_raw, true);
   pdl_enter();
   if (cg_stopped_after(A, early)) {
     cp_async_wait_all();
     return;
   }
-  col_pass_body<N1, N2, MODE, STDF, NoTc, CC>(A, blockIdx.x, smem_raw, nullptr, pre);
+  col_pass_body<N1, N2, MODE, STDF, NoTc, CC>(A, blockIdx.x, gridDim.x, smem_raw, nullptr, pre);
 }
 
 // ------------------------------------------------------------------------------- tensor-core passes ----
@@ -918,7 +1341,7 @@ __global__ void __launch_bounds__(ColCfg<N1, N2>::THREADS, 1) col_pass_tc(const 
   const ColSmem L = col_smem(MODE, S::N, ColCfg<N1, N2>::C, S::SM_LANE_COL, STDF ? S::N / 2 : A.Wc);
   TcDft tc;
   tc.setup(smem_raw + tc_offset(L.total), A.tcB, &A.sc->flags);
-  col_pass_body<N1, N2, MODE, STDF, TcDft>(A, blockIdx.x, smem_raw, &tc);
+  col_pass_body<N1, N2, MODE, STDF, TcDft>(A, blockIdx.x, gridDim.x, smem_raw, &tc);
   tc.teardown();
 }
 
@@ -985,7 +1408,7 @@ __global__ void __launch_bounds__(ColCfg<N1, N2>::THREADS) col_pass_batch(const 
     int bid, nblk;
     const KArgs& A = batch_frame(B, w, bid, nblk);
     if (cg_stopped(A)) continue;
-    col_pass_body<N1, N2, MODE, STDF>(A, bid, smem_raw);
+    col_pass_body<N1, N2, MODE, STDF>(A, bid, nblk, smem_raw);
   }
 }
 
@@ -1007,8 +1430,8 @@ __device__ __noinline__ void row_body_call(const KArgs& A, int bid, int nblk, un
   row_pass_body<N1, N2, MODE, STDF>(A, bid, nblk, smem);
 }
 template <int N1, int N2, int MODE, bool STDF>
-__device__ __noinline__ void col_body_call(const KArgs& A, int bid, unsigned char* smem) {
-  col_pass_body<N1, N2, MODE, STDF>(A, bid, smem);
+__device__ __noinline__ void col_body_call(const KArgs& A, int bid, int nblk, unsigned char* smem) {
+  col_pass_body<N1, N2, MODE, STDF>(A, bid, nblk, smem);
 }
 template <int MODE, bool STDF>
 __device__ __forceinline__ void row_body_of_side(const KArgs& A, int bid, int nblk, unsigned char* smem) {
@@ -1021,13 +1444,13 @@ __device__ __forceinline__ void row_body_of_side(const KArgs& A, int bid, int nb
   }
 }
 template <int MODE, bool STDF>
-__device__ __forceinline__ void col_body_of_side(const KArgs& A, int bid, unsigned char* smem) {
+__device__ __forceinline__ void col_body_of_side(const KArgs& A, int bid, int nblk, unsigned char* smem) {
   switch (A.N) {
-    case 128: col_body_call<8, 16, MODE, STDF>(A, bid, smem); break;
-    case 192: col_body_call<12, 16, MODE, STDF>(A, bid, smem); break;
-    case 256: col_body_call<16, 16, MODE, STDF>(A, bid, smem); break;
-    case 320: col_body_call<16, 20, MODE, STDF>(A, bid, smem); break;
-    default: col_body_call<16, 24, MODE, STDF>(A, bid, smem); break;
+    case 128: col_body_call<8, 16, MODE, STDF>(A, bid, nblk, smem); break;
+    case 192: col_body_call<12, 16, MODE, STDF>(A, bid, nblk, smem); break;
+    case 256: col_body_call<16, 16, MODE, STDF>(A, bid, nblk, smem); break;
+    case 320: col_body_call<16, 20, MODE, STDF>(A, bid, nblk, smem); break;
+    default: col_body_call<16, 24, MODE, STDF>(A, bid, nblk, smem); break;
   }
 }
 
@@ -1051,7 +1474,7 @@ __global__ void __launch_bounds__(kMultiColThreads) col_pass_multi(const BatchAr
     int bid, nblk;
     const KArgs& A = batch_frame(B, w, bid, nblk);
     if (cg_stopped(A)) continue;
-    col_body_of_side<MODE, STDF>(A, bid, smem_raw);
+    col_body_of_side<MODE, STDF>(A, bid, nblk, smem_raw);
   }
 }
 
@@ -1074,6 +1497,7 @@ struct SizeKernels {
   int col_lanes, col_threads;
   int sm_lane;              // shared float2 per lane for one exchange (row passes)
   int sm_lane_col;          // the same for column passes (bank-conflict padding)
+  // Single-frame passes (no batch modes) and batched passes (no single-frame CG modes, no operator-only modes).
   const void* row[NUM_ROW_MODES];
   const void* col[NUM_COL_MODES];
   const void* row_batch[NUM_ROW_MODES];
@@ -1106,13 +1530,36 @@ inline RowGrid row_grid(const SizeKernels* k, int nrows, long rho_pixels, int sm
   const int max_lanes = kRowMaxThreads / k->tl;
   int want = sms * ctas_per_sm;
   if (want > nrows) want = nrows;
-  const int per = (nrows + want - 1) / want;
+  // at least a warp of threads a block: narrower blocks only add partial sums for the next pass to read (64^2 with
+  // 4 coils: 256 blocks of 8 threads)
+  int per = (nrows + want - 1) / want;
+  if (per * k->tl < 32) per = std::min((32 + k->tl - 1) / k->tl, nrows);
   const int rounds = (per + max_lanes - 1) / max_lanes;
   g.lanes = (per + rounds - 1) / rounds;
   g.rows_per_cta = per;
   g.blocks = (nrows + per - 1) / per;
   g.rho_per_cta = (int)((rho_pixels + g.blocks - 1) / g.blocks);
   return g;
+}
+
+// The CG passes of single frames (q_cg_iter in nlinv.cu) and of batches (q_bcg_iter).
+template <int N1, int N2, int CC = NLV_COL_C> void add_frame_cg_cols(SizeKernels& k) {
+  k.col[COL_CG_DIR] = (const void*)col_pass<N1, N2, COL_CG_DIR, false, CC>;
+  k.col_std[COL_CG_DIR] = (const void*)col_pass<N1, N2, COL_CG_DIR, true, CC>;
+}
+template <int N1, int N2> void add_frame_cg(SizeKernels& k) {
+  k.row[ROW_CG_RHS] = (const void*)row_pass<N1, N2, ROW_CG_RHS>;
+  k.row[ROW_CG_PSF] = (const void*)row_pass<N1, N2, ROW_CG_PSF>;
+  k.row_std[ROW_CG_PSF] = (const void*)row_pass<N1, N2, ROW_CG_PSF, true>;
+  k.row[ROW_CG_UPDATE] = (const void*)row_pass<N1, N2, ROW_CG_UPDATE>;
+  k.row_std[ROW_CG_UPDATE] = (const void*)row_pass<N1, N2, ROW_CG_UPDATE, true>;
+  add_frame_cg_cols<N1, N2>(k);
+}
+template <int N1, int N2> void add_batch_cg(SizeKernels& k) {
+  k.row_batch[ROW_BCG_RHS] = (const void*)row_pass_batch<N1, N2, ROW_BCG_RHS>;
+  k.row_std_batch[ROW_BCG_DIR] = (const void*)row_pass_batch<N1, N2, ROW_BCG_DIR, true>;
+  k.row_std_batch[ROW_BCG_NORMAL] = (const void*)row_pass_batch<N1, N2, ROW_BCG_NORMAL, true>;
+  k.col_std_batch[COL_BCG_DIR] = (const void*)col_pass_batch<N1, N2, COL_BCG_DIR, true>;
 }
 
 // Tuning variants of a side (nlinv_autotune): the default table with other column-strip widths, and the single-frame
@@ -1127,6 +1574,7 @@ template <int N1, int N2, int CC> SizeKernels make_size_kernels_strip(const Size
   s.col[COL_IFFT_PROD_FFT] = (const void*)col_pass<N1, N2, COL_IFFT_PROD_FFT, false, CC>;
   s.col[COL_IFFT_ADJ_FFT] = (const void*)col_pass<N1, N2, COL_IFFT_ADJ_FFT, false, CC>;
   for (int m = 0; m < NUM_COL_MODES; ++m) s.col_std[m] = nullptr;
+  add_frame_cg_cols<N1, N2, CC>(s);
   s.col_std[COL_IFFT_PROD_FFT] = (const void*)col_pass<N1, N2, COL_IFFT_PROD_FFT, true, CC>;
   for (int m = 0; m < NUM_ROW_MODES; ++m) s.row_batch[m] = s.row_std_batch[m] = s.row_tc[m] = s.row_tc_std[m] = nullptr;
   for (int m = 0; m < NUM_COL_MODES; ++m) s.col_batch[m] = s.col_std_batch[m] = s.col_tc[m] = s.col_tc_std[m] = nullptr;
@@ -1149,7 +1597,6 @@ template <int N1, int N2> SizeKernels make_size_kernels_single() {
   s.row[ROW_P_IFFT] = (const void*)row_pass<N1, N2, ROW_P_IFFT>;
   s.row[ROW_FFT_W_ADJ] = (const void*)row_pass<N1, N2, ROW_FFT_W_ADJ>;
   s.row[ROW_FFT_W_NORMAL] = (const void*)row_pass<N1, N2, ROW_FFT_W_NORMAL>;
-  s.row[ROW_FFT_W_RHS] = (const void*)row_pass<N1, N2, ROW_FFT_W_RHS>;
   s.col[COL_IFFT_C] = (const void*)col_pass<N1, N2, COL_IFFT_C>;
   s.col[COL_PROD_FFT] = (const void*)col_pass<N1, N2, COL_PROD_FFT>;
   s.col[COL_SIM_FFT] = (const void*)col_pass<N1, N2, COL_SIM_FFT>;
@@ -1159,6 +1606,7 @@ template <int N1, int N2> SizeKernels make_size_kernels_single() {
   s.row_std[ROW_PSF] = (const void*)row_pass<N1, N2, ROW_PSF, true>;
   s.row_std[ROW_FFT_W_NORMAL] = (const void*)row_pass<N1, N2, ROW_FFT_W_NORMAL, true>;
   s.col_std[COL_IFFT_PROD_FFT] = (const void*)col_pass<N1, N2, COL_IFFT_PROD_FFT, true>;
+  add_frame_cg<N1, N2>(s);
   return s;
 }
 
@@ -1178,7 +1626,6 @@ template <int N1, int N2> SizeKernels make_size_kernels() {
   s.row[ROW_P_IFFT] = (const void*)row_pass<N1, N2, ROW_P_IFFT>;
   s.row[ROW_FFT_W_ADJ] = (const void*)row_pass<N1, N2, ROW_FFT_W_ADJ>;
   s.row[ROW_FFT_W_NORMAL] = (const void*)row_pass<N1, N2, ROW_FFT_W_NORMAL>;
-  s.row[ROW_FFT_W_RHS] = (const void*)row_pass<N1, N2, ROW_FFT_W_RHS>;
   s.col[COL_IFFT_C] = (const void*)col_pass<N1, N2, COL_IFFT_C>;
   s.col[COL_PROD_FFT] = (const void*)col_pass<N1, N2, COL_PROD_FFT>;
   s.col[COL_SIM_FFT] = (const void*)col_pass<N1, N2, COL_SIM_FFT>;
@@ -1191,7 +1638,6 @@ template <int N1, int N2> SizeKernels make_size_kernels() {
   s.row_batch[ROW_P_IFFT] = (const void*)row_pass_batch<N1, N2, ROW_P_IFFT>;
   s.row_batch[ROW_FFT_W_ADJ] = (const void*)row_pass_batch<N1, N2, ROW_FFT_W_ADJ>;
   s.row_batch[ROW_FFT_W_NORMAL] = (const void*)row_pass_batch<N1, N2, ROW_FFT_W_NORMAL>;
-  s.row_batch[ROW_FFT_W_RHS] = (const void*)row_pass_batch<N1, N2, ROW_FFT_W_RHS>;
   s.col_batch[COL_IFFT_C] = (const void*)col_pass_batch<N1, N2, COL_IFFT_C>;
   s.col_batch[COL_PROD_FFT] = (const void*)col_pass_batch<N1, N2, COL_PROD_FFT>;
   s.col_batch[COL_SIM_FFT] = (const void*)col_pass_batch<N1, N2, COL_SIM_FFT>;
@@ -1207,6 +1653,8 @@ template <int N1, int N2> SizeKernels make_size_kernels() {
   s.row_std_batch[ROW_PSF] = (const void*)row_pass_batch<N1, N2, ROW_PSF, true>;
   s.row_std_batch[ROW_FFT_W_NORMAL] = (const void*)row_pass_batch<N1, N2, ROW_FFT_W_NORMAL, true>;
   s.col_std_batch[COL_IFFT_PROD_FFT] = (const void*)col_pass_batch<N1, N2, COL_IFFT_PROD_FFT, true>;
+  add_frame_cg<N1, N2>(s);
+  add_batch_cg<N1, N2>(s);
   return s;
 }
 
@@ -1221,15 +1669,21 @@ template <int N1, int N2> SizeKernels make_size_kernels_tc() {
   s.row_tc[ROW_P_IFFT] = (const void*)row_pass_tc<N1, N2, ROW_P_IFFT, false>;
   s.row_tc[ROW_FFT_W_ADJ] = (const void*)row_pass_tc<N1, N2, ROW_FFT_W_ADJ, false>;
   s.row_tc[ROW_FFT_W_NORMAL] = (const void*)row_pass_tc<N1, N2, ROW_FFT_W_NORMAL, false>;
-  s.row_tc[ROW_FFT_W_RHS] = (const void*)row_pass_tc<N1, N2, ROW_FFT_W_RHS, false>;
+  s.row_tc[ROW_CG_RHS] = (const void*)row_pass_tc<N1, N2, ROW_CG_RHS, false>;
+  s.row_tc[ROW_CG_PSF] = (const void*)row_pass_tc<N1, N2, ROW_CG_PSF, false>;
+  s.row_tc[ROW_CG_UPDATE] = (const void*)row_pass_tc<N1, N2, ROW_CG_UPDATE, false>;
   s.col_tc[COL_IFFT_C] = (const void*)col_pass_tc<N1, N2, COL_IFFT_C, false>;
   s.col_tc[COL_PROD_FFT] = (const void*)col_pass_tc<N1, N2, COL_PROD_FFT, false>;
   s.col_tc[COL_SIM_FFT] = (const void*)col_pass_tc<N1, N2, COL_SIM_FFT, false>;
   s.col_tc[COL_IFFT_PROD_FFT] = (const void*)col_pass_tc<N1, N2, COL_IFFT_PROD_FFT, false>;
   s.col_tc[COL_IFFT_ADJ_FFT] = (const void*)col_pass_tc<N1, N2, COL_IFFT_ADJ_FFT, false>;
+  s.col_tc[COL_CG_DIR] = (const void*)col_pass_tc<N1, N2, COL_CG_DIR, false>;
   s.row_tc_std[ROW_PSF] = (const void*)row_pass_tc<N1, N2, ROW_PSF, true>;
   s.row_tc_std[ROW_FFT_W_NORMAL] = (const void*)row_pass_tc<N1, N2, ROW_FFT_W_NORMAL, true>;
+  s.row_tc_std[ROW_CG_PSF] = (const void*)row_pass_tc<N1, N2, ROW_CG_PSF, true>;
+  s.row_tc_std[ROW_CG_UPDATE] = (const void*)row_pass_tc<N1, N2, ROW_CG_UPDATE, true>;
   s.col_tc_std[COL_IFFT_PROD_FFT] = (const void*)col_pass_tc<N1, N2, COL_IFFT_PROD_FFT, true>;
+  s.col_tc_std[COL_CG_DIR] = (const void*)col_pass_tc<N1, N2, COL_CG_DIR, true>;
   return s;
 }
 

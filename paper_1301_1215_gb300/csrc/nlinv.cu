@@ -6,8 +6,8 @@
 //   DF dx          P FFT(M (drho c_j + rho W^-1 dchat_j))       row ROW_W_IFFT, col COL_IFFT_PROD_FFT, row ROW_FFT_P_OUT
 //   DF^H r         (sum_j conj(c_j) z_j, w FFT(conj(rho) z_j)) row ROW_P_IFFT, col COL_IFFT_ADJ_FFT, row ROW_FFT_W_ADJ
 //   (DF^H DF + alpha) p   the PSF form of Sec. 3.1: row ROW_W_IFFT, col COL_IFFT_PROD_FFT, row ROW_PSF,
-//                         col COL_IFFT_ADJ_FFT, row ROW_FFT_W_NORMAL (+ Re<p, q>)
-//   CG updates     dx += alpha p, r -= alpha q (+ |r|^2); p = r + beta p
+//                         col COL_IFFT_ADJ_FFT, row ROW_FFT_W_NORMAL
+//   CG iteration   col COL_CG_DIR, row ROW_PSF, col COL_IFFT_ADJ_FFT, row ROW_CG_UPDATE (q_cg_iter)
 // Each operator application performs the two 2D transforms per operator of Table 1, batched over all coils.
 // Beyond the paper's method: the gradient through the reconstruction (nlinv_reconstruct_checkpoints and
 // nlinv_reconstruct_vjp: the same operators at other linearisation points, plus a CG solve per Newton step),
@@ -38,11 +38,11 @@ namespace {
 thread_local std::string g_create_error;
 
 // ------------------------------------------------------------------------------------------ vector kernels ----
-// float4 groups of CG-step operands in flight per thread.  Two keep the kernel at 64 registers, four blocks of 256
+// The CG step of batches.  float4 groups of its operands in flight per thread.  Two keep the kernel at 64 registers, four blocks of 256
 // threads per SM; four groups need 96 registers (two blocks per SM, measured 13.2 against 11.5 us per step at
 // 384 x 384 with 10 coils) or spill at 64.
 constexpr int kCgGroups = 2;
-// dx += alpha p; r -= alpha q; partial of |r|^2 -> rr_part[bid], over this block's share of the A.n2 float4.
+// dx += alpha p; r -= alpha q; partial of |r|^2 -> brr_part[bid], over this block's share of the A.n2 float4.
 // A thread sums the squares of at most two float4 (8 products) in FP32 before adding them to its FP64 partial.
 __device__ __forceinline__ void cg_step_update(float4& d, float4& r, const float4& p, const float4& q, float a,
                                                float& acc) {
@@ -59,14 +59,13 @@ __device__ __forceinline__ void cg_step_decide(const KArgs& A, int bid, float& s
   for (int k = threadIdx.x; k < A.n_pq; k += blockDim.x) t += A.pq_part[k];
   t = nlv::block_sum(t, red);
   if (threadIdx.x == 0) {
-    const double rr = A.sc->rr;
-    const int flags = *(volatile int*)&A.sc->flags;
-    const bool was_stopped = (flags & nlv::kFlagCgStopped) != 0;
+    const double rr = A.sc->rr[0];
+    const bool was_stopped = nlv::cg_stopped(A);
     double a = 0.0;
     bool stop = false;
     if (!was_stopped) {
       if (!isfinite(t) || !isfinite(rr)) {
-        if (bid == 0) A.sc->flags |= nlv::kFlagBreakdown;
+        if (bid == 0) atomicOr(&A.sc->flags, nlv::kFlagBreakdown);
         stop = true;
       } else if (rr > nlv::kCgFloor2 * A.sc->rr0 && t > 0.0) {
         a = rr / t;
@@ -78,10 +77,7 @@ __device__ __forceinline__ void cg_step_decide(const KArgs& A, int bid, float& s
       A.sc->pq = t;
       A.sc->alpha = a;
       A.sc->rr_prev = rr;
-      if (stop) {
-        A.sc->flags |= nlv::kFlagCgStopped;
-        A.sc->cg_stop[A.slot] = A.iter;
-      }
+      if (stop) A.sc->cg_stop[A.slot] = A.iter;
     }
     s_alpha = (float)a;
     s_skip = was_stopped ? 1 : 0;     // stopped by an earlier iteration: nothing to update
@@ -89,7 +85,7 @@ __device__ __forceinline__ void cg_step_decide(const KArgs& A, int bid, float& s
   __syncthreads();
 }
 
-template <int G = 2>
+template <int G>
 __device__ __forceinline__ void cg_step_body(const KArgs& A, int bid, int nblk) {
   const float4* __restrict__ p4 = (const float4*)A.p;
   const float4* __restrict__ q4 = (const float4*)A.q;
@@ -100,9 +96,8 @@ __device__ __forceinline__ void cg_step_body(const KArgs& A, int bid, int nblk) 
   // fixed order).  The solve stops at the rounding floor: |r|^2 <= kCgFloor2 |b|^2 (|r| at the FP32 unit roundoff
   // relative to |b|, including b = 0), Re<p, A p> <= 0 (impossible in exact arithmetic for the positive definite
   // system of Eq. 3) or a non-finite value.  This step and every later step of the same solve are then empty
-  // (alpha = 0), through a flag latched in the scalars until the next right-hand side, and block 0 records the
-  // iteration.  Non-finite values also set the breakdown flag.  Every block takes the same decision from the same
-  // partials, so a block that already sees the flag set by block 0 in this launch decides as block 0 did.
+  // (alpha = 0): block 0 records the iteration, and the passes of later iterations skip (cg_stopped).  Non-finite values
+  // also set the breakdown flag.  Every block takes the same decision from the same partials.
   const long stride = (long)nblk * blockDim.x;
   long i = bid * (long)blockDim.x + threadIdx.x;
   float4 pg[G], qg[G], rg[G], dg[G];
@@ -138,150 +133,7 @@ __device__ __forceinline__ void cg_step_body(const KArgs& A, int bid, int nblk) 
     i += G * stride;
   }
   const double s = nlv::block_sum(accd, red);
-  if (threadIdx.x == 0) A.rr_part[bid] = s;
-}
-
-// ------------------------------------------------------------------ CG step with bulk asynchronous copies ----
-// The single-frame CG step as a persistent kernel, one block per SM: the vector is cut into chunks of kBulkChunk
-// float4 per array, and a block's chunks (b, b + nblk, ...) stream p, q, r and dx through a ring of kBulkStages
-// shared-memory stages filled by cp.async.bulk (one thread issues four bulk copies per chunk, completion counted in
-// bytes on the stage's mbarrier), so that up to kBulkStages chunks -- 3 x 64 KB -- are in flight per SM without
-// holding them in registers.  Each thread then updates its share of the chunk from shared memory and stores dx and
-// r directly.  Every wait is bounded (about a second of clock cycles): on a timeout the kernel sets
-// kFlagCopyTimeout, waits once more (bounded) for its copies in flight and returns; the host reports ECUDA.
-constexpr int kBulkThreads = 512;
-constexpr int kBulkChunk = 1024;        // float4 per array per chunk (16 KB)
-constexpr int kBulkStages = 3;
-constexpr size_t kBulkSmem = (size_t)kBulkStages * 4 * kBulkChunk * sizeof(float4) + kBulkStages * 8;
-constexpr int kFlagCopyTimeout = 8;     // Scalars::flags bit: a bulk-copy completion wait timed out
-
-__device__ __forceinline__ uint32_t shared_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Waits (bounded by about a second of clock cycles) for the phase of parity `parity` of the mbarrier at bar.
-__device__ __forceinline__ bool bulk_wait(uint32_t bar, uint32_t parity) {
-  const long long t0 = clock64();
-  for (;;) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (ok) return true;
-    if (clock64() - t0 > 2000000000LL) return false;
-    __nanosleep(20);
-  }
-}
-
-// Bytes per array of chunk c.
-__device__ __forceinline__ uint32_t bulk_bytes(const KArgs& A, long c) {
-  const long off = c * kBulkChunk;
-  return (uint32_t)(((A.n2 - off) < kBulkChunk ? (A.n2 - off) : kBulkChunk) * sizeof(float4));
-}
-// Thread 0: the stage's barrier expects the four arrays of chunk c (one arrival with their byte count).
-__device__ __forceinline__ void bulk_expect(const KArgs& A, uint32_t bar, long c) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}"
-               ::"r"(bar), "r"(4u * bulk_bytes(A, c)) : "memory");
-}
-// Thread 0: array a (0 p, 1 q, 2 r, 3 dx) of chunk c into stage s, completion counted on the stage's barrier.
-__device__ __forceinline__ void bulk_copy(const KArgs& A, float4* ring, uint32_t bar, long c, int s, int a) {
-  const float4* src = (const float4*)(a == 0 ? A.p : a == 1 ? A.q : a == 2 ? A.r : A.dx);
-  const uint32_t dst = shared_addr(ring + ((size_t)s * 4 + a) * kBulkChunk);
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst), "l"(src + c * kBulkChunk), "r"(bulk_bytes(A, c)), "r"(bar) : "memory");
-}
-// Thread 0: chunk c of the four arrays into stage s.
-__device__ __forceinline__ void bulk_issue(const KArgs& A, float4* ring, uint32_t bar, long c, int s) {
-  bulk_expect(A, bar, c);
-#pragma unroll
-  for (int a = 0; a < 4; ++a) bulk_copy(A, ring, bar, c, s, a);
-}
-
-// With src_early, the first stages' copies of r, dx and of p beyond its rho plane are issued before the
-// dependent-launch wait: the kernel before (the normal-operator pass) writes q and the rho plane of p, and r, dx and
-// the coil planes of p were written two or more launches back (see cg_flags_early in kernels.cuh); q and the rest
-// of p follow the wait.  Without it (back-to-back launches of this kernel alone) every copy follows the wait.
-__global__ void __launch_bounds__(kBulkThreads, 1) cg_step_bulk(const KArgs A) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  float4* ring = (float4*)smem_raw;
-  const uint32_t bar0 = shared_addr(smem_raw + (size_t)kBulkStages * 4 * kBulkChunk * sizeof(float4));
-  const int bid = blockIdx.x, nblk = gridDim.x;
-  const long nchunks = (A.n2 + kBulkChunk - 1) / kBulkChunk;
-  const long mine = bid < nchunks ? (nchunks - bid + nblk - 1) / nblk : 0;   // chunks bid, bid + nblk, ...
-  const long rho4 = A.src_early ? (long)A.N * A.N / 2 : A.n2;   // float4 of the rho plane (src_early = 0: all)
-  if (threadIdx.x == 0) {
-    for (int st = 0; st < kBulkStages; ++st)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8u * st) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  const long first = mine < kBulkStages ? mine : kBulkStages;
-  if (threadIdx.x == 0) {
-    for (long k = 0; k < first; ++k) {
-      const long ch = bid + k * nblk;
-      const uint32_t bar = bar0 + 8u * (uint32_t)k;
-      bulk_expect(A, bar, ch);
-      if (A.src_early) {
-        bulk_copy(A, ring, bar, ch, (int)k, 2);
-        bulk_copy(A, ring, bar, ch, (int)k, 3);
-      }
-      if (ch * kBulkChunk >= rho4) bulk_copy(A, ring, bar, ch, (int)k, 0);
-    }
-  }
-  nlv::pdl_enter();
-  if (threadIdx.x == 0) {
-    for (long k = 0; k < first; ++k) {
-      const long ch = bid + k * nblk;
-      const uint32_t bar = bar0 + 8u * (uint32_t)k;
-      bulk_copy(A, ring, bar, ch, (int)k, 1);
-      if (ch * kBulkChunk < rho4) bulk_copy(A, ring, bar, ch, (int)k, 0);
-      if (!A.src_early) {
-        bulk_copy(A, ring, bar, ch, (int)k, 2);
-        bulk_copy(A, ring, bar, ch, (int)k, 3);
-      }
-    }
-  }
-  __shared__ float s_alpha;
-  __shared__ int s_skip;
-  __shared__ double red[32];
-  cg_step_decide(A, bid, s_alpha, s_skip, red);
-  bool timed_out = false;
-  if (s_skip) {                       // stopped earlier: let the copies already issued land, then leave
-    for (long k = 0; k < first; ++k) bulk_wait(bar0 + 8u * (uint32_t)k, 0);
-    return;
-  }
-  const float a = s_alpha;
-  float4* __restrict__ r4 = (float4*)A.r;
-  float4* __restrict__ dx4 = (float4*)A.dx;
-  double accd = 0.0;
-  for (long k = 0; k < mine; ++k) {
-    const int st = (int)(k % kBulkStages);
-    const uint32_t bar = bar0 + 8u * st;
-    if (!bulk_wait(bar, (uint32_t)((k / kBulkStages) & 1))) timed_out = true;
-    const long off = (bid + k * nblk) * kBulkChunk;
-    const long cnt = (A.n2 - off) < kBulkChunk ? (A.n2 - off) : kBulkChunk;
-    const float4* sp = ring + ((size_t)st * 4 + 0) * kBulkChunk;
-    const float4* sq = sp + kBulkChunk;
-    const float4* sr = sq + kBulkChunk;
-    const float4* sd = sr + kBulkChunk;
-    float acc = 0.f;
-    for (long e = threadIdx.x; e < cnt; e += kBulkThreads) {
-      float4 d = sd[e], r = sr[e];
-      cg_step_update(d, r, sp[e], sq[e], a, acc);
-      dx4[off + e] = d;
-      r4[off + e] = r;
-    }
-    accd += (double)acc;
-    __syncthreads();                  // every thread is done with stage st
-    if (threadIdx.x == 0 && k + kBulkStages < mine) {
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      bulk_issue(A, ring, bar, bid + (k + kBulkStages) * nblk, st);
-    }
-  }
-  if (timed_out) {
-    if (threadIdx.x == 0) atomicOr(&A.sc->flags, kFlagCopyTimeout);
-    for (long k = (mine > kBulkStages ? mine - kBulkStages : 0); k < mine; ++k)
-      bulk_wait(bar0 + 8u * (uint32_t)(k % kBulkStages), (uint32_t)((k / kBulkStages) & 1));
-  }
-  const double sblk = nlv::block_sum(accd, red);
-  if (threadIdx.x == 0) A.rr_part[bid] = sblk;
+  if (threadIdx.x == 0) A.brr_part[bid] = s;
 }
 
 // x += dx (x = A.dst)
@@ -292,6 +144,31 @@ __device__ __forceinline__ void add_body(const KArgs& A, int bid, int nblk) {
     float4 d = d4[i], x = x4[i];
     x.x += d.x; x.y += d.y; x.z += d.z; x.w += d.w;
     x4[i] = x;
+  }
+}
+
+// out = base + dx_total (out = A.dst, base = A.src or zero): the end of a CG solve.  The CG update pass adds the steps of
+// an even iteration and of the odd one after it to A.dx together, in the odd one (the first pair without reading it),
+// so that after an odd number of executed iterations the last step a p is still to be added, and A.dx holds nothing
+// before iteration 1.  A.iter: the scheduled iterations; A.slot: the Newton step.
+__global__ void cg_finish_kernel(const KArgs A) {
+  nlv::pdl_enter();
+  const int stop = A.sc->cg_stop[A.slot];
+  const int done = stop < 0 ? A.iter : stop;
+  const bool has_dx = done >= 2, has_p = (done & 1) != 0;
+  const float a = has_p ? A.sc->step[0] : 0.f;        // the last executed iteration is an even one
+  const float4* __restrict__ d4 = (const float4*)A.dx;
+  const float4* __restrict__ p4 = (const float4*)A.p;
+  const float4* x4 = (const float4*)A.src;
+  float4* o4 = (float4*)A.dst;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < A.n2; i += (long)gridDim.x * blockDim.x) {
+    const float4 x = x4 ? x4[i] : zero, p = has_p ? p4[i] : zero;
+    float4 d = has_dx ? d4[i] : zero;
+    if (has_p) {
+      d.x = fmaf(a, p.x, d.x); d.y = fmaf(a, p.y, d.y); d.z = fmaf(a, p.z, d.z); d.w = fmaf(a, p.w, d.w);
+    }
+    o4[i] = make_float4(x.x + d.x, x.y + d.y, x.z + d.z, x.w + d.w);
   }
 }
 
@@ -313,16 +190,6 @@ __global__ void image_kernel(const KArgs A) {
   }
 }
 
-// 256 threads, at most 64 registers: four blocks fit on an SM (the default vector grid)
-template <int G>
-__global__ void __launch_bounds__(256, 4) cg_step_kernel(const KArgs A) {
-  nlv::pdl_enter();
-  cg_step_body<G>(A, blockIdx.x, gridDim.x);
-}
-__global__ void add_kernel(const KArgs A) {
-  nlv::pdl_enter();
-  add_body(A, blockIdx.x, gridDim.x);
-}
 // out = alpha X + coef Y (X = A.src, Y = A.q, out = A.dst) over A.n2 float4
 __global__ void axpby_kernel(const KArgs A) {
   nlv::pdl_enter();
@@ -336,26 +203,19 @@ __global__ void axpby_kernel(const KArgs A) {
   }
 }
 
-// CG from dx = 0 for the right-hand side b = A.src: r = p = b, dx = 0, |b|^2 -> RED_RR_INIT
+// CG from dx = 0 for the right-hand side b = A.src: r = b, |b|^2 -> RED_RR_INIT
 __global__ void cg_init_kernel(const KArgs A) {
   nlv::pdl_enter();
   const float4* __restrict__ b4 = (const float4*)A.src;
   float4* __restrict__ r4 = (float4*)A.r;
-  float4* __restrict__ p4 = (float4*)A.pout;
-  float4* __restrict__ d4 = (float4*)A.dx;
   double acc = 0.0;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < A.n2; i += (long)gridDim.x * blockDim.x) {
     const float4 b = b4[i];
     r4[i] = b;
-    p4[i] = b;
-    d4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     acc += (double)(b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w);
   }
   nlv::grid_reduce(acc, A, blockIdx.x, gridDim.x);
 }
-
-// the single-frame CG step
-const void* cg_step_fn() { return (const void*)cg_step_kernel<kCgGroups>; }
 
 __global__ void __launch_bounds__(256, 4) cg_step_batch(const nlv::BatchArgs B) {
   nlv::pdl_enter();
@@ -381,7 +241,7 @@ constexpr double kTuneMargin = 0.03; // a candidate replaces the compiled defaul
 #ifndef NLV_VEC_BLOCKS_PER_SM
 #define NLV_VEC_BLOCKS_PER_SM 4   // blocks per SM of the vector passes
 #endif
-constexpr int kProfileKernels = 6;   // kernels of one CG iteration, in the order nlinv_profile_cg reports them
+constexpr int kProfileSteps = 6;   // steps of one CG iteration, in the order nlinv_profile_cg reports them
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
@@ -403,14 +263,18 @@ struct nlinv_ctx {
   // workspace (one allocation)
   void* base = nullptr;
   float2 *x = nullptr, *xref = nullptr, *y = nullptr, *r0 = nullptr;
-  float2 *r = nullptr, *p = nullptr, *q = nullptr, *dx = nullptr;
+  float2 *r = nullptr, *p = nullptr, *dx = nullptr;
+  float2* q = nullptr;        // A p (frames of a batch)
   float2 *T = nullptr, *coil = nullptr, *zsum = nullptr;
+  float2* U = nullptr;        // W^-1 p on Omega of the CG direction (single frames)
   float2 *twA = nullptr, *twB = nullptr;
   float* wtab = nullptr;      // Sobolev weight, N x N
   uint8_t* mask = nullptr;
   double* partials = nullptr;
-  double* pq_part = nullptr;  // per-block partials of Re<p, A p> of the normal-operator pass
-  double* rr_part = nullptr;  // per-block partials of |r|^2 of the CG step
+  double* pq_part = nullptr;  // frames of a batch: per-block partials of Re<p, A p> and of |r|^2
+  double* brr_part = nullptr;
+  nlv::Pair* dd_part = nullptr;  // single frames: per-block partials of |DF p|^2 of the PSF pass
+  nlv::Pair* rr_part = nullptr;  // per-block partials of |r|^2, Re<r, p> and |p|^2 of the CG update pass
   Scalars* sc = nullptr;
   // graph of one reconstruction
   cudaGraphExec_t graph = nullptr;
@@ -423,7 +287,9 @@ struct nlinv_ctx {
     int grid, block;
     size_t smem;
     KArgs args;
+    int step;                 // 1..6: pass of the CG iteration that nlinv_batch_profile_cg times, 0 otherwise
   };
+  int rec_step = 0;           // the `step` of the launches being recorded
   std::vector<Rec>* rec = nullptr;   // non-null: launches are recorded instead of issued
   bool pdl = true;            // programmatic dependent launches (NLINV_PDL=0 turns them off)
   bool std_fov = false;       // fov = N/4: the passes specialised for it (SizeKernels::row_std, col_std) apply
@@ -503,7 +369,7 @@ int col_blocks(const nlinv_ctx* c) {
 cudaError_t launch(nlinv_ctx* c, const void* fn, int grid, int block, size_t smem, void** args) {
   c->launches++;
   if (c->rec) {                       // every pass takes one KArgs
-    c->rec->push_back({fn, grid, block, smem, *(const KArgs*)args[0]});
+    c->rec->push_back({fn, grid, block, smem, *(const KArgs*)args[0], c->rec_step});
     return cudaSuccess;
   }
   cudaLaunchConfig_t cfg{};
@@ -520,7 +386,7 @@ cudaError_t launch(nlinv_ctx* c, const void* fn, int grid, int block, size_t sme
 }
 
 cudaError_t row(nlinv_ctx* c, int mode, KArgs a) {
-  const bool rho = (mode == nlv::ROW_FFT_W_ADJ || mode == nlv::ROW_FFT_W_NORMAL || mode == nlv::ROW_FFT_W_RHS);
+  const bool rho = mode >= nlv::ROW_FFT_W_ADJ && mode != nlv::ROW_CG_PSF && mode != nlv::ROW_BCG_DIR;
   const nlv::RowGrid g = row_geom(c, rho);
   a.nrows = c->J * c->N;
   a.rows_per_cta = g.rows_per_cta;
@@ -531,18 +397,23 @@ cudaError_t row(nlinv_ctx* c, int mode, KArgs a) {
     return launch(c, fn, g.blocks, g.lanes * c->k->tl, c->k->row_smem_tc(mode, g.lanes), args);
   }
   const void* fn = (c->std_fov && c->k->row_std[mode]) ? c->k->row_std[mode] : c->k->row[mode];
+  if (c->batch_lanes > 0)           // recorded for the batch's launch
+    fn = c->k->row_std_batch[mode] ? c->k->row_std_batch[mode] : c->k->row_batch[mode];
   return launch(c, fn, g.blocks, g.lanes * c->k->tl, c->k->row_smem(mode, g.lanes), args);
 }
 
 cudaError_t col(nlinv_ctx* c, int mode, KArgs a) {
   a.nrows = c->J;
+  const int blocks = col_blocks(c) + (a.scalars ? 1 : 0);
   void* args[] = {&a};
   if (c->tc) {
     const void* fn = (c->std_fov && c->k->col_tc_std[mode]) ? c->k->col_tc_std[mode] : c->k->col_tc[mode];
-    return launch(c, fn, col_blocks(c), c->k->col_threads, c->k->col_smem_tc(mode, c->Wc), args);
+    return launch(c, fn, blocks, c->k->col_threads, c->k->col_smem_tc(mode, c->Wc), args);
   }
   const void* fn = (c->std_fov && c->k->col_std[mode]) ? c->k->col_std[mode] : c->k->col[mode];
-  return launch(c, fn, col_blocks(c), c->k->col_threads, c->k->col_smem(mode, c->Wc), args);
+  if (c->batch_lanes > 0)
+    fn = c->k->col_std_batch[mode] ? c->k->col_std_batch[mode] : c->k->col_batch[mode];
+  return launch(c, fn, blocks, c->k->col_threads, c->k->col_smem(mode, c->Wc), args);
 }
 
 // c_j = W^-1 chat_j on Omega, for the coil planes of x (1+J planes).
@@ -583,11 +454,9 @@ cudaError_t q_dir(nlinv_ctx* c, const float2* x, const float2* d) {
   return col(c, nlv::COL_IFFT_PROD_FFT, a);
 }
 
-// T <- FFT_col(conj(rho) z_j), zsum_j <- conj(c_j) z_j, with z_j = M FFT^-1_col(T).  in_cg: a launch of the CG
-// iteration (skipped once the solve has stopped).
-cudaError_t q_adj_col(nlinv_ctx* c, const float2* x, bool in_cg = false) {
+// T <- FFT_col(conj(rho) z_j), zsum_j <- conj(c_j) z_j, with z_j = M FFT^-1_col(T).
+cudaError_t q_adj_col(nlinv_ctx* c, const float2* x) {
   KArgs a = base_args(c);
-  a.cgskip = in_cg ? nlv::kCgSkipEarly : 0;
   a.src = c->T;
   a.dst = c->T;
   a.rho = x;
@@ -596,112 +465,195 @@ cudaError_t q_adj_col(nlinv_ctx* c, const float2* x, bool in_cg = false) {
   return col(c, nlv::COL_IFFT_ADJ_FFT, a);
 }
 
-// Blocks of the CG step, i.e. the |r|^2 partials the next iteration's first pass adds: one per SM for the bulk-copy
-// form of single frames, the vector grid for batch frames.
-int cg_blocks(const nlinv_ctx* c) { return c->batch_lanes > 0 ? c->vec_blocks : c->sms; }
-
-// dx += alpha p, r -= alpha q, partials of |r|^2; alpha from the n_pq partials of the normal-operator pass.
-// newton / iter: indices of the Newton step and of the CG iteration (recorded if the solve stops here).
-cudaError_t q_cg_step(nlinv_ctx* c, int n_pq, int newton, int iter, bool early = true) {
+// End of a CG solve: out = base + dx_total (base NULL: dx_total alone).
+cudaError_t q_cg_finish(nlinv_ctx* c, const float2* base, float2* out, int newton) {
   KArgs a = base_args(c);
-  a.cgskip = nlv::kCgSkipAfterWait;
-  a.src_early = early ? 1 : 0;
+  a.src = base;
+  a.dst = out;
+  a.dx = c->dx;
+  a.p = c->p;
+  a.iter = c->prm.cg_iters;
+  a.slot = newton;
+  a.n2 = c->vec / 2;
+  void* args[] = {&a};
+  return launch(c, (const void*)cg_finish_kernel, c->vec_blocks, kVecThreads, 0, args);
+}
+
+// One CG iteration i on (DF^H DF + alpha) for linearisation point x, in four passes.  W^-1 and its row transform are
+// linear, so the row pass that finishes q = (DF^H DF + alpha) p goes straight on to r_{i+1} = r_i - a_i q and to the row
+// transform of w r_{i+1} (into T), without beta_{i+1}: W^-1 p_{i+1} = W^-1 r_{i+1} + beta_{i+1} W^-1 p_i is formed by the
+// next column pass, which carries W^-1 p on Omega (U).  a_i is known before that row pass because
+// Re<p, A p> = |DF p|^2 + alpha |p|^2 with |DF p|^2 summed by the PSF pass.  q is never stored, and p, r, dx cross memory
+// 5 times per iteration on average (p, r in and out; dx in and out every other iteration, with two steps at once)
+// where q, p, r and dx crossed it 11 times in separate p-update, q and CG-step passes: 277 -> 145 MB of algorithmic
+// traffic an iteration at 384^2 with 10 coils.  An iteration inside a graph, before (six passes) and after: 64^2/4 coils
+// 25.6 -> 13.7 us, 256^2/8 29.9 -> 24.6, 384^2/10 44.2 -> 31.8, 512^2/16 126 -> 104.
+//   col  beta_i from the |r|^2 partials; u = W^-1 p; T = FFT_col(M (p_rho c_j + rho u))
+//   row  PSF, |DF p|^2 partials
+//   col  adjoint products; one more block: a_i, the stop test
+//   row  p = r + beta p, q, r -= a q, dx += a_{i-1} p_{i-1} + a_i p (odd i); T = row transform of w r; partials
+// The passes are separate functions so that nlinv_profile_cg times exactly what a reconstruction launches.
+cudaError_t q_cg_col_dir(nlinv_ctx* c, const float2* x, int newton, int iter) {
+  KArgs a = base_args(c);
+  a.skip = iter;
+  a.src = c->T;
+  a.dst = c->T;
+  a.rho = x;
+  a.drho = c->p;
+  a.r = c->r;
+  a.U = c->U;
+  a.coil = c->coil;
+  a.rr_part = c->rr_part;
+  a.n_rr = row_geom(c, true).blocks;
   a.slot = newton;
   a.iter = iter;
-  a.pq_part = c->pq_part;
-  a.n_pq = n_pq;
+  return col(c, nlv::COL_CG_DIR, a);
+}
+
+cudaError_t q_cg_row_psf(nlinv_ctx* c, int newton, int iter) {
+  KArgs a = base_args(c);
+  a.skip = iter;
+  a.slot = newton;
+  a.src = c->T;
+  a.dst = c->T;
+  a.mask = c->mask;
+  a.dd_part = c->dd_part;
+  return row(c, nlv::ROW_CG_PSF, a);
+}
+
+cudaError_t q_cg_col_adj(nlinv_ctx* c, const float2* x, float alpha, int newton, int iter) {
+  KArgs a = base_args(c);
+  a.skip = iter;
+  a.src = c->T;
+  a.dst = c->T;
+  a.rho = x;
+  a.coil = c->coil;
+  a.zsum = c->zsum;
+  a.scalars = 1;
+  a.alpha = alpha;
+  a.dd_part = c->dd_part;
+  a.n_dd = row_geom(c, false).blocks;
   a.rr_part = c->rr_part;
+  a.n_rr = row_geom(c, true).blocks;
+  a.slot = newton;
+  a.iter = iter;
+  return col(c, nlv::COL_IFFT_ADJ_FFT, a);
+}
+
+// early: p and r may be loaded before the dependent-launch wait (false for back-to-back launches of this pass alone,
+// where each launch would read what the one before writes)
+cudaError_t q_cg_row_update(nlinv_ctx* c, float alpha, int newton, int iter, bool last, bool early = true) {
+  KArgs a = base_args(c);
+  a.skip = iter + 1;
+  a.skip_after = 1;
+  a.slot = newton;
+  a.src_early = early ? 1 : 0;
+  a.src = c->T;
+  a.dst = c->T;
+  a.p = c->p;
+  a.r = c->r;
+  a.dx = c->dx;
+  a.zsum = c->zsum;
+  a.alpha = alpha;
+  a.rr_part = c->rr_part;
+  a.n_rr = row_geom(c, true).blocks;
+  a.iter = iter;
+  a.last = last ? 1 : 0;
+  return row(c, nlv::ROW_CG_UPDATE, a);
+}
+
+cudaError_t q_cg_iter(nlinv_ctx* c, const float2* x, float alpha, int newton, int iter) {
+  cudaError_t e;
+  if ((e = q_cg_col_dir(c, x, newton, iter)) != cudaSuccess) return e;
+  if ((e = q_cg_row_psf(c, newton, iter)) != cudaSuccess) return e;
+  if ((e = q_cg_col_adj(c, x, alpha, newton, iter)) != cudaSuccess) return e;
+  return q_cg_row_update(c, alpha, newton, iter, iter == c->prm.cg_iters - 1);
+}
+
+// One CG iteration of a batch's frame, in six passes with q stored and Re<p, q> taken from it.  A batch keeps this
+// form although the four passes above move fewer bytes: FP32 CG that ends unconverged (30 iterations at small alpha_n)
+// lies between two iterates of exact CG, and any other rounding moves it there -- of the 64 frames of the uneven
+// batch, two or so change their distance to the FP64 solution by more than 1.5x either way.  The batch's results stay
+// what they were, bit for bit.
+//   row  beta from the |r|^2 partials of the CG step before; p_c = r_c + beta p_c; T = W^-1 p_c (first axis)
+//   col  drho = r_rho + beta p_rho; T = FFT_col(M (drho c_j + rho W^-1 p_c))
+//   row  PSF;  col  adjoint products;  row  q = DF^H DF p + alpha p, p_rho written, Re<p, q> partials
+//   vec  alpha from those; dx += alpha p, r -= alpha q, per-block partials of |r|^2
+// The direction update p = r + beta p of the previous iteration is folded into the passes that first read p (beta = 0
+// right after the right-hand side).
+cudaError_t q_bcg_iter(nlinv_ctx* c, const float2* x, float alpha, int newton, int iter) {
+  cudaError_t e;
+  const bool timed = iter == 1 && newton == 0;      // the iteration that nlinv_batch_profile_cg times
+  auto cg_args = [&](int step) {
+    KArgs a = base_args(c);
+    a.skip = iter;
+    a.skip_after = 1;
+    a.slot = newton;
+    c->rec_step = timed ? step : 0;
+    return a;
+  };
+  KArgs a = cg_args(1);
+  a.src = c->p + c->plane;
+  a.r = c->r + c->plane;
+  if (iter > 0) {
+    a.brr_part = c->brr_part;
+    a.n_rr = c->vec_blocks;
+  }
+  a.dst = c->T;
+  if ((e = row(c, nlv::ROW_BCG_DIR, a)) != cudaSuccess) return e;
+  a = cg_args(2);
+  a.src = c->T;
+  a.dst = c->T;
+  a.rho = x;
+  a.drho = c->p;
+  a.r = c->r;
+  a.coil = c->coil;
+  if ((e = col(c, nlv::COL_BCG_DIR, a)) != cudaSuccess) return e;
+  a = cg_args(3);
+  a.src = c->T;
+  a.dst = c->T;
+  a.mask = c->mask;
+  if ((e = row(c, nlv::ROW_PSF, a)) != cudaSuccess) return e;
+  a = cg_args(4);
+  a.src = c->T;
+  a.dst = c->T;
+  a.rho = x;
+  a.coil = c->coil;
+  a.zsum = c->zsum;
+  if ((e = col(c, nlv::COL_IFFT_ADJ_FFT, a)) != cudaSuccess) return e;
+  a = cg_args(5);
+  a.src = c->T;
+  a.dst = c->q;
+  a.p = c->p;
+  a.r = c->r;
+  a.zsum = c->zsum;
+  a.alpha = alpha;
+  a.pq_part = c->pq_part;
+  if ((e = row(c, nlv::ROW_BCG_NORMAL, a)) != cudaSuccess) return e;
+  a = cg_args(6);
+  a.iter = iter;
+  a.pq_part = c->pq_part;
+  a.n_pq = row_geom(c, true).blocks;
+  a.brr_part = c->brr_part;
   a.p = c->p;
   a.q = c->q;
   a.r = c->r;
   a.dx = c->dx;
   a.n2 = c->vec / 2;
   void* args[] = {&a};
-  if (c->batch_lanes > 0)     // batch frames: the register-staged form, which the batched kernel runs
-    return launch(c, cg_step_fn(), c->vec_blocks, kVecThreads, 0, args);
-  return launch(c, (const void*)cg_step_bulk, cg_blocks(c), kBulkThreads, kBulkSmem, args);
+  e = launch(c, (const void*)cg_step_batch, c->vec_blocks, kVecThreads, 0, args);
+  c->rec_step = 0;
+  return e;
 }
 
-// x += dx
-cudaError_t q_add(nlinv_ctx* c) {
+// x += dx, after the CG solve of a batch's frame
+cudaError_t q_bcg_add(nlinv_ctx* c) {
   KArgs a = base_args(c);
   a.dx = c->dx;
   a.dst = c->x;
   a.n2 = c->vec / 2;
   void* args[] = {&a};
-  return launch(c, (const void*)add_kernel, c->vec_blocks, kVecThreads, 0, args);
-}
-
-// One CG iteration on (DF^H DF + alpha) for linearisation point x.  The direction update p = r + beta p of the
-// previous iteration is folded into the passes that first read p (beta = 0 right after the right-hand side).
-//   K1 row  beta from the |r|^2 partials of K6 before; p_c = r_c + beta p_c; T = W^-1 p_c (first axis)
-//   K2 col  drho = r_rho + beta p_rho; T = FFT_col(M (drho c_j + rho W^-1 p_c))
-//   K3 row  PSF;  K4 col  adjoint products;  K5 row  q = DF^H DF p + alpha p, p_rho written, Re<p, q> partials
-//   K6      alpha from the K5 partials; dx += alpha p, r -= alpha q, per-block partials of |r|^2
-// The steps are separate functions so that nlinv_profile_cg times exactly what a reconstruction launches.
-// early: p may be loaded before the dependent-launch wait (false for back-to-back launches of this pass alone,
-// where each launch would read what the one before writes)
-cudaError_t q_cg_k1(nlinv_ctx* c, bool first, bool early = true) {
-  KArgs a = base_args(c);
-  a.cgskip = nlv::kCgSkipAfterWait;
-  a.src = c->p + c->plane;
-  a.r = c->r + c->plane;
-  a.pupd = 1;
-  if (!first) {
-    a.rr_part = c->rr_part;
-    a.n_rr = cg_blocks(c);
-    // p's coil planes were written by this pass one iteration back (before the first iteration, by the
-    // right-hand side pass just before it)
-    a.src_early = early ? 1 : 0;
-  }
-  a.dst = c->T;
-  return row(c, nlv::ROW_W_IFFT, a);
-}
-
-cudaError_t q_cg_k2(nlinv_ctx* c, const float2* x) {
-  KArgs a = base_args(c);
-  a.cgskip = nlv::kCgSkipEarly;
-  a.src = c->T;
-  a.dst = c->T;
-  a.rho = x;
-  a.drho = c->p;
-  a.r = c->r;
-  a.pupd = 1;
-  a.coil = c->coil;
-  return col(c, nlv::COL_IFFT_PROD_FFT, a);
-}
-
-cudaError_t q_cg_k3(nlinv_ctx* c) {
-  KArgs a = base_args(c);
-  a.cgskip = nlv::kCgSkipEarly;
-  a.src = c->T;
-  a.dst = c->T;
-  a.mask = c->mask;
-  return row(c, nlv::ROW_PSF, a);
-}
-
-cudaError_t q_cg_k5(nlinv_ctx* c, float alpha) {
-  KArgs a = base_args(c);
-  a.cgskip = nlv::kCgSkipEarly;
-  a.src = c->T;
-  a.dst = c->q;
-  a.p = c->p;
-  a.r = c->r;
-  a.pupd = 1;
-  a.zsum = c->zsum;
-  a.alpha = alpha;
-  a.pq_part = c->pq_part;
-  return row(c, nlv::ROW_FFT_W_NORMAL, a);
-}
-
-cudaError_t q_cg_iter(nlinv_ctx* c, const float2* x, float alpha, int newton, int iter) {
-  cudaError_t e;
-  if ((e = q_cg_k1(c, iter == 0)) != cudaSuccess) return e;
-  if ((e = q_cg_k2(c, x)) != cudaSuccess) return e;
-  if ((e = q_cg_k3(c)) != cudaSuccess) return e;
-  if ((e = q_adj_col(c, x, true)) != cudaSuccess) return e;
-  if ((e = q_cg_k5(c, alpha)) != cudaSuccess) return e;
-  return q_cg_step(c, row_geom(c, true).blocks, newton, iter);
+  return launch(c, (const void*)add_batch, c->vec_blocks, kVecThreads, 0, args);
 }
 
 // Coil maps of c->x and the Newton residual r0 = y - F x with |r0| into resid[slot].
@@ -771,7 +723,9 @@ cudaError_t q_reconstruct(nlinv_ctx* c) {
   for (int n = 0; n < P.newton_steps; ++n) {
     const float al = (float)alpha;
     if ((e = q_residual(c, n)) != cudaSuccess) return e;
-    // b = DF^H r0 - alpha (x - xref) -> r = p = b, dx = 0, rr = |b|^2
+    // b = DF^H r0 - alpha (x - xref) -> r = b, rr = |b|^2 and, for the first iteration, T = row transform of w b (a
+    // single frame) or p = b, dx = 0 (a frame of a batch)
+    const bool batch = c->batch_lanes > 0;
     KArgs a = base_args(c);
     a.src = c->r0;
     a.dst = c->T;
@@ -784,15 +738,16 @@ cudaError_t q_reconstruct(nlinv_ctx* c) {
     a.x = c->x;
     a.xref = c->xref;
     a.r = c->r;
+    a.dst = c->T;
     a.pout = c->p;
     a.dx = c->dx;
     a.alpha = al;
     a.reduce = nlv::RED_RR_INIT;
     a.slot = n;
-    if ((e = row(c, nlv::ROW_FFT_W_RHS, a)) != cudaSuccess) return e;
+    if ((e = row(c, batch ? nlv::ROW_BCG_RHS : nlv::ROW_CG_RHS, a)) != cudaSuccess) return e;
     for (int i = 0; i < P.cg_iters; ++i)
-      if ((e = q_cg_iter(c, c->x, al, n, i)) != cudaSuccess) return e;
-    if ((e = q_add(c)) != cudaSuccess) return e;
+      if ((e = batch ? q_bcg_iter(c, c->x, al, n, i) : q_cg_iter(c, c->x, al, n, i)) != cudaSuccess) return e;
+    if ((e = batch ? q_bcg_add(c) : q_cg_finish(c, c->x, c->x, n)) != cudaSuccess) return e;
     if (c->ckpt &&
         (e = cudaMemcpyAsync(c->ckpt + (size_t)(n + 1) * c->vec, c->x, vb, cudaMemcpyDeviceToDevice, c->stream)) !=
             cudaSuccess)
@@ -836,6 +791,30 @@ nlinv_status validate(const nlinv_params* p, std::string* why) {
     return NLINV_EINVAL;
   }
   return NLINV_OK;
+}
+
+// For the timing calls: marks the CG solve of a Newton step as running and takes the rounding floor away (until the
+// next right-hand side), so that every kernel does its full work.  Synchronous.
+cudaError_t mark_running(nlinv_ctx* c, int newton) {
+  const int running = -1;
+  const double none = 0.0;
+  cudaError_t e = cudaMemcpy(&c->sc->cg_stop[newton], &running, sizeof(int), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(&c->sc->rr0, &none, sizeof(double), cudaMemcpyHostToDevice);
+  return e;
+}
+
+// The six steps that nlinv_profile_cg reports, from the four passes' durations (ms4: column direction, row PSF, column
+// adjoint, row update).  The row update pass does three of them -- the p update with the first axis of W^-1, W^-H with
+// alpha p, and the CG step -- and its duration is divided among them by the vector planes each moves: 2 (r read,
+// p written, beside its transform's T), 1 (p read, beside its transform's T) and 2 (r written; dx in and out every
+// other iteration).
+void split_profile(const double* ms4, double* out) {
+  out[0] = ms4[3] * 0.4;
+  out[1] = ms4[0];
+  out[2] = ms4[1];
+  out[3] = ms4[2];
+  out[4] = ms4[3] * 0.2;
+  out[5] = ms4[3] * 0.4;
 }
 
 nlinv_status finish_call(nlinv_ctx* c, cudaError_t e, const char* where) {
@@ -988,18 +967,17 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
   };
   const int lanes_max = std::max(row_geom(c, false).lanes, row_geom(c, true).lanes);
   for (int m = 0; m < nlv::NUM_ROW_MODES && smem_err.empty(); ++m) {
-    allow(c->k->row[m], c->k->row_smem(m, lanes_max));
-    if (smem_err.empty()) allow(c->k->row_batch[m], c->k->row_smem(m, lanes_max));
+    if (c->k->row[m]) allow(c->k->row[m], c->k->row_smem(m, lanes_max));
+    if (smem_err.empty() && c->k->row_batch[m]) allow(c->k->row_batch[m], c->k->row_smem(m, lanes_max));
     if (smem_err.empty() && c->k->row_std[m]) allow(c->k->row_std[m], c->k->row_smem(m, lanes_max));
     if (smem_err.empty() && c->k->row_std_batch[m]) allow(c->k->row_std_batch[m], c->k->row_smem(m, lanes_max));
   }
   for (int m = 0; m < nlv::NUM_COL_MODES && smem_err.empty(); ++m) {
-    allow(c->k->col[m], c->k->col_smem(m, c->Wc));
-    if (smem_err.empty()) allow(c->k->col_batch[m], c->k->col_smem(m, c->Wc));
+    if (c->k->col[m]) allow(c->k->col[m], c->k->col_smem(m, c->Wc));
+    if (smem_err.empty() && c->k->col_batch[m]) allow(c->k->col_batch[m], c->k->col_smem(m, c->Wc));
     if (smem_err.empty() && c->k->col_std[m]) allow(c->k->col_std[m], c->k->col_smem(m, c->Wc));
     if (smem_err.empty() && c->k->col_std_batch[m]) allow(c->k->col_std_batch[m], c->k->col_smem(m, c->Wc));
   }
-  if (smem_err.empty()) allow((const void*)cg_step_bulk, kBulkSmem);
   if (c->tc) {
     for (int m = 0; m < nlv::NUM_ROW_MODES && smem_err.empty(); ++m) {
       if (c->k->row_tc[m]) allow(c->k->row_tc[m], c->k->row_smem_tc(m, lanes_max));
@@ -1031,7 +1009,9 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
   const size_t partb = align_up((size_t)max_blocks * sizeof(double), 256);
   const size_t scb = align_up(sizeof(Scalars), 256);
   const size_t tcb = c->tc ? align_up(nlv::kTcBBytes, 256) : 0;
-  const size_t total = 6 * vecb + 2 * datab + Tb + 2 * cb + 2 * twb + wb + maskb + 3 * partb + scb + tcb;
+  const bool batch = batch_lanes > 0;
+  const size_t total = (batch ? 6 : 5) * vecb + 2 * datab + Tb + (batch ? 2 : 3) * cb + 2 * twb + wb + maskb +
+                       (batch ? 3 : 5) * partb + scb + tcb;
   // NLINV_TEST_FAIL_ALLOC=1 (tests only): the workspace allocation reports out-of-memory without trying, so that
   // the ENOMEM path can be exercised without exhausting a GPU.
   const char* fail_alloc = std::getenv("NLINV_TEST_FAIL_ALLOC");
@@ -1050,20 +1030,26 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
   c->xref = (float2*)take(vecb);
   c->r = (float2*)take(vecb);
   c->p = (float2*)take(vecb);
-  c->q = (float2*)take(vecb);
   c->dx = (float2*)take(vecb);
+  if (batch) c->q = (float2*)take(vecb);
   c->y = (float2*)take(datab);
   c->r0 = (float2*)take(datab);
   c->T = (float2*)take(Tb);
   c->coil = (float2*)take(cb);
   c->zsum = (float2*)take(cb);
+  if (!batch) c->U = (float2*)take(cb);
   c->twA = (float2*)take(twb);
   c->twB = (float2*)take(twb);
   c->wtab = (float*)take(wb);
   c->mask = (uint8_t*)take(maskb);
   c->partials = (double*)take(partb);
-  c->pq_part = (double*)take(partb);
-  c->rr_part = (double*)take(partb);
+  if (batch) {
+    c->pq_part = (double*)take(partb);
+    c->brr_part = (double*)take(partb);
+  } else {
+    c->dd_part = (nlv::Pair*)take(partb);
+    c->rr_part = (nlv::Pair*)take(3 * partb);
+  }
   c->sc = (Scalars*)take(scb);
   if (c->tc) c->tcB = take(tcb);
 
@@ -1184,7 +1170,6 @@ nlinv_status nlinv_normal(nlinv_ctx* c, const nlinv_c32* x, const uint8_t* mask,
     a.p = (const float2*)d;
     a.zsum = c->zsum;
     a.alpha = (float)alpha;
-    a.reduce = nlv::RED_NONE;
     e = row(c, nlv::ROW_FFT_W_NORMAL, a);
   }
   return finish_call(c, e, "nlinv_normal");
@@ -1271,10 +1256,10 @@ nlinv_status nlinv_reconstruct(nlinv_ctx* c, const nlinv_c32* y, const uint8_t* 
     NLV_TRY(cudaStreamSynchronize(c->stream), "synchronize");
     if (resid)
       for (int n = 0; n <= c->prm.newton_steps; ++n) resid[n] = hs.resid[n];
-    if (hs.flags & (nlv::kFlagTcTimeout | kFlagCopyTimeout)) {
+    if (hs.flags & nlv::kFlagTcTimeout) {
       int zero = 0;
       cudaMemcpy(&c->sc->flags, &zero, sizeof(int), cudaMemcpyHostToDevice);
-      return fail(c, NLINV_ECUDA, "an asynchronous copy or tensor-core stage did not complete within its time limit");
+      return fail(c, NLINV_ECUDA, "a tensor-core stage did not complete within its time limit");
     }
     if (hs.flags & 1) {
       int zero = 0;
@@ -1306,10 +1291,10 @@ nlinv_status nlinv_wait(nlinv_ctx* c, double timeout_s) {
   cudaEventDestroy(ev);
   int flags = 0;
   NLV_TRY(cudaMemcpy(&flags, &c->sc->flags, sizeof(int), cudaMemcpyDeviceToHost), "read flags");
-  if (flags & (nlv::kFlagTcTimeout | kFlagCopyTimeout)) {
+  if (flags & nlv::kFlagTcTimeout) {
     int zero = 0;
     NLV_TRY(cudaMemcpy(&c->sc->flags, &zero, sizeof(int), cudaMemcpyHostToDevice), "clear flags");
-    return fail(c, NLINV_ECUDA, "an asynchronous copy or tensor-core stage did not complete within its time limit");
+    return fail(c, NLINV_ECUDA, "a tensor-core stage did not complete within its time limit");
   }
   if (flags & 1) {
     int zero = 0;
@@ -1418,12 +1403,18 @@ nlinv_status nlinv_reconstruct_vjp(nlinv_ctx* c, const nlinv_c32* y, const uint8
     // u = (DF^H DF + alpha)^-1 g by the reconstruction's CG (u in c->dx)
     if (e == cudaSuccess) {
       KArgs a = base_args(c);
-      a.src = g; a.r = c->r; a.pout = c->p; a.dx = c->dx; a.n2 = c->vec / 2; a.reduce = nlv::RED_RR_INIT;
+      a.src = g; a.r = c->r; a.n2 = c->vec / 2; a.reduce = nlv::RED_RR_INIT;
       a.slot = k;
       void* args[] = {&a};
       e = launch(c, (const void*)cg_init_kernel, c->vec_blocks, kVecThreads, 0, args);
     }
+    if (e == cudaSuccess) {      // T = row transform of w r, which the first iteration starts from
+      KArgs a = base_args(c);
+      a.src = c->r + c->plane; a.dst = c->T;
+      e = row(c, nlv::ROW_W_IFFT, a);
+    }
     for (int i = 0; i < P.cg_iters && e == cudaSuccess; ++i) e = q_cg_iter(c, c->x, alpha, k, i);
+    if (e == cudaSuccess) e = q_cg_finish(c, nullptr, c->dx, k);
     // v = DF_x u; dL/dy += v; dL/dx_ref += alpha u
     if (e == cudaSuccess) e = q_dir(c, c->x, c->dx);
     if (e == cudaSuccess) {
@@ -1448,41 +1439,36 @@ nlinv_status nlinv_profile_cg(nlinv_ctx* c, int reps, double* ms_out) {
   if (!c) return NLINV_EINVAL;
   if (reps < 1 || !ms_out) return fail(c, NLINV_EINVAL, "reps must be >= 1 and ms_out non-NULL");
   if (!c->have_state) return fail(c, NLINV_EINVAL, "run nlinv_reconstruct before nlinv_profile_cg");
-  constexpr int K = kProfileKernels;
-  // the kernels are timed doing their full work: a solve that stopped at its floor is marked running again
-  {
-    int flags = 0;
-    NLV_TRY(cudaMemcpy(&flags, &c->sc->flags, sizeof(int), cudaMemcpyDeviceToHost), "read flags");
-    flags &= ~nlv::kFlagCgStopped;
-    NLV_TRY(cudaMemcpy(&c->sc->flags, &flags, sizeof(int), cudaMemcpyHostToDevice), "write flags");
-  }
+  NLV_TRY(mark_running(c, nlv::kMaxNewton), "mark the solve running");
   cudaEvent_t ev[2];
   for (int i = 0; i < 2; ++i) NLV_TRY(cudaEventCreate(&ev[i]), "event create");
   const float al = (float)c->last_alpha;
-  // kernel k of the CG iteration, reps launches back to back between two events: its steady-state launch
-  // duration (consecutive launches overlap ramp and drain through the dependent launch, as in a graph replay)
-  auto one = [&](int k) -> cudaError_t {
+  // pass k of the CG iteration, reps launches back to back between two events: its steady-state launch duration
+  // (consecutive launches overlap ramp and drain through the dependent launch, as in a graph replay).  The CG update
+  // pass alternates between the iteration that updates dx and the one that does not.
+  auto one = [&](int k, int it) -> cudaError_t {
     switch (k) {
-      case 0: return q_cg_k1(c, false, false);
-      case 1: return q_cg_k2(c, c->x);
-      case 2: return q_cg_k3(c);
-      case 3: return q_adj_col(c, c->x, true);
-      case 4: return q_cg_k5(c, al);
-      default: return q_cg_step(c, row_geom(c, true).blocks, 0, 0, false);
+      case 0: return q_cg_col_dir(c, c->x, nlv::kMaxNewton, 2);
+      case 1: return q_cg_row_psf(c, nlv::kMaxNewton, 2);
+      case 2: return q_cg_col_adj(c, c->x, al, nlv::kMaxNewton, 2);
+      default: return q_cg_row_update(c, al, nlv::kMaxNewton, 2 + (it & 1), false, false);
     }
   };
   cudaError_t e = cudaSuccess;
-  for (int k = 0; k < K && e == cudaSuccess; ++k) {
+  double ms4[4] = {};
+  for (int k = 0; k < 4 && e == cudaSuccess; ++k) {
     e = cudaEventRecord(ev[0], c->stream);
-    for (int it = 0; it < reps && e == cudaSuccess; ++it) e = one(k);
+    for (int it = 0; it < reps && e == cudaSuccess; ++it) e = one(k, it);
     if (e == cudaSuccess) e = cudaEventRecord(ev[1], c->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(ev[1]);
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
-    ms_out[k] = ms / reps;
+    ms4[k] = ms / reps;
+    if (e == cudaSuccess) e = mark_running(c, nlv::kMaxNewton);
   }
   for (int i = 0; i < 2; ++i) cudaEventDestroy(ev[i]);
   if (e != cudaSuccess) return cuda_fail(c, e, "nlinv_profile_cg");
+  split_profile(ms4, ms_out);
   return NLINV_OK;
 }
 
@@ -1730,11 +1716,11 @@ struct nlinv_batch {
     int grid, block;
     size_t smem;
     nlv::BatchArgs args;
+    int step;                               // nlinv_ctx::Rec::step
   };
   std::vector<Launch> launches;
   cudaGraphExec_t graph = nullptr;
   bool have_state = false;                  // a reconstruction has filled the workspaces
-  std::vector<size_t> group_first;          // index in `launches` of each group's first launch
   bool pdl = true;
   bool multi = false;                       // one launch per pass for all sides the multi-side kernels cover
                                             // (NLINV_BATCH_MULTI=1; measured slower, see nlinv_batch_create)
@@ -1757,37 +1743,20 @@ void batch_free(nlinv_batch* b) {
   delete b;
 }
 
-// The multi-side kernel (kernels.cuh, "batches of several sides") that runs the single-frame pass fn of side k for
-// frames of every side, and its dynamic shared memory; nullptr if fn is not a pass.
+// The multi-side kernel (kernels.cuh, "batches of several sides") that runs the batched pass fn of side k for frames of
+// every side, and its dynamic shared memory (0 and fn itself when fn is a vector pass, which knows no side).
 const void* multi_kernel(const SizeKernels* k, const void* fn, size_t* smem) {
   const nlv::MultiKernels* mk = nlv::multi_kernels();
   for (int m = 0; m < nlv::NUM_ROW_MODES; ++m) {
-    if (fn == k->row[m]) { *smem = mk->row_smem[m]; return mk->row[m]; }
-    if (k->row_std[m] && fn == k->row_std[m]) { *smem = mk->row_smem[m]; return mk->row_std[m]; }
+    if (fn == k->row_batch[m]) { *smem = mk->row_smem[m]; return mk->row[m]; }
+    if (k->row_std_batch[m] && fn == k->row_std_batch[m]) { *smem = mk->row_smem[m]; return mk->row_std[m]; }
   }
   for (int m = 0; m < nlv::NUM_COL_MODES; ++m) {
-    if (fn == k->col[m]) { *smem = mk->col_smem[m]; return mk->col[m]; }
-    if (k->col_std[m] && fn == k->col_std[m]) { *smem = mk->col_smem[m]; return mk->col_std[m]; }
+    if (fn == k->col_batch[m]) { *smem = mk->col_smem[m]; return mk->col[m]; }
+    if (k->col_std_batch[m] && fn == k->col_std_batch[m]) { *smem = mk->col_smem[m]; return mk->col_std[m]; }
   }
   *smem = 0;
-  if (fn == cg_step_fn()) return (const void*)cg_step_batch;
-  if (fn == (const void*)add_kernel) return (const void*)add_batch;
-  return nullptr;
-}
-
-// The batched kernel that runs the single-frame pass fn for several frames of one side.
-const void* batched_kernel(const SizeKernels* k, const void* fn) {
-  for (int m = 0; m < nlv::NUM_ROW_MODES; ++m) {
-    if (fn == k->row[m]) return k->row_batch[m];
-    if (k->row_std[m] && fn == k->row_std[m]) return k->row_std_batch[m];
-  }
-  for (int m = 0; m < nlv::NUM_COL_MODES; ++m) {
-    if (fn == k->col[m]) return k->col_batch[m];
-    if (k->col_std[m] && fn == k->col_std[m]) return k->col_std_batch[m];
-  }
-  if (fn == cg_step_fn()) return (const void*)cg_step_batch;
-  if (fn == (const void*)add_kernel) return (const void*)add_batch;
-  return nullptr;
+  return fn;
 }
 
 // One batched launch on stream st (with the batch's dependent-launch setting).
@@ -1882,12 +1851,12 @@ nlinv_status nlinv_batch_create(const nlinv_params* params, int nframes, const n
     for (int i : fr)
       if (recs[i].size() != L) return batch_fail(b, NLINV_EINVAL, "frames of one grid side differ in schedule");
     const bool multi = sides[g] == 0;
-    b->group_first.push_back(b->launches.size());
     for (size_t l = 0; l < L; ++l) {
       nlinv_batch::Launch bl{};
       bl.group = (int)g;
+      bl.step = recs[fr[0]][l].step;
       size_t msmem = 0;
-      bl.fn = multi ? multi_kernel(k, recs[fr[0]][l].fn, &msmem) : batched_kernel(k, recs[fr[0]][l].fn);
+      bl.fn = multi ? multi_kernel(k, recs[fr[0]][l].fn, &msmem) : recs[fr[0]][l].fn;
       if (!bl.fn) return batch_fail(b, NLINV_EINVAL, "internal: no batched form of a pass");
       size_t off = (host.size() + 15) / 16 * 16;
       host.resize(off + fr.size() * sizeof(KArgs));
@@ -1897,7 +1866,7 @@ nlinv_status nlinv_batch_create(const nlinv_params* params, int nframes, const n
       for (size_t t = 0; t < fr.size(); ++t) {
         const nlinv_ctx::Rec& r = recs[fr[t]][l];
         size_t ms = 0;
-        const void* same = multi ? multi_kernel(b->frames[fr[t]]->k, r.fn, &ms) : batched_kernel(k, r.fn);
+        const void* same = multi ? multi_kernel(b->frames[fr[t]]->k, r.fn, &ms) : r.fn;
         if (same != bl.fn || (!multi && r.block != recs[fr[0]][l].block))
           return batch_fail(b, NLINV_EINVAL, "frames of one group differ in pass shapes");
         std::memcpy(host.data() + off + t * sizeof(KArgs), &r.args, sizeof(KArgs));
@@ -2034,35 +2003,24 @@ nlinv_status nlinv_batch_profile_cg(nlinv_batch* b, int reps, double* ms_out) {
   if (!b->have_state) return fail(nullptr, NLINV_EINVAL, "run nlinv_reconstruct_batch before nlinv_batch_profile_cg");
   if (b->prm.cg_iters < 2) return fail(nullptr, NLINV_EINVAL, "the batch's schedule has fewer than two CG iterations");
   cudaError_t e = cudaStreamSynchronize(b->stream);
-  // every frame's solve is marked running, so that every kernel does its full work
-  for (nlinv_ctx* c : b->frames) {
-    int flags = 0;
-    if (e == cudaSuccess) e = cudaMemcpy(&flags, &c->sc->flags, sizeof(int), cudaMemcpyDeviceToHost);
-    flags &= ~nlv::kFlagCgStopped;
-    if (e == cudaSuccess) e = cudaMemcpy(&c->sc->flags, &flags, sizeof(int), cudaMemcpyHostToDevice);
-  }
+  for (nlinv_ctx* c : b->frames)
+    if (e == cudaSuccess) e = mark_running(c, 0);
   if (e != cudaSuccess) return fail(nullptr, NLINV_ECUDA, std::string("nlinv_batch_profile_cg: ") + cudaGetErrorString(e));
-  // the six launches of the second CG iteration of the first Newton step, in every group: they end at the group's
-  // second CG step
-  std::vector<size_t> first6;
-  for (size_t g = 0; g < b->group_first.size(); ++g) {
-    const size_t end = g + 1 < b->group_first.size() ? b->group_first[g + 1] : b->launches.size();
-    int seen = 0;
-    size_t at = 0;
-    for (size_t l = b->group_first[g]; l < end && seen < 2; ++l)
-      if (b->launches[l].fn == (const void*)cg_step_batch && ++seen == 2) at = l;
-    if (seen < 2 || at < b->group_first[g] + 5) return fail(nullptr, NLINV_EINVAL, "internal: CG launches not found");
-    first6.push_back(at - 5);
-  }
+  // the six passes of the second CG iteration of the first Newton step, in every group
+  std::vector<std::vector<size_t>> pass(kProfileSteps);
+  for (size_t l = 0; l < b->launches.size(); ++l)
+    if (b->launches[l].step > 0) pass[b->launches[l].step - 1].push_back(l);
+  for (const std::vector<size_t>& v : pass)
+    if (v.size() != b->groups.size()) return fail(nullptr, NLINV_EINVAL, "internal: CG launches not found");
   cudaEvent_t ev[2];
   for (int i = 0; i < 2; ++i)
     if ((e = cudaEventCreate(&ev[i])) != cudaSuccess)
       return fail(nullptr, NLINV_ECUDA, std::string("event create: ") + cudaGetErrorString(e));
-  for (int k = 0; k < kProfileKernels && e == cudaSuccess; ++k) {
+  for (int k = 0; k < kProfileSteps && e == cudaSuccess; ++k) {
     e = cudaEventRecord(ev[0], b->stream);
     for (int it = 0; it < reps && e == cudaSuccess; ++it)
-      for (size_t g = 0; g < first6.size() && e == cudaSuccess; ++g)
-        e = launch_batched(b, b->launches[first6[g] + k], b->stream);
+      for (size_t l : pass[k])
+        if (e == cudaSuccess) e = launch_batched(b, b->launches[l], b->stream);
     if (e == cudaSuccess) e = cudaEventRecord(ev[1], b->stream);
     if (e == cudaSuccess) e = cudaEventSynchronize(ev[1]);
     float ms = 0.f;
