@@ -104,6 +104,18 @@ NLINV_API nlinv_status nlinv_create(const nlinv_params* params, void* stream, nl
 /* Waits for the context's stream, then frees the context and its workspace.  NULL is accepted. */
 NLINV_API nlinv_status nlinv_destroy(nlinv_ctx* ctx);
 
+/* Chooses the stream of the next operator call on ctx (nlinv_forward, nlinv_derivative, nlinv_adjoint, nlinv_normal,
+ * nlinv_image, nlinv_simulate): it is then queued on `stream` (a cudaStream_t of the context's device, NULL the legacy
+ * default stream) instead of the context's own, ordered after the context's last call wherever that ran, and saves the
+ * caller the two events that order another stream's work around the context's.  Calls that are not operator calls
+ * always use the context's own stream, after the context's last call.  Returns 1 when the choice is taken, 0 when the
+ * next call will use the context's own stream: `stream` is that stream, or is being captured into a graph (a captured
+ * call is ordered by the capture's own events), or ctx is NULL. */
+NLINV_API int nlinv_use_stream(nlinv_ctx* ctx, void* stream);
+
+/* Orders the context's own stream after the context's last call, wherever it ran.  Errors: EINVAL, ECUDA. */
+NLINV_API nlinv_status nlinv_join(nlinv_ctx* ctx);
+
 /* F x of Eq. 2: y_out_j = P FFT(M rho c_j), c_j = W^-1 chat_j.  x: 1+J planes; y_out: J planes. */
 NLINV_API nlinv_status nlinv_forward(nlinv_ctx* ctx, const nlinv_c32* x, const uint8_t* mask, nlinv_c32* y_out);
 
@@ -192,13 +204,17 @@ typedef struct nlinv_gridder nlinv_gridder;
 NLINV_API nlinv_status nlinv_gridder_create(int n, int nspokes, const double* directions, void* stream,
                                             nlinv_gridder** out);
 
+/* Chooses the stream of the next nlinv_grid call on g, as nlinv_use_stream does for operator calls.  The gridder's
+ * tables are only read; calls on a caller's stream are ordered after one another all the same, for the destructor. */
+NLINV_API int nlinv_gridder_use_stream(nlinv_gridder* g, void* stream);
+
 /* y_out (DEVICE, ncoils x n x n) and mask_out (DEVICE, n x n) from samples (DEVICE, ncoils x nspokes x 2n, spoke-major
  * within a coil).  Queued on the gridder's stream.  Errors: EINVAL (NULL or host pointers, ncoils outside 1..64),
  * ECUDA. */
 NLINV_API nlinv_status nlinv_grid(nlinv_gridder* g, int ncoils, const nlinv_c32* samples, nlinv_c32* y_out,
                                   uint8_t* mask_out);
 
-/* Waits for the gridder's stream and frees it.  NULL is accepted. */
+/* Waits for the gridder's work and frees it.  NULL is accepted. */
 NLINV_API nlinv_status nlinv_gridder_destroy(nlinv_gridder* g);
 
 /* ---------------------------------------------------------------------------------------------- batches ----

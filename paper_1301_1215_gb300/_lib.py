@@ -46,6 +46,8 @@ SIGNATURES = {
     "nlinv_default_params": (_int, [C.POINTER(Params), _int, _int]),
     "nlinv_create": (_int, [C.POINTER(Params), _vp, C.POINTER(_vp)]),
     "nlinv_destroy": (_int, [_vp]),
+    "nlinv_use_stream": (_int, [_vp, _vp]),
+    "nlinv_join": (_int, [_vp]),
     "nlinv_forward": (_int, [_vp, _vp, _vp, _vp]),
     "nlinv_derivative": (_int, [_vp, _vp, _vp, _vp, _vp]),
     "nlinv_adjoint": (_int, [_vp, _vp, _vp, _vp, _vp]),
@@ -66,6 +68,7 @@ SIGNATURES = {
     "nlinv_last_launch_count": (_long, [_vp]),
     "nlinv_cg_stops": (_int, [_vp, C.POINTER(_int), _int]),
     "nlinv_gridder_create": (_int, [_int, _int, C.POINTER(_dbl), _vp, C.POINTER(_vp)]),
+    "nlinv_gridder_use_stream": (_int, [_vp, _vp]),
     "nlinv_grid": (_int, [_vp, _int, _vp, _vp, _vp]),
     "nlinv_gridder_destroy": (_int, [_vp]),
     "nlinv_autotune": (_int, [_vp, _vp, _vp, _vp, _int, C.POINTER(Tuning), C.POINTER(Tuning), _int]),

@@ -256,6 +256,14 @@ struct nlinv_ctx {
   const SizeKernels* k = nullptr;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
+  // Operator calls on a caller's stream (nlinv_use_stream).  All streams share the workspace, so every call is ordered
+  // after the call before it: `done` marks the end of the last one, which ran on `last`.  Kept only once a caller's
+  // stream has been used.
+  cudaStream_t run = nullptr;      // where launches go: `stream` outside an operator call
+  cudaStream_t next = nullptr;     // the stream of the next operator call, if next_set
+  bool next_set = false;
+  cudaStream_t last = nullptr;
+  cudaEvent_t done = nullptr;
   int device = 0;
   int vec_blocks = 0;         // grid of the vector kernels
   int sms = 0;                // streaming multiprocessors of the device
@@ -376,7 +384,7 @@ cudaError_t launch(nlinv_ctx* c, const void* fn, int grid, int block, size_t sme
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
-  cfg.stream = c->stream;
+  cfg.stream = c->run;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = c->pdl ? 1 : 0;
@@ -384,6 +392,40 @@ cudaError_t launch(nlinv_ctx* c, const void* fn, int grid, int block, size_t sme
   cfg.numAttrs = 1;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
+
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+}
+
+// Orders the context's next work, on stream s, after its last call and sends launches there.  A stream that is being
+// captured takes no dependency on work outside its capture (nlinv_use_stream never picks one).
+cudaError_t enter_stream(nlinv_ctx* c, cudaStream_t s) {
+  c->run = s;
+  if (!c->done || c->last == s || capturing(s)) return cudaSuccess;
+  return cudaStreamWaitEvent(s, c->done, 0);
+}
+cudaError_t enter_own(nlinv_ctx* c) {
+  c->next_set = false;
+  return enter_stream(c, c->stream);
+}
+// The end of a call's work on c->run; launches go to the context's own stream again.
+cudaError_t leave_stream(nlinv_ctx* c) {
+  cudaError_t e = cudaSuccess;
+  if (c->done && !(c->run == c->stream && capturing(c->run))) {
+    e = cudaEventRecord(c->done, c->run);
+    c->last = c->run;
+  }
+  c->run = c->stream;
+  return e;
+}
+// Scope of a call on the context's own stream.
+struct OwnStream {
+  nlinv_ctx* c;
+  cudaError_t err;
+  explicit OwnStream(nlinv_ctx* ctx) : c(ctx), err(enter_own(ctx)) {}
+  ~OwnStream() { leave_stream(c); }
+};
 
 cudaError_t row(nlinv_ctx* c, int mode, KArgs a) {
   const bool rho = mode >= nlv::ROW_FFT_W_ADJ && mode != nlv::ROW_CG_PSF && mode != nlv::ROW_BCG_DIR;
@@ -822,6 +864,22 @@ nlinv_status finish_call(nlinv_ctx* c, cudaError_t e, const char* where) {
   return NLINV_OK;
 }
 
+// Begin and end of an operator call: on the stream that nlinv_use_stream chose for it (taken first thing, so that a
+// refused call uses the choice up too), else on the context's own.
+cudaStream_t op_stream(nlinv_ctx* c) {
+  const cudaStream_t s = c->next_set ? c->next : c->stream;
+  c->next_set = false;
+  return s;
+}
+cudaError_t op_begin(nlinv_ctx* c, cudaStream_t s) {
+  c->launches = 0;
+  return enter_stream(c, s);
+}
+nlinv_status op_end(nlinv_ctx* c, cudaError_t e, const char* where) {
+  const cudaError_t e2 = leave_stream(c);
+  return finish_call(c, e != cudaSuccess ? e : e2, where);
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------- C-ABI ----
@@ -940,6 +998,7 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
     if (e != cudaSuccess) { g_create_error = std::string("cudaStreamCreate: ") + cudaGetErrorString(e); delete c; return NLINV_ECUDA; }
     c->own_stream = true;
   }
+  c->run = c->stream;
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   if (const char* v = std::getenv("NLINV_PDL")) c->pdl = std::strcmp(v, "0") != 0;
@@ -1093,9 +1152,41 @@ nlinv_status nlinv_create(const nlinv_params* params, void* stream, nlinv_ctx** 
   return create_ctx(params, stream, 0, out);
 }
 
+int nlinv_use_stream(nlinv_ctx* c, void* stream) {
+  if (!c) return 0;
+  const cudaStream_t s = (cudaStream_t)stream;
+  c->next_set = false;
+  if (s == c->stream || capturing(s)) return 0;
+  if (!c->done) {              // from here on the end of every call is marked
+    if (capturing(c->stream)) return 0;
+    if (cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventRecord(c->done, c->stream) != cudaSuccess) {
+      cudaGetLastError();
+      if (c->done) cudaEventDestroy(c->done);
+      c->done = nullptr;
+      return 0;
+    }
+    c->last = c->stream;
+  }
+  c->next = s;
+  c->next_set = true;
+  return 1;
+}
+
+nlinv_status nlinv_join(nlinv_ctx* c) {
+  if (!c) return NLINV_EINVAL;
+  OwnStream on(c);
+  NLV_TRY(on.err, "order after the last call");
+  return NLINV_OK;
+}
+
 nlinv_status nlinv_destroy(nlinv_ctx* c) {
   if (!c) return NLINV_OK;
   cudaStreamSynchronize(c->stream);
+  if (c->done) {
+    cudaEventSynchronize(c->done);
+    cudaEventDestroy(c->done);
+  }
   if (c->graph) cudaGraphExecDestroy(c->graph);
   cudaFree(c->base);
   if (c->vjp_base) cudaFree(c->vjp_base);
@@ -1106,11 +1197,12 @@ nlinv_status nlinv_destroy(nlinv_ctx* c) {
 
 nlinv_status nlinv_forward(nlinv_ctx* c, const nlinv_c32* x, const uint8_t* mask, nlinv_c32* y_out) {
   if (!c) return NLINV_EINVAL;
+  const cudaStream_t on = op_stream(c);
   nlinv_status s;
   if ((s = check_dev(c, x, "x")) || (s = check_dev(c, mask, "mask")) || (s = check_dev(c, y_out, "y_out"))) return s;
-  c->launches = 0;
   const float2* xv = (const float2*)x;
-  cudaError_t e = q_coils(c, xv);
+  cudaError_t e = op_begin(c, on);
+  if (e == cudaSuccess) e = q_coils(c, xv);
   if (e == cudaSuccess) e = q_prod(c, xv);
   if (e == cudaSuccess) {
     KArgs a = base_args(c);
@@ -1119,44 +1211,47 @@ nlinv_status nlinv_forward(nlinv_ctx* c, const nlinv_c32* x, const uint8_t* mask
     a.mask = mask;
     e = row(c, nlv::ROW_FFT_P_OUT, a);
   }
-  return finish_call(c, e, "nlinv_forward");
+  return op_end(c, e, "nlinv_forward");
 }
 
 nlinv_status nlinv_derivative(nlinv_ctx* c, const nlinv_c32* x, const uint8_t* mask, const nlinv_c32* dx,
                               nlinv_c32* out) {
   if (!c) return NLINV_EINVAL;
+  const cudaStream_t on = op_stream(c);
   nlinv_status s;
   if ((s = check_dev(c, x, "x")) || (s = check_dev(c, mask, "mask")) || (s = check_dev(c, dx, "dx")) ||
       (s = check_dev(c, out, "out")))
     return s;
-  c->launches = 0;
-  const cudaError_t e = q_derivative_to(c, (const float2*)x, (const float2*)dx, mask, (float2*)out);
-  return finish_call(c, e, "nlinv_derivative");
+  cudaError_t e = op_begin(c, on);
+  if (e == cudaSuccess) e = q_derivative_to(c, (const float2*)x, (const float2*)dx, mask, (float2*)out);
+  return op_end(c, e, "nlinv_derivative");
 }
 
 nlinv_status nlinv_adjoint(nlinv_ctx* c, const nlinv_c32* x, const uint8_t* mask, const nlinv_c32* r,
                            nlinv_c32* out) {
   if (!c) return NLINV_EINVAL;
+  const cudaStream_t on = op_stream(c);
   nlinv_status s;
   if ((s = check_dev(c, x, "x")) || (s = check_dev(c, mask, "mask")) || (s = check_dev(c, r, "r")) ||
       (s = check_dev(c, out, "out")))
     return s;
-  c->launches = 0;
-  const cudaError_t e = q_adjoint_to(c, (const float2*)x, (const float2*)r, mask, (float2*)out);
-  return finish_call(c, e, "nlinv_adjoint");
+  cudaError_t e = op_begin(c, on);
+  if (e == cudaSuccess) e = q_adjoint_to(c, (const float2*)x, (const float2*)r, mask, (float2*)out);
+  return op_end(c, e, "nlinv_adjoint");
 }
 
 nlinv_status nlinv_normal(nlinv_ctx* c, const nlinv_c32* x, const uint8_t* mask, const nlinv_c32* d, double alpha,
                           nlinv_c32* out) {
   if (!c) return NLINV_EINVAL;
+  const cudaStream_t on = op_stream(c);
   nlinv_status s;
   if ((s = check_dev(c, x, "x")) || (s = check_dev(c, mask, "mask")) || (s = check_dev(c, d, "d")) ||
       (s = check_dev(c, out, "out")))
     return s;
   if (!std::isfinite(alpha)) return fail(c, NLINV_EINVAL, "alpha must be finite");
-  c->launches = 0;
   const float2* xv = (const float2*)x;
-  cudaError_t e = q_coils(c, xv);
+  cudaError_t e = op_begin(c, on);
+  if (e == cudaSuccess) e = q_coils(c, xv);
   if (e == cudaSuccess) e = q_dir(c, xv, (const float2*)d);
   if (e == cudaSuccess) {
     KArgs a = base_args(c);
@@ -1175,15 +1270,16 @@ nlinv_status nlinv_normal(nlinv_ctx* c, const nlinv_c32* x, const uint8_t* mask,
     a.alpha = (float)alpha;
     e = row(c, nlv::ROW_FFT_W_NORMAL, a);
   }
-  return finish_call(c, e, "nlinv_normal");
+  return op_end(c, e, "nlinv_normal");
 }
 
 nlinv_status nlinv_image(nlinv_ctx* c, const nlinv_c32* x, nlinv_c32* image_out) {
   if (!c) return NLINV_EINVAL;
+  const cudaStream_t on = op_stream(c);
   nlinv_status s;
   if ((s = check_dev(c, x, "x")) || (s = check_dev(c, image_out, "image_out"))) return s;
-  c->launches = 0;
-  cudaError_t e = q_coils(c, (const float2*)x);
+  cudaError_t e = op_begin(c, on);
+  if (e == cudaSuccess) e = q_coils(c, (const float2*)x);
   if (e == cudaSuccess) {
     KArgs a = base_args(c);
     a.rho = (const float2*)x;
@@ -1192,22 +1288,23 @@ nlinv_status nlinv_image(nlinv_ctx* c, const nlinv_c32* x, nlinv_c32* image_out)
     void* args[] = {&a};
     e = launch(c, (const void*)image_kernel, c->vec_blocks, kVecThreads, 0, args);
   }
-  return finish_call(c, e, "nlinv_image");
+  return op_end(c, e, "nlinv_image");
 }
 
 nlinv_status nlinv_simulate(nlinv_ctx* c, const nlinv_c32* rho, const nlinv_c32* coil_img, const uint8_t* mask,
                             nlinv_c32* y_out) {
   if (!c) return NLINV_EINVAL;
+  const cudaStream_t on = op_stream(c);
   nlinv_status s;
   if ((s = check_dev(c, rho, "rho")) || (s = check_dev(c, coil_img, "coil_img")) ||
       (s = check_dev(c, mask, "mask")) || (s = check_dev(c, y_out, "y_out")))
     return s;
-  c->launches = 0;
   KArgs a = base_args(c);
   a.rho = (const float2*)rho;
   a.cimg = (const float2*)coil_img;
   a.dst = c->T;
-  cudaError_t e = col(c, nlv::COL_SIM_FFT, a);
+  cudaError_t e = op_begin(c, on);
+  if (e == cudaSuccess) e = col(c, nlv::COL_SIM_FFT, a);
   if (e == cudaSuccess) {
     a = base_args(c);
     a.src = c->T;
@@ -1215,7 +1312,7 @@ nlinv_status nlinv_simulate(nlinv_ctx* c, const nlinv_c32* rho, const nlinv_c32*
     a.mask = mask;
     e = row(c, nlv::ROW_FFT_P_OUT, a);
   }
-  return finish_call(c, e, "nlinv_simulate");
+  return op_end(c, e, "nlinv_simulate");
 }
 
 nlinv_status nlinv_reconstruct(nlinv_ctx* c, const nlinv_c32* y, const uint8_t* mask, const nlinv_c32* x_ref,
@@ -1224,6 +1321,8 @@ nlinv_status nlinv_reconstruct(nlinv_ctx* c, const nlinv_c32* y, const uint8_t* 
   if (!y || !mask || !x_inout) return fail(c, NLINV_EINVAL, "y, mask and x_inout must not be NULL");
   const size_t vb = c->vec * sizeof(float2), db = (size_t)c->J * c->plane * sizeof(float2);
   const bool host_x = !is_device_ptr(x_inout);
+  OwnStream on(c);
+  NLV_TRY(on.err, "order after the last call");
   NLV_TRY(cudaMemcpyAsync(c->y, y, db, cudaMemcpyDefault, c->stream), "copy y");
   NLV_TRY(cudaMemcpyAsync(c->mask, mask, (size_t)c->plane, cudaMemcpyDefault, c->stream), "copy mask");
   NLV_TRY(cudaMemcpyAsync(c->x, x_inout, vb, cudaMemcpyDefault, c->stream), "copy x");
@@ -1275,6 +1374,8 @@ nlinv_status nlinv_reconstruct(nlinv_ctx* c, const nlinv_c32* y, const uint8_t* 
 
 nlinv_status nlinv_wait(nlinv_ctx* c, double timeout_s) {
   if (!c) return NLINV_EINVAL;
+  OwnStream on(c);
+  NLV_TRY(on.err, "order after the last call");
   cudaEvent_t ev;
   NLV_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "event create");
   cudaError_t e = cudaEventRecord(ev, c->stream);
@@ -1317,6 +1418,8 @@ nlinv_status nlinv_reconstruct_checkpoints(nlinv_ctx* c, const nlinv_c32* y, con
     return s;
   if (x_ref && (s = check_dev(c, x_ref, "x_ref"))) return s;
   const size_t vb = c->vec * sizeof(float2), db = (size_t)c->J * c->plane * sizeof(float2);
+  OwnStream on(c);
+  NLV_TRY(on.err, "order after the last call");
   NLV_TRY(cudaMemcpyAsync(c->y, y, db, cudaMemcpyDeviceToDevice, c->stream), "copy y");
   NLV_TRY(cudaMemcpyAsync(c->mask, mask, (size_t)c->plane, cudaMemcpyDeviceToDevice, c->stream), "copy mask");
   NLV_TRY(cudaMemcpyAsync(c->x, x_inout, vb, cudaMemcpyDeviceToDevice, c->stream), "copy x");
@@ -1372,6 +1475,8 @@ nlinv_status nlinv_reconstruct_vjp(nlinv_ctx* c, const nlinv_c32* y, const uint8
   float2* v = sres + J * c->plane;
   const float2* X = (const float2*)ckpt;
   c->launches = 0;
+  OwnStream on(c);
+  NLV_TRY(on.err, "order after the last call");
   NLV_TRY(cudaMemcpyAsync(c->y, y, db, cudaMemcpyDeviceToDevice, c->stream), "copy y");
   NLV_TRY(cudaMemcpyAsync(c->mask, mask, (size_t)c->plane, cudaMemcpyDeviceToDevice, c->stream), "copy mask");
   NLV_TRY(cudaMemcpyAsync(g, grad_x, vb, cudaMemcpyDeviceToDevice, c->stream), "copy grad_x");
@@ -1442,6 +1547,8 @@ nlinv_status nlinv_profile_cg(nlinv_ctx* c, int reps, double* ms_out) {
   if (!c) return NLINV_EINVAL;
   if (reps < 1 || !ms_out) return fail(c, NLINV_EINVAL, "reps must be >= 1 and ms_out non-NULL");
   if (!c->have_state) return fail(c, NLINV_EINVAL, "run nlinv_reconstruct before nlinv_profile_cg");
+  OwnStream on(c);
+  NLV_TRY(on.err, "order after the last call");
   NLV_TRY(mark_running(c, nlv::kMaxNewton), "mark the solve running");
   cudaEvent_t ev[2];
   for (int i = 0; i < 2; ++i) NLV_TRY(cudaEventCreate(&ev[i]), "event create");
@@ -1481,6 +1588,8 @@ nlinv_status nlinv_cg_stops(nlinv_ctx* c, int* out, int len) {
   if (!c) return NLINV_EINVAL;
   if (!out || len < c->prm.newton_steps) return fail(c, NLINV_EINVAL, "out must hold newton_steps entries");
   if (!c->have_state) return fail(c, NLINV_EINVAL, "no reconstruction has run on this context");
+  OwnStream on(c);
+  NLV_TRY(on.err, "order after the last call");
   Scalars hs{};
   NLV_TRY(cudaMemcpyAsync(&hs, c->sc, sizeof(Scalars), cudaMemcpyDeviceToHost, c->stream), "read scalars");
   NLV_TRY(cudaStreamSynchronize(c->stream), "synchronize");
@@ -1562,6 +1671,8 @@ nlinv_status nlinv_autotune(nlinv_ctx* c, const nlinv_c32* y, const uint8_t* mas
         return NLINV_OK;
       }
   }
+  OwnStream on(c);
+  NLV_TRY(on.err, "order after the last call");
   // Whole reconstructions of the caller's frame, replayed as graphs (each replay starts from the same start value):
   // only the whole graph shows how neighbouring passes overlap, and an all-zero workspace times differently from
   // data.  Every timed replay starts with a cold L2 (a write of twice its size outside the events), as a frame of a
