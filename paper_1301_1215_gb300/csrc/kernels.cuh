@@ -27,17 +27,25 @@ enum Reduce : int {
 constexpr int kMaxNewton = 64;
 
 // Scalars of the CG and Newton iterations, kept in device memory (FP64).
+// An unevaluated sum of two floats (see pair_add).
+struct Pair {
+  float h, l;
+};
+
 // The values that one launch writes while its other blocks still read the value of the iteration before have two
 // slots, indexed by the parity of the CG iteration.
 struct Scalars {
-  double rr[2];                  // |r_i|^2 of iteration i in slot i & 1 (batches: slot 0)
+  double rr;                     // |b|^2 of the current solve; batches: |r|^2 of the current CG residual
   double rr0;                    // |b|^2 of the current CG solve (the reference of the rounding floor)
   double rr_prev;                // batches: |r|^2 of the previous CG residual (denominator of the next beta)
   double alpha;                  // batches: CG step length
   double beta;                   // CG direction update
   double pq;                     // last Re<p, A p>
-  float step[2];                 // CG step length a_i of iteration i in slot i & 1, as the FP32 updates use it
-  float beta_f;                  // beta likewise
+  // Single frames (pairs in units of the sums over a launch, kPairScale; the step lengths as the FP32 updates use them):
+  Pair rr_pair;                  // |b|^2 of the current CG solve
+  Pair rr_i[2];                  // |r_i|^2 of iteration i in slot i & 1
+  Pair beta_p;                   // beta of the current direction
+  float step[2];                 // CG step length a_i of iteration i in slot i & 1
   double last;                   // result of a RED_NONE reduction
   double resid[kMaxNewton + 1];  // |y - F x_n| per Newton step
   int cg_stop[kMaxNewton + 1];   // per Newton step: the CG iteration that reached the rounding floor, -1 if none
@@ -51,11 +59,6 @@ constexpr int kFlagBreakdown = 1;
 // relative to |b| (further iterations cannot improve a single-precision solution; left to run, the recursive
 // residual decays into the FP32 denormal range, where the step lengths lose their precision).
 constexpr double kCgFloor2 = 0x1p-48;
-
-// An unevaluated sum of two floats (see pair_add).
-struct Pair {
-  float h, l;
-};
 
 struct KArgs {
   int N, J, f, Wc;          // grid side, coils, half-width of Omega, compact width 2f
@@ -193,9 +196,11 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 
 // Sums over the threads and blocks of a CG iteration are kept as an unevaluated pair of floats h + l: Knuth's two-sum
 // gives the exact rounding error of every addition to h, which collects in l, so a sum of n terms is good to about
-// n 2^-48.  The terms themselves are FP32 sums of at most 16 products, good to 2^-22 or so, and the scalars formed
-// from the sums (|r|^2, beta, the step length) are FP64.  FP64 additions run at 1/64 of the FP32 rate on sm_103a: a
-// tree sum in FP64 cost the PSF pass 1.2 us of 7.4 at 384 x 384 with 10 coils, and the update pass, with three, 3 us.
+// n 2^-48.  The terms themselves are FP32 sums of at most 16 products, good to 2^-22 or so.  The scalars formed from the
+// sums (beta, the step length) are pairs as well; the updates use them rounded to FP32.  FP64 runs at 1/90 of the FP32
+// rate on sm_103a (1.4 additions a clock and SM), and a dependent chain at some hundred cycles an operation: a tree sum
+// in FP64 cost the PSF pass 1.2 us of 7.4 at 384 x 384 with 10 coils, the update pass, with three, 3 us, and the
+// scalars' two quotients of an iteration 4 us where nothing hides them.
 __device__ __forceinline__ void pair_add(Pair& s, float x, float lo) {
   const float t = __fadd_rn(s.h, x);
   const float z = __fsub_rn(t, s.h);
@@ -203,12 +208,36 @@ __device__ __forceinline__ void pair_add(Pair& s, float x, float lo) {
   s.h = t;
   s.l = __fadd_rn(s.l, __fadd_rn(e, lo));
 }
+// Arithmetic on pairs, relative error about 2^-45: products by fused multiply-add (exact low part), quotients by one
+// correction of the FP32 quotient.
+__device__ __forceinline__ Pair pair_norm(float h, float l) {            // |l| at most |h|
+  const float t = __fadd_rn(h, l);
+  return {t, __fsub_rn(l, __fsub_rn(t, h))};
+}
+__device__ __forceinline__ Pair pair_sum(Pair a, Pair b) {
+  pair_add(a, b.h, b.l);
+  return pair_norm(a.h, a.l);
+}
+__device__ __forceinline__ Pair pair_mul(Pair a, Pair b) {
+  const float t = __fmul_rn(a.h, b.h);
+  const float e = fmaf(a.h, b.h, -t);
+  return pair_norm(t, fmaf(a.h, b.l, fmaf(a.l, b.h, e)));
+}
+__device__ __forceinline__ Pair pair_scale(Pair a, float s) { return {a.h * s, a.l * s}; }      // s a power of two
+__device__ __forceinline__ Pair pair_div(Pair a, Pair b) {
+  const float q = a.h / b.h;
+  const float r = __fadd_rn(fmaf(-q, b.h, a.h), fmaf(-q, b.l, a.l));    // the first difference is exact
+  return pair_norm(q, r / b.h);
+}
+__device__ __forceinline__ bool pair_gt(Pair a, Pair b) { return a.h > b.h || (a.h == b.h && a.l > b.l); }
 // The sums over a block carry a factor kBlockScale and those over the blocks of a launch kGridScale more, so that no
 // FP32 sum overflows where its terms do not (at most 2^13 terms of a block's threads, 2^12 blocks); powers of two, so
 // nothing is rounded short of the denormal range.
-constexpr float kBlockScale = 0x1p-13f, kGridScale = 0x1p-12f;
-// The value of a sum over the blocks of a launch.
-__device__ __forceinline__ double grid_value(const Pair& s) { return ((double)s.h + (double)s.l) * 0x1p25; }
+constexpr float kBlockScale = 0x1p-13f, kGridScale = 0x1p-12f, kPairScale = kBlockScale * kGridScale;
+// |p|^2 of p = r + beta p_old from |r|^2, beta, Re<r, p_old> and |p_old|^2.
+__device__ __forceinline__ Pair cg_direction_norm(Pair rr, Pair beta, Pair rp, Pair pp) {
+  return pair_sum(rr, pair_mul(beta, pair_sum(pair_scale(rp, 2.f), pair_mul(beta, pp))));
+}
 // Butterfly sum over the existing lanes of the calling warp (all of them call it), valid in lane 0.
 __device__ __forceinline__ Pair warp_sum(Pair s, int cnt) {
   const unsigned mask = cnt >= 32 ? 0xffffffffu : (1u << cnt) - 1u;
@@ -255,9 +284,12 @@ __device__ __forceinline__ void finalize_scalar(Scalars* sc, int reduce, int slo
   switch (reduce) {
     case RED_RESID: sc->resid[slot] = sqrt(total); break;
     case RED_RR_INIT:           // a new CG solve starts: nothing has stopped yet
-      sc->rr[0] = total;
+      sc->rr = total;
       sc->rr0 = total;
       sc->beta = 0.0;
+      sc->rr_pair.h = (float)(total * kPairScale);
+      sc->rr_pair.l = (float)(total * kPairScale - (double)sc->rr_pair.h);
+      sc->rr_i[0] = sc->rr_pair;
       sc->cg_stop[slot] = -1;
       break;
     default: sc->last = total; break;
@@ -556,11 +588,11 @@ __device__ __forceinline__ float2 cg_point(const CgStep& c, float2 z, float2 r, 
 // dx += g (odd iterations; the first one, iteration 1, writes it).  The addition happens in L2, so no thread waits for
 // dx or holds it: read and written by the pass it cost 6 of 55 us at 512 x 512 with 16 coils and, held in registers
 // across the second transform, spilled 300 bytes a thread.
-__device__ __forceinline__ void cg_add_dx(const KArgs& A, int o, float2 g) {
-  if (A.iter > 1)
-    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(A.dx + o), "f"(g.x), "f"(g.y) : "memory");
+__device__ __forceinline__ void cg_add_dx(float2* dx, float2 g, bool add) {
+  if (add)
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(dx), "f"(g.x), "f"(g.y) : "memory");
   else
-    A.dx[o] = g;
+    *dx = g;
 }
 
 // Adds a thread's products to its three sums at sums[k * blockDim.x]; first: they hold nothing yet.
@@ -573,6 +605,12 @@ __device__ __forceinline__ void cg_flush(CgDots& d, Pair* sums, bool first) {
     dot_flush(*v[k], s);
     sums[k * blockDim.x] = s;
   }
+}
+
+__device__ __forceinline__ void cg_flush(CgDots& d, Pair (&sums)[3]) {
+  dot_flush(d.rr, sums[0]);
+  dot_flush(d.rp, sums[1]);
+  dot_flush(d.pp, sums[2]);
 }
 
 // The rho plane's slice of the CG update pass.
@@ -607,7 +645,7 @@ __device__ __forceinline__ void rho_cg_slice(const KArgs& A, int bid, const CgSt
       float2 g;
       A.r[o] = cg_point(c, z[k], r[k], p[k], g, acc);
       const_cast<float2*>(A.p)[o] = p[k];
-      if (c.odd) cg_add_dx(A, o, g);
+      if (c.odd) cg_add_dx(A.dx + o, g, A.iter > 1);
     }
     cg_flush(acc, sums, false);
   }
@@ -757,7 +795,7 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
       cg.alpha = A.alpha;
       cg.a = A.sc->step[A.iter & 1];
       cg.a_prev = cg.first ? 0.f : A.sc->step[(A.iter & 1) ^ 1];
-      cg.beta = cg.first ? 0.f : A.sc->beta_f;
+      cg.beta = cg.first ? 0.f : A.sc->beta_p.h;
       s_cg = cg;
     }
   }
@@ -774,7 +812,7 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
           const double rp = A.sc->rr_prev;
           const double b = (rp != 0.0) ? t / rp : 0.0;
           s_beta = (float)b;
-          if (bid == 0) { A.sc->rr[0] = t; A.sc->beta = b; }
+          if (bid == 0) { A.sc->rr = t; A.sc->beta = b; }
         }
       } else if (threadIdx.x == 0) {
         s_beta = (float)A.sc->beta;
@@ -875,7 +913,7 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
           const float2 rn = cg_point(cg, cscale(v[m], w), rB[m], p, g, dots);
           A.r[rowB + N2 * m] = rn;
           const_cast<float2*>(A.p)[rowB + N2 * m] = p;
-          if (cg.odd) cg_add_dx(A, rowB + N2 * m, g);
+          if (cg.odd) cg_add_dx(A.dx + rowB + N2 * m, g, A.iter > 1);
           out = cscale(rn, w);
         }
         v[m] = out;
@@ -1091,21 +1129,19 @@ __device__ __forceinline__ void col_stage_side(const KArgs& A, int bid, unsigned
 // s_stop: the same for every block.
 __device__ __forceinline__ void cg_direction_scalars(const KArgs& A, int bid, float& s_beta, int& s_stop) {
   if (threadIdx.x < ((blockDim.x - 1) & ~31u)) return;
-  const double rp = A.sc->rr[(A.iter & 1) ^ 1], rr0 = A.sc->rr0;
-  const Pair s = warp_sum_of(A.rr_part, A.n_rr, kGridScale);
+  const Pair rp = A.sc->rr_i[(A.iter & 1) ^ 1], floor = pair_scale(A.sc->rr_pair, (float)kCgFloor2);
+  const Pair t = warp_sum_of(A.rr_part, A.n_rr, kGridScale);
   if ((threadIdx.x & 31) == 0) {
-    const double t = grid_value(s);
-    const double b = (rp != 0.0) ? t / rp : 0.0;
-    const bool stop = !(t > kCgFloor2 * rr0) || !isfinite(t);
-    s_beta = (float)b;
+    const Pair b = rp.h != 0.f ? pair_div(t, rp) : Pair{0.f, 0.f};
+    const bool stop = !pair_gt(t, floor) || !isfinite(t.h);
+    s_beta = b.h;
     s_stop = stop ? 1 : 0;
     if (bid == 0) {
-      A.sc->rr[A.iter & 1] = t;
-      A.sc->beta = b;
-      A.sc->beta_f = (float)b;
+      A.sc->rr_i[A.iter & 1] = t;
+      A.sc->beta_p = b;
       if (stop) {
         A.sc->cg_stop[A.slot] = A.iter;
-        if (!isfinite(t)) atomicOr(&A.sc->flags, kFlagBreakdown);
+        if (!isfinite(t.h)) atomicOr(&A.sc->flags, kFlagBreakdown);
       }
     }
   }
@@ -1131,16 +1167,16 @@ __device__ __forceinline__ void cg_decide(const KArgs& A) {
     }
   __syncthreads();
   if (threadIdx.x != 0 || A.sc->cg_stop[A.slot] == A.iter) return;    // stopped by the direction pass already
-  const double rr = A.sc->rr[A.iter & 1], beta = A.iter > 0 ? A.sc->beta : 0.0;
-  const double pp = rr + beta * (2.0 * grid_value(tot[1]) + beta * grid_value(tot[2]));
+  const Pair none = {0.f, 0.f};
+  const Pair rr = A.sc->rr_i[A.iter & 1], beta = A.iter > 0 ? A.sc->beta_p : none;
+  const Pair pp = cg_direction_norm(rr, beta, tot[1], tot[2]);
   // the PSF pass's values carry one more transform factor rs ~ 1/sqrt(N) than DF p; it is divided out as the passes
   // round it (N in its place is off by up to 5e-7, and CG loses its orthogonality that much sooner)
-  const double rs = (double)rsqrtf((float)N);
-  const double t = grid_value(tot[0]) / (rs * rs) + (double)A.alpha * pp;
-  const bool finite = isfinite(t) && isfinite(rr);
-  A.sc->pq = t;
-  if (finite && rr > kCgFloor2 * A.sc->rr0 && t > 0.0) {
-    A.sc->step[A.iter & 1] = (float)(rr / t);
+  const float rs = rsqrtf((float)N);
+  const Pair t = pair_sum(pair_div(tot[0], pair_mul({rs, 0.f}, {rs, 0.f})), pair_mul(pp, {A.alpha, 0.f}));
+  const bool finite = isfinite(t.h) && isfinite(rr.h);
+  if (finite && pair_gt(rr, pair_scale(A.sc->rr_pair, (float)kCgFloor2)) && t.h > 0.f) {
+    A.sc->step[A.iter & 1] = pair_div(rr, t).h;
   } else {
     A.sc->cg_stop[A.slot] = A.iter;
     if (!finite) atomicOr(&A.sc->flags, kFlagBreakdown);
@@ -1516,6 +1552,10 @@ struct SizeKernels {
   const void* col_tc[NUM_COL_MODES];
   const void* row_tc_std[NUM_ROW_MODES];
   const void* col_tc_std[NUM_COL_MODES];
+  // The whole CG solve of a small single frame as one cluster launch (cg_cluster.cuh); nullptr where not compiled.
+  const void* cluster;
+  int cluster_threads;
+  size_t (*cluster_smem)(int J);
   size_t row_smem(int mode, int lanes) const { return nlv::row_smem(mode, N1 * N2, lanes, sm_lane).total; }
   size_t col_smem(int mode, int Wc) const { return nlv::col_smem(mode, N1 * N2, col_lanes, sm_lane_col, Wc).total; }
   size_t row_smem_tc(int mode, int lanes) const { return tc_offset(row_smem(mode, lanes)) + tc_smem_bytes(lanes * tl); }

@@ -59,7 +59,7 @@ __device__ __forceinline__ void cg_step_decide(const KArgs& A, int bid, float& s
   for (int k = threadIdx.x; k < A.n_pq; k += blockDim.x) t += A.pq_part[k];
   t = nlv::block_sum(t, red);
   if (threadIdx.x == 0) {
-    const double rr = A.sc->rr[0];
+    const double rr = A.sc->rr;
     const bool was_stopped = nlv::cg_stopped(A);
     double a = 0.0;
     bool stop = false;
@@ -301,6 +301,7 @@ struct nlinv_ctx {
   std::vector<Rec>* rec = nullptr;   // non-null: launches are recorded instead of issued
   bool pdl = true;            // programmatic dependent launches (NLINV_PDL=0 turns them off)
   bool std_fov = false;       // fov = N/4: the passes specialised for it (SizeKernels::row_std, col_std) apply
+  bool cluster = false;       // the CG solves run as one cluster launch each (cluster_fits)
   bool tc = false;            // radix-16 DFT stages on the tensor cores (params.tensor_dft)
   void* tcB = nullptr;        // their B tiles (workspace)
   double last_alpha = 0.0;    // alpha_n of the last Newton step
@@ -374,7 +375,8 @@ int col_blocks(const nlinv_ctx* c) {
 // Launches with programmatic stream serialisation (see pdl_enter in kernels.cuh): the next pass is scheduled while
 // the current one drains (about 1% per frame on the 384 x 384, 10-coil series).  Every kernel launched here must
 // call nlv::pdl_enter() before its first global memory access.
-cudaError_t launch(nlinv_ctx* c, const void* fn, int grid, int block, size_t smem, void** args) {
+// cluster > 1: the grid in clusters of that many blocks.
+cudaError_t launch(nlinv_ctx* c, const void* fn, int grid, int block, size_t smem, void** args, int cluster = 1) {
   c->launches++;
   if (c->rec) {                       // every pass takes one KArgs
     c->rec->push_back({fn, grid, block, smem, *(const KArgs*)args[0], c->rec_step});
@@ -385,11 +387,14 @@ cudaError_t launch(nlinv_ctx* c, const void* fn, int grid, int block, size_t sme
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = c->run;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = c->pdl ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
@@ -612,6 +617,62 @@ cudaError_t q_cg_iter(nlinv_ctx* c, const float2* x, float alpha, int newton, in
   return q_cg_row_update(c, alpha, newton, iter, iter == c->prm.cg_iters - 1);
 }
 
+// The CG solve of a Newton step and out = base + dx (base NULL: dx alone): one cluster launch, or one launch per pass.
+cudaError_t q_cg_solve(nlinv_ctx* c, const float2* x, float alpha, int newton, const float2* base, float2* out) {
+  if (!c->cluster || c->prm.cg_iters == 0) {
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < c->prm.cg_iters && e == cudaSuccess; ++i) e = q_cg_iter(c, x, alpha, newton, i);
+    return e == cudaSuccess ? q_cg_finish(c, base, out, newton) : e;
+  }
+  KArgs a = base_args(c);
+  a.src = c->T;
+  a.rho = x;
+  a.coil = c->coil;
+  a.mask = c->mask;
+  a.r = c->r;
+  a.x = base;
+  a.dst = out;
+  a.alpha = alpha;
+  a.slot = newton;
+  a.iter = c->prm.cg_iters;
+  void* args[] = {&a};
+  return launch(c, c->k->cluster, c->J, c->k->cluster_threads, c->k->cluster_smem(c->J), args, c->J);
+}
+
+// Whether the CG solves of a single frame run as one cluster launch each: the side has that kernel, the field of view is
+// n/4, one block per coil makes a cluster the device can hold, and the transforms run in FP32.  Sets the kernel's limits.
+bool cluster_fits(nlinv_ctx* c) {
+  if (!c->k->cluster || !c->std_fov || c->tc || c->batch_lanes > 0 || c->J > nlv::kClusterMaxCoils) return false;
+  const void* fn = c->k->cluster;
+  int n = 0, smem_optin = 0;
+  cudaFuncAttributes fa{};
+  if (cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device) != cudaSuccess ||
+      cudaFuncGetAttributes(&fa, fn) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const int dyn_max = smem_optin - (int)fa.sharedSizeBytes;
+  if ((size_t)dyn_max < c->k->cluster_smem(c->J)) return false;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = c->J;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(c->J);
+  cfg.blockDim = dim3(c->k->cluster_threads);
+  cfg.dynamicSmemBytes = c->k->cluster_smem(c->J);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const bool ok =
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_max) == cudaSuccess &&
+      cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) ==
+          cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n >= 1;
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+
 // One CG iteration of a batch's frame, in six passes with q stored and Re<p, q> taken from it.  A batch keeps this
 // form although the four passes above move fewer bytes: FP32 CG that ends unconverged (30 iterations at small alpha_n)
 // lies between two iterates of exact CG, and any other rounding moves it there -- of the 64 frames of the uneven
@@ -787,9 +848,9 @@ cudaError_t q_reconstruct(nlinv_ctx* c) {
     a.reduce = nlv::RED_RR_INIT;
     a.slot = n;
     if ((e = row(c, batch ? nlv::ROW_BCG_RHS : nlv::ROW_CG_RHS, a)) != cudaSuccess) return e;
-    for (int i = 0; i < P.cg_iters; ++i)
-      if ((e = batch ? q_bcg_iter(c, c->x, al, n, i) : q_cg_iter(c, c->x, al, n, i)) != cudaSuccess) return e;
-    if ((e = batch ? q_bcg_add(c) : q_cg_finish(c, c->x, c->x, n)) != cudaSuccess) return e;
+    for (int i = 0; i < P.cg_iters && batch; ++i)
+      if ((e = q_bcg_iter(c, c->x, al, n, i)) != cudaSuccess) return e;
+    if ((e = batch ? q_bcg_add(c) : q_cg_solve(c, c->x, al, n, c->x, c->x)) != cudaSuccess) return e;
     if (c->ckpt &&
         (e = cudaMemcpyAsync(c->ckpt + (size_t)(n + 1) * c->vec, c->x, vb, cudaMemcpyDeviceToDevice, c->stream)) !=
             cudaSuccess)
@@ -840,8 +901,10 @@ nlinv_status validate(const nlinv_params* p, std::string* why) {
 cudaError_t mark_running(nlinv_ctx* c, int newton) {
   const int running = -1;
   const double none = 0.0;
+  const nlv::Pair none_p = {0.f, 0.f};
   cudaError_t e = cudaMemcpy(&c->sc->cg_stop[newton], &running, sizeof(int), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(&c->sc->rr0, &none, sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(&c->sc->rr_pair, &none_p, sizeof(none_p), cudaMemcpyHostToDevice);
   return e;
 }
 
@@ -1057,6 +1120,8 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
     delete c;
     return NLINV_EINVAL;
   }
+
+  c->cluster = cluster_fits(c);
 
   // workspace layout
   const size_t cplx = sizeof(float2);
@@ -1521,8 +1586,7 @@ nlinv_status nlinv_reconstruct_vjp(nlinv_ctx* c, const nlinv_c32* y, const uint8
       a.src = c->r + c->plane; a.dst = c->T;
       e = row(c, nlv::ROW_W_IFFT, a);
     }
-    for (int i = 0; i < P.cg_iters && e == cudaSuccess; ++i) e = q_cg_iter(c, c->x, alpha, k, i);
-    if (e == cudaSuccess) e = q_cg_finish(c, nullptr, c->dx, k);
+    if (e == cudaSuccess) e = q_cg_solve(c, c->x, alpha, k, nullptr, c->dx);
     // v = DF_x u; dL/dy += v; dL/dx_ref += alpha u
     if (e == cudaSuccess) e = q_dir(c, c->x, c->dx);
     if (e == cudaSuccess) {

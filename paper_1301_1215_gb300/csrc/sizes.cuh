@@ -1,9 +1,20 @@
 // Grid sides with compiled transforms and their four-step splits N = N1 * N2.  Each sizes_*.cu file instantiates
 // the pass kernels of a few sides so that they compile in parallel.
 #pragma once
+#include "cg_cluster.cuh"
 #include "kernels.cuh"
 
 namespace nlv {
+
+// A side with the cluster CG solve added.
+template <int N1, int N2> SizeKernels make_size_kernels_cluster() {
+  static_assert(N1 * N2 <= kClusterMaxSide, "the cluster solve is for small sides");
+  SizeKernels s = make_size_kernels<N1, N2>();
+  s.cluster = (const void*)cg_solve_cluster<N1, N2>;
+  s.cluster_threads = ClusterSmem<N1, N2>::T;
+  s.cluster_smem = cluster_smem_bytes<N1, N2>;
+  return s;
+}
 
 // Lookup functions defined by the sizes_*.cu files: the kernel table of side n, or nullptr if that file does not
 // hold n.
@@ -40,6 +51,11 @@ inline const SizeKernels* find_size(int n) {
 #define NLV_SIZE_CASE(n, a, b)                                      \
   case n: {                                                         \
     static const ::nlv::SizeKernels k = ::nlv::make_size_kernels<a, b>(); \
+    return &k;                                                      \
+  }
+#define NLV_SIZE_CASE_SMALL(n, a, b)                                \
+  case n: {                                                         \
+    static const ::nlv::SizeKernels k = ::nlv::make_size_kernels_cluster<a, b>(); \
     return &k;                                                      \
   }
 // A side that also has the passes with tensor-core radix-16 stages.
