@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <type_traits>
 #include "fft_core.cuh"
 #include "tc_dft.cuh"
 
@@ -35,15 +36,9 @@ struct Pair {
 // The values that one launch writes while its other blocks still read the value of the iteration before have two
 // slots, indexed by the parity of the CG iteration.
 struct Scalars {
-  double rr;                     // |b|^2 of the current solve; batches: |r|^2 of the current CG residual
-  double rr0;                    // |b|^2 of the current CG solve (the reference of the rounding floor)
-  double rr_prev;                // batches: |r|^2 of the previous CG residual (denominator of the next beta)
-  double alpha;                  // batches: CG step length
-  double beta;                   // CG direction update
-  double pq;                     // last Re<p, A p>
-  // Single frames (pairs in units of the sums over a launch, kPairScale; the step lengths as the FP32 updates use them):
+  // Pairs in units of the sums over a launch (kPairScale); the step lengths as the FP32 updates use them.
   Pair rr_pair;                  // |b|^2 of the current CG solve
-  Pair rr_i[2];                  // |r_i|^2 of iteration i in slot i & 1
+  Pair rr_i[2];                  // |r_i|^2 of iteration i in slot i & 1 (batches: current and previous |r|^2)
   Pair beta_p;                   // beta of the current direction
   float step[2];                 // CG step length a_i of iteration i in slot i & 1
   double last;                   // result of a RED_NONE reduction
@@ -93,12 +88,12 @@ struct KArgs {
   int scalars;              // DF^H column pass of a CG iteration: one more block forms the step length (cg_decide)
   const float2* q;          // vector passes: second operand; batch CG step: A p
   float2* pout;             // batches: CG direction written by the right-hand side pass
-  // Batches: the normal-operator pass writes one FP64 partial of Re<p, A p> per block into pq_part (the CG step adds
-  // the n_pq partials to form alpha), the CG step one of |r|^2 into brr_part (the first pass of the next iteration adds
-  // the n_rr partials to form beta; NULL: beta from Scalars).
-  double* pq_part;
+  // Batches: the normal-operator pass writes one partial of Re<p, A p> per block into pq_part (the CG step adds the n_pq
+  // partials to form alpha), the CG step one of |r|^2 into brr_part (the first pass of the next iteration adds the n_rr
+  // partials to form beta; NULL: beta from Scalars).
+  Pair* pq_part;
   int n_pq;
-  double* brr_part;
+  Pair* brr_part;
   long n2;                  // vector passes: number of float4 (two complex values each)
   // Sums without a last-block tail: a pass writes one partial per block and a later launch adds them.
   Pair* dd_part;            // PSF pass: partials of |P FFT(...)|^2 = |DF p|^2 (n_dd of them)
@@ -284,9 +279,7 @@ __device__ __forceinline__ void finalize_scalar(Scalars* sc, int reduce, int slo
   switch (reduce) {
     case RED_RESID: sc->resid[slot] = sqrt(total); break;
     case RED_RR_INIT:           // a new CG solve starts: nothing has stopped yet
-      sc->rr = total;
-      sc->rr0 = total;
-      sc->beta = 0.0;
+      sc->beta_p = {0.f, 0.f};
       sc->rr_pair.h = (float)(total * kPairScale);
       sc->rr_pair.l = (float)(total * kPairScale - (double)sc->rr_pair.h);
       sc->rr_i[0] = sc->rr_pair;
@@ -433,8 +426,8 @@ __host__ __device__ constexpr int w_pitch(int mode, int N) { return mode == ROW_
 // o + blockDim.x) and issues every load of both before the first use; the coil sum of a pixel runs over even and
 // odd coils in two partial sums added at the end.
 // Dot-product partials: a thread sums at most 32 products in FP32 (one row round, or two pixels of the rho slice)
-// before adding them to its FP64 partial, so the FP32 summation length is bounded whatever the problem size.  In the
-// single-frame CG passes the real and imaginary products of a thread go to two FP32 sums of at most 16 products each
+// before adding them to its FP64 or pair partial, so the FP32 summation length is bounded whatever the problem size.  In
+// the single-frame CG passes the real and imaginary products of a thread go to two FP32 sums of at most 16 products each
 // (one row round of at most 16 complex values, or one step of the rho slice) before they are added to its pair.
 __device__ __forceinline__ void dot_acc(float2& acc, float2 a, float2 b) {     // acc += (Re a Re b, Im a Im b)
   acc.x = fmaf(a.x, b.x, acc.x);
@@ -503,15 +496,18 @@ __device__ __forceinline__ void rho_channel_sum(const KArgs& A, const bool (&om)
   z[1] = cadd(s[1][0], s[1][1]);
 }
 
-template <int N, int MODE, bool STDF>
-__device__ __forceinline__ double rho_slice(const KArgs& A, int bid) {
+// Adds a thread's FP32 partial to its FP64 sum or its pair.
+__device__ __forceinline__ void acc_add(double& s, float v) { s += (double)v; }
+__device__ __forceinline__ void acc_add(Pair& s, float v) { pair_add(s, v * kBlockScale, 0.f); }
+
+template <int N, int MODE, bool STDF, class Sum>
+__device__ __forceinline__ void rho_slice(const KArgs& A, int bid, Sum& sum) {
   const int f = STDF ? N / 4 : A.f, Wc = STDF ? N / 2 : A.Wc;
   constexpr int plane = N * N;
   const int e_begin = bid * A.rho_per_cta;
   const int e_end = min(e_begin + A.rho_per_cta, plane);
-  const float beta = MODE == ROW_BCG_NORMAL ? (float)A.sc->beta : 0.f;
+  const float beta = MODE == ROW_BCG_NORMAL ? A.sc->beta_p.h : 0.f;
   const int bd = blockDim.x;
-  double accd = 0.0;
   for (int o0 = e_begin + threadIdx.x; o0 < e_end; o0 += 2 * bd) {
     float acc = 0.f;
     float2 a[2], b[2], z[2];
@@ -557,9 +553,8 @@ __device__ __forceinline__ double rho_slice(const KArgs& A, int bid) {
         acc += bb.x * bb.x + bb.y * bb.y;
       }
     }
-    accd += (double)acc;
+    if constexpr (RowTraits<MODE>::reduces) acc_add(sum, acc);
   }
-  return accd;
 }
 
 // The scalars of one CG update (see cg_point).
@@ -721,7 +716,9 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
   const bool mapB = (int)threadIdx.x < LANES * N2;           // threads beyond the whole lanes stay idle
   const int f = STDF ? N / 4 : A.f, Wc = STDF ? N / 2 : A.Wc;
   float acc = 0.f;        // this round's products (at most N1 <= 16 complex values per thread)
-  double accd = 0.0;      // FP64 sum of the rounds
+  // sum of the rounds: FP64 outside the CG iteration, a pair inside
+  using Sum = std::conditional_t<MODE == ROW_BCG_NORMAL, Pair, double>;
+  Sum sum{};
   const RowSmem L = row_smem(MODE, N, LANES, S::SM_LANE);
   float2* smA = (float2*)(smem_raw + L.xch) + laneA * S::SM_LANE;
   float2* smB = (float2*)(smem_raw + L.xch) + laneB * S::SM_LANE;
@@ -750,7 +747,7 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
   }
   __shared__ CgStep s_cg;          // CG update: its scalars, and the threads' sums (live registers across the transforms
   [[maybe_unused]] Pair* sums = (Pair*)(smem_raw + L.sums) + threadIdx.x;      // would spill)
-  __shared__ Pair s_pairs[MODE == ROW_CG_PSF ? kRowMaxThreads : 1];
+  __shared__ Pair s_pairs[MODE == ROW_CG_PSF || MODE == ROW_BCG_NORMAL ? kRowMaxThreads : 1];
   [[maybe_unused]] float2 dd = make_float2(0.f, 0.f);      // PSF pass: this round's |DF p|^2
   __shared__ float s_beta;       // beta of the batches' direction update p = r + beta p
 
@@ -803,19 +800,19 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
   // every block; block 0 publishes |r|^2 and beta for the CG step and the later passes of this iteration)
   if constexpr (MODE == ROW_BCG_DIR) {
     if (R0 == r_begin) {
-      if (A.brr_part) {
-        __shared__ double red[32];
-        double t = 0.0;
-        for (int k = threadIdx.x; k < A.n_rr; k += blockDim.x) t += A.brr_part[k];
-        t = block_sum(t, red);
-        if (threadIdx.x == 0) {
-          const double rp = A.sc->rr_prev;
-          const double b = (rp != 0.0) ? t / rp : 0.0;
-          s_beta = (float)b;
-          if (bid == 0) { A.sc->rr = t; A.sc->beta = b; }
+      if (!A.brr_part) {
+        if (threadIdx.x == 0) s_beta = A.sc->beta_p.h;
+      } else if (threadIdx.x >= ((blockDim.x - 1) & ~31u)) {       // the last warp has the least to load
+        const Pair t = warp_sum_of(A.brr_part, A.n_rr, kGridScale);
+        if ((threadIdx.x & 31) == 0) {
+          const Pair rp = A.sc->rr_i[1];
+          const Pair b = rp.h != 0.f ? pair_div(t, rp) : Pair{0.f, 0.f};
+          s_beta = b.h;
+          if (bid == 0) {
+            A.sc->rr_i[0] = t;
+            A.sc->beta_p = b;
+          }
         }
-      } else if (threadIdx.x == 0) {
-        s_beta = (float)A.sc->beta;
       }
     }
   }
@@ -994,12 +991,12 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
   }
   if (R0 + LANES < r_end) __syncthreads();   // the next round restages the side rows and reuses the exchange
   if constexpr (T::reduces) {
-    accd += (double)acc;
+    acc_add(sum, acc);
     acc = 0.f;
   }
   }  // rounds
 
-  if constexpr (T::has_rho) accd += rho_slice<N, MODE, STDF>(A, bid);
+  if constexpr (T::has_rho) rho_slice<N, MODE, STDF>(A, bid, sum);
   if constexpr (CG) {
     rho_cg_slice<N, STDF>(A, bid, s_cg, sums);
     __syncthreads();
@@ -1008,11 +1005,11 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
   // the pairs were stored before the second transform's barrier
   if constexpr (MODE == ROW_CG_PSF) block_pairs<1>(s_pairs, {A.dd_part + bid});
   if constexpr (MODE == ROW_BCG_NORMAL) {
-    __shared__ double red[32];
-    const double sblk = block_sum(accd, red);
-    if (threadIdx.x == 0) A.pq_part[bid] = sblk;
+    s_pairs[threadIdx.x] = sum;
+    __syncthreads();
+    block_pairs<1>(s_pairs, {A.pq_part + bid});
   } else if constexpr (T::reduces) {
-    grid_reduce(accd, A, bid, nblk);
+    grid_reduce(sum, A, bid, nblk);
   }
 }
 
@@ -1285,7 +1282,7 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, int nblk,
           beta = s_beta;
         }
       }
-      if constexpr (MODE == COL_BCG_DIR) beta = (float)A.sc->beta;
+      if constexpr (MODE == COL_BCG_DIR) beta = A.sc->beta_p.h;
       const size_t sstride = (size_t)Wc * C;
       if (idx < N2) {
 #pragma unroll

@@ -38,12 +38,14 @@ namespace {
 thread_local std::string g_create_error;
 
 // ------------------------------------------------------------------------------------------ vector kernels ----
+constexpr int kVecThreads = 256;     // threads per block of the vector kernels
+
 // The CG step of batches.  float4 groups of its operands in flight per thread.  Two keep the kernel at 64 registers, four blocks of 256
 // threads per SM; four groups need 96 registers (two blocks per SM, measured 13.2 against 11.5 us per step at
 // 384 x 384 with 10 coils) or spill at 64.
 constexpr int kCgGroups = 2;
 // dx += alpha p; r -= alpha q; partial of |r|^2 -> brr_part[bid], over this block's share of the A.n2 float4.
-// A thread sums the squares of at most two float4 (8 products) in FP32 before adding them to its FP64 partial.
+// A thread sums the squares of at most two float4 (8 products) in FP32 before adding them to its pair.
 __device__ __forceinline__ void cg_step_update(float4& d, float4& r, const float4& p, const float4& q, float a,
                                                float& acc) {
   d.x = fmaf(a, p.x, d.x); d.y = fmaf(a, p.y, d.y); d.z = fmaf(a, p.z, d.z); d.w = fmaf(a, p.w, d.w);
@@ -52,35 +54,34 @@ __device__ __forceinline__ void cg_step_update(float4& d, float4& r, const float
 }
 
 // The CG step's scalars, the same in every block: t = Re<p, A p> from the n_pq partials, alpha = |r|^2 / t, and the
-// rounding-floor test (see cg_step_body).  Block 0 publishes them; s_alpha and s_skip (stopped by an earlier
+// rounding-floor test (see cg_step_body), formed as pairs by the block's first warp (in FP64, a tree over the block and a
+// quotient, each some thousand cycles a block).  Block 0 publishes them; s_alpha and s_skip (stopped by an earlier
 // iteration) are valid for every thread of the block on return.
-__device__ __forceinline__ void cg_step_decide(const KArgs& A, int bid, float& s_alpha, int& s_skip, double* red) {
-  double t = 0.0;
-  for (int k = threadIdx.x; k < A.n_pq; k += blockDim.x) t += A.pq_part[k];
-  t = nlv::block_sum(t, red);
-  if (threadIdx.x == 0) {
-    const double rr = A.sc->rr;
-    const bool was_stopped = nlv::cg_stopped(A);
-    double a = 0.0;
-    bool stop = false;
-    if (!was_stopped) {
-      if (!isfinite(t) || !isfinite(rr)) {
-        if (bid == 0) atomicOr(&A.sc->flags, nlv::kFlagBreakdown);
-        stop = true;
-      } else if (rr > nlv::kCgFloor2 * A.sc->rr0 && t > 0.0) {
-        a = rr / t;
-      } else {
-        stop = true;
+__device__ __forceinline__ void cg_step_decide(const KArgs& A, int bid, float& s_alpha, int& s_skip) {
+  if (threadIdx.x < 32) {
+    const nlv::Pair t = nlv::warp_sum_of(A.pq_part, A.n_pq, nlv::kGridScale);
+    if (threadIdx.x == 0) {
+      const nlv::Pair rr = A.sc->rr_i[0], floor = nlv::pair_scale(A.sc->rr_pair, (float)nlv::kCgFloor2);
+      const bool was_stopped = nlv::cg_stopped(A);
+      float a = 0.f;
+      bool stop = false;
+      if (!was_stopped) {
+        if (!isfinite(t.h) || !isfinite(rr.h)) {
+          if (bid == 0) atomicOr(&A.sc->flags, nlv::kFlagBreakdown);
+          stop = true;
+        } else if (nlv::pair_gt(rr, floor) && t.h > 0.f) {
+          a = nlv::pair_div(rr, t).h;
+        } else {
+          stop = true;
+        }
       }
+      if (bid == 0) {
+        A.sc->rr_i[1] = rr;
+        if (stop) A.sc->cg_stop[A.slot] = A.iter;
+      }
+      s_alpha = a;
+      s_skip = was_stopped ? 1 : 0;     // stopped by an earlier iteration: nothing to update
     }
-    if (bid == 0) {
-      A.sc->pq = t;
-      A.sc->alpha = a;
-      A.sc->rr_prev = rr;
-      if (stop) A.sc->cg_stop[A.slot] = A.iter;
-    }
-    s_alpha = (float)a;
-    s_skip = was_stopped ? 1 : 0;     // stopped by an earlier iteration: nothing to update
   }
   __syncthreads();
 }
@@ -109,11 +110,11 @@ __device__ __forceinline__ void cg_step_body(const KArgs& A, int bid, int nblk) 
     }
   __shared__ float s_alpha;
   __shared__ int s_skip;
-  __shared__ double red[32];
-  cg_step_decide(A, bid, s_alpha, s_skip, red);
+  __shared__ nlv::Pair s_pairs[kVecThreads];
+  cg_step_decide(A, bid, s_alpha, s_skip);
   if (s_skip) return;                 // the same for the whole block (thread 0 decided for it)
   const float a = s_alpha;
-  double accd = 0.0;
+  nlv::Pair sum = {0.f, 0.f};
   // G groups in flight per thread; each group's operands for the next round are loaded right after it is stored,
   // while the other groups of this round are processed
   while (i < A.n2) {
@@ -129,11 +130,12 @@ __device__ __forceinline__ void cg_step_body(const KArgs& A, int bid, int nblk) 
         if (kn < A.n2) { pg[g] = p4[kn]; qg[g] = q4[kn]; rg[g] = r4[kn]; dg[g] = dx4[kn]; }
       }
     }
-    accd += (double)acc;
+    nlv::acc_add(sum, acc);
     i += G * stride;
   }
-  const double s = nlv::block_sum(accd, red);
-  if (threadIdx.x == 0) A.brr_part[bid] = s;
+  s_pairs[threadIdx.x] = sum;
+  __syncthreads();
+  nlv::block_pairs<1>(s_pairs, {A.brr_part + bid});
 }
 
 // x += dx (x = A.dst)
@@ -234,7 +236,6 @@ __global__ void add_batch(const nlv::BatchArgs B) {
   }
 }
 
-constexpr int kVecThreads = 256;
 constexpr int kTuneVecMax = 8;       // largest vector-kernel blocks per SM that nlinv_autotune tries
 constexpr int kTuneMaxCandidates = 16;   // most candidates it times (2 splits + 3 strips + 3 row + 6 vector shapes)
 constexpr double kTuneMargin = 0.03; // a candidate replaces the compiled default only when this much faster
@@ -279,8 +280,8 @@ struct nlinv_ctx {
   float* wtab = nullptr;      // Sobolev weight, N x N
   uint8_t* mask = nullptr;
   double* partials = nullptr;
-  double* pq_part = nullptr;  // frames of a batch: per-block partials of Re<p, A p> and of |r|^2
-  double* brr_part = nullptr;
+  nlv::Pair* pq_part = nullptr;  // frames of a batch: per-block partials of Re<p, A p> and of |r|^2
+  nlv::Pair* brr_part = nullptr;
   nlv::Pair* dd_part = nullptr;  // single frames: per-block partials of |DF p|^2 of the PSF pass
   nlv::Pair* rr_part = nullptr;  // per-block partials of |r|^2, Re<r, p> and |p|^2 of the CG update pass
   Scalars* sc = nullptr;
@@ -900,11 +901,9 @@ nlinv_status validate(const nlinv_params* p, std::string* why) {
 // next right-hand side), so that every kernel does its full work.  Synchronous.
 cudaError_t mark_running(nlinv_ctx* c, int newton) {
   const int running = -1;
-  const double none = 0.0;
-  const nlv::Pair none_p = {0.f, 0.f};
+  const nlv::Pair none = {0.f, 0.f};
   cudaError_t e = cudaMemcpy(&c->sc->cg_stop[newton], &running, sizeof(int), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(&c->sc->rr0, &none, sizeof(double), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(&c->sc->rr_pair, &none_p, sizeof(none_p), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(&c->sc->rr_pair, &none, sizeof(none), cudaMemcpyHostToDevice);
   return e;
 }
 
@@ -1075,7 +1074,7 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
   cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
   // (the limit is raised to the device maximum so that contexts with different fov can share the kernels)
   std::string smem_err;
-  auto allow = [&](const void* fn, size_t need) {
+  auto allow = [&](const void* fn, size_t need, bool frame = true) {
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) { smem_err = "cudaFuncGetAttributes failed"; return; }
     const int dyn_max = smem_optin - (int)fa.sharedSizeBytes;
@@ -1086,22 +1085,25 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
     }
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_max) != cudaSuccess)
       smem_err = "cudaFuncSetAttribute failed";
-    // one carve-out for all passes: with the driver's own choice consecutive passes differ, and an SM changes its
-    // carve-out only when it is empty (256^2 with 8 coils: 4.41 -> 4.07 ms a frame; other sides within 1 %)
-    cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    // one carve-out for all single-frame passes: with the driver's own choice consecutive passes differ, and an SM changes
+    // its carve-out only when it is empty (256^2 with 8 coils: 4.41 -> 4.07 ms a frame; other sides within 2 %).  The
+    // batched passes run long enough to keep the driver's choice, which leaves more L1 for loads in flight (64 uneven
+    // frames, column DF^H pass: 203 us an iteration, 241 with the largest carve-out)
+    if (frame)
+      cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   };
   const int lanes_max = std::max(row_geom(c, false).lanes, row_geom(c, true).lanes);
   for (int m = 0; m < nlv::NUM_ROW_MODES && smem_err.empty(); ++m) {
     if (c->k->row[m]) allow(c->k->row[m], c->k->row_smem(m, lanes_max));
-    if (smem_err.empty() && c->k->row_batch[m]) allow(c->k->row_batch[m], c->k->row_smem(m, lanes_max));
+    if (smem_err.empty() && c->k->row_batch[m]) allow(c->k->row_batch[m], c->k->row_smem(m, lanes_max), false);
     if (smem_err.empty() && c->k->row_std[m]) allow(c->k->row_std[m], c->k->row_smem(m, lanes_max));
-    if (smem_err.empty() && c->k->row_std_batch[m]) allow(c->k->row_std_batch[m], c->k->row_smem(m, lanes_max));
+    if (smem_err.empty() && c->k->row_std_batch[m]) allow(c->k->row_std_batch[m], c->k->row_smem(m, lanes_max), false);
   }
   for (int m = 0; m < nlv::NUM_COL_MODES && smem_err.empty(); ++m) {
     if (c->k->col[m]) allow(c->k->col[m], c->k->col_smem(m, c->Wc));
-    if (smem_err.empty() && c->k->col_batch[m]) allow(c->k->col_batch[m], c->k->col_smem(m, c->Wc));
+    if (smem_err.empty() && c->k->col_batch[m]) allow(c->k->col_batch[m], c->k->col_smem(m, c->Wc), false);
     if (smem_err.empty() && c->k->col_std[m]) allow(c->k->col_std[m], c->k->col_smem(m, c->Wc));
-    if (smem_err.empty() && c->k->col_std_batch[m]) allow(c->k->col_std_batch[m], c->k->col_smem(m, c->Wc));
+    if (smem_err.empty() && c->k->col_std_batch[m]) allow(c->k->col_std_batch[m], c->k->col_smem(m, c->Wc), false);
   }
   if (c->tc) {
     for (int m = 0; m < nlv::NUM_ROW_MODES && smem_err.empty(); ++m) {
@@ -1171,8 +1173,8 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
   c->mask = (uint8_t*)take(maskb);
   c->partials = (double*)take(partb);
   if (batch) {
-    c->pq_part = (double*)take(partb);
-    c->brr_part = (double*)take(partb);
+    c->pq_part = (nlv::Pair*)take(partb);
+    c->brr_part = (nlv::Pair*)take(partb);
   } else {
     c->dd_part = (nlv::Pair*)take(partb);
     c->rr_part = (nlv::Pair*)take(3 * partb);
