@@ -55,11 +55,14 @@ constexpr int kFlagBreakdown = 1;
 // residual decays into the FP32 denormal range, where the step lengths lose their precision).
 constexpr double kCgFloor2 = 0x1p-48;
 
-struct KArgs {
+struct alignas(16) KArgs {
   int N, J, f, Wc;          // grid side, coils, half-width of Omega, compact width 2f
   int nrows;                // row passes: rows of the coil planes (J*N); column passes: J
   int rows_per_cta;         // row passes: consecutive coil rows handled by one block
   int rho_per_cta;          // row passes with a rho part: consecutive rho-plane pixels handled by one block
+  // Row passes of batches: the rows and the rho slice of such a block are shared by `sub` blocks of sub_lanes lanes, which
+  // together stand for its group_threads threads (see rho_slice); sub = 0: single frames, no sharing.
+  int sub, sub_lanes, group_threads;
   const float* wtab;        // Sobolev weight w(k) = (1 + a |k|^2)^(-l/2), N x N natural order
   float alpha;              // alpha_n of Eq. 3 for the normal operator and the right-hand side
   const float2* src;        // main input planes
@@ -378,6 +381,12 @@ enum RowMode : int {
 // threads) and loops over its share of rows when they do not fit at once.
 constexpr int kRowMaxThreads = 320;
 constexpr int kRowCtasPerSM = 2;
+// Row passes of batches: the same warps per SM in twice the blocks of half the size.  A block of these passes waits for its
+// loads, then for its exchanges; more and smaller blocks are more often at different points.  64 uneven frames: 288 ms with
+// 320 threads, 281 with 160, 292 with 96 (the launch of one side alone is faster with 320, 1.67 against 1.93 ms an
+// iteration over all sides, but in the batch's graph the sides run side by side).
+constexpr int kRowBatchThreads = 160;
+constexpr int kRowBatchCtasPerSM = 4;
 
 template <int MODE> struct RowTraits {
   static constexpr bool inverse_first = (MODE == ROW_W_IFFT || MODE == ROW_P_IFFT || MODE == ROW_BCG_DIR);
@@ -440,14 +449,15 @@ __device__ __forceinline__ void dot_flush(float2& acc, Pair& sum) {
   acc = make_float2(0.f, 0.f);
 }
 
-// The two pixels o0 and o0 + blockDim.x of a rho-plane step: which exist (ok), which lie on Omega (om, with their
+// The two pixels o0 and o0 + bd of a rho-plane step: which exist (ok), which lie on Omega (om, with their
 // compact offset zo).  Pixel and channel-product offsets fit 32 bits: a plane has at most 1024^2 pixels, the J
 // channel-product planes at most 64 x 512^2 entries.
 template <int N>
-__device__ __forceinline__ void rho_pixels(int o0, int e_end, int f, int Wc, bool (&ok)[2], bool (&om)[2], int (&zo)[2]) {
+__device__ __forceinline__ void rho_pixels(int o0, int bd, int e_end, int f, int Wc, bool (&ok)[2], bool (&om)[2],
+                                           int (&zo)[2]) {
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    const int o = o0 + k * (int)blockDim.x;
+    const int o = o0 + k * bd;
     const int e1 = o / N, e2 = o - e1 * N;
     ok[k] = o < e_end;
     om[k] = ok[k] && in_omega(e1, N, f) && in_omega(e2, N, f);
@@ -500,20 +510,22 @@ __device__ __forceinline__ void rho_channel_sum(const KArgs& A, const bool (&om)
 __device__ __forceinline__ void acc_add(double& s, float v) { s += (double)v; }
 __device__ __forceinline__ void acc_add(Pair& s, float v) { pair_add(s, v * kBlockScale, 0.f); }
 
+// t, bd: the thread's index in the block and the block's threads.  Blocks that share a slice (KArgs::sub) pass their
+// threads' places in the undivided block, so that a thread's two pixels, whose products it adds in FP32, stay the same
+// pair however the block is divided.
 template <int N, int MODE, bool STDF, class Sum>
-__device__ __forceinline__ void rho_slice(const KArgs& A, int bid, Sum& sum) {
+__device__ __forceinline__ void rho_slice(const KArgs& A, int bid, int t, int bd, Sum& sum) {
   const int f = STDF ? N / 4 : A.f, Wc = STDF ? N / 2 : A.Wc;
   constexpr int plane = N * N;
   const int e_begin = bid * A.rho_per_cta;
   const int e_end = min(e_begin + A.rho_per_cta, plane);
   const float beta = MODE == ROW_BCG_NORMAL ? A.sc->beta_p.h : 0.f;
-  const int bd = blockDim.x;
-  for (int o0 = e_begin + threadIdx.x; o0 < e_end; o0 += 2 * bd) {
+  for (int o0 = e_begin + t; o0 < e_end; o0 += 2 * bd) {
     float acc = 0.f;
     float2 a[2], b[2], z[2];
     int zo[2];
     bool ok[2], om[2];
-    rho_pixels<N>(o0, e_end, f, Wc, ok, om, zo);
+    rho_pixels<N>(o0, bd, e_end, f, Wc, ok, om, zo);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int o = o0 + k * bd;
@@ -622,7 +634,7 @@ __device__ __forceinline__ void rho_cg_slice(const KArgs& A, int bid, const CgSt
     float2 p[2], r[2], z[2];
     int zo[2];
     bool ok[2], om[2];
-    rho_pixels<N>(o0, e_end, f, Wc, ok, om, zo);
+    rho_pixels<N>(o0, bd, e_end, f, Wc, ok, om, zo);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int o = o0 + k * bd;
@@ -699,9 +711,10 @@ __device__ __forceinline__ void row_pass_prestage(const KArgs& A, int bid, unsig
 // plane.  All threads of the block run every round (inactive lanes carry zeros) because of the barriers.
 // PRE: the twiddles and the first round's side rows were staged by row_pass_prestage, and the body itself waits for
 // the kernel before (pdl_enter) and applies the stop test before its first loads.
+// tw_ready: the block has staged the twiddles already (a batched launch, for all its work items).
 template <int N1, int N2, int MODE, bool STDF = false, class TC = NoTc, bool PRE = false>
 __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk, unsigned char* smem_raw,
-                                              TC* tc = nullptr) {
+                                              TC* tc = nullptr, bool tw_ready = false) {
   using S = Split<N1, N2>;
   using T = RowTraits<MODE>;
   constexpr int N = S::N, TL = S::TL, E = S::E;
@@ -725,9 +738,13 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
   const float2* twA = (const float2*)(smem_raw + L.tw);
   const float2* twB = twA + N;
   const float rs = rsqrtf((float)N);
-  const int r_begin = bid * A.rows_per_cta;
-  const int r_end = min(r_begin + A.rows_per_cta, A.nrows);
-  if (!PRE) {
+  const int group = !PRE && A.sub > 0 ? bid / A.sub : bid, part = bid - group * A.sub;
+  int r_begin = group * A.rows_per_cta, r_end = min(r_begin + A.rows_per_cta, A.nrows);
+  if (!PRE && A.sub > 0) {
+    r_begin += part * A.sub_lanes;
+    r_end = min(r_begin + A.sub_lanes, r_end);
+  }
+  if (!PRE && !tw_ready) {
     stage_bytes(smem_raw + L.tw, A.twA, N * 8);
     stage_bytes(smem_raw + L.tw + N * 8, A.twB, N * 8);
   }
@@ -996,7 +1013,15 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
   }
   }  // rounds
 
-  if constexpr (T::has_rho) rho_slice<N, MODE, STDF>(A, bid, sum);
+  if constexpr (T::has_rho) {
+    if (PRE || A.sub == 0) {
+      rho_slice<N, MODE, STDF>(A, bid, threadIdx.x, blockDim.x, sum);
+    } else {
+      const int t = threadIdx.x + part * A.sub_lanes * TL;
+      if ((int)threadIdx.x < A.sub_lanes * TL && t < A.group_threads)
+        rho_slice<N, MODE, STDF>(A, group, t, A.group_threads, sum);
+    }
+  }
   if constexpr (CG) {
     rho_cg_slice<N, STDF>(A, bid, s_cg, sums);
     __syncthreads();
@@ -1091,7 +1116,8 @@ __device__ __forceinline__ void stage_natural_cols(float2* sdst, const float2* p
 // rho), which a single-frame pass stages before its dependent-launch wait; else the rest: drho, for the CG direction
 // pass the rho planes of p and r that the CG update pass just before has written.
 template <int N1, int N2, int MODE, bool STDF, int CC>
-__device__ __forceinline__ void col_stage_side(const KArgs& A, int bid, unsigned char* smem_raw, bool before) {
+__device__ __forceinline__ void col_stage_side(const KArgs& A, int bid, unsigned char* smem_raw, bool before,
+                                               bool tw_ready = false) {
   using S = Split<N1, N2>;
   constexpr int N = S::N, C = ColCfg<N1, N2, CC>::C;
   const int f = STDF ? N / 4 : A.f, Wc = STDF ? N / 2 : A.Wc;
@@ -1102,8 +1128,10 @@ __device__ __forceinline__ void col_stage_side(const KArgs& A, int bid, unsigned
   float2* sd = (float2*)(smem_raw + L.side);
   const size_t sstride = (size_t)Wc * C;
   if (before) {
-    stage_bytes(smem_raw + L.tw, A.twA, N * 8);
-    stage_bytes(smem_raw + L.tw + N * 8, A.twB, N * 8);
+    if (!tw_ready) {
+      stage_bytes(smem_raw + L.tw, A.twA, N * 8);
+      stage_bytes(smem_raw + L.tw + N * 8, A.twB, N * 8);
+    }
     if constexpr (MODE == COL_IFFT_PROD_FFT || MODE == COL_IFFT_ADJ_FFT || MODE == COL_CG_DIR || MODE == COL_BCG_DIR) {
       if (j < A.nrows) {
         stage_compact_cols(sd, A.coil + (size_t)j * Wc * Wc, cc0, C, Wc);
@@ -1184,7 +1212,7 @@ __device__ __forceinline__ void cg_decide(const KArgs& A) {
 // the dependent-launch wait.
 template <int N1, int N2, int MODE, bool STDF = false, class TC = NoTc, int CC = NLV_COL_C>
 __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, int nblk, unsigned char* smem_raw,
-                                              TC* tc = nullptr, bool prestaged = false) {
+                                              TC* tc = nullptr, bool prestaged = false, bool tw_ready = false) {
   using S = Split<N1, N2>;
   constexpr int N = S::N, E = S::E, C = ColCfg<N1, N2, CC>::C;
   if constexpr (MODE == COL_IFFT_ADJ_FFT) {
@@ -1246,7 +1274,7 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, int nblk,
     }
   }
   // ---- staged side inputs (Omega rows of this block's columns) and twiddles
-  if (!prestaged) col_stage_side<N1, N2, MODE, STDF, CC>(A, bid, smem_raw, true);
+  if (!prestaged) col_stage_side<N1, N2, MODE, STDF, CC>(A, bid, smem_raw, true, tw_ready);
   col_stage_side<N1, N2, MODE, STDF, CC>(A, bid, smem_raw, false);
   if constexpr (MODE == COL_CG_DIR) {      // while the loads above are in flight; read after the first transform
     if (A.iter > 0) cg_direction_scalars(A, bid, s_beta, s_stop);
@@ -1387,64 +1415,118 @@ __global__ void __launch_bounds__(ColCfg<N1, N2>::THREADS, 1) col_pass_tc(const 
 struct BatchArgs {
   const KArgs* args;       // per-frame arguments (device)
   const int* first;        // nframes + 1 block offsets (device)
+  const int* const* stops; // per-frame Scalars::cg_stop (device)
   int nframes;
   int total;               // work items = first[nframes]; a block takes items blockIdx.x, + gridDim.x, ...
+  int slot, skip;          // a launch of a CG iteration: its Newton step, and KArgs::skip
 };
 
-// Work item w of a batched launch: its frame's arguments (copied to shared memory), its block index within the
-// frame and the frame's block count.  Every thread of the block calls it (barriers).
-__device__ __forceinline__ const KArgs& batch_frame(const BatchArgs& B, int w, int& bid, int& nblk) {
-  __shared__ KArgs sa;
-  __shared__ int sf, sb, sn;
-  __syncthreads();         // the previous work item of this block is done with sa
-  // the frame is the number of block offsets first[1 .. nframes-1] at or below this item (offsets increase):
-  // the first warp tests 32 of them per step, all loads of a step in flight together
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x, nl = warp_lanes();
-    const unsigned live = nl >= 32 ? 0xffffffffu : (1u << nl) - 1u;
-    int f = 0;
-    for (int base = 1; base < B.nframes; base += nl) {
-      const int k = base + lane;
-      const bool le = lane < nl && k < B.nframes && B.first[k] <= w;
-      f += __popc(__ballot_sync(live, le));
-    }
-    if (lane == 0) {
-      sf = f;
-      sb = w - B.first[f];
-      sn = B.first[f + 1] - B.first[f];
-    }
+// The work items of a block: the arguments of the next item are fetched into shared memory while the block works on the
+// current one, by its last warp (in most splits that warp has no part in the first half of a transform), so that an item
+// starts without waiting for the chain offsets -> arguments -> stop -> inputs.  Before, that chain and the twiddles staged
+// anew for every item took 299 ms of 64 uneven frames; so, 288.  The row passes' next inputs, consecutive rows, go to L2
+// meanwhile (281 -> 275 ms; the column passes' 64-byte pieces did not gain from it).
+struct BatchQueue {
+  KArgs args[2];
+  int bid[2], nblk[2];
+  int stop[2];             // Scalars::cg_stop of the item's frame
+};
+
+// The calling warp fetches work item w into slot k (asynchronous copies: the caller waits, then a block barrier).
+__device__ __forceinline__ void batch_fetch(const BatchArgs& B, int w, BatchQueue& q, int k) {
+  const int lane = threadIdx.x & 31, nl = warp_lanes();
+  const unsigned live = nl >= 32 ? 0xffffffffu : (1u << nl) - 1u;
+  // the frame is the number of block offsets first[1 .. nframes-1] at or below this item (offsets increase): a warp tests
+  // 32 of them per step, all loads of a step in flight together
+  int f = 0;
+  for (int base = 1; base < B.nframes; base += nl) {
+    const int i = base + lane;
+    const bool le = lane < nl && i < B.nframes && B.first[i] <= w;
+    f += __popc(__ballot_sync(live, le));
   }
+  static_assert(sizeof(KArgs) % 16 == 0, "copied in 16-byte pieces");
+  for (int i = lane; i < (int)(sizeof(KArgs) / 16); i += nl) cp_async16((char*)&q.args[k] + 16 * i, (const char*)(B.args + f) + 16 * i);
+  if (lane == 0) {
+    q.stop[k] = B.skip > 0 ? *(volatile const int*)(B.stops[f] + B.slot) : -1;
+    q.bid[k] = w - B.first[f];
+    q.nblk[k] = B.first[f + 1] - B.first[f];
+  }
+}
+
+// Prefetches nbytes (a multiple of 16, 16-byte aligned) into L2.
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned nbytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(nbytes) : "memory");
+}
+// By one thread: the inputs of a row-pass work item that lie in consecutive rows, into L2.
+template <int N1, int N2, int MODE, bool STDF>
+__device__ __forceinline__ void row_prefetch(const KArgs& A, int bid) {
+  using T = RowTraits<MODE>;
+  constexpr int N = N1 * N2;
+  const int Wc = STDF ? N / 2 : A.Wc;
+  const int group = A.sub > 0 ? bid / A.sub : bid;
+  const int r0 = group * A.rows_per_cta + (bid - group * A.sub) * A.sub_lanes;
+  const int nr = min(min(A.sub > 0 ? A.sub_lanes : A.rows_per_cta, (group + 1) * A.rows_per_cta - r0), A.nrows - r0);
+  if (nr <= 0) return;
+  if constexpr (T::load_compact) prefetch_l2(A.src + (size_t)r0 * Wc, (unsigned)(nr * Wc * 8));
+  else prefetch_l2(A.src + (size_t)r0 * N, (unsigned)(nr * N * 8));
+  if constexpr (MODE == ROW_BCG_DIR) prefetch_l2(A.r + (size_t)r0 * N, (unsigned)(nr * N * 8));
+  if constexpr (MODE == ROW_BCG_NORMAL) prefetch_l2(A.p + (size_t)(N + r0) * N, (unsigned)(nr * N * 8));
+}
+
+// Runs item(args, bid, nblk, stopped) for every work item of this block; stopped: the item's frame has stopped before this
+// CG iteration (see cg_stopped).  ahead(args, bid): one thread, for the next item once it is fetched.
+struct NoAhead {
+  __device__ __forceinline__ void operator()(const KArgs&, int) const {}
+};
+template <class Item, class Ahead = NoAhead>
+__device__ __forceinline__ void batch_items(const BatchArgs& B, BatchQueue& q, Item&& item, Ahead&& ahead = NoAhead()) {
+  const bool fetcher = threadIdx.x >= ((blockDim.x - 1) & ~31u);
+  int w = blockIdx.x, k = 0;
+  if (fetcher && w < B.total) batch_fetch(B, w, q, 0);
+  cp_async_wait_all();
   __syncthreads();
-  const int* src = (const int*)(B.args + sf);
-  for (int i = threadIdx.x; i < (int)(sizeof(KArgs) / sizeof(int)); i += blockDim.x) ((int*)&sa)[i] = src[i];
-  bid = sb;
-  nblk = sn;
-  __syncthreads();
-  return sa;
+  for (; w < B.total; w += gridDim.x, k ^= 1) {
+    if (fetcher && w + (int)gridDim.x < B.total) {
+      batch_fetch(B, w + gridDim.x, q, k ^ 1);
+      if constexpr (!std::is_same_v<std::decay_t<Ahead>, NoAhead>) {
+        cp_async_wait_all();
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0 && (unsigned)q.stop[k ^ 1] >= (unsigned)B.skip) ahead(q.args[k ^ 1], q.bid[k ^ 1]);
+      }
+    }
+    item(q.args[k], q.bid[k], q.nblk[k], (unsigned)q.stop[k] < (unsigned)B.skip);
+    cp_async_wait_all();
+    __syncthreads();       // the next item is fetched, and this block is done with this one's shared memory
+  }
 }
 
 template <int N1, int N2, int MODE, bool STDF = false>
-__global__ void __launch_bounds__(kRowMaxThreads, kRowCtasPerSM) row_pass_batch(const BatchArgs B) {
+__global__ void __launch_bounds__(kRowBatchThreads, kRowBatchCtasPerSM) row_pass_batch(const BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ BatchQueue q;
+  using S = Split<N1, N2>;
+  const RowSmem L = row_smem(MODE, S::N, blockDim.x / S::TL, S::SM_LANE);
+  // the tables are the same for every frame of the side
+  stage_bytes(smem_raw + L.tw, B.args[0].twA, S::N * 8);
+  stage_bytes(smem_raw + L.tw + S::N * 8, B.args[0].twB, S::N * 8);
   pdl_enter();
-  for (int w = blockIdx.x; w < B.total; w += gridDim.x) {
-    int bid, nblk;
-    const KArgs& A = batch_frame(B, w, bid, nblk);
-    if (cg_stopped(A)) continue;
-    row_pass_body<N1, N2, MODE, STDF>(A, bid, nblk, smem_raw);
-  }
+  batch_items(B, q, [&](const KArgs& A, int bid, int nblk, bool stopped) {
+    if (!stopped) row_pass_body<N1, N2, MODE, STDF>(A, bid, nblk, smem_raw, (NoTc*)nullptr, true);
+  }, [&](const KArgs& A, int bid) { row_prefetch<N1, N2, MODE, STDF>(A, bid); });
 }
 
 template <int N1, int N2, int MODE, bool STDF = false>
 __global__ void __launch_bounds__(ColCfg<N1, N2>::THREADS) col_pass_batch(const BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ BatchQueue q;
+  using S = Split<N1, N2>;
+  const ColSmem L = col_smem(MODE, S::N, ColCfg<N1, N2>::C, S::SM_LANE_COL, S::N / 2);
+  stage_bytes(smem_raw + L.tw, B.args[0].twA, S::N * 8);
+  stage_bytes(smem_raw + L.tw + S::N * 8, B.args[0].twB, S::N * 8);
   pdl_enter();
-  for (int w = blockIdx.x; w < B.total; w += gridDim.x) {
-    int bid, nblk;
-    const KArgs& A = batch_frame(B, w, bid, nblk);
-    if (cg_stopped(A)) continue;
-    col_pass_body<N1, N2, MODE, STDF>(A, bid, nblk, smem_raw);
-  }
+  batch_items(B, q, [&](const KArgs& A, int bid, int nblk, bool stopped) {
+    if (!stopped) col_pass_body<N1, N2, MODE, STDF>(A, bid, nblk, smem_raw, (NoTc*)nullptr, false, true);
+  });
 }
 
 // ------------------------------------------------------------------------- batches of several sides ----
@@ -1492,25 +1574,21 @@ __device__ __forceinline__ void col_body_of_side(const KArgs& A, int bid, int nb
 template <int MODE, bool STDF>
 __global__ void __launch_bounds__(kRowMaxThreads, kRowCtasPerSM) row_pass_multi(const BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ BatchQueue q;
   pdl_enter();
-  for (int w = blockIdx.x; w < B.total; w += gridDim.x) {
-    int bid, nblk;
-    const KArgs& A = batch_frame(B, w, bid, nblk);
-    if (cg_stopped(A)) continue;
-    row_body_of_side<MODE, STDF>(A, bid, nblk, smem_raw);
-  }
+  batch_items(B, q, [&](const KArgs& A, int bid, int nblk, bool stopped) {
+    if (!stopped) row_body_of_side<MODE, STDF>(A, bid, nblk, smem_raw);
+  });
 }
 
 template <int MODE, bool STDF>
 __global__ void __launch_bounds__(kMultiColThreads) col_pass_multi(const BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ BatchQueue q;
   pdl_enter();
-  for (int w = blockIdx.x; w < B.total; w += gridDim.x) {
-    int bid, nblk;
-    const KArgs& A = batch_frame(B, w, bid, nblk);
-    if (cg_stopped(A)) continue;
-    col_body_of_side<MODE, STDF>(A, bid, nblk, smem_raw);
-  }
+  batch_items(B, q, [&](const KArgs& A, int bid, int nblk, bool stopped) {
+    if (!stopped) col_body_of_side<MODE, STDF>(A, bid, nblk, smem_raw);
+  });
 }
 
 // The multi-side kernels of every pass (defined in batch_multi.cu) and their dynamic shared memory (the largest
@@ -1563,6 +1641,7 @@ struct SizeKernels {
 // pixels of the rho plane when the pass has one), so that the rows are split evenly over ctas_per_sm blocks per SM.
 struct RowGrid {
   int blocks, lanes, rows_per_cta, rho_per_cta;
+  int sub;       // batches: blocks that share one block's rows and slice (KArgs::sub)
 };
 inline RowGrid row_grid(const SizeKernels* k, int nrows, long rho_pixels, int sms, int ctas_per_sm) {
   RowGrid g{};

@@ -55,32 +55,21 @@ __device__ __forceinline__ void cg_step_update(float4& d, float4& r, const float
 
 // The CG step's scalars, the same in every block: t = Re<p, A p> from the n_pq partials, alpha = |r|^2 / t, and the
 // rounding-floor test (see cg_step_body), formed as pairs by the block's first warp (in FP64, a tree over the block and a
-// quotient, each some thousand cycles a block).  Block 0 publishes them; s_alpha and s_skip (stopped by an earlier
-// iteration) are valid for every thread of the block on return.
-__device__ __forceinline__ void cg_step_decide(const KArgs& A, int bid, float& s_alpha, int& s_skip) {
+// quotient, each some thousand cycles a block).  Block 0 publishes them; s_alpha is valid for every thread of the block
+// on return.
+__device__ __forceinline__ void cg_step_decide(const KArgs& A, int bid, float& s_alpha) {
   if (threadIdx.x < 32) {
     const nlv::Pair t = nlv::warp_sum_of(A.pq_part, A.n_pq, nlv::kGridScale);
     if (threadIdx.x == 0) {
       const nlv::Pair rr = A.sc->rr_i[0], floor = nlv::pair_scale(A.sc->rr_pair, (float)nlv::kCgFloor2);
-      const bool was_stopped = nlv::cg_stopped(A);
-      float a = 0.f;
-      bool stop = false;
-      if (!was_stopped) {
-        if (!isfinite(t.h) || !isfinite(rr.h)) {
-          if (bid == 0) atomicOr(&A.sc->flags, nlv::kFlagBreakdown);
-          stop = true;
-        } else if (nlv::pair_gt(rr, floor) && t.h > 0.f) {
-          a = nlv::pair_div(rr, t).h;
-        } else {
-          stop = true;
-        }
-      }
+      const bool finite = isfinite(t.h) && isfinite(rr.h);
+      const bool go = finite && nlv::pair_gt(rr, floor) && t.h > 0.f;
       if (bid == 0) {
         A.sc->rr_i[1] = rr;
-        if (stop) A.sc->cg_stop[A.slot] = A.iter;
+        if (!go) A.sc->cg_stop[A.slot] = A.iter;
+        if (!finite) atomicOr(&A.sc->flags, nlv::kFlagBreakdown);
       }
-      s_alpha = a;
-      s_skip = was_stopped ? 1 : 0;     // stopped by an earlier iteration: nothing to update
+      s_alpha = go ? nlv::pair_div(rr, t).h : 0.f;
     }
   }
   __syncthreads();
@@ -109,10 +98,8 @@ __device__ __forceinline__ void cg_step_body(const KArgs& A, int bid, int nblk) 
       pg[g] = p4[k]; qg[g] = q4[k]; rg[g] = r4[k]; dg[g] = dx4[k];
     }
   __shared__ float s_alpha;
-  __shared__ int s_skip;
   __shared__ nlv::Pair s_pairs[kVecThreads];
-  cg_step_decide(A, bid, s_alpha, s_skip);
-  if (s_skip) return;                 // the same for the whole block (thread 0 decided for it)
+  cg_step_decide(A, bid, s_alpha);
   const float a = s_alpha;
   nlv::Pair sum = {0.f, 0.f};
   // G groups in flight per thread; each group's operands for the next round are loaded right after it is stored,
@@ -220,20 +207,18 @@ __global__ void cg_init_kernel(const KArgs A) {
 }
 
 __global__ void __launch_bounds__(256, 4) cg_step_batch(const nlv::BatchArgs B) {
+  __shared__ nlv::BatchQueue q;
   nlv::pdl_enter();
-  for (int w = blockIdx.x; w < B.total; w += gridDim.x) {
-    int bid, nblk;
-    const KArgs& A = nlv::batch_frame(B, w, bid, nblk);
-    cg_step_body<kCgGroups>(A, bid, nblk);
-  }
+  nlv::batch_items(B, q, [&](const KArgs& A, int bid, int nblk, bool stopped) {
+    if (!stopped) cg_step_body<kCgGroups>(A, bid, nblk);
+  });
 }
 __global__ void add_batch(const nlv::BatchArgs B) {
+  __shared__ nlv::BatchQueue q;
   nlv::pdl_enter();
-  for (int w = blockIdx.x; w < B.total; w += gridDim.x) {
-    int bid, nblk;
-    const KArgs& A = nlv::batch_frame(B, w, bid, nblk);
-    add_body(A, bid, nblk);
-  }
+  nlv::batch_items(B, q, [&](const KArgs& A, int bid, int nblk, bool stopped) {
+    if (!stopped) add_body(A, bid, nblk);
+  });
 }
 
 constexpr int kTuneVecMax = 8;       // largest vector-kernel blocks per SM that nlinv_autotune tries
@@ -355,10 +340,13 @@ nlv::RowGrid row_geom(const nlinv_ctx* c, bool with_rho) {
   if (c->batch_lanes > 0) {           // batch frames: equal block shapes for every frame of a grid side
     nlv::RowGrid g{};
     const int rows = c->J * c->N;
-    g.lanes = std::min(c->batch_lanes, rows);
-    g.rows_per_cta = g.lanes;
-    g.blocks = (rows + g.lanes - 1) / g.lanes;
-    g.rho_per_cta = with_rho ? (int)((c->plane + g.blocks - 1) / g.blocks) : 0;
+    g.rows_per_cta = std::min(c->batch_lanes, rows);
+    const int groups = (rows + g.rows_per_cta - 1) / g.rows_per_cta;
+    g.sub = 1;
+    while ((g.rows_per_cta + g.sub - 1) / g.sub * c->k->tl > nlv::kRowBatchThreads) ++g.sub;
+    g.lanes = (g.rows_per_cta + g.sub - 1) / g.sub;
+    g.blocks = groups * g.sub;
+    g.rho_per_cta = with_rho ? (int)((c->plane + groups - 1) / groups) : 0;
     return g;
   }
   nlv::RowGrid g = nlv::row_grid(c->k, c->J * c->N, with_rho ? c->plane : 0, c->sms, c->row_ctas_per_sm);
@@ -439,6 +427,9 @@ cudaError_t row(nlinv_ctx* c, int mode, KArgs a) {
   a.nrows = c->J * c->N;
   a.rows_per_cta = g.rows_per_cta;
   a.rho_per_cta = g.rho_per_cta;
+  a.sub = g.sub;
+  a.sub_lanes = g.lanes;
+  a.group_threads = g.rows_per_cta * c->k->tl;
   void* args[] = {&a};
   if (c->tc) {
     const void* fn = (c->std_fov && c->k->row_tc_std[mode]) ? c->k->row_tc_std[mode] : c->k->row_tc[mode];
@@ -2023,7 +2014,7 @@ nlinv_status nlinv_batch_create(const nlinv_params* params, int nframes, const n
     if (e != cudaSuccess) return batch_fail(b, NLINV_ECUDA, std::string("recording: ") + cudaGetErrorString(e));
   }
   std::vector<char> host;
-  std::vector<size_t> arg_off, first_off;
+  std::vector<size_t> arg_off, first_off, stop_off;
   for (size_t g = 0; g < b->groups.size(); ++g) {
     const std::vector<int>& fr = b->groups[g];
     const size_t L = recs[fr[0]].size();
@@ -2031,6 +2022,12 @@ nlinv_status nlinv_batch_create(const nlinv_params* params, int nframes, const n
     for (int i : fr)
       if (recs[i].size() != L) return batch_fail(b, NLINV_EINVAL, "frames of one grid side differ in schedule");
     const bool multi = sides[g] == 0;
+    stop_off.push_back((host.size() + 15) / 16 * 16);
+    host.resize(stop_off.back() + fr.size() * sizeof(const int*));
+    for (size_t t = 0; t < fr.size(); ++t) {
+      const int* at = b->frames[fr[t]]->sc->cg_stop;      // a device address
+      std::memcpy(host.data() + stop_off.back() + t * sizeof(at), &at, sizeof(at));
+    }
     for (size_t l = 0; l < L; ++l) {
       nlinv_batch::Launch bl{};
       bl.group = (int)g;
@@ -2081,6 +2078,8 @@ nlinv_status nlinv_batch_create(const nlinv_params* params, int nframes, const n
       first_off.push_back(off);
       bl.args.nframes = (int)fr.size();
       bl.args.total = first.back();
+      bl.args.slot = recs[fr[0]][l].args.slot;
+      bl.args.skip = recs[fr[0]][l].args.skip;
       b->launches.push_back(bl);
     }
   }
@@ -2091,6 +2090,7 @@ nlinv_status nlinv_batch_create(const nlinv_params* params, int nframes, const n
   for (size_t l = 0; l < b->launches.size(); ++l) {
     b->launches[l].args.args = (const KArgs*)((char*)b->tables + arg_off[l]);
     b->launches[l].args.first = (const int*)((char*)b->tables + first_off[l]);
+    b->launches[l].args.stops = (const int* const*)((char*)b->tables + stop_off[b->launches[l].group]);
   }
   // one graph: the groups as parallel branches
   const size_t G = b->groups.size();
