@@ -341,6 +341,10 @@ __device__ __forceinline__ void stage_bytes(void* sdst, const void* gsrc, int nb
     cp_async16((char*)sdst + 16 * i, (const char*)gsrc + 16 * i);
 }
 
+// Prefetches nbytes (a multiple of 16, 16-byte aligned) into L2.
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned nbytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(nbytes) : "memory");
+}
 __host__ __device__ constexpr size_t align16(size_t v) { return (v + 15) / 16 * 16; }
 
 // Rows R0 .. R0+nr-1 of rb bytes each (rb a multiple of 16) into consecutive rows of sdst: row R of gsrc, or row
@@ -1453,10 +1457,6 @@ __device__ __forceinline__ void batch_fetch(const BatchArgs& B, int w, BatchQueu
   }
 }
 
-// Prefetches nbytes (a multiple of 16, 16-byte aligned) into L2.
-__device__ __forceinline__ void prefetch_l2(const void* p, unsigned nbytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(nbytes) : "memory");
-}
 // By one thread: the inputs of a row-pass work item that lie in consecutive rows, into L2.
 template <int N1, int N2, int MODE, bool STDF>
 __device__ __forceinline__ void row_prefetch(const KArgs& A, int bid) {

@@ -6,13 +6,14 @@
 
 namespace nlv {
 
-// A side with the cluster CG solve added.
-template <int N1, int N2> SizeKernels make_size_kernels_cluster() {
-  static_assert(N1 * N2 <= kClusterMaxSide, "the cluster solve is for small sides");
+// The kernel table of a side, with the cluster CG solve where the side is small enough for it.
+template <int N1, int N2> SizeKernels make_side() {
   SizeKernels s = make_size_kernels<N1, N2>();
-  s.cluster = (const void*)cg_solve_cluster<N1, N2>;
-  s.cluster_threads = ClusterSmem<N1, N2>::T;
-  s.cluster_smem = cluster_smem_bytes<N1, N2>;
+  if constexpr (N1 * N2 <= kClusterMaxSide) {
+    s.cluster = (const void*)cg_solve_cluster<N1, N2>;
+    s.cluster_threads = ClusterSmem<N1, N2>::T;
+    s.cluster_smem = cluster_smem_bytes<N1, N2>;
+  }
   return s;
 }
 
@@ -50,12 +51,7 @@ inline const SizeKernels* find_size(int n) {
 
 #define NLV_SIZE_CASE(n, a, b)                                      \
   case n: {                                                         \
-    static const ::nlv::SizeKernels k = ::nlv::make_size_kernels<a, b>(); \
-    return &k;                                                      \
-  }
-#define NLV_SIZE_CASE_SMALL(n, a, b)                                \
-  case n: {                                                         \
-    static const ::nlv::SizeKernels k = ::nlv::make_size_kernels_cluster<a, b>(); \
+    static const ::nlv::SizeKernels k = ::nlv::make_side<a, b>(); \
     return &k;                                                      \
   }
 // A side that also has the passes with tensor-core radix-16 stages.
