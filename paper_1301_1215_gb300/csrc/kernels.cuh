@@ -67,6 +67,10 @@ struct alignas(16) KArgs {
   float alpha;              // alpha_n of Eq. 3 for the normal operator and the right-hand side
   const float2* src;        // main input planes
   float2* dst;              // main output planes
+  const float2* src2;       // passes with two inputs: the second (row passes: rows nrows1 .. nrows-1, into dst2)
+  float2* dst2;
+  int nrows1;
+  float2* coil_out;         // column passes that form the coil maps: where they go (compact J x Wc x Wc), or NULL
   const float2* rho;        // rho of the linearisation point (natural N x N)
   const float2* drho;       // rho part of the direction (natural N x N)
   const float2* coil;       // c_j on Omega, compact J x Wc x Wc
@@ -378,7 +382,10 @@ enum RowMode : int {
   ROW_BCG_RHS = 10,      // as ADJ, minus alpha (x - xref); r = p = b, dx = 0, |b|^2     (right-hand side)
   ROW_BCG_DIR = 11,      // p = r + beta p; T <- compact cols of FFT^-1_row(w p / sqrt N)
   ROW_BCG_NORMAL = 12,   // as NORMAL with the rho part of p = r + beta p; Re<p, q>
-  NUM_ROW_MODES = 13
+  // operators: two arrays in one launch
+  ROW_W_W_IFFT = 13,     // T <- W_IFFT of src, T2 <- W_IFFT of src2
+  ROW_W_P_IFFT = 14,     // T <- W_IFFT of src, T2 <- P_IFFT of src2
+  NUM_ROW_MODES = 15
 };
 
 // Row passes run kRowCtasPerSM blocks per SM; a block holds up to kRowMaxThreads threads (whole lanes of TL
@@ -393,7 +400,8 @@ constexpr int kRowBatchThreads = 160;
 constexpr int kRowBatchCtasPerSM = 4;
 
 template <int MODE> struct RowTraits {
-  static constexpr bool inverse_first = (MODE == ROW_W_IFFT || MODE == ROW_P_IFFT || MODE == ROW_BCG_DIR);
+  static constexpr bool both = (MODE == ROW_W_W_IFFT || MODE == ROW_W_P_IFFT);
+  static constexpr bool inverse_first = (MODE == ROW_W_IFFT || MODE == ROW_P_IFFT || MODE == ROW_BCG_DIR || both);
   static constexpr bool load_compact = !inverse_first;
   static constexpr bool psf = (MODE == ROW_PSF || MODE == ROW_CG_PSF);
   static constexpr bool normal = (MODE == ROW_FFT_W_NORMAL || MODE == ROW_BCG_NORMAL);
@@ -404,7 +412,7 @@ template <int MODE> struct RowTraits {
   static constexpr bool two = (psf || MODE == ROW_CG_RHS || MODE == ROW_CG_UPDATE);
   // side inputs staged per row: sampling-pattern row (bytes), weight row (floats), complex rows
   static constexpr bool s_mask = (psf || MODE == ROW_FFT_P_OUT || MODE == ROW_FFT_RESID);
-  static constexpr bool s_w = has_rho || MODE == ROW_W_IFFT || MODE == ROW_BCG_DIR || MODE == ROW_CG_UPDATE;
+  static constexpr bool s_w = has_rho || MODE == ROW_W_IFFT || MODE == ROW_BCG_DIR || MODE == ROW_CG_UPDATE || both;
 };
 
 // Shared-memory layout of a row pass (byte offsets), identical on host and device.
@@ -782,6 +790,10 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
   // ---- batches' direction update: the rows of r go to the exchange buffer (natural order, pitch N) while p is loaded
   if constexpr (MODE == ROW_BCG_DIR) stage_rows(smem_raw + L.xch, A.r, R0, min(LANES, r_end - R0), N * 8, N, false);
 
+  // passes over two arrays: which one this thread's layout-A row belongs to
+  [[maybe_unused]] const bool second = T::both && RA >= A.nrows1;
+  [[maybe_unused]] const float2* srcA = nullptr;
+  if constexpr (T::both) srcA = second ? A.src2 + (size_t)(RA - A.nrows1) * N : A.src + (size_t)RA * N;
   // ---- main loads, layout A: thread a < N1 holds row elements a + N1*m (no stores until all are issued)
   if (mapA) {
 #pragma unroll
@@ -791,6 +803,10 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
       if (activeA) {
         if constexpr (T::load_compact) {
           if (in_omega(e2, N, f)) val = A.src[(size_t)RA * Wc + to_compact(e2, N, f)];
+        } else if constexpr (T::both) {
+          val = srcA[e2];
+          if constexpr (MODE == ROW_W_P_IFFT)
+            if (second) val = A.mask[(size_t)e1A * N + e2] ? val : make_float2(0.f, 0.f);
         } else if constexpr (MODE != ROW_P_IFFT) {
           val = A.src[(size_t)RA * N + e2];
         } else {
@@ -854,11 +870,12 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
       }
     }
     __syncthreads();   // the exchange below overwrites the staged rows of r
-  } else if constexpr (MODE == ROW_W_IFFT) {
+  } else if constexpr (MODE == ROW_W_IFFT || T::both) {
     const float* sw = (const float*)(smem_raw + L.w) + (size_t)laneA * N;
     if (activeA) {
 #pragma unroll
-      for (int m = 0; m < N2; ++m) v[m] = cscale(v[m], sw[idxA + N1 * m] * rs);
+      for (int m = 0; m < N2; ++m)
+        v[m] = cscale(v[m], MODE == ROW_W_P_IFFT && second ? rs : sw[idxA + N1 * m] * rs);
     }
   } else if constexpr (MODE == ROW_P_IFFT) {
     if (mapA) {
@@ -870,7 +887,16 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
   if constexpr (T::inverse_first) {
     fft_AtoB2<N1, N2, +1, E, TC, false>(v, smA, idxA, mapA, smB, idxB, mapB, twA, tc);
     // layout B: thread b < N2 holds elements b + N2*m; keep the Omega columns
-    if (activeB) {
+    if constexpr (T::both) {
+      float2* d = RB >= A.nrows1 ? A.dst2 + (size_t)(RB - A.nrows1) * Wc : A.dst + (size_t)RB * Wc;
+      if (activeB) {
+#pragma unroll
+        for (int m = 0; m < N1; ++m) {
+          const int e2 = idxB + N2 * m;
+          if (in_omega(e2, N, f)) d[to_compact(e2, N, f)] = v[m];
+        }
+      }
+    } else if (activeB) {
 #pragma unroll
       for (int m = 0; m < N1; ++m) {
         const int e2 = idxB + N2 * m;
@@ -1062,22 +1088,33 @@ enum ColMode : int {
   COL_IFFT_ADJ_FFT = 4,   // z = M FFT^-1_col(T); zsum_j = conj(c_j) z; T <- FFT_col(conj(rho) z)   (DF^H)
   COL_CG_DIR = 5,         // single frames: U <- FFT^-1_col(T) + beta U;  T <- FFT_col(M ((r + beta p)_rho c_j + rho U))
   COL_BCG_DIR = 6,        // batches: COL_IFFT_PROD_FFT for the rho part of p = r + beta p
-  NUM_COL_MODES = 7
+  // operators: the coil maps c = FFT^-1_col(T) and what follows them in one pass (c to coil_out, if given)
+  COL_COIL_PROD = 7,      // T <- FFT_col(M rho c)                                               (F)
+  COL_COIL_DIR = 8,       // u = FFT^-1_col(T2);  T <- FFT_col(M (drho c + rho u))                (DF)
+  COL_COIL_ADJ = 9,       // z = M FFT^-1_col(T2);  zsum = conj(c) z;  T <- FFT_col(conj(rho) z)  (DF^H)
+  NUM_COL_MODES = 10
 };
 
 // Shared-memory layout of a column pass (byte offsets): exchange, twiddles, then `nside` side arrays of
-// Wc x C complex values (Omega rows of the block's columns: coil map, rho, drho, r).
+// Wc x C complex values (Omega rows of the block's columns: coil map, rho, drho, r; passes that form the coil maps: rho,
+// drho), and for two inputs the block's columns of the second.
 struct ColSmem {
-  size_t xch, tw, side, total;
+  size_t xch, tw, side, t2, total;
   int nside;
 };
+__host__ __device__ constexpr bool col_forms_coils(int mode) { return mode >= COL_COIL_PROD && mode <= COL_COIL_ADJ; }
+
 __host__ __device__ inline ColSmem col_smem(int mode, int N, int C, int sm_lane, int Wc) {
   ColSmem L{};
-  L.nside = (mode == COL_CG_DIR || mode == COL_BCG_DIR) ? 4 : (mode == COL_IFFT_PROD_FFT) ? 3 : (mode == COL_IFFT_ADJ_FFT) ? 2 : 0;
+  L.nside = (mode == COL_CG_DIR || mode == COL_BCG_DIR) ? 4
+            : (mode == COL_IFFT_PROD_FFT) ? 3
+            : (mode == COL_IFFT_ADJ_FFT || mode == COL_COIL_DIR) ? 2
+            : col_forms_coils(mode) ? 1 : 0;
   L.xch = 0;
   L.tw = align16((size_t)C * sm_lane * 8);
   L.side = L.tw + align16((size_t)2 * N * 8);
-  L.total = L.side + (size_t)L.nside * Wc * C * 8;
+  L.t2 = L.side + (size_t)L.nside * Wc * C * 8;
+  L.total = L.t2 + (mode == COL_COIL_DIR || mode == COL_COIL_ADJ ? (size_t)N * C * 8 : 0);
   return L;
 }
 
@@ -1136,11 +1173,24 @@ __device__ __forceinline__ void col_stage_side(const KArgs& A, int bid, unsigned
       stage_bytes(smem_raw + L.tw, A.twA, N * 8);
       stage_bytes(smem_raw + L.tw + N * 8, A.twB, N * 8);
     }
-    if constexpr (MODE == COL_IFFT_PROD_FFT || MODE == COL_IFFT_ADJ_FFT || MODE == COL_CG_DIR || MODE == COL_BCG_DIR) {
+    if constexpr (col_forms_coils(MODE)) {
+      if (j < A.nrows) stage_natural_cols(sd, A.rho, cc0, C, Wc, N, f);
+    } else if constexpr (MODE == COL_IFFT_PROD_FFT || MODE == COL_IFFT_ADJ_FFT || MODE == COL_CG_DIR ||
+                         MODE == COL_BCG_DIR) {
       if (j < A.nrows) {
         stage_compact_cols(sd, A.coil + (size_t)j * Wc * Wc, cc0, C, Wc);
         stage_natural_cols(sd + sstride, A.rho, cc0, C, Wc, N, f);
       }
+    }
+  } else if constexpr (MODE == COL_COIL_DIR || MODE == COL_COIL_ADJ) {
+    if (j < A.nrows) {
+      if constexpr (MODE == COL_COIL_DIR) stage_natural_cols(sd + sstride, A.drho, cc0, C, Wc, N, f);
+      // the columns of the second input, every row
+      float2* t2 = (float2*)(smem_raw + L.t2);
+      const int k = threadIdx.x % (C / 2), cc = cc0 + 2 * k, step = blockDim.x / (C / 2);
+      if (cc < Wc)
+        for (int e = threadIdx.x / (C / 2); e < N; e += step)
+          cp_async16(t2 + (size_t)e * C + 2 * k, A.src2 + ((size_t)j * N + e) * Wc + cc);
     }
   } else if constexpr (MODE == COL_IFFT_PROD_FFT) {
     if (j < A.nrows) stage_natural_cols(sd + 2 * sstride, A.drho, cc0, C, Wc, N, f);
@@ -1316,7 +1366,51 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, int nblk,
       }
       if constexpr (MODE == COL_BCG_DIR) beta = A.sc->beta_p.h;
       const size_t sstride = (size_t)Wc * C;
-      if (idx < N2) {
+      if constexpr (col_forms_coils(MODE)) {
+        float2 c[N1];                       // the coil map on this thread's Omega elements (layout B)
+        if (idx < N2) {
+#pragma unroll
+          for (int m = 0; m < N1; ++m) {
+            const int e1 = idx + N2 * m;
+            c[m] = make_float2(0.f, 0.f);
+            if (active && in_omega(e1, N, f)) {
+              c[m] = cscale(v[m], rs);
+              if (A.coil_out) A.coil_out[cbase + (size_t)to_compact(e1, N, f) * Wc] = c[m];
+            }
+          }
+        }
+        if constexpr (MODE != COL_COIL_PROD) {
+          const float2* t2 = (const float2*)(smem_raw + L.t2) + lane;
+          if (idx < N1) {
+#pragma unroll
+            for (int m = 0; m < N2; ++m) v[m] = active ? t2[(size_t)(idx + N1 * m) * C] : make_float2(0.f, 0.f);
+          }
+          fft_AtoB<N1, N2, +1, true>(v, sm, twA, idx, tc);
+        }
+        if (idx < N2) {
+#pragma unroll
+          for (int m = 0; m < N1; ++m) {
+            const int e1 = idx + N2 * m;
+            float2 out = make_float2(0.f, 0.f);
+            if (active && in_omega(e1, N, f)) {
+              const int cr = to_compact(e1, N, f);
+              const float2 rh = side[(size_t)cr * C + lane];
+              if constexpr (MODE == COL_COIL_PROD) {
+                out = cmul(rh, c[m]);
+              } else {
+                const float2 u = cscale(v[m], rs);
+                if constexpr (MODE == COL_COIL_DIR) {
+                  out = cadd(cmul(side[sstride + (size_t)cr * C + lane], c[m]), cmul(rh, u));
+                } else {
+                  A.zsum[cbase + (size_t)cr * Wc] = cmulc(c[m], u);
+                  out = cmulc(rh, u);
+                }
+              }
+            }
+            v[m] = out;
+          }
+        }
+      } else if (idx < N2) {
 #pragma unroll
         for (int m = 0; m < N1; ++m) {
           const int e1 = idx + N2 * m;
@@ -1660,6 +1754,22 @@ inline RowGrid row_grid(const SizeKernels* k, int nrows, long rho_pixels, int sm
   return g;
 }
 
+// The operators' passes with two inputs or with the coil maps formed on the way (q_op_* in nlinv.cu).
+template <int N1, int N2, int CC = NLV_COL_C> void add_op_cols(SizeKernels& k) {
+  k.col[COL_COIL_PROD] = (const void*)col_pass<N1, N2, COL_COIL_PROD, false, CC>;
+  k.col[COL_COIL_DIR] = (const void*)col_pass<N1, N2, COL_COIL_DIR, false, CC>;
+  k.col[COL_COIL_ADJ] = (const void*)col_pass<N1, N2, COL_COIL_ADJ, false, CC>;
+  k.col_std[COL_COIL_PROD] = (const void*)col_pass<N1, N2, COL_COIL_PROD, true, CC>;
+  k.col_std[COL_COIL_DIR] = (const void*)col_pass<N1, N2, COL_COIL_DIR, true, CC>;
+  k.col_std[COL_COIL_ADJ] = (const void*)col_pass<N1, N2, COL_COIL_ADJ, true, CC>;
+}
+template <int N1, int N2> void add_op_passes(SizeKernels& k) {
+  k.row[ROW_W_W_IFFT] = (const void*)row_pass<N1, N2, ROW_W_W_IFFT>;
+  k.row[ROW_W_P_IFFT] = (const void*)row_pass<N1, N2, ROW_W_P_IFFT>;
+  k.row_std[ROW_W_W_IFFT] = (const void*)row_pass<N1, N2, ROW_W_W_IFFT, true>;
+  k.row_std[ROW_W_P_IFFT] = (const void*)row_pass<N1, N2, ROW_W_P_IFFT, true>;
+  add_op_cols<N1, N2>(k);
+}
 // The CG passes of single frames (q_cg_iter in nlinv.cu) and of batches (q_bcg_iter).
 template <int N1, int N2, int CC = NLV_COL_C> void add_frame_cg_cols(SizeKernels& k) {
   k.col[COL_CG_DIR] = (const void*)col_pass<N1, N2, COL_CG_DIR, false, CC>;
@@ -1693,6 +1803,7 @@ template <int N1, int N2, int CC> SizeKernels make_size_kernels_strip(const Size
   s.col[COL_IFFT_ADJ_FFT] = (const void*)col_pass<N1, N2, COL_IFFT_ADJ_FFT, false, CC>;
   for (int m = 0; m < NUM_COL_MODES; ++m) s.col_std[m] = nullptr;
   add_frame_cg_cols<N1, N2, CC>(s);
+  add_op_cols<N1, N2, CC>(s);
   s.col_std[COL_IFFT_PROD_FFT] = (const void*)col_pass<N1, N2, COL_IFFT_PROD_FFT, true, CC>;
   for (int m = 0; m < NUM_ROW_MODES; ++m) s.row_batch[m] = s.row_std_batch[m] = s.row_tc[m] = s.row_tc_std[m] = nullptr;
   for (int m = 0; m < NUM_COL_MODES; ++m) s.col_batch[m] = s.col_std_batch[m] = s.col_tc[m] = s.col_tc_std[m] = nullptr;
@@ -1725,6 +1836,7 @@ template <int N1, int N2> SizeKernels make_size_kernels_single() {
   s.row_std[ROW_FFT_W_NORMAL] = (const void*)row_pass<N1, N2, ROW_FFT_W_NORMAL, true>;
   s.col_std[COL_IFFT_PROD_FFT] = (const void*)col_pass<N1, N2, COL_IFFT_PROD_FFT, true>;
   add_frame_cg<N1, N2>(s);
+  add_op_passes<N1, N2>(s);
   return s;
 }
 
@@ -1772,6 +1884,7 @@ template <int N1, int N2> SizeKernels make_size_kernels() {
   s.row_std_batch[ROW_FFT_W_NORMAL] = (const void*)row_pass_batch<N1, N2, ROW_FFT_W_NORMAL, true>;
   s.col_std_batch[COL_IFFT_PROD_FFT] = (const void*)col_pass_batch<N1, N2, COL_IFFT_PROD_FFT, true>;
   add_frame_cg<N1, N2>(s);
+  add_op_passes<N1, N2>(s);
   add_batch_cg<N1, N2>(s);
   return s;
 }

@@ -336,7 +336,7 @@ KArgs base_args(const nlinv_ctx* c) {
   return a;
 }
 
-nlv::RowGrid row_geom(const nlinv_ctx* c, bool with_rho) {
+nlv::RowGrid row_geom(const nlinv_ctx* c, bool with_rho, int arrays = 1) {
   if (c->batch_lanes > 0) {           // batch frames: equal block shapes for every frame of a grid side
     nlv::RowGrid g{};
     const int rows = c->J * c->N;
@@ -349,7 +349,7 @@ nlv::RowGrid row_geom(const nlinv_ctx* c, bool with_rho) {
     g.rho_per_cta = with_rho ? (int)((c->plane + groups - 1) / groups) : 0;
     return g;
   }
-  nlv::RowGrid g = nlv::row_grid(c->k, c->J * c->N, with_rho ? c->plane : 0, c->sms, c->row_ctas_per_sm);
+  nlv::RowGrid g = nlv::row_grid(c->k, arrays * c->J * c->N, with_rho ? c->plane : 0, c->sms, c->row_ctas_per_sm);
   // tensor-core passes: whole warps (every lane of a warp takes part in tcgen05.ld), the extra lanes idle
   if (c->tc)
     while ((g.lanes * c->k->tl) % 32 != 0) ++g.lanes;
@@ -422,9 +422,11 @@ struct OwnStream {
 };
 
 cudaError_t row(nlinv_ctx* c, int mode, KArgs a) {
-  const bool rho = mode >= nlv::ROW_FFT_W_ADJ && mode != nlv::ROW_CG_PSF && mode != nlv::ROW_BCG_DIR;
-  const nlv::RowGrid g = row_geom(c, rho);
-  a.nrows = c->J * c->N;
+  const bool both = mode == nlv::ROW_W_W_IFFT || mode == nlv::ROW_W_P_IFFT;
+  const bool rho = mode >= nlv::ROW_FFT_W_ADJ && mode != nlv::ROW_CG_PSF && mode != nlv::ROW_BCG_DIR && !both;
+  const nlv::RowGrid g = row_geom(c, rho, both ? 2 : 1);
+  a.nrows1 = c->J * c->N;
+  a.nrows = (both ? 2 : 1) * a.nrows1;
   a.rows_per_cta = g.rows_per_cta;
   a.rho_per_cta = g.rho_per_cta;
   a.sub = g.sub;
@@ -475,6 +477,68 @@ cudaError_t q_prod(nlinv_ctx* c, const float2* rho) {
   a.coil = c->coil;
   a.dst = c->T;
   return col(c, nlv::COL_PROD_FFT, a);
+}
+
+// The operators' passes that form the coil maps on the way (the FP32 transforms of single frames): W^-1 of the coil
+// planes and the other operator's input go through one row launch, and the column pass transforms both, where coil maps,
+// then the operator, took two launches each and a pass over the maps.  The calls are bound by launches and by each
+// pass's latency (1.5 to 6 us a launch, against 1 to 4 us of arithmetic).  Before and after: normal operator 384^2/10
+// coils 47.4 -> 40.0 us, 512^2/16 113.6 -> 109.8; DF^H 192^2/13 23.4 -> 18.1, DF 26.6 -> 21.5; F 64^2/4 19.3 -> 16.6.
+// The results of the operators are the same bit for bit.  The tensor-core passes have one input, and the batch's item
+// tables one launch per pass for all frames: both keep the separate passes.
+bool fused_ops(const nlinv_ctx* c) { return !c->tc && c->batch_lanes == 0; }
+
+// T <- FFT_col(M rho c_j), c_j = W^-1 chat_j of x (1+J planes); the maps to c->coil if keep.
+cudaError_t q_op_prod(nlinv_ctx* c, const float2* x, bool keep) {
+  KArgs a = base_args(c);
+  a.src = x + c->plane;
+  a.dst = c->T;
+  cudaError_t e = row(c, nlv::ROW_W_IFFT, a);
+  if (e != cudaSuccess) return e;
+  a = base_args(c);
+  a.src = c->T;
+  a.dst = c->T;
+  a.rho = x;
+  a.coil_out = keep ? c->coil : nullptr;
+  return col(c, nlv::COL_COIL_PROD, a);
+}
+
+// T <- FFT_col(M (drho c_j + rho W^-1 dchat_j)), c_j of x, for direction d; the maps to c->coil if keep.
+cudaError_t q_op_dir(nlinv_ctx* c, const float2* x, const float2* d, bool keep) {
+  KArgs a = base_args(c);
+  a.src = x + c->plane;
+  a.src2 = d + c->plane;
+  a.dst = c->T;
+  a.dst2 = c->r0;                 // the data residual's buffer, free outside a Newton step
+  cudaError_t e = row(c, nlv::ROW_W_W_IFFT, a);
+  if (e != cudaSuccess) return e;
+  a = base_args(c);
+  a.src = c->T;
+  a.src2 = c->r0;
+  a.dst = c->T;
+  a.rho = x;
+  a.drho = d;
+  a.coil_out = keep ? c->coil : nullptr;
+  return col(c, nlv::COL_COIL_DIR, a);
+}
+
+// T <- FFT_col(conj(rho) z_j), zsum_j <- conj(c_j) z_j with z_j = M FFT^-1(P r_j), c_j of x.
+cudaError_t q_op_adj(nlinv_ctx* c, const float2* x, const float2* r, const uint8_t* mask) {
+  KArgs a = base_args(c);
+  a.src = x + c->plane;
+  a.src2 = r;
+  a.mask = mask;
+  a.dst = c->T;
+  a.dst2 = c->r0;
+  cudaError_t e = row(c, nlv::ROW_W_P_IFFT, a);
+  if (e != cudaSuccess) return e;
+  a = base_args(c);
+  a.src = c->T;
+  a.src2 = c->r0;
+  a.dst = c->T;
+  a.rho = x;
+  a.zsum = c->zsum;
+  return col(c, nlv::COL_COIL_ADJ, a);
 }
 
 // T <- FFT_col(M (drho c_j + rho W^-1 dchat_j)) for direction d and linearisation point x
@@ -753,9 +817,9 @@ cudaError_t q_bcg_add(nlinv_ctx* c) {
 
 // Coil maps of c->x and the Newton residual r0 = y - F x with |r0| into resid[slot].
 cudaError_t q_residual(nlinv_ctx* c, int slot) {
-  cudaError_t e = q_coils(c, c->x);
+  cudaError_t e = fused_ops(c) ? q_op_prod(c, c->x, true) : q_coils(c, c->x);
+  if (e == cudaSuccess && !fused_ops(c)) e = q_prod(c, c->x);
   if (e != cudaSuccess) return e;
-  if ((e = q_prod(c, c->x)) != cudaSuccess) return e;
   KArgs a = base_args(c);
   a.src = c->T;
   a.dst = c->r0;
@@ -781,8 +845,8 @@ cudaError_t q_axpby(nlinv_ctx* c, float2* out, float a, const float2* X, float b
 
 // out = DF_z d (J data planes) at the linearisation point z.
 cudaError_t q_derivative_to(nlinv_ctx* c, const float2* z, const float2* d, const uint8_t* mask, float2* out) {
-  cudaError_t e = q_coils(c, z);
-  if (e == cudaSuccess) e = q_dir(c, z, d);
+  cudaError_t e = fused_ops(c) ? q_op_dir(c, z, d, false) : q_coils(c, z);
+  if (e == cudaSuccess && !fused_ops(c)) e = q_dir(c, z, d);
   if (e != cudaSuccess) return e;
   KArgs a = base_args(c);
   a.src = c->T;
@@ -793,14 +857,18 @@ cudaError_t q_derivative_to(nlinv_ctx* c, const float2* z, const float2* d, cons
 
 // out = DF_z^H r (one unknown-space vector) at the linearisation point z.
 cudaError_t q_adjoint_to(nlinv_ctx* c, const float2* z, const float2* r, const uint8_t* mask, float2* out) {
-  cudaError_t e = q_coils(c, z);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   KArgs a = base_args(c);
-  a.src = r;
-  a.dst = c->T;
-  a.mask = mask;
-  if ((e = row(c, nlv::ROW_P_IFFT, a)) != cudaSuccess) return e;
-  if ((e = q_adj_col(c, z)) != cudaSuccess) return e;
+  if (fused_ops(c)) {
+    if ((e = q_op_adj(c, z, r, mask)) != cudaSuccess) return e;
+  } else {
+    if ((e = q_coils(c, z)) != cudaSuccess) return e;
+    a.src = r;
+    a.dst = c->T;
+    a.mask = mask;
+    if ((e = row(c, nlv::ROW_P_IFFT, a)) != cudaSuccess) return e;
+    if ((e = q_adj_col(c, z)) != cudaSuccess) return e;
+  }
   a = base_args(c);
   a.src = c->T;
   a.dst = out;
@@ -988,7 +1056,7 @@ bool allow_passes(nlinv_ctx* c, const SizeKernels* k) {
   cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
   const SizeKernels* saved = c->k;
   c->k = k;
-  const int lanes = std::max(row_geom(c, false).lanes, row_geom(c, true).lanes);
+  const int lanes = std::max({row_geom(c, false).lanes, row_geom(c, true).lanes, row_geom(c, false, 2).lanes});
   c->k = saved;
   auto allow = [&](const void* fn, size_t need) {
     if (!fn) return true;
@@ -1083,7 +1151,7 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
     if (frame)
       cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   };
-  const int lanes_max = std::max(row_geom(c, false).lanes, row_geom(c, true).lanes);
+  const int lanes_max = std::max({row_geom(c, false).lanes, row_geom(c, true).lanes, row_geom(c, false, 2).lanes});
   for (int m = 0; m < nlv::NUM_ROW_MODES && smem_err.empty(); ++m) {
     if (c->k->row[m]) allow(c->k->row[m], c->k->row_smem(m, lanes_max));
     if (smem_err.empty() && c->k->row_batch[m]) allow(c->k->row_batch[m], c->k->row_smem(m, lanes_max), false);
@@ -1260,8 +1328,8 @@ nlinv_status nlinv_forward(nlinv_ctx* c, const nlinv_c32* x, const uint8_t* mask
   if ((s = check_dev(c, x, "x")) || (s = check_dev(c, mask, "mask")) || (s = check_dev(c, y_out, "y_out"))) return s;
   const float2* xv = (const float2*)x;
   cudaError_t e = op_begin(c, on);
-  if (e == cudaSuccess) e = q_coils(c, xv);
-  if (e == cudaSuccess) e = q_prod(c, xv);
+  if (e == cudaSuccess) e = fused_ops(c) ? q_op_prod(c, xv, false) : q_coils(c, xv);
+  if (e == cudaSuccess && !fused_ops(c)) e = q_prod(c, xv);
   if (e == cudaSuccess) {
     KArgs a = base_args(c);
     a.src = c->T;
@@ -1309,8 +1377,8 @@ nlinv_status nlinv_normal(nlinv_ctx* c, const nlinv_c32* x, const uint8_t* mask,
   if (!std::isfinite(alpha)) return fail(c, NLINV_EINVAL, "alpha must be finite");
   const float2* xv = (const float2*)x;
   cudaError_t e = op_begin(c, on);
-  if (e == cudaSuccess) e = q_coils(c, xv);
-  if (e == cudaSuccess) e = q_dir(c, xv, (const float2*)d);
+  if (e == cudaSuccess) e = fused_ops(c) ? q_op_dir(c, xv, (const float2*)d, true) : q_coils(c, xv);
+  if (e == cudaSuccess && !fused_ops(c)) e = q_dir(c, xv, (const float2*)d);
   if (e == cudaSuccess) {
     KArgs a = base_args(c);
     a.src = c->T;
