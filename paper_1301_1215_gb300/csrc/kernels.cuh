@@ -1609,8 +1609,12 @@ __global__ void __launch_bounds__(kRowBatchThreads, kRowBatchCtasPerSM) row_pass
   }, [&](const KArgs& A, int bid) { row_prefetch<N1, N2, MODE, STDF>(A, bid); });
 }
 
+// Column passes of batches are bound by the loads in flight: blocks per SM are asked for by the block's threads (left to
+// the compiler, sides 320 and 384 took registers for 3 and 2).  64 frames (5 Newton steps of 12 iterations) 100.0 -> 98.7
+// ms, three 384^2 frames 11.9 -> 11.7.
+constexpr int col_batch_ctas(int threads) { return threads <= 128 ? 5 : threads <= 160 ? 4 : threads <= 192 ? 3 : 1; }
 template <int N1, int N2, int MODE, bool STDF = false>
-__global__ void __launch_bounds__(ColCfg<N1, N2>::THREADS) col_pass_batch(const BatchArgs B) {
+__global__ void __launch_bounds__(ColCfg<N1, N2>::THREADS, col_batch_ctas(ColCfg<N1, N2>::THREADS)) col_pass_batch(const BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ BatchQueue q;
   using S = Split<N1, N2>;

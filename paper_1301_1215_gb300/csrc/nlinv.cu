@@ -227,6 +227,12 @@ constexpr double kTuneMargin = 0.03; // a candidate replaces the compiled defaul
 #ifndef NLV_VEC_BLOCKS_PER_SM
 #define NLV_VEC_BLOCKS_PER_SM 4   // blocks per SM of the vector passes
 #endif
+// One shared-memory carve-out for every pass of a batch (percent of an SM's; 72 to 84 select the same one): a launch that
+// asks for another split of the L1 than its predecessor's waits until the SM is empty, and streams of different sides then
+// hold each other up.  Left to the driver, per pass, or at the maximum, whose 28 KB of L1 limit the loads in flight, 64
+// frames (5 Newton steps of 12 iterations) take 107.3 ms, at 50 percent 107.8, at 60 102.8, here 100.0; three 384^2
+// frames 12.7, 13.3, 12.5 and 11.9.
+constexpr int kBatchCarveout = 76;
 constexpr int kProfileSteps = 6;   // steps of one CG iteration, in the order nlinv_profile_cg reports them
 
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -1146,8 +1152,7 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
       smem_err = "cudaFuncSetAttribute failed";
     // one carve-out for all single-frame passes: with the driver's own choice consecutive passes differ, and an SM changes
     // its carve-out only when it is empty (256^2 with 8 coils: 4.41 -> 4.07 ms a frame; other sides within 2 %).  The
-    // batched passes run long enough to keep the driver's choice, which leaves more L1 for loads in flight (64 uneven
-    // frames, column DF^H pass: 203 us an iteration, 241 with the largest carve-out)
+    // batched passes have their own (kBatchCarveout)
     if (frame)
       cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   };
@@ -2134,6 +2139,7 @@ nlinv_status nlinv_batch_create(const nlinv_params* params, int nframes, const n
       cudaFuncAttributes fa{};
       if (cudaFuncGetAttributes(&fa, bl.fn) == cudaSuccess && bl.smem > 0)
         cudaFuncSetAttribute(bl.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - (int)fa.sharedSizeBytes);
+      cudaFuncSetAttribute(bl.fn, cudaFuncAttributePreferredSharedMemoryCarveout, kBatchCarveout);
       int occ = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, bl.fn, bl.block, bl.smem) != cudaSuccess || occ < 1) {
         cudaGetLastError();
