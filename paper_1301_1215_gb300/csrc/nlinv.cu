@@ -260,6 +260,7 @@ struct nlinv_ctx {
   int vec_blocks = 0;         // grid of the vector kernels
   int sms = 0;                // streaming multiprocessors of the device
   int row_ctas_per_sm = nlv::kRowCtasPerSM;   // blocks per SM of the row passes
+  int carveout = 100;         // shared-memory carve-out of the launches, percent (choose_carveout)
   // workspace (one allocation)
   void* base = nullptr;
   float2 *x = nullptr, *xref = nullptr, *y = nullptr, *r0 = nullptr;
@@ -382,14 +383,16 @@ cudaError_t launch(nlinv_ctx* c, const void* fn, int grid, int block, size_t sme
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = c->run;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[3];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = c->pdl ? 1 : 0;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = cluster;
-  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  attr[1].val.sharedMemCarveout = c->carveout;
+  attr[2].id = cudaLaunchAttributeClusterDimension;
+  attr[2].val.clusterDim.x = cluster;
+  attr[2].val.clusterDim.y = attr[2].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cfg.numAttrs = cluster > 1 ? 3 : 2;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
@@ -427,9 +430,41 @@ struct OwnStream {
   ~OwnStream() { leave_stream(c); }
 };
 
+bool row_two_arrays(int mode) { return mode == nlv::ROW_W_W_IFFT || mode == nlv::ROW_W_P_IFFT; }
+bool row_has_rho(int mode) {
+  return mode >= nlv::ROW_FFT_W_ADJ && mode != nlv::ROW_CG_PSF && mode != nlv::ROW_BCG_DIR && !row_two_arrays(mode);
+}
+
+// One shared-memory carve-out for all launches of a single frame (with the driver's own choice consecutive passes differ,
+// and an SM changes its carve-out only when it is empty): the smallest of 164, 196 and 228 KB per SM that holds the row
+// passes' resident blocks, and the column passes' where 228 KB holds them all at once.  What is left is L1, which holds the
+// loads in flight.  Four Newton steps of 20 iterations with 164 / 196 / 228 KB: 192^2/13 coils 1450 / 1516 / 1625 us,
+// 320^2/7 2007 / 2016 / 2119, 384^2/22 6227 / 5334 / 5629, 512^2/3 2442 / 2432 / 2673, 320^2/22 4201 / 3718 / 3611; 7 x 30
+// iterations, 384^2/10 7240 / 7302 / 6526, 512^2/16 22.2 / 22.7 / 18.6 ms.  Side 256 does not go below 196: reconstruction
+// and gradient, 9 coils, 3242 / 3172 / 3158, frame with 9 coils and a wide field of view 2604 / 2563 / 2636.  Sides up to
+// 128 gain nothing (128^2/3 1027 / 1011 / 1019, /22 1230 / 1281 / 1240) and keep the largest, as do the tensor-core passes.
+void choose_carveout(nlinv_ctx* c) {
+  c->carveout = 100;
+  if (c->tc || c->N <= 128) return;
+  size_t need = 0;
+  for (int m = 0; m < nlv::NUM_ROW_MODES; ++m) {
+    if (!c->k->row[m]) continue;
+    const nlv::RowGrid g = row_geom(c, row_has_rho(m), row_two_arrays(m) ? 2 : 1);
+    const size_t resident = (size_t)std::min(c->row_ctas_per_sm, (g.blocks + c->sms - 1) / c->sms);
+    need = std::max(need, resident * (c->k->row_smem(m, g.lanes) + 2048));     // static and system use: under 2 KB a block
+  }
+  // column blocks that the full 228 KB would hold all at once stay resident together (320^2/22: 440 blocks, three per SM)
+  const size_t blocks = col_blocks(c) + 1;
+  for (int m = 0; m < nlv::NUM_COL_MODES; ++m) {
+    if (!c->k->col[m]) continue;
+    const size_t per = c->k->col_smem(m, c->Wc) + 2048, resident = (blocks + c->sms - 1) / c->sms;
+    if (resident * per <= (size_t)228 << 10) need = std::max(need, resident * per);
+  }
+  c->carveout = need <= (size_t)164 << 10 && c->N != 256 ? 66 : need <= (size_t)196 << 10 ? 84 : 100;
+}
+
 cudaError_t row(nlinv_ctx* c, int mode, KArgs a) {
-  const bool both = mode == nlv::ROW_W_W_IFFT || mode == nlv::ROW_W_P_IFFT;
-  const bool rho = mode >= nlv::ROW_FFT_W_ADJ && mode != nlv::ROW_CG_PSF && mode != nlv::ROW_BCG_DIR && !both;
+  const bool both = row_two_arrays(mode), rho = row_has_rho(mode);
   const nlv::RowGrid g = row_geom(c, rho, both ? 2 : 1);
   a.nrows1 = c->J * c->N;
   a.nrows = (both ? 2 : 1) * a.nrows1;
@@ -1091,6 +1126,7 @@ bool use_variant(nlinv_ctx* c, const SizeKernels* k) {
   if (!allow_passes(c, k)) return false;
   const bool resplit = k->N1 != c->k->N1;
   c->k = k;
+  choose_carveout(c);
   if (resplit && upload_twiddles(c) != cudaSuccess) return false;
   if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
   return true;
@@ -1139,7 +1175,7 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
   cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
   // (the limit is raised to the device maximum so that contexts with different fov can share the kernels)
   std::string smem_err;
-  auto allow = [&](const void* fn, size_t need, bool frame = true) {
+  auto allow = [&](const void* fn, size_t need) {
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) { smem_err = "cudaFuncGetAttributes failed"; return; }
     const int dyn_max = smem_optin - (int)fa.sharedSizeBytes;
@@ -1150,24 +1186,19 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
     }
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_max) != cudaSuccess)
       smem_err = "cudaFuncSetAttribute failed";
-    // one carve-out for all single-frame passes: with the driver's own choice consecutive passes differ, and an SM changes
-    // its carve-out only when it is empty (256^2 with 8 coils: 4.41 -> 4.07 ms a frame; other sides within 2 %).  The
-    // batched passes have their own (kBatchCarveout)
-    if (frame)
-      cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   };
   const int lanes_max = std::max({row_geom(c, false).lanes, row_geom(c, true).lanes, row_geom(c, false, 2).lanes});
   for (int m = 0; m < nlv::NUM_ROW_MODES && smem_err.empty(); ++m) {
     if (c->k->row[m]) allow(c->k->row[m], c->k->row_smem(m, lanes_max));
-    if (smem_err.empty() && c->k->row_batch[m]) allow(c->k->row_batch[m], c->k->row_smem(m, lanes_max), false);
+    if (smem_err.empty() && c->k->row_batch[m]) allow(c->k->row_batch[m], c->k->row_smem(m, lanes_max));
     if (smem_err.empty() && c->k->row_std[m]) allow(c->k->row_std[m], c->k->row_smem(m, lanes_max));
-    if (smem_err.empty() && c->k->row_std_batch[m]) allow(c->k->row_std_batch[m], c->k->row_smem(m, lanes_max), false);
+    if (smem_err.empty() && c->k->row_std_batch[m]) allow(c->k->row_std_batch[m], c->k->row_smem(m, lanes_max));
   }
   for (int m = 0; m < nlv::NUM_COL_MODES && smem_err.empty(); ++m) {
     if (c->k->col[m]) allow(c->k->col[m], c->k->col_smem(m, c->Wc));
-    if (smem_err.empty() && c->k->col_batch[m]) allow(c->k->col_batch[m], c->k->col_smem(m, c->Wc), false);
+    if (smem_err.empty() && c->k->col_batch[m]) allow(c->k->col_batch[m], c->k->col_smem(m, c->Wc));
     if (smem_err.empty() && c->k->col_std[m]) allow(c->k->col_std[m], c->k->col_smem(m, c->Wc));
-    if (smem_err.empty() && c->k->col_std_batch[m]) allow(c->k->col_std_batch[m], c->k->col_smem(m, c->Wc), false);
+    if (smem_err.empty() && c->k->col_std_batch[m]) allow(c->k->col_std_batch[m], c->k->col_smem(m, c->Wc));
   }
   if (c->tc) {
     for (int m = 0; m < nlv::NUM_ROW_MODES && smem_err.empty(); ++m) {
@@ -1188,6 +1219,7 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
   }
 
   c->cluster = cluster_fits(c);
+  choose_carveout(c);
 
   // workspace layout
   const size_t cplx = sizeof(float2);
@@ -1745,10 +1777,12 @@ nlinv_status nlinv_set_shapes(nlinv_ctx* c, const nlinv_tuning* t) {
   c->row_ctas_per_sm = t->row_blocks_per_sm;
   if (!use_variant(c, pick) || !allow_passes(c, c->k)) {
     c->row_ctas_per_sm = saved_rc;
+    choose_carveout(c);
     return fail(c, NLINV_EINVAL, "the passes of these shapes do not fit in shared memory");
   }
   c->vec_blocks = c->sms * t->vec_blocks_per_sm;
   c->pdl = t->pdl != 0;
+  choose_carveout(c);
   if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
   return NLINV_OK;
 }
@@ -1785,6 +1819,7 @@ nlinv_status nlinv_autotune(nlinv_ctx* c, const nlinv_c32* y, const uint8_t* mas
     c->vec_blocks = c->sms * vbk;
     c->pdl = pdl;
     c->row_ctas_per_sm = row_ctas;
+    choose_carveout(c);
     if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
   };
   {
