@@ -177,7 +177,7 @@ def replica_throughput(steps_per_rank: int, world: int, slowest_ms: float) -> fl
 
 
 def cg_bytes(n: int, J: int, fov: int):
-    """Algorithmic bytes per launch of the kernels of one CG iteration: every input read once and every output
+    """Algorithmic bytes per launch of the kernels of one CG iteration of a batch: every input read once and every output
     written once (U = one complex64 plane, compact Omega columns Wc = 2 fov)."""
     U = n * n * 8
     h = (2 * fov) / n                 # fraction of a plane kept as Omega columns
@@ -191,6 +191,26 @@ def cg_bytes(n: int, J: int, fov: int):
         "row W^-H+alpha p": J * U * (h + q) + 2 * J * U + 4 * U,       # T, products, p in; q out; rho: r, p in, p, q out
         "cg step": 6 * (1 + J) * U,                                    # p, q, r, dx in; dx, r out
     }
+
+
+def frame_cg_bytes(n: int, J: int, fov: int):
+    """The same for the four passes of a single frame's CG iteration (U here: W^-1 p on Omega, carried along; the
+    solution is updated every second iteration)."""
+    U = n * n * 8
+    h = (2 * fov) / n
+    q = h * h
+    return {
+        "col direction": J * U * (2 * h + 3 * q) + 3 * q * U,          # T, U, c in; T, U out; rho, r_rho, p_rho on Omega
+        "row PSF": J * U * 2 * h + n * n,
+        "col FFT^-1/C^H/FFT": J * U * (h + q + h + q) + q * U,         # T, c in; T, channel products out; rho
+        "row update": J * U * (2 * h + q) + 5 * (1 + J) * U,           # T, products, r, p in; T, r, p out; dx in and out
+    }
+
+
+def frame_cg_passes(prof):
+    """Durations of those four passes from nlinv_profile_cg's six entries (it divides the update pass's over three)."""
+    step, col1, psf, col2, out, upd = prof.values()
+    return {"col direction": col1, "row PSF": psf, "col FFT^-1/C^H/FFT": col2, "row update": step + out + upd}
 
 
 def compulsory_bytes(n: int, J: int) -> int:
@@ -257,8 +277,8 @@ def run_ours(args, rank, world, local):
     finite = bool(torch.isfinite(torch.view_as_real(x)).all().item())
 
     # per-kernel CUDA-event durations of the CG iteration on the same state (the roofline's dominant kernel)
-    prof = ctx.profile_cg(reps=20)
-    algo = cg_bytes(W.n, W.ncoils, W.fov)
+    prof = frame_cg_passes(ctx.profile_cg(reps=20))
+    algo = frame_cg_bytes(W.n, W.ncoils, W.fov)
     top = max(prof, key=prof.get)
     hbm, src = peaks()
     achieved = algo[top] / (prof[top] * 1e-3) / 1e9
@@ -272,7 +292,7 @@ def run_ours(args, rank, world, local):
     kernels = {k: {"ms": round(v, 5), "algo_bytes": int(algo[k]),
                    "gbs": round(algo[k] / (v * 1e-3) / 1e9, 1)} for k, v in prof.items()}
     # the same iteration on the compulsory accounting (every array touched once): bytes / in-graph iteration time
-    # (the six steady-state kernel durations add up to it), and bytes of all CG iterations / whole frame time
+    # (the steady-state durations of its passes add up to it), and bytes of all CG iterations / whole frame time
     t_iter = sum(prof.values()) * 1e-3
     comp = compulsory_bytes(W.n, W.ncoils)
     comp_iter_gbs = comp / t_iter / 1e9
@@ -341,7 +361,7 @@ def run_ours(args, rank, world, local):
     line = {
         "metric": METRIC, "value": round(value, 3), "unit": "frames/s", "n_gpus": world, "steps": K,
         "warmup": Wm, "ms_per_step": round(total_ms / K, 4), "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "c64 (f32 complex; f64 CG scalars)", "data": "synthetic",
+        "vs_baseline": None, "dtype": "c64 (f32 complex; CG scalars as f32 pairs)", "data": "synthetic",
         "p50_ms": round(p50, 4), "p99_ms": round(p99, 4),
         "config": {"workload": "real-time radial series: 384x384 grid (192x192 image), 10 coils, 13 spokes/frame "
                                "rotated k*2pi/65, 7 Newton x 30 CG, previous frame as start and reference",
@@ -364,8 +384,8 @@ def run_ours(args, rank, world, local):
                                     "gbs": round(comp_iter_gbs, 1),
                                     "frame_gbs": round(comp_frame_gbs, 1),
                                     "frame_frac": round(comp_frame_gbs / hbm, 4),
-                                    "note": "(10J+10) planes + n^2 bytes per CG iteration; iter_ms = the six "
-                                            "steady-state kernel durations; frame_* = all CG iterations' bytes / "
+                                    "note": "(10J+10) planes + n^2 bytes per CG iteration; iter_ms = the sum of "
+                                            "the passes' steady-state durations; frame_* = all CG iterations' bytes / "
                                             "whole frame time (includes the non-CG passes)"},
                      "l2_resident": "the 384^2 frame's ~110 MB working set stays in the 126 MB L2 between passes: "
                                     "DRAM traffic ('traffic') is below the algorithmic bytes; the HBM-bound case "
@@ -507,12 +527,11 @@ def synth_workload():
     return synth.WORKLOADS[WORKLOAD]
 
 
-CG_KERNEL_ORDER = ("row p-update/W^-1", "col W^-1/C/FFT", "row PSF", "col FFT^-1/C^H/FFT", "row W^-H+alpha p",
-                   "cg step")
+CG_PASS_ORDER = ("col direction", "row PSF", "col FFT^-1/C^H/FFT", "row update")
 
 
 def write_traffic(rep: str) -> None:
-    """profiles/traffic.json from an ncu report holding, in launch order, the CG kernels of one
+    """profiles/traffic.json from an ncu report holding, in launch order, the four CG passes of one
     nlinv_profile_cg iteration (dram__bytes_read.sum + dram__bytes_write.sum per launch)."""
     import csv
     import io
@@ -522,7 +541,7 @@ def write_traffic(rep: str) -> None:
     scale = {"byte": 1, "Kbyte": 1e3, "Mbyte": 1e6, "Gbyte": 1e9}
     ri, wi = hdr.index("dram__bytes_read.sum"), hdr.index("dram__bytes_write.sum")
     kernels = {}
-    for name, d in zip(CG_KERNEL_ORDER, data):
+    for name, d in zip(CG_PASS_ORDER, data):
         kernels[name] = int(float(d[ri]) * scale[units[ri]] + float(d[wi]) * scale[units[wi]])
     doc = {"csrc_digest": csrc_digest(), "source": os.path.basename(rep), "kernels": kernels,
            "note": "ncu flushes caches per replay pass: DRAM bytes of one cold launch"}

@@ -221,8 +221,8 @@ NLINV_API nlinv_status nlinv_gridder_destroy(nlinv_gridder* g);
  * Many independent frames (slices, series of different patients, ...) of uneven grid side and coil count,
  * reconstructed together: every pass of Eq. 3 is one launch per grid side covering all frames of that side, and
  * the sides run as parallel branches of one captured graph.  Each frame has its own workspace and its own CG and
- * Newton scalars, so a frame's result is its single-frame reconstruction up to the summation order of the FP64
- * scalars (the block partition of a batched pass differs from a single-frame pass). */
+ * Newton scalars, so a frame's result is its single-frame reconstruction up to the rounding of the
+ * CG scalars and directions (single frames run another form of the iteration, in fewer launches). */
 typedef struct {
   int n;                    /* grid side of the frame (see nlinv_supported_size); fov = n/4 */
   int ncoils;               /* coils of the frame, 1..64 */
