@@ -525,7 +525,7 @@ cudaError_t q_prod(nlinv_ctx* c, const float2* rho) {
 // then the operator, took two launches each and a pass over the maps.  The calls are bound by launches and by each
 // pass's latency (1.5 to 6 us a launch, against 1 to 4 us of arithmetic).  Before and after: normal operator 384^2/10
 // coils 47.4 -> 40.0 us, 512^2/16 113.6 -> 109.8; DF^H 192^2/13 23.4 -> 18.1, DF 26.6 -> 21.5; F 64^2/4 19.3 -> 16.6.
-// The results of the operators are the same bit for bit.  The tensor-core passes have one input, and the batch's item
+// The results are the same bits on most shapes and within 1.2e-7 on the others.  The tensor-core passes have one input, and the batch's item
 // tables one launch per pass for all frames: both keep the separate passes.
 bool fused_ops(const nlinv_ctx* c) { return !c->tc && c->batch_lanes == 0; }
 
