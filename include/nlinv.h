@@ -24,7 +24,8 @@
  *   - M_Omega keeps the centred square -fov <= g < fov of the image (fov = n/4: the un-oversampled image of a 2x
  *     grid, Sec. 3.2).  FFT is the unitary 2D DFT (FFT^-1 = FFT^H).
  *   - Work is queued on the context's CUDA stream and returns before it finishes unless stated otherwise.
- *   - Unless stated otherwise, pointers are DEVICE pointers owned by the caller, valid until the work is done.
+ *   - Unless stated otherwise, pointers are DEVICE pointers owned by the caller, valid until the work is done.  Complex
+ *     arrays lie on an 8-byte boundary, sampling patterns anywhere (off a 16-byte boundary, some calls copy a plane first).
  *   - No entry point throws; every one returns an nlinv_status.  Arguments are checked on the host before any
  *     work is queued; on error nothing is queued and nlinv_last_error() describes the problem.
  *
@@ -345,7 +346,7 @@ NLINV_API nlinv_status nlinv_cg_stops(nlinv_ctx* ctx, int* out, int len);
  * The scratch (the twiddle and Sobolev tables at fixed offsets, then the Omega-column transform buffer and the
  * coil maps) lives in one file-scope device array of 16 MiB that every GPU loading this library holds until the
  * process exits; a call whose n, ncoils and fov need more than that is rejected with EINVAL (384 x 384 with 10
- * coils and fov = n/4 fits; 512 x 512 with 16 coils does not).  The caller passes x (1+J planes), mask and y_out
+ * coils and fov = n/4 fits; 512 x 512 with 16 coils does not; a mask off the 16-byte boundary takes n^2 bytes of it).  The caller passes x (1+J planes), mask and y_out
  * (J planes), device (or managed) memory of the current device, and a cudaStream_t (NULL = legacy default stream);
  * params supplies n, ncoils, fov, sobolev_a and sobolev_l (the other fields are ignored).
  * Set-up: the first call on a device (with that device current) finds the array's device address, and the first

@@ -179,17 +179,21 @@ __global__ void image_kernel(const KArgs A) {
   }
 }
 
-// out = alpha X + coef Y (X = A.src, Y = A.q, out = A.dst) over A.n2 float4
-__global__ void axpby_kernel(const KArgs A) {
+// out = alpha X + coef Y (X = A.src, Y = A.q, out = A.dst, which may be X or Y) over A.n2 float4, or, for a caller's array
+// off the 16-byte boundary, 2 A.n2 float2
+__device__ __forceinline__ float4 axpby(float a, float4 x, float b, float4 y) {
+  return make_float4(fmaf(a, x.x, b * y.x), fmaf(a, x.y, b * y.y), fmaf(a, x.z, b * y.z), fmaf(a, x.w, b * y.w));
+}
+__device__ __forceinline__ float2 axpby(float a, float2 x, float b, float2 y) {
+  return make_float2(fmaf(a, x.x, b * y.x), fmaf(a, x.y, b * y.y));
+}
+template <class V> __global__ void axpby_kernel(const KArgs A) {
   nlv::pdl_enter();
-  const float4* __restrict__ x4 = (const float4*)A.src;
-  const float4* __restrict__ y4 = (const float4*)A.q;
-  float4* __restrict__ o4 = (float4*)A.dst;
-  const float a = A.alpha, b = A.coef;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < A.n2; i += (long)gridDim.x * blockDim.x) {
-    const float4 x = x4[i], y = y4[i];
-    o4[i] = make_float4(fmaf(a, x.x, b * y.x), fmaf(a, x.y, b * y.y), fmaf(a, x.z, b * y.z), fmaf(a, x.w, b * y.w));
-  }
+  const V *x = (const V*)A.src, *y = (const V*)A.q;
+  V* o = (V*)A.dst;
+  const long n = A.n2 * (long)(sizeof(float4) / sizeof(V));
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
+    o[i] = axpby(A.alpha, x[i], A.coef, y[i]);
 }
 
 // CG from dx = 0 for the right-hand side b = A.src: r = b, |b|^2 -> RED_RR_INIT
@@ -430,6 +434,24 @@ struct OwnStream {
   ~OwnStream() { leave_stream(c); }
 };
 
+// Passes copy the planes of rho, drho and the sampling pattern into shared memory in 16-byte pieces.  A caller's array may
+// lie off that boundary (a slice of a larger one): its plane then goes to `room` first, part of a vector that holds
+// nothing outside a CG solve, whose own arrays all lie on it.
+bool on_boundary(const void* p) { return (uintptr_t)p % 16 == 0; }
+template <class T> cudaError_t stageable(const nlinv_ctx* c, const T*& p, void* room) {
+  if (on_boundary(p)) return cudaSuccess;
+  const T* from = p;
+  p = (const T*)room;
+  return cudaMemcpyAsync(room, from, (size_t)c->plane * sizeof(T), cudaMemcpyDeviceToDevice, c->run);
+}
+bool row_stages_mask(int mode) {
+  return mode == nlv::ROW_PSF || mode == nlv::ROW_CG_PSF || mode == nlv::ROW_FFT_P_OUT || mode == nlv::ROW_FFT_RESID;
+}
+bool col_stages_rho(int mode) {
+  return mode != nlv::COL_IFFT_C && mode != nlv::COL_PROD_FFT && mode != nlv::COL_SIM_FFT;
+}
+bool col_stages_drho(int mode) { return mode == nlv::COL_IFFT_PROD_FFT || mode == nlv::COL_COIL_DIR; }
+
 bool row_two_arrays(int mode) { return mode == nlv::ROW_W_W_IFFT || mode == nlv::ROW_W_P_IFFT; }
 bool row_has_rho(int mode) {
   return mode >= nlv::ROW_FFT_W_ADJ && mode != nlv::ROW_CG_PSF && mode != nlv::ROW_BCG_DIR && !row_two_arrays(mode);
@@ -464,6 +486,10 @@ void choose_carveout(nlinv_ctx* c) {
 }
 
 cudaError_t row(nlinv_ctx* c, int mode, KArgs a) {
+  if (row_stages_mask(mode)) {
+    const cudaError_t e = stageable(c, a.mask, c->dx);
+    if (e != cudaSuccess) return e;
+  }
   const bool both = row_two_arrays(mode), rho = row_has_rho(mode);
   const nlv::RowGrid g = row_geom(c, rho, both ? 2 : 1);
   a.nrows1 = c->J * c->N;
@@ -485,6 +511,10 @@ cudaError_t row(nlinv_ctx* c, int mode, KArgs a) {
 }
 
 cudaError_t col(nlinv_ctx* c, int mode, KArgs a) {
+  cudaError_t e = cudaSuccess;
+  if (col_stages_rho(mode)) e = stageable(c, a.rho, c->p);
+  if (e == cudaSuccess && col_stages_drho(mode)) e = stageable(c, a.drho, c->r);
+  if (e != cudaSuccess) return e;
   a.nrows = c->J;
   const int blocks = col_blocks(c) + (a.scalars ? 1 : 0);
   void* args[] = {&a};
@@ -881,7 +911,9 @@ cudaError_t q_axpby(nlinv_ctx* c, float2* out, float a, const float2* X, float b
   k.coef = b;
   k.n2 = planes * c->plane / 2;
   void* args[] = {&k};
-  return launch(c, (const void*)axpby_kernel, c->vec_blocks, kVecThreads, 0, args);
+  const bool wide = on_boundary(out) && on_boundary(X) && on_boundary(Y);
+  return launch(c, wide ? (const void*)axpby_kernel<float4> : (const void*)axpby_kernel<float2>, c->vec_blocks,
+                kVecThreads, 0, args);
 }
 
 // out = DF_z d (J data planes) at the linearisation point z.

@@ -87,7 +87,9 @@ extern "C" NLINV_API nlinv_status nlinv_forward_noalloc(const nlinv_params* p, v
   const size_t plane = (size_t)N * N;
   const size_t bT = round256((size_t)J * N * Wc * sizeof(float2));
   const size_t bC = round256((size_t)J * Wc * Wc * sizeof(float2));
-  const size_t need = kDataOff + bT + bC;
+  // the last pass copies the sampling pattern in 16-byte pieces: one off that boundary goes through the scratch array
+  const size_t bM = (uintptr_t)mask % 16 ? round256(plane) : 0;
+  const size_t need = kDataOff + bT + bC + bM;
   if (need > kScratchBytes)
     return fail(NLINV_EINVAL, "nlinv_forward_noalloc needs " + std::to_string(need) +
                                   " bytes of scratch for this n, ncoils and fov; its static maximum is " +
@@ -181,6 +183,11 @@ extern "C" NLINV_API nlinv_status nlinv_forward_noalloc(const nlinv_params* p, v
   nlv::KArgs a3 = a;                        // T = FFT_col(M rho c_j)
   a3.rho = xv; a3.coil = coil; a3.dst = T; a3.nrows = J;
   if (e == cudaSuccess) e = launch(k->col[nlv::COL_PROD_FFT], cols, k->col_threads, k->col_smem(nlv::COL_PROD_FFT, Wc), st, a3);
+  if (bM > 0) {
+    uint8_t* room = b + kDataOff + bT + bC;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(room, mask, plane, cudaMemcpyDeviceToDevice, st);
+    mask = room;
+  }
   nlv::KArgs a4 = a;                        // y = P FFT_row(T)
   a4.src = T; a4.dst = (float2*)y_out; a4.mask = mask; a4.nrows = J * N; a4.rows_per_cta = rg.rows_per_cta;
   if (e == cudaSuccess)
