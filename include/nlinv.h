@@ -111,7 +111,8 @@ NLINV_API nlinv_status nlinv_destroy(nlinv_ctx* ctx);
  * caller the two events that order another stream's work around the context's.  Calls that are not operator calls
  * always use the context's own stream, after the context's last call.  Returns 1 when the choice is taken, 0 when the
  * next call will use the context's own stream: `stream` is that stream, or is being captured into a graph (a captured
- * call is ordered by the capture's own events), or ctx is NULL. */
+ * call is ordered by the capture's own events), or another device than the context's is current (a handle like that of
+ * the default stream then names that device's; the call's launches are refused with ECUDA), or ctx is NULL. */
 NLINV_API int nlinv_use_stream(nlinv_ctx* ctx, void* stream);
 
 /* Orders the context's own stream after the context's last call, wherever it ran.  Errors: EINVAL, ECUDA. */

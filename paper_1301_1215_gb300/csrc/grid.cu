@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "nlinv.h"
+#include "call_order.h"
 #include "kernels.cuh"
 
 void nlv_set_global_error(const std::string& msg);
@@ -22,10 +23,7 @@ struct nlinv_gridder {
   int* idx = nullptr;            // device: sample indices s * 2n + i, grouped by grid point
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  cudaStream_t next = nullptr;   // the stream of the next call, if next_set (nlinv_gridder_use_stream)
-  bool next_set = false;
-  cudaStream_t last = nullptr;   // once a caller's stream has been used: the stream of the last call, and its end
-  cudaEvent_t done = nullptr;
+  nlv::StreamOrder order;        // calls on a caller's stream (nlinv_gridder_use_stream)
 };
 
 namespace {
@@ -55,10 +53,7 @@ nlinv_status gfail(nlinv_status s, const std::string& msg) {
 void gridder_free(nlinv_gridder* g) {
   if (!g) return;
   if (g->stream) cudaStreamSynchronize(g->stream);
-  if (g->done) {
-    cudaEventSynchronize(g->done);
-    cudaEventDestroy(g->done);
-  }
+  g->order.finish();
   if (g->off) cudaFree(g->off);
   if (g->idx) cudaFree(g->idx);
   if (g->own_stream && g->stream) cudaStreamDestroy(g->stream);
@@ -118,6 +113,9 @@ nlinv_status nlinv_gridder_create(int n, int nspokes, const double* directions, 
     g->own_stream = e == cudaSuccess;
     if (e != cudaSuccess) g->stream = nullptr;
   }
+  int dev = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  g->order.init(g->stream, dev);
   if (e == cudaSuccess) e = cudaMalloc(&g->off, (size_t)(cells + 1) * sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&g->idx, idx.size() * sizeof(int));
   if (e == cudaSuccess)
@@ -134,33 +132,13 @@ nlinv_status nlinv_gridder_create(int n, int nspokes, const double* directions, 
 }
 
 int nlinv_gridder_use_stream(nlinv_gridder* g, void* stream) {
-  if (!g) return 0;
-  const cudaStream_t s = (cudaStream_t)stream;
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  g->next_set = false;
-  if (s == g->stream || cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return 0;
-  if (!g->done) {
-    if (cudaStreamIsCapturing(g->stream, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return 0;
-    if (cudaEventCreateWithFlags(&g->done, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventRecord(g->done, g->stream) != cudaSuccess) {
-      cudaGetLastError();
-      if (g->done) cudaEventDestroy(g->done);
-      g->done = nullptr;
-      return 0;
-    }
-    g->last = g->stream;
-  }
-  g->next = s;
-  g->next_set = true;
-  return 1;
+  return g && g->order.choose((cudaStream_t)stream) ? 1 : 0;
 }
 
 nlinv_status nlinv_grid(nlinv_gridder* g, int ncoils, const nlinv_c32* samples, nlinv_c32* y_out,
                         uint8_t* mask_out) {
   if (!g) return gfail(NLINV_EINVAL, "gridder is NULL");
-  const bool chosen = g->next_set;
-  const cudaStream_t st = chosen ? g->next : g->stream;
-  g->next_set = false;
+  const cudaStream_t st = g->order.take();
   if (ncoils < 1 || ncoils > 64) return gfail(NLINV_EINVAL, "ncoils must be in 1..64");
   if (!samples || !y_out || !mask_out) return gfail(NLINV_EINVAL, "samples, y_out and mask_out are required");
   if (!device_ptr(samples) || !device_ptr(y_out) || !device_ptr(mask_out))
@@ -169,15 +147,14 @@ nlinv_status nlinv_grid(nlinv_gridder* g, int ncoils, const nlinv_c32* samples, 
   const long threads = (long)ncoils * cells;
   const int block = 256;
   const unsigned grid = (unsigned)((threads + block - 1) / block);
-  // each call on a caller's stream follows the call before, so that `done` marks the end of them all
-  if (chosen && g->last != st) cudaStreamWaitEvent(st, g->done, 0);
-  grid_gather_kernel<<<grid, block, 0, st>>>((const float2*)samples, g->off, g->idx, cells, ncoils,
-                                                    g->nspokes * 2 * g->n, (float2*)y_out, mask_out);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && chosen) {
-    e = cudaEventRecord(g->done, st);
-    g->last = st;
-  }
+  // the tables are only read, but each call follows the call before, so that one event marks the end of them all
+  cudaError_t e = g->order.enter(st);
+  if (e == cudaSuccess)
+    grid_gather_kernel<<<grid, block, 0, st>>>((const float2*)samples, g->off, g->idx, cells, ncoils,
+                                               g->nspokes * 2 * g->n, (float2*)y_out, mask_out);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  const cudaError_t e2 = g->order.leave();
+  if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) return gfail(NLINV_ECUDA, std::string("nlinv_grid: ") + cudaGetErrorString(e));
   return NLINV_OK;
 }

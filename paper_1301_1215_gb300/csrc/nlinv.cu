@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "nlinv.h"
+#include "call_order.h"
 #include "sizes.cuh"
 
 using nlv::KArgs;
@@ -252,14 +253,7 @@ struct nlinv_ctx {
   const SizeKernels* k = nullptr;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  // Operator calls on a caller's stream (nlinv_use_stream).  All streams share the workspace, so every call is ordered
-  // after the call before it: `done` marks the end of the last one, which ran on `last`.  Kept only once a caller's
-  // stream has been used.
-  cudaStream_t run = nullptr;      // where launches go: `stream` outside an operator call
-  cudaStream_t next = nullptr;     // the stream of the next operator call, if next_set
-  bool next_set = false;
-  cudaStream_t last = nullptr;
-  cudaEvent_t done = nullptr;
+  nlv::StreamOrder order;     // operator calls on a caller's stream (nlinv_use_stream): all share the workspace
   int device = 0;
   int vec_blocks = 0;         // grid of the vector kernels
   int sms = 0;                // streaming multiprocessors of the device
@@ -386,7 +380,7 @@ cudaError_t launch(nlinv_ctx* c, const void* fn, int grid, int block, size_t sme
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
-  cfg.stream = c->run;
+  cfg.stream = c->order.run;
   cudaLaunchAttribute attr[3];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = c->pdl ? 1 : 0;
@@ -400,38 +394,12 @@ cudaError_t launch(nlinv_ctx* c, const void* fn, int grid, int block, size_t sme
   return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
-bool capturing(cudaStream_t s) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
-}
-
-// Orders the context's next work, on stream s, after its last call and sends launches there.  A stream that is being
-// captured takes no dependency on work outside its capture (nlinv_use_stream never picks one).
-cudaError_t enter_stream(nlinv_ctx* c, cudaStream_t s) {
-  c->run = s;
-  if (!c->done || c->last == s || capturing(s)) return cudaSuccess;
-  return cudaStreamWaitEvent(s, c->done, 0);
-}
-cudaError_t enter_own(nlinv_ctx* c) {
-  c->next_set = false;
-  return enter_stream(c, c->stream);
-}
-// The end of a call's work on c->run; launches go to the context's own stream again.
-cudaError_t leave_stream(nlinv_ctx* c) {
-  cudaError_t e = cudaSuccess;
-  if (c->done && !(c->run == c->stream && capturing(c->run))) {
-    e = cudaEventRecord(c->done, c->run);
-    c->last = c->run;
-  }
-  c->run = c->stream;
-  return e;
-}
 // Scope of a call on the context's own stream.
 struct OwnStream {
   nlinv_ctx* c;
   cudaError_t err;
-  explicit OwnStream(nlinv_ctx* ctx) : c(ctx), err(enter_own(ctx)) {}
-  ~OwnStream() { leave_stream(c); }
+  explicit OwnStream(nlinv_ctx* ctx) : c(ctx), err(ctx->order.enter_own()) {}
+  ~OwnStream() { c->order.leave(); }
 };
 
 // Passes copy the planes of rho, drho and the sampling pattern into shared memory in 16-byte pieces.  A caller's array may
@@ -442,7 +410,7 @@ template <class T> cudaError_t stageable(const nlinv_ctx* c, const T*& p, void* 
   if (on_boundary(p)) return cudaSuccess;
   const T* from = p;
   p = (const T*)room;
-  return cudaMemcpyAsync(room, from, (size_t)c->plane * sizeof(T), cudaMemcpyDeviceToDevice, c->run);
+  return cudaMemcpyAsync(room, from, (size_t)c->plane * sizeof(T), cudaMemcpyDeviceToDevice, c->order.run);
 }
 bool row_stages_mask(int mode) {
   return mode == nlv::ROW_PSF || mode == nlv::ROW_CG_PSF || mode == nlv::ROW_FFT_P_OUT || mode == nlv::ROW_FFT_RESID;
@@ -1060,17 +1028,13 @@ nlinv_status finish_call(nlinv_ctx* c, cudaError_t e, const char* where) {
 
 // Begin and end of an operator call: on the stream that nlinv_use_stream chose for it (taken first thing, so that a
 // refused call uses the choice up too), else on the context's own.
-cudaStream_t op_stream(nlinv_ctx* c) {
-  const cudaStream_t s = c->next_set ? c->next : c->stream;
-  c->next_set = false;
-  return s;
-}
+cudaStream_t op_stream(nlinv_ctx* c) { return c->order.take(); }
 cudaError_t op_begin(nlinv_ctx* c, cudaStream_t s) {
   c->launches = 0;
-  return enter_stream(c, s);
+  return c->order.enter(s);
 }
 nlinv_status op_end(nlinv_ctx* c, cudaError_t e, const char* where) {
-  const cudaError_t e2 = leave_stream(c);
+  const cudaError_t e2 = c->order.leave();
   return finish_call(c, e != cudaSuccess ? e : e2, where);
 }
 
@@ -1193,7 +1157,7 @@ nlinv_status create_ctx(const nlinv_params* params, void* stream, int batch_lane
     if (e != cudaSuccess) { g_create_error = std::string("cudaStreamCreate: ") + cudaGetErrorString(e); delete c; return NLINV_ECUDA; }
     c->own_stream = true;
   }
-  c->run = c->stream;
+  c->order.init(c->stream, c->device);
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
   if (const char* v = std::getenv("NLINV_PDL")) c->pdl = std::strcmp(v, "0") != 0;
@@ -1347,26 +1311,7 @@ nlinv_status nlinv_create(const nlinv_params* params, void* stream, nlinv_ctx** 
   return create_ctx(params, stream, 0, out);
 }
 
-int nlinv_use_stream(nlinv_ctx* c, void* stream) {
-  if (!c) return 0;
-  const cudaStream_t s = (cudaStream_t)stream;
-  c->next_set = false;
-  if (s == c->stream || capturing(s)) return 0;
-  if (!c->done) {              // from here on the end of every call is marked
-    if (capturing(c->stream)) return 0;
-    if (cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventRecord(c->done, c->stream) != cudaSuccess) {
-      cudaGetLastError();
-      if (c->done) cudaEventDestroy(c->done);
-      c->done = nullptr;
-      return 0;
-    }
-    c->last = c->stream;
-  }
-  c->next = s;
-  c->next_set = true;
-  return 1;
-}
+int nlinv_use_stream(nlinv_ctx* c, void* stream) { return c && c->order.choose((cudaStream_t)stream) ? 1 : 0; }
 
 nlinv_status nlinv_join(nlinv_ctx* c) {
   if (!c) return NLINV_EINVAL;
@@ -1378,10 +1323,7 @@ nlinv_status nlinv_join(nlinv_ctx* c) {
 nlinv_status nlinv_destroy(nlinv_ctx* c) {
   if (!c) return NLINV_OK;
   cudaStreamSynchronize(c->stream);
-  if (c->done) {
-    cudaEventSynchronize(c->done);
-    cudaEventDestroy(c->done);
-  }
+  c->order.finish();
   if (c->graph) cudaGraphExecDestroy(c->graph);
   cudaFree(c->base);
   if (c->vjp_base) cudaFree(c->vjp_base);
