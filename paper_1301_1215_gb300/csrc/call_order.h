@@ -4,6 +4,10 @@
 // share the object's device memory, so each follows the one before it: `done` marks the end of the last call, and a call
 // on another stream waits for it.  The event is there only once a caller's stream has been used.
 //
+// Whether two calls share a stream is told by the stream's id, which the runtime never gives out twice.  The handle does
+// not tell: that of a destroyed stream, whose work may still be running, can come back for a new one, and
+// cudaStreamPerThread is one handle for a stream per host thread (it has no id here: a call on it always waits).
+//
 // Api supplies the runtime calls, so that the decisions can be tested without a GPU (tests/test_call_order_host.py).
 #pragma once
 
@@ -42,7 +46,7 @@ template <class Api> struct CallOrder {
         done = {};
         return false;
       }
-      last = own;
+      mark(own);
     }
     next = s;
     next_set = true;
@@ -57,7 +61,8 @@ template <class Api> struct CallOrder {
   // Orders the call's work, on stream s, after the call before it and sends launches there.
   Error enter(Stream s) {
     run = s;
-    if (!done || last == s || capturing(s)) return Api::kSuccess;
+    unsigned long long id = 0;
+    if (!done || capturing(s) || (last_known && Api::stream_id(s, &id) && id == last)) return Api::kSuccess;
     return Api::wait(s, done);
   }
   Error enter_own() {
@@ -69,7 +74,7 @@ template <class Api> struct CallOrder {
     Error e = Api::kSuccess;
     if (done && !(run == own && capturing(run))) {
       e = Api::record(done, run);
-      last = run;
+      mark(run);
     }
     run = own;
     return e;
@@ -83,13 +88,15 @@ template <class Api> struct CallOrder {
   }
 
  private:
+  void mark(Stream s) { last_known = Api::stream_id(s, &last); }
   static bool capturing(Stream s) {
     bool yes = false;
     return Api::is_capturing(s, &yes) != Api::kSuccess || yes;
   }
   Stream next = {};          // the stream of the next call, if next_set
   bool next_set = false;
-  Stream last = {};          // where `done` was recorded
+  unsigned long long last = 0;     // the id of the stream where `done` was recorded, if it has one
+  bool last_known = false;
 };
 
 #if defined(__CUDACC__)
@@ -104,6 +111,12 @@ struct CudaOrderApi {
     const Error e = cudaStreamIsCapturing(s, &st);
     *yes = st != cudaStreamCaptureStatusNone;
     return e;
+  }
+  static bool stream_id(Stream s, unsigned long long* id) {
+    if (s == cudaStreamPerThread) return false;
+    if (cudaStreamGetId(s, id) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
   }
   static Error create(Event* e) { return cudaEventCreateWithFlags(e, cudaEventDisableTiming); }
   static Error record(Event e, Stream s) { return cudaEventRecord(e, s); }

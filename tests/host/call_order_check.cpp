@@ -5,7 +5,7 @@
 #include "call_order.h"
 
 struct Fake {
-  using Stream = int;            // 0: the default stream
+  using Stream = int;            // 0: the default stream; 9: the per-thread stream, which has no id
   using Event = int;
   using Error = int;
   static constexpr Error kSuccess = 0;
@@ -13,6 +13,12 @@ struct Fake {
   static inline std::string log;
   static Error current_device(int* d) { *d = device; return device_error; }
   static Error is_capturing(Stream s, bool* yes) { *yes = s == capturing; return 0; }
+  static inline int reborn = -1;         // a handle whose stream was destroyed and created anew
+  static bool stream_id(Stream s, unsigned long long* id) {
+    if (s == 9) return false;
+    *id = 1000ull + (unsigned long long)s + (s == reborn ? 100000ull : 0ull);
+    return true;
+  }
   static Error create(Event* e) { *e = 7; return 0; }
   static Error record(Event, Stream s) { log += "record" + std::to_string(s) + " "; return 0; }
   static Error wait(Stream s, Event) { log += "wait" + std::to_string(s) + " "; return 0; }
@@ -63,6 +69,18 @@ int main() {
     Fake::log.clear();
     check(!o.choose(0) && Fake::log == "clear ", "unknown device: not taken, the error is not left behind");
     Fake::device_error = 0;
+  }
+  {                                                 // one handle, another stream
+    nlv::CallOrder<Fake> o;
+    o.init(own, 0);
+    call(o, 1);
+    Fake::reborn = 1;
+    check(call(o, 1) == "wait1 record1 ran1", "a new stream at an old handle follows the call on the old one");
+    check(call(o, 1) == "record1 ran1", "and needs no wait after itself");
+    Fake::reborn = -1;
+    check(call(o, 9) == "wait9 record9 ran9", "the per-thread stream follows");
+    check(call(o, 9) == "wait9 record9 ran9", "the per-thread stream, perhaps another thread's, follows again");
+    check(call(o, 1) == "wait1 record1 ran1", "a stream follows the per-thread one");
   }
   {                                                 // captured streams
     nlv::CallOrder<Fake> o;
