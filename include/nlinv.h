@@ -206,8 +206,8 @@ typedef struct nlinv_gridder nlinv_gridder;
 NLINV_API nlinv_status nlinv_gridder_create(int n, int nspokes, const double* directions, void* stream,
                                             nlinv_gridder** out);
 
-/* Chooses the stream of the next nlinv_grid call on g, as nlinv_use_stream does for operator calls.  The gridder's
- * tables are only read; calls on a caller's stream are ordered after one another all the same, for the destructor. */
+/* Chooses the stream of the next nlinv_grid call on g, as nlinv_use_stream does for operator calls.  A gridder holds one
+ * choice, whichever host thread made it: several threads use nlinv_grid_on. */
 NLINV_API int nlinv_gridder_use_stream(nlinv_gridder* g, void* stream);
 
 /* y_out (DEVICE, ncoils x n x n) and mask_out (DEVICE, n x n) from samples (DEVICE, ncoils x nspokes x 2n, spoke-major
@@ -215,6 +215,15 @@ NLINV_API int nlinv_gridder_use_stream(nlinv_gridder* g, void* stream);
  * ECUDA. */
 NLINV_API nlinv_status nlinv_grid(nlinv_gridder* g, int ncoils, const nlinv_c32* samples, nlinv_c32* y_out,
                                   uint8_t* mask_out);
+
+/* nlinv_grid queued on `stream` (a cudaStream_t of the gridder's device, NULL the legacy default stream), after the
+ * gridder's last call wherever that ran; on a stream that is being captured, in the capture's order alone.  Host threads
+ * may call it on one gridder at the same time.  Errors: as nlinv_grid, and ECUDA while another device is current. */
+NLINV_API nlinv_status nlinv_grid_on(nlinv_gridder* g, void* stream, int ncoils, const nlinv_c32* samples,
+                                     nlinv_c32* y_out, uint8_t* mask_out);
+
+/* Orders the gridder's own stream after its last call, wherever it ran.  Errors: EINVAL, ECUDA. */
+NLINV_API nlinv_status nlinv_gridder_join(nlinv_gridder* g);
 
 /* Waits for the gridder's work and frees it.  NULL is accepted. */
 NLINV_API nlinv_status nlinv_gridder_destroy(nlinv_gridder* g);

@@ -70,6 +70,8 @@ SIGNATURES = {
     "nlinv_gridder_create": (_int, [_int, _int, C.POINTER(_dbl), _vp, C.POINTER(_vp)]),
     "nlinv_gridder_use_stream": (_int, [_vp, _vp]),
     "nlinv_grid": (_int, [_vp, _int, _vp, _vp, _vp]),
+    "nlinv_grid_on": (_int, [_vp, _vp, _int, _vp, _vp, _vp]),
+    "nlinv_gridder_join": (_int, [_vp]),
     "nlinv_gridder_destroy": (_int, [_vp]),
     "nlinv_autotune": (_int, [_vp, _vp, _vp, _vp, _int, C.POINTER(Tuning), C.POINTER(Tuning), _int]),
     "nlinv_set_shapes": (_int, [_vp, C.POINTER(Tuning)]),

@@ -7,6 +7,7 @@
 // without atomics, so the result does not depend on scheduling.
 #include <cmath>
 #include <cstdlib>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -23,7 +24,8 @@ struct nlinv_gridder {
   int* idx = nullptr;            // device: sample indices s * 2n + i, grouped by grid point
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  nlv::StreamOrder order;        // calls on a caller's stream (nlinv_gridder_use_stream)
+  std::mutex lock;               // calls may come from several host threads
+  nlv::StreamOrder order;        // calls on a caller's stream (nlinv_grid_on, nlinv_gridder_use_stream)
 };
 
 namespace {
@@ -67,6 +69,35 @@ bool device_ptr(const void* p) {
     return false;
   }
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
+nlinv_status check_grid(int ncoils, const nlinv_c32* samples, nlinv_c32* y_out, uint8_t* mask_out) {
+  if (ncoils < 1 || ncoils > 64) return gfail(NLINV_EINVAL, "ncoils must be in 1..64");
+  if (!samples || !y_out || !mask_out) return gfail(NLINV_EINVAL, "samples, y_out and mask_out are required");
+  if (!device_ptr(samples) || !device_ptr(y_out) || !device_ptr(mask_out))
+    return gfail(NLINV_EINVAL, "samples, y_out and mask_out must be device pointers");
+  return NLINV_OK;
+}
+
+cudaError_t gather(const nlinv_gridder* g, cudaStream_t st, int ncoils, const nlinv_c32* samples, nlinv_c32* y_out,
+                   uint8_t* mask_out) {
+  const int cells = g->n * g->n, block = 256;
+  const unsigned grid = (unsigned)(((long)ncoils * cells + block - 1) / block);
+  grid_gather_kernel<<<grid, block, 0, st>>>((const float2*)samples, g->off, g->idx, cells, ncoils,
+                                             g->nspokes * 2 * g->n, (float2*)y_out, mask_out);
+  return cudaGetLastError();
+}
+
+// One call on stream st (under the gridder's lock): the tables are only read, but each call follows the call before, so
+// that one event marks the end of them all.
+nlinv_status run_ordered(nlinv_gridder* g, cudaStream_t st, int ncoils, const nlinv_c32* samples, nlinv_c32* y_out,
+                         uint8_t* mask_out) {
+  cudaError_t e = g->order.enter(st);
+  if (e == cudaSuccess) e = gather(g, st, ncoils, samples, y_out, mask_out);
+  const cudaError_t e2 = g->order.leave();
+  if (e == cudaSuccess) e = e2;
+  if (e != cudaSuccess) return gfail(NLINV_ECUDA, std::string("nlinv_grid: ") + cudaGetErrorString(e));
+  return NLINV_OK;
 }
 
 }  // namespace
@@ -132,30 +163,49 @@ nlinv_status nlinv_gridder_create(int n, int nspokes, const double* directions, 
 }
 
 int nlinv_gridder_use_stream(nlinv_gridder* g, void* stream) {
-  return g && g->order.choose((cudaStream_t)stream) ? 1 : 0;
+  if (!g) return 0;
+  std::lock_guard<std::mutex> hold(g->lock);
+  return g->order.choose((cudaStream_t)stream) ? 1 : 0;
 }
 
 nlinv_status nlinv_grid(nlinv_gridder* g, int ncoils, const nlinv_c32* samples, nlinv_c32* y_out,
                         uint8_t* mask_out) {
   if (!g) return gfail(NLINV_EINVAL, "gridder is NULL");
+  std::lock_guard<std::mutex> hold(g->lock);
   const cudaStream_t st = g->order.take();
-  if (ncoils < 1 || ncoils > 64) return gfail(NLINV_EINVAL, "ncoils must be in 1..64");
-  if (!samples || !y_out || !mask_out) return gfail(NLINV_EINVAL, "samples, y_out and mask_out are required");
-  if (!device_ptr(samples) || !device_ptr(y_out) || !device_ptr(mask_out))
-    return gfail(NLINV_EINVAL, "samples, y_out and mask_out must be device pointers");
-  const int cells = g->n * g->n;
-  const long threads = (long)ncoils * cells;
-  const int block = 256;
-  const unsigned grid = (unsigned)((threads + block - 1) / block);
-  // the tables are only read, but each call follows the call before, so that one event marks the end of them all
-  cudaError_t e = g->order.enter(st);
-  if (e == cudaSuccess)
-    grid_gather_kernel<<<grid, block, 0, st>>>((const float2*)samples, g->off, g->idx, cells, ncoils,
-                                               g->nspokes * 2 * g->n, (float2*)y_out, mask_out);
-  if (e == cudaSuccess) e = cudaGetLastError();
-  const cudaError_t e2 = g->order.leave();
-  if (e == cudaSuccess) e = e2;
-  if (e != cudaSuccess) return gfail(NLINV_ECUDA, std::string("nlinv_grid: ") + cudaGetErrorString(e));
+  const nlinv_status bad = check_grid(ncoils, samples, y_out, mask_out);
+  if (bad != NLINV_OK) return bad;
+  return run_ordered(g, st, ncoils, samples, y_out, mask_out);
+}
+
+nlinv_status nlinv_grid_on(nlinv_gridder* g, void* stream, int ncoils, const nlinv_c32* samples, nlinv_c32* y_out,
+                           uint8_t* mask_out) {
+  if (!g) return gfail(NLINV_EINVAL, "gridder is NULL");
+  const nlinv_status bad = check_grid(ncoils, samples, y_out, mask_out);
+  if (bad != NLINV_OK) return bad;
+  const cudaStream_t st = (cudaStream_t)stream;
+  int dev = -1;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess && dev != g->order.device) return gfail(NLINV_ECUDA, "nlinv_grid_on: another device is current");
+  if (e == cudaSuccess) e = cudaStreamIsCapturing(st, &cap);
+  if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) e = gather(g, st, ncoils, samples, y_out, mask_out);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return gfail(NLINV_ECUDA, std::string("nlinv_grid_on: ") + cudaGetErrorString(e));
+  }
+  if (cap != cudaStreamCaptureStatusNone) return NLINV_OK;      // the capture orders what it holds
+  std::lock_guard<std::mutex> hold(g->lock);
+  if (st != g->stream && !g->order.choose(st)) return gfail(NLINV_ECUDA, "nlinv_grid_on: the stream cannot be ordered");
+  return run_ordered(g, g->order.take(), ncoils, samples, y_out, mask_out);
+}
+
+nlinv_status nlinv_gridder_join(nlinv_gridder* g) {
+  if (!g) return gfail(NLINV_EINVAL, "gridder is NULL");
+  std::lock_guard<std::mutex> hold(g->lock);
+  const cudaError_t e = g->order.enter_own(), e2 = g->order.leave();
+  if (e != cudaSuccess || e2 != cudaSuccess)
+    return gfail(NLINV_ECUDA, std::string("nlinv_gridder_join: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
   return NLINV_OK;
 }
 

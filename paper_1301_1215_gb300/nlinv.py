@@ -441,9 +441,10 @@ class Gridder:
 
     @property
     def stream(self) -> "torch.cuda.Stream":
-        """The gridder's CUDA stream, ordered after the current stream; later calls run on it (until it is read, calls
-        run on the current stream)."""
+        """The gridder's CUDA stream, ordered after its earlier calls and the current stream; later calls run on it (until
+        it is read, calls run on the current stream)."""
         if not self._stream_seen:
+            _lib.check(self._lib.nlinv_gridder_join(self._h))
             self._stream.wait_stream(torch.cuda.current_stream(self.device))
             self._stream_seen = True
         return self._stream
@@ -457,8 +458,9 @@ class Gridder:
         J = samples.shape[0]
         y = torch.empty((J, self.n, self.n), dtype=torch.complex64, device=self.device)
         m = torch.empty((self.n, self.n), dtype=torch.uint8, device=self.device)
-        if not self._stream_seen and self._lib.nlinv_gridder_use_stream(self._h, _raw_stream(self.device.index)):
-            _lib.check(self._lib.nlinv_grid(self._h, int(J), _ptr(samples), _ptr(y), _ptr(m)))
+        if not self._stream_seen:
+            _lib.check(self._lib.nlinv_grid_on(self._h, _raw_stream(self.device.index), int(J), _ptr(samples), _ptr(y),
+                                               _ptr(m)))
         else:
             self._stream.wait_stream(torch.cuda.current_stream(self.device))
             _lib.check(self._lib.nlinv_grid(self._h, int(J), _ptr(samples), _ptr(y), _ptr(m)))

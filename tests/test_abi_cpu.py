@@ -115,6 +115,8 @@ def test_gridder_create_rejects_bad_arguments_on_the_host(lib):
     nan = (C.c_double * 2)(float("nan"), 0.0)
     assert lib.nlinv_gridder_create(16, 1, nan, None, C.byref(h)) == _lib.EINVAL
     assert lib.nlinv_grid(None, 1, None, None, None) == _lib.EINVAL
+    assert lib.nlinv_grid_on(None, None, 1, None, None, None) == _lib.EINVAL
+    assert lib.nlinv_gridder_join(None) == _lib.EINVAL
     assert lib.nlinv_gridder_destroy(None) == _lib.OK
 
 

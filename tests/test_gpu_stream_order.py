@@ -107,3 +107,57 @@ def test_per_thread_stream(env):
     assert status == [1, 0, 1, 0]
     for o, w in zip(out, want):
         assert torch.equal(o.cpu(), w)
+
+
+def _spokes(k=4):
+    return [(np.cos(a), np.sin(a)) for a in np.arange(k) * 0.7]
+
+
+def test_gridder_shared_by_two_threads(env):
+    """Each thread grids samples that its own stream produces after a delay, again and again, on one gridder."""
+    torch = env[0]
+    import threading
+    from paper_1301_1215_gb300.nlinv import Gridder
+    base = torch.randn((J, 4, 2 * N), dtype=torch.complex64, device="cuda")
+    with Gridder(N, _spokes()) as gr:
+        want = gr.grid(base)[0] * 2.0           # powers of two below: exact
+        torch.cuda.synchronize()
+        got, errors = [[], []], []
+
+        def work(i):
+            try:
+                s = torch.cuda.Stream()
+                with torch.cuda.stream(s):
+                    for k in range(40):
+                        if k % 10 == 0:
+                            torch.cuda._sleep(DELAY // 10)
+                        got[i].append(gr.grid(base * 2.0)[0])
+                s.synchronize()
+            except Exception as e:              # reported by the main thread
+                errors.append(e)
+        threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        assert not errors, errors
+        torch.cuda.synchronize()
+        for y in got[0] + got[1]:
+            assert torch.equal(y, want)
+
+
+def test_gridders_stream_follows_calls_on_other_streams(env):
+    torch = env[0]
+    from paper_1301_1215_gb300.nlinv import Gridder
+    smp = torch.randn((J, 4, 2 * N), dtype=torch.complex64, device="cuda")
+    side = torch.cuda.Stream()
+    with Gridder(N, _spokes()) as gr:
+        gr.grid(smp)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(DELAY)
+            gr.grid(smp)
+        own = gr.stream                          # read with the default stream current, which has nothing to wait for
+        assert not own.query()
+        own.synchronize()
+        assert side.query()
