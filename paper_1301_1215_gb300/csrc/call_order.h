@@ -91,7 +91,9 @@ template <class Api> struct CallOrder {
   void mark(Stream s) { last_known = Api::stream_id(s, &last); }
   static bool capturing(Stream s) {
     bool yes = false;
-    return Api::is_capturing(s, &yes) != Api::kSuccess || yes;
+    if (Api::is_capturing(s, &yes) == Api::kSuccess) return yes;
+    Api::clear_error();      // (the default stream while a stream that it blocks is captured; not this call's error)
+    return true;
   }
   Stream next = {};          // the stream of the next call, if next_set
   bool next_set = false;

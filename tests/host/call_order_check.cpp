@@ -9,10 +9,10 @@ struct Fake {
   using Event = int;
   using Error = int;
   static constexpr Error kSuccess = 0;
-  static inline int device = 0, device_error = 0, capturing = -1;
+  static inline int device = 0, device_error = 0, capturing = -1, capture_error = 0;
   static inline std::string log;
   static Error current_device(int* d) { *d = device; return device_error; }
-  static Error is_capturing(Stream s, bool* yes) { *yes = s == capturing; return 0; }
+  static Error is_capturing(Stream s, bool* yes) { *yes = s == capturing; return capture_error; }
   static inline int reborn = -1;         // a handle whose stream was destroyed and created anew
   static bool stream_id(Stream s, unsigned long long* id) {
     if (s == 9) return false;
@@ -94,6 +94,10 @@ int main() {
     Fake::capturing = own;
     check(call(o, own) == "ran50", "a captured call on the own stream: no wait on, no mark of, work outside the capture");
     Fake::capturing = -1;
+    Fake::capture_error = 4;
+    Fake::log.clear();
+    check(!o.choose(0) && Fake::log == "clear ", "unknown capture: not taken, the error is not left behind");
+    Fake::capture_error = 0;
     check(o.choose(1) && o.take() == 1 && o.take() == own, "a choice is for one call");
     o.choose(1);
     o.enter_own();
