@@ -134,15 +134,16 @@ __global__ void __launch_bounds__(ClusterSmem<N1, N2>::T, 1) cg_solve_cluster(co
     const int cr = i / (Wc / 2), k = i % (Wc / 2);
     cp_async16(srho + cr * Wc + 2 * k, A.rho + (size_t)to_natural(cr, N, f) * N + to_natural(2 * k, N, f));
   }
+  const float unit = A.sc->unit;
   for (int o = tid; o < o_cnt; o += T) {
-    qr[o] = A.r[o_begin + o];
+    qr[o] = cscale(A.r[o_begin + o], unit);
     qp[o] = qd[o] = make_float2(0.f, 0.f);
   }
   float2 r[N1], p[N1], dx[N1];
   float w[N1];
 #pragma unroll
   for (int m = 0; m < N1; ++m) {
-    r[m] = A.r[coil0 + ob + N2 * m];
+    r[m] = cscale(A.r[coil0 + ob + N2 * m], unit);
     w[m] = A.wtab[ob + N2 * m] * rs;
     p[m] = dx[m] = make_float2(0.f, 0.f);
   }
@@ -155,11 +156,11 @@ __global__ void __launch_bounds__(ClusterSmem<N1, N2>::T, 1) cg_solve_cluster(co
     ro_at[h] = cluster_addr(qr + (o - own * share), own);
   }
   // The scalars live in thread 0 of every block, formed there from the same sums in the same order: pairs, all in the
-  // units of the block sums (kBlockScale).  s_cg and s_stop pass the decisions on (s_stop: 1 the solve stops before
+  // unit of the solve (cg_unit), as r, p and dx.  s_cg and s_stop pass the decisions on (s_stop: 1 the solve stops before
   // iteration `it` takes its step, 2 on a non-finite value).  In FP64 they took 15000 of 34600 cycles an iteration.
   Pair rr = {0.f, 0.f}, floor = rr, pp = rr, beta = rr, inv_rs2 = rr;
   if (tid == 0) {
-    rr = pp = pair_scale(A.sc->rr_pair, kBlockScale / kPairScale);
+    rr = pp = A.sc->rr_pair;
     floor = pair_scale(rr, (float)kCgFloor2);
     inv_rs2 = pair_div({1.f, 0.f}, pair_mul({rs, 0.f}, {rs, 0.f}));
     s_cg.a = s_cg.a_prev = s_cg.beta = 0.f;
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(ClusterSmem<N1, N2>::T, 1) cg_solve_cluster(co
           if (m < H / 2 || m >= N1 - H / 2) {                    // Omega
             const int h = m < H / 2 ? m : m - (N1 - H);
             const int o = to_compact(e1, N, f) * Wc + cl;
-            float2 u = cscale(v[m], rs), dr = ro[h];
+            float2 u = cscale(v[m], first ? rs * unit : rs), dr = ro[h];      // (T as staged holds b)
             if (!first) {
               const float2 uo = su[o];
               dr = make_float2(fmaf(bf, po[h].x, dr.x), fmaf(bf, po[h].y, dr.y));
@@ -296,6 +297,7 @@ __global__ void __launch_bounds__(ClusterSmem<N1, N2>::T, 1) cg_solve_cluster(co
     cg.a_prev = 0.f;
     cg.beta = bf;
     cg.alpha = A.alpha;
+    cg.unit = 1.f;
     cg.first = first;
     CgDots dots;
     dots.rr = dots.rp = dots.pp = make_float2(0.f, 0.f);
@@ -354,12 +356,17 @@ __global__ void __launch_bounds__(ClusterSmem<N1, N2>::T, 1) cg_solve_cluster(co
     __syncthreads();
   }
   // ---- x + dx
+  const float inv = 1.f / unit;
 #pragma unroll
   for (int m = 0; m < N1; ++m) {
     const size_t o = coil0 + ob + N2 * m;
-    A.dst[o] = A.x ? cadd(A.x[o], dx[m]) : dx[m];
+    const float2 d = cscale(dx[m], inv);
+    A.dst[o] = A.x ? cadd(A.x[o], d) : d;
   }
-  for (int o = tid; o < o_cnt; o += T) A.dst[o_begin + o] = A.x ? cadd(A.x[o_begin + o], qd[o]) : qd[o];
+  for (int o = tid; o < o_cnt; o += T) {
+    const float2 d = cscale(qd[o], inv);
+    A.dst[o_begin + o] = A.x ? cadd(A.x[o_begin + o], d) : d;
+  }
   if (j == 0 && tid == 0) {
     // (`it` iterations took a step; a floor reached by the last scheduled one is not a stop)
     A.sc->cg_stop[A.slot] = it < A.iter ? it : -1;

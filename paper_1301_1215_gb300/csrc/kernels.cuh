@@ -27,16 +27,16 @@ enum Reduce : int {
 
 constexpr int kMaxNewton = 64;
 
-// Scalars of the CG and Newton iterations, kept in device memory (FP64).
 // An unevaluated sum of two floats (see pair_add).
 struct Pair {
   float h, l;
 };
 
+// Scalars of the CG and Newton iterations, kept in device memory: those of CG as pairs, the residual norms in FP64.
 // The values that one launch writes while its other blocks still read the value of the iteration before have two
 // slots, indexed by the parity of the CG iteration.
 struct Scalars {
-  // Pairs in units of the sums over a launch (kPairScale); the step lengths as the FP32 updates use them.
+  float unit;                    // of the current CG solve, see cg_unit: r, p, dx and the pairs below are in it
   Pair rr_pair;                  // |b|^2 of the current CG solve
   Pair rr_i[2];                  // |r_i|^2 of iteration i in slot i & 1 (batches: current and previous |r|^2)
   Pair beta_p;                   // beta of the current direction
@@ -232,10 +232,18 @@ __device__ __forceinline__ Pair pair_div(Pair a, Pair b) {
   return pair_norm(q, r / b.h);
 }
 __device__ __forceinline__ bool pair_gt(Pair a, Pair b) { return a.h > b.h || (a.h == b.h && a.l > b.l); }
-// The sums over a block carry a factor kBlockScale and those over the blocks of a launch kGridScale more, so that no
-// FP32 sum overflows where its terms do not (at most 2^13 terms of a block's threads, 2^12 blocks); powers of two, so
-// nothing is rounded short of the denormal range.
-constexpr float kBlockScale = 0x1p-13f, kGridScale = 0x1p-12f, kPairScale = kBlockScale * kGridScale;
+// The unit of a CG solve: the power of two that takes |b| to between 1/2 and 1 (kept so small that its square and the
+// inverse of that are ordinary floats).  A solve is linear in b: it runs on unit b, the first iteration's passes
+// multiplying what the right-hand side pass left by it, and the result is divided by it.  Nothing is rounded by that, and
+// neither the sums of squares nor the rounding floor of |r|^2, 2^-48 of its start, meet the ends of the FP32 range,
+// whatever units the data are in: with raw data and a fixed factor of 2^-25 on the sums, a frame with |b| near 1e-12 never
+// met its floor or met it two iterations early.
+__device__ __forceinline__ float cg_unit(double bb) {
+  if (!(bb > 0.0) || !isfinite(bb)) return 1.f;
+  const int e = ((__double2hiint(bb) >> 20) & 0x7ff) - 1022;       // bb in [2^(e-1), 2^e)
+  const int half = min(max((e + 1) >> 1, -62), 62);
+  return __int_as_float((127 - half) << 23);
+}
 // |p|^2 of p = r + beta p_old from |r|^2, beta, Re<r, p_old> and |p_old|^2.
 __device__ __forceinline__ Pair cg_direction_norm(Pair rr, Pair beta, Pair rp, Pair pp) {
   return pair_sum(rr, pair_mul(beta, pair_sum(pair_scale(rp, 2.f), pair_mul(beta, pp))));
@@ -251,9 +259,8 @@ __device__ __forceinline__ Pair warp_sum(Pair s, int cnt) {
   }
   return s;
 }
-// scale times the sum of the n pairs at src (global or shared memory) by the calling warp, in a fixed order, valid in
-// lane 0.
-__device__ __forceinline__ Pair warp_sum_of(const Pair* src, int n, float scale) {
+// The sum of the n pairs at src (global or shared memory) by the calling warp, in a fixed order, valid in lane 0.
+__device__ __forceinline__ Pair warp_sum_of(const Pair* src, int n) {
   constexpr int D = 12;            // loads in flight
   const int lane = threadIdx.x & 31, nl = warp_lanes();
   Pair s = {0.f, 0.f};
@@ -266,7 +273,7 @@ __device__ __forceinline__ Pair warp_sum_of(const Pair* src, int n, float scale)
       t[d].l = ok ? src[k0 + d * nl].l : 0.f;
     }
 #pragma unroll
-    for (int d = 0; d < D; ++d) pair_add(s, t[d].h * scale, t[d].l * scale);
+    for (int d = 0; d < D; ++d) pair_add(s, t[d].h, t[d].l);
   }
   return warp_sum(s, nl);
 }
@@ -277,7 +284,7 @@ template <int K> __device__ __forceinline__ void block_pairs(const Pair* sums, P
 #pragma unroll
   for (int k = 0; k < K; ++k)
     if (warp == nw - 1 - k % nw) {
-      const Pair s = warp_sum_of(sums + k * blockDim.x, blockDim.x, 1.f);
+      const Pair s = warp_sum_of(sums + k * blockDim.x, blockDim.x);
       if ((threadIdx.x & 31) == 0) *out[k] = s;
     }
 }
@@ -287,8 +294,10 @@ __device__ __forceinline__ void finalize_scalar(Scalars* sc, int reduce, int slo
     case RED_RESID: sc->resid[slot] = sqrt(total); break;
     case RED_RR_INIT:           // a new CG solve starts: nothing has stopped yet
       sc->beta_p = {0.f, 0.f};
-      sc->rr_pair.h = (float)(total * kPairScale);
-      sc->rr_pair.l = (float)(total * kPairScale - (double)sc->rr_pair.h);
+      sc->unit = cg_unit(total);
+      total *= (double)sc->unit * (double)sc->unit;
+      sc->rr_pair.h = (float)total;
+      sc->rr_pair.l = (float)(total - (double)sc->rr_pair.h);
       sc->rr_i[0] = sc->rr_pair;
       sc->cg_stop[slot] = -1;
       break;
@@ -456,8 +465,8 @@ __device__ __forceinline__ void dot_acc(float2& acc, float2 a, float2 b) {     /
 }
 
 __device__ __forceinline__ void dot_flush(float2& acc, Pair& sum) {
-  pair_add(sum, acc.x * kBlockScale, 0.f);
-  pair_add(sum, acc.y * kBlockScale, 0.f);
+  pair_add(sum, acc.x, 0.f);
+  pair_add(sum, acc.y, 0.f);
   acc = make_float2(0.f, 0.f);
 }
 
@@ -520,7 +529,7 @@ __device__ __forceinline__ void rho_channel_sum(const KArgs& A, const bool (&om)
 
 // Adds a thread's FP32 partial to its FP64 sum or its pair.
 __device__ __forceinline__ void acc_add(double& s, float v) { s += (double)v; }
-__device__ __forceinline__ void acc_add(Pair& s, float v) { pair_add(s, v * kBlockScale, 0.f); }
+__device__ __forceinline__ void acc_add(Pair& s, float v) { pair_add(s, v, 0.f); }
 
 // t, bd: the thread's index in the block and the block's threads.  Blocks that share a slice (KArgs::sub) pass their
 // threads' places in the undivided block, so that a thread's two pixels, whose products it adds in FP32, stay the same
@@ -532,6 +541,7 @@ __device__ __forceinline__ void rho_slice(const KArgs& A, int bid, int t, int bd
   const int e_begin = bid * A.rho_per_cta;
   const int e_end = min(e_begin + A.rho_per_cta, plane);
   const float beta = MODE == ROW_BCG_NORMAL ? A.sc->beta_p.h : 0.f;
+  const float unit = MODE == ROW_BCG_NORMAL && A.iter == 0 ? A.sc->unit : 1.f;      // r holds b
   for (int o0 = e_begin + t; o0 < e_end; o0 += 2 * bd) {
     float acc = 0.f;
     float2 a[2], b[2], z[2];
@@ -561,7 +571,7 @@ __device__ __forceinline__ void rho_slice(const KArgs& A, int bid, int t, int bd
       } else if constexpr (RowTraits<MODE>::normal) {
         float2 pv = a[k];
         if constexpr (MODE == ROW_BCG_NORMAL) {
-          pv = make_float2(fmaf(beta, pv.x, b[k].x), fmaf(beta, pv.y, b[k].y));
+          pv = make_float2(fmaf(beta, pv.x, unit * b[k].x), fmaf(beta, pv.y, unit * b[k].y));
           const_cast<float2*>(A.p)[o] = pv;
         }
         const float2 q = make_float2(fmaf(A.alpha, pv.x, z[k].x), fmaf(A.alpha, pv.y, z[k].y));
@@ -584,16 +594,18 @@ __device__ __forceinline__ void rho_slice(const KArgs& A, int bid, int t, int bd
 // The scalars of one CG update (see cg_point).
 struct CgStep {
   float a, a_prev, beta, alpha;
+  float unit;                   // of the solve (iteration 0: r holds b)
   bool first, odd;              // iteration 0 (p = r); an odd iteration (the one that updates dx)
 };
 struct CgDots {                 // sums of |r|^2, Re<r, p> and |p|^2 of the new r and p
   float2 rr, rp, pp;
 };
-// One element of the CG update:  p = r + beta p_old;  q = z + alpha p (z: the element of DF^H DF p);  r -= a q.
+// One element of the CG update (in iteration 0 after r *= unit):  p = r + beta p_old;  q = z + alpha p (z: the element of DF^H DF p);  r -= a q.
 // Returns the new r; p: in the old, out the new direction; g: what the pair of iterations adds to dx (odd
 // iterations: a_prev p_old + a p).
 __device__ __forceinline__ float2 cg_point(const CgStep& c, float2 z, float2 r, float2& p, float2& g, CgDots& acc) {
   const float2 po = p;
+  if (c.first) r = cscale(r, c.unit);
   p = c.first ? r : make_float2(fmaf(c.beta, po.x, r.x), fmaf(c.beta, po.y, r.y));
   const float2 q = make_float2(fmaf(c.alpha, p.x, z.x), fmaf(c.alpha, p.y, z.y));
   r = make_float2(fmaf(-c.a, q.x, r.x), fmaf(-c.a, q.y, r.y));
@@ -827,6 +839,7 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
       cg.first = A.iter == 0;
       cg.odd = (A.iter & 1) != 0;
       cg.alpha = A.alpha;
+      cg.unit = cg.first ? A.sc->unit : 1.f;
       cg.a = A.sc->step[A.iter & 1];
       cg.a_prev = cg.first ? 0.f : A.sc->step[(A.iter & 1) ^ 1];
       cg.beta = cg.first ? 0.f : A.sc->beta_p.h;
@@ -840,7 +853,7 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
       if (!A.brr_part) {
         if (threadIdx.x == 0) s_beta = A.sc->beta_p.h;
       } else if (threadIdx.x >= ((blockDim.x - 1) & ~31u)) {       // the last warp has the least to load
-        const Pair t = warp_sum_of(A.brr_part, A.n_rr, kGridScale);
+        const Pair t = warp_sum_of(A.brr_part, A.n_rr);
         if ((threadIdx.x & 31) == 0) {
           const Pair rp = A.sc->rr_i[1];
           const Pair b = rp.h != 0.f ? pair_div(t, rp) : Pair{0.f, 0.f};
@@ -861,9 +874,10 @@ __device__ __forceinline__ void row_pass_body(const KArgs& A, int bid, int nblk,
     const float* sw = (const float*)(smem_raw + L.w) + (size_t)laneA * N;
     const float2* sr = (const float2*)(smem_raw + L.xch) + (size_t)laneA * N;
     if (activeA) {
+      const float unit = A.iter == 0 ? A.sc->unit : 1.f;      // r holds b
 #pragma unroll
       for (int m = 0; m < N2; ++m) {
-        const float2 rv = sr[idxA + N1 * m];
+        const float2 rv = cscale(sr[idxA + N1 * m], unit);
         v[m] = make_float2(fmaf(s_beta, v[m].x, rv.x), fmaf(s_beta, v[m].y, rv.y));
         const_cast<float2*>(A.src)[(size_t)RA * N + idxA + N1 * m] = v[m];
         v[m] = cscale(v[m], sw[idxA + N1 * m] * rs);
@@ -1209,7 +1223,7 @@ __device__ __forceinline__ void col_stage_side(const KArgs& A, int bid, unsigned
 __device__ __forceinline__ void cg_direction_scalars(const KArgs& A, int bid, float& s_beta, int& s_stop) {
   if (threadIdx.x < ((blockDim.x - 1) & ~31u)) return;
   const Pair rp = A.sc->rr_i[(A.iter & 1) ^ 1], floor = pair_scale(A.sc->rr_pair, (float)kCgFloor2);
-  const Pair t = warp_sum_of(A.rr_part, A.n_rr, kGridScale);
+  const Pair t = warp_sum_of(A.rr_part, A.n_rr);
   if ((threadIdx.x & 31) == 0) {
     const Pair b = rp.h != 0.f ? pair_div(t, rp) : Pair{0.f, 0.f};
     const bool stop = !pair_gt(t, floor) || !isfinite(t.h);
@@ -1240,8 +1254,8 @@ __device__ __forceinline__ void cg_decide(const KArgs& A) {
 #pragma unroll
   for (int k = 0; k < 3; ++k)
     if (warp == k % nw) {
-      const Pair s = k == 0 ? warp_sum_of(A.dd_part, A.n_dd, kGridScale)
-                            : warp_sum_of(A.rr_part + k * A.n_rr, A.iter > 0 ? A.n_rr : 0, kGridScale);
+      const Pair s = k == 0 ? warp_sum_of(A.dd_part, A.n_dd)
+                            : warp_sum_of(A.rr_part + k * A.n_rr, A.iter > 0 ? A.n_rr : 0);
       if (lane == 0) tot[k] = s;
     }
   __syncthreads();
@@ -1365,6 +1379,9 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, int nblk,
         }
       }
       if constexpr (MODE == COL_BCG_DIR) beta = A.sc->beta_p.h;
+      [[maybe_unused]] float unit = 1.f;           // iteration 0: r, and T of single frames, hold b
+      if constexpr (MODE == COL_CG_DIR || MODE == COL_BCG_DIR)
+        if (A.iter == 0) unit = A.sc->unit;
       const size_t sstride = (size_t)Wc * C;
       if constexpr (col_forms_coils(MODE)) {
         float2 c[N1];                       // the coil map on this thread's Omega elements (layout B)
@@ -1417,7 +1434,7 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, int nblk,
           float2 out = make_float2(0.f, 0.f);
           if (active && in_omega(e1, N, f)) {
             const int cr = to_compact(e1, N, f);
-            float2 u = cscale(v[m], rs);
+            float2 u = cscale(v[m], MODE == COL_CG_DIR ? rs * unit : rs);
             const float2 c = side[(size_t)cr * C + lane];
             const float2 rh = side[sstride + (size_t)cr * C + lane];
             if constexpr (MODE == COL_IFFT_ADJ_FFT) {
@@ -1426,7 +1443,7 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, int nblk,
             } else {
               float2 dr;
               if constexpr (MODE == COL_CG_DIR) {      // W^-1 p and the rho part of p = r + beta p
-                dr = side[3 * sstride + (size_t)cr * C + lane];
+                dr = cscale(side[3 * sstride + (size_t)cr * C + lane], unit);
                 if (A.iter > 0) {
                   const float2 po = side[2 * sstride + (size_t)cr * C + lane];
                   dr = make_float2(fmaf(beta, po.x, dr.x), fmaf(beta, po.y, dr.y));
@@ -1436,7 +1453,7 @@ __device__ __forceinline__ void col_pass_body(const KArgs& A, int bid, int nblk,
               } else {
                 dr = side[2 * sstride + (size_t)cr * C + lane];
                 if constexpr (MODE == COL_BCG_DIR) {   // the rho part of p = r + beta p (written by the last row pass)
-                  const float2 rv = side[3 * sstride + (size_t)cr * C + lane];
+                  const float2 rv = cscale(side[3 * sstride + (size_t)cr * C + lane], unit);
                   dr = make_float2(fmaf(beta, dr.x, rv.x), fmaf(beta, dr.y, rv.y));
                 }
               }

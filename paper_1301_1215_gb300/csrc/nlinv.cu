@@ -57,11 +57,12 @@ __device__ __forceinline__ void cg_step_update(float4& d, float4& r, const float
 // The CG step's scalars, the same in every block: t = Re<p, A p> from the n_pq partials, alpha = |r|^2 / t, and the
 // rounding-floor test (see cg_step_body), formed as pairs by the block's first warp (in FP64, a tree over the block and a
 // quotient, each some thousand cycles a block).  Block 0 publishes them; s_alpha is valid for every thread of the block
-// on return.
-__device__ __forceinline__ void cg_step_decide(const KArgs& A, int bid, float& s_alpha) {
+// on return, as is s_unit, the solve's unit.
+__device__ __forceinline__ void cg_step_decide(const KArgs& A, int bid, float& s_alpha, float& s_unit) {
   if (threadIdx.x < 32) {
-    const nlv::Pair t = nlv::warp_sum_of(A.pq_part, A.n_pq, nlv::kGridScale);
+    const nlv::Pair t = nlv::warp_sum_of(A.pq_part, A.n_pq);
     if (threadIdx.x == 0) {
+      s_unit = A.sc->unit;
       const nlv::Pair rr = A.sc->rr_i[0], floor = nlv::pair_scale(A.sc->rr_pair, (float)nlv::kCgFloor2);
       const bool finite = isfinite(t.h) && isfinite(rr.h);
       const bool go = finite && nlv::pair_gt(rr, floor) && t.h > 0.f;
@@ -98,10 +99,11 @@ __device__ __forceinline__ void cg_step_body(const KArgs& A, int bid, int nblk) 
       const long k = i + g * stride;
       pg[g] = p4[k]; qg[g] = q4[k]; rg[g] = r4[k]; dg[g] = dx4[k];
     }
-  __shared__ float s_alpha;
+  __shared__ float s_alpha, s_unit;
   __shared__ nlv::Pair s_pairs[kVecThreads];
-  cg_step_decide(A, bid, s_alpha);
+  cg_step_decide(A, bid, s_alpha, s_unit);
   const float a = s_alpha;
+  const bool first = A.iter == 0;        // r holds b
   nlv::Pair sum = {0.f, 0.f};
   // G groups in flight per thread; each group's operands for the next round are loaded right after it is stored,
   // while the other groups of this round are processed
@@ -111,6 +113,7 @@ __device__ __forceinline__ void cg_step_body(const KArgs& A, int bid, int nblk) 
     for (int g = 0; g < G; ++g) {
       const long k = i + g * stride;
       if (k < A.n2) {
+        if (first) rg[g] = make_float4(rg[g].x * s_unit, rg[g].y * s_unit, rg[g].z * s_unit, rg[g].w * s_unit);
         cg_step_update(dg[g], rg[g], pg[g], qg[g], a, acc);
         dx4[k] = dg[g];
         r4[k] = rg[g];
@@ -126,18 +129,19 @@ __device__ __forceinline__ void cg_step_body(const KArgs& A, int bid, int nblk) 
   nlv::block_pairs<1>(s_pairs, {A.brr_part + bid});
 }
 
-// x += dx (x = A.dst)
+// x += dx (x = A.dst; dx in the unit of the solve)
 __device__ __forceinline__ void add_body(const KArgs& A, int bid, int nblk) {
   const float4* __restrict__ d4 = (const float4*)A.dx;
   float4* __restrict__ x4 = (float4*)A.dst;
+  const float inv = 1.f / A.sc->unit;
   for (long i = bid * (long)blockDim.x + threadIdx.x; i < A.n2; i += (long)nblk * blockDim.x) {
     float4 d = d4[i], x = x4[i];
-    x.x += d.x; x.y += d.y; x.z += d.z; x.w += d.w;
+    x.x = fmaf(inv, d.x, x.x); x.y = fmaf(inv, d.y, x.y); x.z = fmaf(inv, d.z, x.z); x.w = fmaf(inv, d.w, x.w);
     x4[i] = x;
   }
 }
 
-// out = base + dx_total (out = A.dst, base = A.src or zero): the end of a CG solve.  The CG update pass adds the steps of
+// out = base + dx_total (out = A.dst, base = A.src or zero): the end of a CG solve, which leaves its unit.  The CG update pass adds the steps of
 // an even iteration and of the odd one after it to A.dx together, in the odd one (the first pair without reading it),
 // so that after an odd number of executed iterations the last step a p is still to be added, and A.dx holds nothing
 // before iteration 1.  A.iter: the scheduled iterations; A.slot: the Newton step.
@@ -147,6 +151,7 @@ __global__ void cg_finish_kernel(const KArgs A) {
   const int done = stop < 0 ? A.iter : stop;
   const bool has_dx = done >= 2, has_p = (done & 1) != 0;
   const float a = has_p ? A.sc->step[0] : 0.f;        // the last executed iteration is an even one
+  const float inv = 1.f / A.sc->unit;
   const float4* __restrict__ d4 = (const float4*)A.dx;
   const float4* __restrict__ p4 = (const float4*)A.p;
   const float4* x4 = (const float4*)A.src;
@@ -158,7 +163,7 @@ __global__ void cg_finish_kernel(const KArgs A) {
     if (has_p) {
       d.x = fmaf(a, p.x, d.x); d.y = fmaf(a, p.y, d.y); d.z = fmaf(a, p.z, d.z); d.w = fmaf(a, p.w, d.w);
     }
-    o4[i] = make_float4(x.x + d.x, x.y + d.y, x.z + d.z, x.w + d.w);
+    o4[i] = make_float4(fmaf(inv, d.x, x.x), fmaf(inv, d.y, x.y), fmaf(inv, d.z, x.z), fmaf(inv, d.w, x.w));
   }
 }
 
@@ -787,6 +792,7 @@ cudaError_t q_bcg_iter(nlinv_ctx* c, const float2* x, float alpha, int newton, i
     a.skip = iter;
     a.skip_after = 1;
     a.slot = newton;
+    a.iter = iter;
     c->rec_step = timed ? step : 0;
     return a;
   };
@@ -829,7 +835,6 @@ cudaError_t q_bcg_iter(nlinv_ctx* c, const float2* x, float alpha, int newton, i
   a.pq_part = c->pq_part;
   if ((e = row(c, nlv::ROW_BCG_NORMAL, a)) != cudaSuccess) return e;
   a = cg_args(6);
-  a.iter = iter;
   a.pq_part = c->pq_part;
   a.n_pq = row_geom(c, true).blocks;
   a.brr_part = c->brr_part;
