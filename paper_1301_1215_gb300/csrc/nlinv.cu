@@ -1012,6 +1012,23 @@ cudaError_t mark_running(nlinv_ctx* c, int newton) {
   return e;
 }
 
+// The same for a single frame's passes, with a CG state that none of them takes for a stopped or broken solve: what the
+// passes find otherwise depends on the solve before (the cluster solve writes no partial sums at all; a diverged or
+// finished one leaves NaN or zeros).  Synchronous; the context's stream is idle.
+cudaError_t seed_running(nlinv_ctx* c, int newton) {
+  const nlv::Pair one = {1.f, 0.f};
+  const int n_dd = row_geom(c, false).blocks, n_rr = row_geom(c, true).blocks;
+  const std::vector<nlv::Pair> part(std::max(n_dd, 3 * n_rr), one);
+  Scalars hs{};
+  cudaError_t e = mark_running(c, newton);
+  if (e == cudaSuccess) e = cudaMemcpy(&hs, c->sc, sizeof(hs), cudaMemcpyDeviceToHost);
+  hs.rr_i[0] = hs.rr_i[1] = hs.beta_p = one;
+  if (e == cudaSuccess) e = cudaMemcpy(c->sc, &hs, sizeof(hs), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(c->dd_part, part.data(), n_dd * sizeof(one), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(c->rr_part, part.data(), 3 * n_rr * sizeof(one), cudaMemcpyHostToDevice);
+  return e;
+}
+
 // The six steps that nlinv_profile_cg reports, from the four passes' durations (ms4: column direction, row PSF, column
 // adjoint, row update).  The row update pass does three of them -- the p update with the first axis of W^-1, W^-H with
 // alpha p, and the CG step -- and its duration is divided among them by the vector planes each moves: 2 (r read,
@@ -1690,7 +1707,8 @@ nlinv_status nlinv_profile_cg(nlinv_ctx* c, int reps, double* ms_out) {
   if (!c->have_state) return fail(c, NLINV_EINVAL, "run nlinv_reconstruct before nlinv_profile_cg");
   OwnStream on(c);
   NLV_TRY(on.err, "order after the last call");
-  NLV_TRY(mark_running(c, nlv::kMaxNewton), "mark the solve running");
+  NLV_TRY(cudaStreamSynchronize(c->stream), "synchronize");      // a reconstruction may still be running
+  NLV_TRY(seed_running(c, nlv::kMaxNewton), "mark the solve running");
   cudaEvent_t ev[2];
   for (int i = 0; i < 2; ++i) NLV_TRY(cudaEventCreate(&ev[i]), "event create");
   const float al = (float)c->last_alpha;
@@ -1715,7 +1733,7 @@ nlinv_status nlinv_profile_cg(nlinv_ctx* c, int reps, double* ms_out) {
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
     ms4[k] = ms / reps;
-    if (e == cudaSuccess) e = mark_running(c, nlv::kMaxNewton);
+    if (e == cudaSuccess) e = seed_running(c, nlv::kMaxNewton);
   }
   for (int i = 0; i < 2; ++i) cudaEventDestroy(ev[i]);
   if (e != cudaSuccess) return cuda_fail(c, e, "nlinv_profile_cg");

@@ -1,0 +1,53 @@
+"""nlinv_profile_cg times full passes whatever the solve before left: on small contexts, whose solves run as one cluster
+launch, after a solve that broke down, and again after itself.  A pass that takes the solve for a stopped one leaves early
+and is a fifth to a third shorter; repeated timings of the same pass differ by a few percent."""
+import numpy as np
+import pytest
+
+from tests.helpers import ensure_built, noisy_data
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,J", [(64, 4), (96, 2)])
+@pytest.mark.parametrize("broken", [False, True])
+def test_repeated_profiles_agree(n, J, broken):
+    ensure_built()
+    import torch
+    from paper_1301_1215_gb300.nlinv import Nlinv, NlinvError
+    _, fr, y = noisy_data(n, J, 11, seed=5)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    y = y.astype(np.complex64)
+    with Nlinv(n, J, newton_steps=2, cg_iters=6) as ctx:
+        ctx.reconstruct(t(y), t(fr.mask))
+        ctx.profile_cg(reps=20)                                   # warm-up
+        want = [list(ctx.profile_cg(reps=300).values()) for _ in range(2)]
+        if broken:
+            y[0, 0, 0] = np.nan
+            ctx.reconstruct(t(y), t(fr.mask | 1))
+            with pytest.raises(NlinvError):
+                ctx.wait()
+        else:
+            ctx.reconstruct(t(y), t(fr.mask))
+        got = [list(ctx.profile_cg(reps=300).values()) for _ in range(3)]
+    for k in (1, 2, 3):                                           # column, row, column pass
+        ms = [v[k] for v in want + got]
+        assert max(ms) < 1.15 * min(ms), (k, ms)
+
+
+def test_cluster_contexts_time_the_passes_of_the_others():
+    """16 and 17 coils of 64 x 64: 64 and 68 column blocks, fewer than there are SMs, so that a pass takes as long; the
+    first context solves in one cluster launch, the second in passes."""
+    ensure_built()
+    import torch
+    from paper_1301_1215_gb300.nlinv import Nlinv
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    ms = []
+    for J in (16, 17):
+        _, fr, y = noisy_data(64, J, 11, seed=6)
+        with Nlinv(64, J, newton_steps=2, cg_iters=6) as ctx:
+            ctx.reconstruct(t(y.astype(np.complex64)), t(fr.mask))
+            ctx.profile_cg(reps=20)
+            ms.append(list(ctx.profile_cg(reps=300).values()))
+    for k in (1, 2, 3):
+        assert max(ms[0][k], ms[1][k]) < 1.15 * min(ms[0][k], ms[1][k]), (k, ms)
