@@ -208,9 +208,9 @@ def frame_cg_bytes(n: int, J: int, fov: int):
 
 
 def frame_cg_passes(prof):
-    """Durations of those four passes from nlinv_profile_cg's six entries (it divides the update pass's over three)."""
-    step, col1, psf, col2, out, upd = prof.values()
-    return {"col direction": col1, "row PSF": psf, "col FFT^-1/C^H/FFT": col2, "row update": step + out + upd}
+    """Durations of those four passes from nlinv_profile_cg's six entries (two are 0 for a single frame)."""
+    _, col1, psf, col2, _, upd = prof.values()
+    return {"col direction": col1, "row PSF": psf, "col FFT^-1/C^H/FFT": col2, "row update": upd}
 
 
 def compulsory_bytes(n: int, J: int) -> int:

@@ -290,13 +290,12 @@ NLINV_API nlinv_status nlinv_wait(nlinv_ctx* ctx, double timeout_s);
  * passes of a graph replay do; the row update pass issues its loads of p and r after its wait here, since back to back
  * each launch would read what the one before writes, while in a reconstruction it issues them before).  An iteration is
  * four passes: a column pass [1], a row pass [2], a column pass [3] and a row update pass that does the work of [0], [4]
- * and [5]; its duration is divided among those three in proportion to the vector planes each part moves (2 : 1 : 2), so
- * the six entries add up to the iteration.  (Small frames -- n up to 64, up to 16 coils, fov = n/4 -- run a whole solve as
+ * and [5]; its duration is in [5], and [0] and [4] are 0, so the six entries add up to the iteration.  (Small frames -- n up to 64, up to 16 coils, fov = n/4 -- run a whole solve as
  * one launch instead; these passes are timed all the same.)  ms_out (HOST, 6 doubles) receives the mean duration in milliseconds of:
  *   [0] row pass  p = r + beta p, W^-1 (first axis)   [1] column pass  W^-1, C (products), FFT
  *   [2] row pass  PSF                                  [3] column pass  FFT^-1, C^H (channel products), FFT
  *   [4] row pass  W^-H + alpha p                       [5] CG step  dx += alpha p, r -= alpha q, |r|^2
- * Waits for the stream.  Errors: EINVAL (reps < 1, NULL pointers, no reconstruction yet), ECUDA. */
+ * (a batch has all six, see nlinv_batch_profile_cg).  Waits for the stream.  Errors: EINVAL (reps < 1, NULL pointers, no reconstruction yet), ECUDA. */
 NLINV_API nlinv_status nlinv_profile_cg(nlinv_ctx* ctx, int reps, double* ms_out);
 
 /* Launch shapes picked by nlinv_autotune (one record per timed candidate in its table). */

@@ -1029,20 +1029,6 @@ cudaError_t seed_running(nlinv_ctx* c, int newton) {
   return e;
 }
 
-// The six steps that nlinv_profile_cg reports, from the four passes' durations (ms4: column direction, row PSF, column
-// adjoint, row update).  The row update pass does three of them -- the p update with the first axis of W^-1, W^-H with
-// alpha p, and the CG step -- and its duration is divided among them by the vector planes each moves: 2 (r read,
-// p written, beside its transform's T), 1 (p read, beside its transform's T) and 2 (r written; dx in and out every
-// other iteration).
-void split_profile(const double* ms4, double* out) {
-  out[0] = ms4[3] * 0.4;
-  out[1] = ms4[0];
-  out[2] = ms4[1];
-  out[3] = ms4[2];
-  out[4] = ms4[3] * 0.2;
-  out[5] = ms4[3] * 0.4;
-}
-
 nlinv_status finish_call(nlinv_ctx* c, cudaError_t e, const char* where) {
   if (e != cudaSuccess) return cuda_fail(c, e, where);
   return NLINV_OK;
@@ -1737,7 +1723,8 @@ nlinv_status nlinv_profile_cg(nlinv_ctx* c, int reps, double* ms_out) {
   }
   for (int i = 0; i < 2; ++i) cudaEventDestroy(ev[i]);
   if (e != cudaSuccess) return cuda_fail(c, e, "nlinv_profile_cg");
-  split_profile(ms4, ms_out);
+  const double six[kProfileSteps] = {0.0, ms4[0], ms4[1], ms4[2], 0.0, ms4[3]};   // the update pass does [0] and [4] too
+  std::copy(six, six + kProfileSteps, ms_out);
   return NLINV_OK;
 }
 

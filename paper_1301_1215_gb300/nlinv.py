@@ -263,7 +263,7 @@ class Nlinv:
     def profile_cg(self, reps: int = 20) -> dict:
         """Steady-state CUDA-event duration (ms) of each step of one CG iteration: each pass is launched ``reps``
         times back to back on the state of the last reconstruction (which it advances), as in a graph replay.  The row
-        update pass does three of the steps; its duration is divided among them."""
+        update pass does three of the steps; its duration is under "cg step", the other two are 0."""
         ms = (C.c_double * len(self.CG_KERNELS))()
         self._begin()
         self._check(self._lib.nlinv_profile_cg(self._h, int(reps), ms))

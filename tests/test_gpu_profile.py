@@ -30,6 +30,8 @@ def test_repeated_profiles_agree(n, J, broken):
         else:
             ctx.reconstruct(t(y), t(fr.mask))
         got = [list(ctx.profile_cg(reps=300).values()) for _ in range(3)]
+    for v in want + got:                # the passes of a single frame: nothing but measured durations
+        assert v[0] == 0 and v[4] == 0 and min(v[1], v[2], v[3], v[5]) > 0
     for k in (1, 2, 3):                                           # column, row, column pass
         ms = [v[k] for v in want + got]
         assert max(ms) < 1.15 * min(ms), (k, ms)
