@@ -401,12 +401,12 @@ enum RowMode : int {
 // threads) and loops over its share of rows when they do not fit at once.
 constexpr int kRowMaxThreads = 320;
 constexpr int kRowCtasPerSM = 2;
-// Row passes of batches: the same warps per SM in twice the blocks of half the size.  A block of these passes waits for its
-// loads, then for its exchanges; more and smaller blocks are more often at different points.  64 uneven frames: 288 ms with
-// 320 threads, 281 with 160, 292 with 96 (the launch of one side alone is faster with 320, 1.67 against 1.93 ms an
-// iteration over all sides, but in the batch's graph the sides run side by side).
+// Row passes of batches: where a block's rows divide evenly, the same warps per SM in twice the blocks of half the size.  A
+// block of these passes waits for its loads, then for its exchanges; more and smaller blocks are more often at different
+// points: 2 Newton steps of 15 iterations of 8 frames of 192^2/6 with 8 of 256^2/8 4.81 ms whole, 4.68 divided.  The 13
+// rows of a block of side 384, the one side where they do not divide, would make parts of 5, 5 and 3 rows that hold a
+// block of 5 each: 4 frames of 384^2/10 6.78 ms divided, 6.10 whole; 16 22.9 and 21.4; 8 with 8 of 320^2/8 16.8 and 15.0.
 constexpr int kRowBatchThreads = 160;
-constexpr int kRowBatchCtasPerSM = 4;
 
 template <int MODE> struct RowTraits {
   static constexpr bool both = (MODE == ROW_W_W_IFFT || MODE == ROW_W_P_IFFT);
@@ -1612,7 +1612,7 @@ __device__ __forceinline__ void batch_items(const BatchArgs& B, BatchQueue& q, I
 }
 
 template <int N1, int N2, int MODE, bool STDF = false>
-__global__ void __launch_bounds__(kRowBatchThreads, kRowBatchCtasPerSM) row_pass_batch(const BatchArgs B) {
+__global__ void __launch_bounds__(kRowMaxThreads, kRowCtasPerSM) row_pass_batch(const BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ BatchQueue q;
   using S = Split<N1, N2>;
@@ -1751,6 +1751,12 @@ struct SizeKernels {
   size_t row_smem_tc(int mode, int lanes) const { return tc_offset(row_smem(mode, lanes)) + tc_smem_bytes(lanes * tl); }
   size_t col_smem_tc(int mode, int Wc) const { return tc_offset(col_smem(mode, Wc)) + tc_smem_bytes(col_threads); }
 };
+
+// Parts of a batch's row block of `rows` rows: as many as kRowBatchThreads asks for, if they come out equal.
+inline int batch_row_split(const SizeKernels* k, int rows) {
+  const int sub = (rows * k->tl + kRowBatchThreads - 1) / kRowBatchThreads;
+  return rows % sub == 0 ? sub : 1;
+}
 
 // Launch geometry of a row pass: `blocks` blocks of `lanes` lanes, each taking rows_per_cta rows (and rho_per_cta
 // pixels of the rho plane when the pass has one), so that the rows are split evenly over ctas_per_sm blocks per SM.

@@ -286,6 +286,8 @@ struct nlinv_ctx {
   long launches = 0;
   bool have_state = false;    // a reconstruction has filled the workspace
   int batch_lanes = 0;        // > 0: frame of a batch; row passes use this many lanes and one round per block
+  bool batch_split = true;    // those blocks may be divided (batch_row_split); not under the multi-side kernels, which
+                              // run kRowMaxThreads threads whatever the side
   struct Rec {
     const void* fn;
     int grid, block;
@@ -352,9 +354,8 @@ nlv::RowGrid row_geom(const nlinv_ctx* c, bool with_rho, int arrays = 1) {
     const int rows = c->J * c->N;
     g.rows_per_cta = std::min(c->batch_lanes, rows);
     const int groups = (rows + g.rows_per_cta - 1) / g.rows_per_cta;
-    g.sub = 1;
-    while ((g.rows_per_cta + g.sub - 1) / g.sub * c->k->tl > nlv::kRowBatchThreads) ++g.sub;
-    g.lanes = (g.rows_per_cta + g.sub - 1) / g.sub;
+    g.sub = c->batch_split ? nlv::batch_row_split(c->k, g.rows_per_cta) : 1;
+    g.lanes = g.rows_per_cta / g.sub;
     g.blocks = groups * g.sub;
     g.rho_per_cta = with_rho ? (int)((c->plane + groups - 1) / groups) : 0;
     return g;
@@ -2084,6 +2085,7 @@ nlinv_status nlinv_batch_create(const nlinv_params* params, int nframes, const n
     b->frames.push_back(c);
     // frames of the sides the multi-side kernels cover form one group (side key 0); other sides one group each
     const int key = (b->multi && nlv::multi_side(fp.n)) ? 0 : fp.n;
+    c->batch_split = key != 0;
     size_t g = 0;
     while (g < sides.size() && sides[g] != key) ++g;
     if (g == sides.size()) {

@@ -72,6 +72,9 @@ int main() {
         }
       }
       const int batch_lanes = kRowMaxThreads / k.tl;    // batch frames: fixed lanes
+      const int brows = batch_lanes < nrows ? batch_lanes : nrows, parts = batch_row_split(&k, brows);
+      CHECK(parts >= 1 && brows % parts == 0, "n=%d J=%d batch rows %d in %d parts", N, J, brows, parts);
+      CHECK(parts == 1 || brows / parts * k.tl <= kRowBatchThreads, "n=%d J=%d batch part too large", N, J);
       for (int m = 0; m < NUM_ROW_MODES; ++m)
         CHECK(k.row_smem(m, batch_lanes) <= kSmemLimit, "n=%d batch row mode %d", N, m);
       for (int f : {1, N / 4, N / 2}) {
