@@ -541,7 +541,6 @@ __device__ __forceinline__ void rho_slice(const KArgs& A, int bid, int t, int bd
   const int e_begin = bid * A.rho_per_cta;
   const int e_end = min(e_begin + A.rho_per_cta, plane);
   const float beta = MODE == ROW_BCG_NORMAL ? A.sc->beta_p.h : 0.f;
-  const float unit = MODE == ROW_BCG_NORMAL && A.iter == 0 ? A.sc->unit : 1.f;      // r holds b
   for (int o0 = e_begin + t; o0 < e_end; o0 += 2 * bd) {
     float acc = 0.f;
     float2 a[2], b[2], z[2];
@@ -571,7 +570,9 @@ __device__ __forceinline__ void rho_slice(const KArgs& A, int bid, int t, int bd
       } else if constexpr (RowTraits<MODE>::normal) {
         float2 pv = a[k];
         if constexpr (MODE == ROW_BCG_NORMAL) {
-          pv = make_float2(fmaf(beta, pv.x, unit * b[k].x), fmaf(beta, pv.y, unit * b[k].y));
+          if (A.iter == 0) b[k] = cscale(b[k], A.sc->unit);      // r holds b (the unit held in a register spilled 76 bytes
+                                                                 // a thread at side 320)
+          pv = make_float2(fmaf(beta, pv.x, b[k].x), fmaf(beta, pv.y, b[k].y));
           const_cast<float2*>(A.p)[o] = pv;
         }
         const float2 q = make_float2(fmaf(A.alpha, pv.x, z[k].x), fmaf(A.alpha, pv.y, z[k].y));
