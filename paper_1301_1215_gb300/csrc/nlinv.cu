@@ -152,7 +152,7 @@ __global__ void cg_finish_kernel(const KArgs A) {
   const bool has_dx = done >= 2, has_p = (done & 1) != 0;
   const float a = has_p ? A.sc->step[0] : 0.f;        // the last executed iteration is an even one
   const float inv = 1.f / A.sc->unit;
-  const float4* __restrict__ d4 = (const float4*)A.dx;
+  const float4* d4 = (const float4*)A.dx;        // A.dst itself in the gradient
   const float4* __restrict__ p4 = (const float4*)A.p;
   const float4* x4 = (const float4*)A.src;
   float4* o4 = (float4*)A.dst;
