@@ -46,7 +46,7 @@ template <class Api> struct CallOrder {
         done = {};
         return false;
       }
-      mark(own);
+      last_known = Api::stream_id(own, &last);
     }
     next = s;
     next_set = true;
@@ -61,9 +61,11 @@ template <class Api> struct CallOrder {
   // Orders the call's work, on stream s, after the call before it and sends launches there.
   Error enter(Stream s) {
     run = s;
-    unsigned long long id = 0;
-    if (!done || capturing(s) || (last_known && Api::stream_id(s, &id) && id == last)) return Api::kSuccess;
-    return Api::wait(s, done);
+    run_known = false;
+    // (a chosen stream is not captured; the runtime takes asking a captured one for its id as an error of the capture)
+    if (!done || (s == own && capturing(s))) return Api::kSuccess;
+    run_known = Api::stream_id(s, &run_id);
+    return run_known && last_known && run_id == last ? Api::kSuccess : Api::wait(s, done);
   }
   Error enter_own() {
     next_set = false;
@@ -74,7 +76,8 @@ template <class Api> struct CallOrder {
     Error e = Api::kSuccess;
     if (done && !(run == own && capturing(run))) {
       e = Api::record(done, run);
-      mark(run);
+      last_known = run_known;
+      last = run_id;
     }
     run = own;
     return e;
@@ -88,7 +91,6 @@ template <class Api> struct CallOrder {
   }
 
  private:
-  void mark(Stream s) { last_known = Api::stream_id(s, &last); }
   static bool capturing(Stream s) {
     bool yes = false;
     if (Api::is_capturing(s, &yes) == Api::kSuccess) return yes;
@@ -97,8 +99,9 @@ template <class Api> struct CallOrder {
   }
   Stream next = {};          // the stream of the next call, if next_set
   bool next_set = false;
-  unsigned long long last = 0;     // the id of the stream where `done` was recorded, if it has one
-  bool last_known = false;
+  // the ids of `run` and of the stream where `done` was recorded, if they have one
+  unsigned long long run_id = 0, last = 0;
+  bool run_known = false, last_known = false;
 };
 
 #if defined(__CUDACC__)

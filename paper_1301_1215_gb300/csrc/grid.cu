@@ -184,20 +184,21 @@ nlinv_status nlinv_grid_on(nlinv_gridder* g, void* stream, int ncoils, const nli
   const nlinv_status bad = check_grid(ncoils, samples, y_out, mask_out);
   if (bad != NLINV_OK) return bad;
   const cudaStream_t st = (cudaStream_t)stream;
+  std::lock_guard<std::mutex> hold(g->lock);
+  if (st == g->stream || g->order.choose(st))
+    return run_ordered(g, g->order.take(), ncoils, samples, y_out, mask_out);
+  // not taken: another device is current, or the stream is captured, which orders what it holds by itself
   int dev = -1;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess && dev != g->order.device) return gfail(NLINV_ECUDA, "nlinv_grid_on: another device is current");
   if (e == cudaSuccess) e = cudaStreamIsCapturing(st, &cap);
-  if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) e = gather(g, st, ncoils, samples, y_out, mask_out);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return gfail(NLINV_ECUDA, std::string("nlinv_grid_on: ") + cudaGetErrorString(e));
-  }
-  if (cap != cudaStreamCaptureStatusNone) return NLINV_OK;      // the capture orders what it holds
-  std::lock_guard<std::mutex> hold(g->lock);
-  if (st != g->stream && !g->order.choose(st)) return gfail(NLINV_ECUDA, "nlinv_grid_on: the stream cannot be ordered");
-  return run_ordered(g, g->order.take(), ncoils, samples, y_out, mask_out);
+  if (e == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+    return gfail(NLINV_ECUDA, "nlinv_grid_on: the stream cannot be ordered");
+  if (e == cudaSuccess) e = gather(g, st, ncoils, samples, y_out, mask_out);
+  if (e == cudaSuccess) return NLINV_OK;
+  cudaGetLastError();
+  return gfail(NLINV_ECUDA, std::string("nlinv_grid_on: ") + cudaGetErrorString(e));
 }
 
 nlinv_status nlinv_gridder_join(nlinv_gridder* g) {

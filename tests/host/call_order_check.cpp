@@ -15,6 +15,7 @@ struct Fake {
   static Error is_capturing(Stream s, bool* yes) { *yes = s == capturing; return capture_error; }
   static inline int reborn = -1;         // a handle whose stream was destroyed and created anew
   static bool stream_id(Stream s, unsigned long long* id) {
+    if (s == capturing) log += "id-of-captured ";
     if (s == 9) return false;
     *id = 1000ull + (unsigned long long)s + (s == reborn ? 100000ull : 0ull);
     return true;
