@@ -62,3 +62,30 @@ def test_cluster_and_four_pass_solves_agree_on_the_stop():
     assert all(p >= 0 and q >= 0 and abs(p - q) <= 1 for p, q in zip(a, b)), (a, b)
     assert rel(xb[:17], xa) < 1e-4
     assert np.abs(xb[17]).max() < 1e-6 * np.abs(xa[1:]).max()
+
+
+@pytest.mark.parametrize("n,J", [(64, 4), (96, 2)])
+def test_nan_in_a_solve_is_flagged_and_leaves_nothing_behind(n, J):
+    """NaN data break the first solve down (cluster solve, four passes): no step is taken, nlinv_wait says so once, and the
+    next reconstruction on the context is that of a fresh one."""
+    ensure_built()
+    import torch
+    from paper_1301_1215_gb300 import _lib
+    from paper_1301_1215_gb300.nlinv import Nlinv, NlinvError
+    s, fr, y = noisy_data(n, J, 11, seed=78)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to("cuda")
+    y = y.astype(np.complex64)
+    bad = y.copy()
+    bad[0, 0, 0] = np.nan                                # the centre of k-space, which every spoke samples
+    x0 = synth.initial_guess(n, J).astype(np.complex64)
+    with Nlinv(n, J, newton_steps=3, cg_iters=8) as ctx:
+        want = ctx.reconstruct(t(y), t(fr.mask)).cpu().numpy()
+    with Nlinv(n, J, newton_steps=3, cg_iters=8) as ctx:
+        x = ctx.reconstruct(t(bad), t(fr.mask), t(x0)).cpu().numpy()
+        assert np.array_equal(x, x0)
+        assert ctx.cg_stops() == [0, 0, 0]
+        with pytest.raises(NlinvError) as e:
+            ctx.wait()
+        assert e.value.status == _lib.EBREAKDOWN
+        ctx.wait()
+        assert np.array_equal(ctx.reconstruct(t(y), t(fr.mask)).cpu().numpy(), want)
