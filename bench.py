@@ -337,10 +337,10 @@ def run_ours(args, rank, world, local):
             gr.grid(smp)
         torch.cuda.synchronize()
         gs, ge = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        gs.record(gr.stream)
+        gs.record()                       # grid() runs on the current stream until gr.stream is read
         for _ in range(100):
             gr.grid(smp)
-        ge.record(gr.stream)
+        ge.record()
         torch.cuda.synchronize()
         grid_us = gs.elapsed_time(ge) / 100 * 1e3
     gbytes = smp.numel() * 8 + W.ncoils * W.n * W.n * 8 + W.n * W.n
