@@ -436,9 +436,11 @@ bool row_has_rho(int mode) {
 // passes' resident blocks, and the column passes' where 228 KB holds them all at once.  What is left is L1, which holds the
 // loads in flight.  Four Newton steps of 20 iterations with 164 / 196 / 228 KB: 192^2/13 coils 1450 / 1516 / 1625 us,
 // 320^2/7 2007 / 2016 / 2119, 384^2/22 6227 / 5334 / 5629, 512^2/3 2442 / 2432 / 2673, 320^2/22 4201 / 3718 / 3611; 7 x 30
-// iterations, 384^2/10 7240 / 7302 / 6526, 512^2/16 22.2 / 22.7 / 18.6 ms.  Side 256 does not go below 196: reconstruction
-// and gradient, 9 coils, 3242 / 3172 / 3158, frame with 9 coils and a wide field of view 2604 / 2563 / 2636.  Sides up to
-// 128 gain nothing (128^2/3 1027 / 1011 / 1019, /22 1230 / 1281 / 1240) and keep the largest, as do the tensor-core passes.
+// iterations, 384^2/10 7240 / 7302 / 6526, 512^2/16 22.2 / 22.7 / 18.6 ms.  Two lines rest on measurements without a mechanism behind them, both
+// within a few percent either way (3 Newton steps of 20): side 256 does not go below 196 -- 164 / 196 KB: 4 coils 1110 / 1082,
+// gradient with 9 1444 / 1391, normal operator with 16 and half-width 100 37.2 / 34.3, but 12 coils 1313 / 1379, 24 1927 /
+// 2080 --, and sides up to 128 keep the largest -- 164 / 228 KB: 128^2/3 726 / 710, /6 714 / 712, /12 737 / 747, /22 821 /
+// 832, 96^2/8 646 / 647 --, as do the tensor-core passes.
 void choose_carveout(nlinv_ctx* c) {
   c->carveout = 100;
   if (c->tc || c->N <= 128) return;
