@@ -119,6 +119,10 @@ struct CudaOrderApi {
   }
   static bool stream_id(Stream s, unsigned long long* id) {
     if (s == cudaStreamPerThread) return false;
+    if (s == nullptr || s == cudaStreamLegacy) {      // one stream that lasts: no need to ask (0.2 us)
+      *id = ~0ull;
+      return true;
+    }
     if (cudaStreamGetId(s, id) == cudaSuccess) return true;
     cudaGetLastError();
     return false;

@@ -1,12 +1,22 @@
 """nlinv_profile_cg times full passes whatever the solve before left: on small contexts, whose solves run as one cluster
 launch, after a solve that broke down, and again after itself.  A pass that takes the solve for a stopped one leaves early
-and is a fifth to a third shorter; repeated timings of the same pass differ by a few percent."""
+and is a fifth to a third shorter; repeated timings of the same pass differ by a few percent, and a measurement that
+something else on the machine disturbed is taken again, twice at most."""
 import numpy as np
 import pytest
 
 from tests.helpers import ensure_built, noisy_data
 
 pytestmark = pytest.mark.gpu
+
+
+def _agree(measure):
+    """measure() returns timings of the column, row and column pass by several calls; those of a pass agree within 15 %."""
+    for _ in range(3):
+        calls = measure()
+        if all(max(v[k] for v in calls) < 1.15 * min(v[k] for v in calls) for k in (1, 2, 3)):
+            return
+    pytest.fail(f"timings of one pass differ: {calls}")
 
 
 @pytest.mark.parametrize("n,J", [(64, 4), (96, 2)])
@@ -18,23 +28,22 @@ def test_repeated_profiles_agree(n, J, broken):
     _, fr, y = noisy_data(n, J, 11, seed=5)
     t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
     y = y.astype(np.complex64)
+    bad = y.copy()
+    bad[0, 0, 0] = np.nan
     with Nlinv(n, J, newton_steps=2, cg_iters=6) as ctx:
-        ctx.reconstruct(t(y), t(fr.mask))
-        ctx.profile_cg(reps=20)                                   # warm-up
-        want = [list(ctx.profile_cg(reps=300).values()) for _ in range(2)]
-        if broken:
-            y[0, 0, 0] = np.nan
-            ctx.reconstruct(t(y), t(fr.mask | 1))
-            with pytest.raises(NlinvError):
-                ctx.wait()
-        else:
+        def measure():
             ctx.reconstruct(t(y), t(fr.mask))
-        got = [list(ctx.profile_cg(reps=300).values()) for _ in range(3)]
-    for v in want + got:                # the passes of a single frame: nothing but measured durations
-        assert v[0] == 0 and v[4] == 0 and min(v[1], v[2], v[3], v[5]) > 0
-    for k in (1, 2, 3):                                           # column, row, column pass
-        ms = [v[k] for v in want + got]
-        assert max(ms) < 1.15 * min(ms), (k, ms)
+            ctx.profile_cg(reps=20)                                   # warm-up
+            calls = [list(ctx.profile_cg(reps=300).values()) for _ in range(2)]
+            ctx.reconstruct(t(bad if broken else y), t(fr.mask | 1))
+            if broken:
+                with pytest.raises(NlinvError):
+                    ctx.wait()
+            calls += [list(ctx.profile_cg(reps=300).values()) for _ in range(3)]
+            for v in calls:             # the passes of a single frame: nothing but measured durations
+                assert v[0] == 0 and v[4] == 0 and min(v[1], v[2], v[3], v[5]) > 0
+            return calls
+        _agree(measure)
 
 
 def test_cluster_contexts_time_the_passes_of_the_others():
@@ -44,12 +53,14 @@ def test_cluster_contexts_time_the_passes_of_the_others():
     import torch
     from paper_1301_1215_gb300.nlinv import Nlinv
     t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
-    ms = []
-    for J in (16, 17):
-        _, fr, y = noisy_data(64, J, 11, seed=6)
-        with Nlinv(64, J, newton_steps=2, cg_iters=6) as ctx:
-            ctx.reconstruct(t(y.astype(np.complex64)), t(fr.mask))
-            ctx.profile_cg(reps=20)
-            ms.append(list(ctx.profile_cg(reps=300).values()))
-    for k in (1, 2, 3):
-        assert max(ms[0][k], ms[1][k]) < 1.15 * min(ms[0][k], ms[1][k]), (k, ms)
+
+    def measure():
+        calls = []
+        for J in (16, 17):
+            _, fr, y = noisy_data(64, J, 11, seed=6)
+            with Nlinv(64, J, newton_steps=2, cg_iters=6) as ctx:
+                ctx.reconstruct(t(y.astype(np.complex64)), t(fr.mask))
+                ctx.profile_cg(reps=20)
+                calls.append(list(ctx.profile_cg(reps=300).values()))
+        return calls
+    _agree(measure)
