@@ -73,7 +73,8 @@ class Nlinv:
     def stream(self) -> "torch.cuda.Stream":
         """The context's CUDA stream, ordered after the context's last call; later calls run on it."""
         if not self._stream_seen:
-            self._check(self._lib.nlinv_join(self._h))
+            if self._h:                      # closed: nothing is queued any more
+                self._check(self._lib.nlinv_join(self._h))
             self._stream_seen = True
         return self._stream
 
@@ -444,7 +445,8 @@ class Gridder:
         """The gridder's CUDA stream, ordered after its earlier calls and the current stream; later calls run on it (until
         it is read, calls run on the current stream)."""
         if not self._stream_seen:
-            _lib.check(self._lib.nlinv_gridder_join(self._h))
+            if self._h:                      # closed: nothing is queued any more
+                _lib.check(self._lib.nlinv_gridder_join(self._h))
             self._stream.wait_stream(torch.cuda.current_stream(self.device))
             self._stream_seen = True
         return self._stream

@@ -161,3 +161,13 @@ def test_gridders_stream_follows_calls_on_other_streams(env):
         assert not own.query()
         own.synchronize()
         assert side.query()
+
+
+def test_the_stream_of_a_closed_context_can_still_be_read(env):
+    torch, xs, mask, want = env
+    from paper_1301_1215_gb300.nlinv import Gridder, Nlinv
+    with Nlinv(N, J) as ctx, Gridder(N, _spokes()) as gr:
+        y = ctx.forward(xs[0], mask)
+    ctx.stream.synchronize()
+    gr.stream.synchronize()
+    assert torch.equal(y.cpu(), want[0])
